@@ -163,6 +163,29 @@ struct mj_ctx {
   uint64_t fixed_N = 0;
   Buf in_bytes, in_offsets;  // staging for mj_join_host
   uint64_t n_part = 0, n_cand = 0, n_out = 0;
+  // pairs listed for verification in cand_i/cand_j: all candidates, or (plain
+  // joins by strings) those the lower bounds leave, in any order
+  uint64_t n_list = 0;
+  bool list_bounded = false;      // made under the lower bounds of mj_pairs.cu
+  // plain joins by strings (mj_pairs.cu): lengths and ids by rank, ranks by
+  // id, windows by rank, first records by string, sorted records, windows,
+  // signatures, counters
+  Buf rk_len, rk_len_alt, rk_sid, rk_sid_alt, rk_of, rk_hi, rk_first, rk_delta, rk_scan, rk_len_rank;
+  Buf rk_a, rk_b, rk_skr, rk_win, rk_sig1, rk_sig2, rk_cnt, rk_list;
+  Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
+  bool by_strings = false;        // this call builds the rank tables
+  bool rk_alt = false;            // rk_len_alt / rk_sid_alt hold the sorted strings
+  uint32_t rk_widest = 0;
+  uint32_t rep_first[65] = {0};   // first record of every repetition
+  uint64_t code_counts[256] = {0};   // input symbols by rank code
+  // A plain join by strings lists no candidates: mj_candidates_copy makes them
+  // on demand from the join's records, kept in cand_recs once mj_partition
+  // replaces recs.
+  bool cand_on_demand = false, cand_recs_kept = false;
+  Derived cand_d;
+  uint64_t cand_n_part = 0;
+  uint32_t cand_n_str = 0;
+  Buf cand_recs;
   // bit-planes written by the partition kernel for the verifier
   mj_verify_config vcfg{MJ_VERIFY_KERNEL_AUTO, 0, 0, 0};
   // autotuned kernel per length bucket
@@ -172,8 +195,8 @@ struct mj_ctx {
   Buf branges;   // bucket counts [32] then ranges [64]
   // CUDA graph of the plain verification stage
   cudaGraphExec_t graph_exec = nullptr;
-  uint64_t graph_sig[23] = {};
-  uint64_t last_sig[23] = {};
+  uint64_t graph_sig[27] = {};
+  uint64_t last_sig[27] = {};
   uint64_t graph_launches = 0;
   // learned first-pass band: parameters P, Adam moments M and V, gradient G, loss
   Buf band;
@@ -262,7 +285,9 @@ void begin_call(mj_ctx* c, bool timing) {
   c->geo_valid = false;
   c->planes_ready = false;
   c->codes_ready = false;
+  c->planes_pw = c->planes_gw = 0;
   c->work_started = false;
+  c->by_strings = c->list_bounded = false;
   c->timing = timing;
   for (bool& u : c->sec_used) u = false;
   c->launches_at_start = launch_count();
@@ -314,6 +339,9 @@ int derive(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t
       if (c->h_small[b]) d.rank[b] = (uint8_t)sigma++;
     }
   }
+  for (int b = 0; b < 256; ++b) c->code_counts[b] = 0;
+  for (int b = 0; b < 256; ++b)
+    if (c->h_small[b]) c->code_counts[d.rank[b]] = c->h_small[b];
   d.sigma = sigma;
   d.bits = 1;
   while ((1u << d.bits) < sigma) ++d.bits;
@@ -421,8 +449,11 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
                                      c->scan_tmp.p, total, s));
     MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small, total, 4, cudaMemcpyDeviceToHost, s));
     MJ_CUDA_TRY(cudaMemcpyAsync((char*)c->h_small + 8, c->dev_flags.p, 4, cudaMemcpyDeviceToHost, s));
+    if (c->by_strings)
+      MJ_CUDA_TRY(cudaMemcpyAsync((char*)c->h_small + 16, c->rk_cnt.p, 4, cudaMemcpyDeviceToHost, s));
     MJ_CUDA_TRY(cudaStreamSynchronize(s));
     const uint32_t n_anchor = *(uint32_t*)c->h_small;
+    if (c->by_strings) c->rk_widest = *(uint32_t*)((char*)c->h_small + 16);
     c->stats.device_flags |= *(uint32_t*)((char*)c->h_small + 8);
     if (c->stats.device_flags) return MJ_ERR_DEVICE;
     if (n_total + n_anchor >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;   // record indexes are 32-bit
@@ -432,8 +463,14 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
                                     c->tile_first.as<uint32_t>(), key_base_for(d.seed),
                                     c->recs.as<PRec>() + n_total, s));
     tstop(c, 1, s);
+    if (c->by_strings) {
+      MJ_TRY(launch_string_first(d_offsets, n, nbytes, c->bitmap.as<uint32_t>(), c->tile_off.as<uint32_t>(), n_anchor,
+                                 (uint32_t)n_total, c->rk_first.as<uint32_t>() + (uint64_t)k * (n + 1), s));
+      c->rep_first[k] = (uint32_t)n_total;
+    }
     n_total += n_anchor;
   }
+  c->rep_first[R] = (uint32_t)n_total;
   c->n_part = n_total;
   c->stats.n_partitions = n_total;
   return MJ_OK;
@@ -608,6 +645,162 @@ int candidates(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint
   return MJ_OK;
 }
 
+// Whether the lower bounds can exceed K: unrelated strings of length N differ
+// by about 0.8 sqrt(2 N / 256) counts in each of the second level's 256
+// buckets, 18 sqrt(N) in all, and the bound needs more than 2 q K.
+bool bounds_reach(uint64_t N, uint32_t sigma, uint32_t K) {
+  const double q = (double)signature_grams(sigma, 256);
+  return 2.0 * q * K < 18.0 * sqrt((double)N);
+}
+
+constexpr uint64_t kLenRankMax = 1u << 22;   // longest string up to which ranks are found by length from a table
+
+// Rank tables of a plain join by strings (before its partition step, whose
+// readback also returns the widest window).
+int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s) {
+  const size_t b = (size_t)n * 4 + 16;
+  for (Buf* x : {&c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi}) MJ_TRY(x->reserve(b, s));
+  MJ_TRY(c->rk_cnt.reserve(128, s));
+  MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(n), s));
+  const bool by_len = c->d.N <= kLenRankMax;
+  if (by_len) {
+    MJ_TRY(c->rk_len_rank.reserve(((size_t)c->d.N + 1) * 4, s));
+    if (c->fixed_alpha)   // N may be above this input's longest
+      MJ_CUDA_TRY(cudaMemsetAsync(c->rk_len_rank.p, 0xff, ((size_t)c->d.N + 1) * 4, s));
+  }
+  MJ_TRY(c->rk_first.reserve((size_t)c->d.repeats * ((size_t)n + 1) * 4, s));
+  return launch_string_ranks(d_offsets, n, c->d.K, bits_for(c->d.N), c->rk_len.as<uint32_t>(),
+                             c->rk_len_alt.as<uint32_t>(), c->rk_sid.as<uint32_t>(), c->rk_sid_alt.as<uint32_t>(),
+                             c->sort_tmp.p, c->rk_of.as<uint32_t>(), c->rk_hi.as<uint32_t>(),
+                             by_len ? c->rk_len_rank.as<uint32_t>() : nullptr, c->rk_cnt.as<unsigned int>(), &c->rk_alt,
+                             s);
+}
+
+// a5-a7 by strings (after partition and string_ranks): the candidates counted,
+// those that may be within K listed in c->cand_i/j (n_list of them).
+int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s) {
+  const Derived& d = c->d;
+  const uint32_t nr = (uint32_t)c->n_part;
+  c->n_cand = c->n_list = 0;
+  c->cand_on_demand = true;
+  c->cand_recs_kept = false;
+  c->cand_d = d;
+  c->cand_n_part = nr;
+  c->cand_n_str = n;
+  if (nr == 0) return MJ_OK;
+  // position buckets of width W >= K / 2 in at most 8 of the 32 key bits, so that
+  // at least 24 hash bits keep most (len, key) classes apart (the visits
+  // compare both)
+  uint32_t W = d.K / 2 + (d.K & 1u);
+  if (d.N / W > 255) W = (uint32_t)(d.N / 255 + 1);
+  const int pb_bits = bits_for(d.N / W);
+  const uint32_t* sid_of = c->rk_alt ? c->rk_sid_alt.as<uint32_t>() : c->rk_sid.as<uint32_t>();
+  const uint32_t* rlen = c->rk_alt ? c->rk_len_alt.as<uint32_t>() : c->rk_len.as<uint32_t>();
+  const uint32_t* rank_of = c->rk_of.as<uint32_t>();
+  unsigned long long* cnt = c->rk_cnt.as<unsigned long long>();   // 0 widest, 1 visits, 2 listed, 3-5 totals, 6 listed after the second bound
+  MJ_TRY(c->keys.reserve((size_t)nr * 4, s));
+  MJ_TRY(c->keys_alt.reserve((size_t)nr * 4, s));
+  c->geo_valid = false;   // c->idx is reused by the record sort
+  MJ_TRY(c->idx.reserve((size_t)nr * 4, s));
+  MJ_TRY(c->idx_alt.reserve((size_t)nr * 4, s));
+  MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(nr), s));
+  MJ_TRY(c->rk_delta.reserve((size_t)d.repeats * ((size_t)n + 1) * 4, s));
+  MJ_TRY(c->rk_scan.reserve((size_t)n * 4 + 16, s));
+  MJ_TRY(c->scan_tmp.reserve(scan_temp_bytes(n), s));
+  MJ_TRY(c->rk_a.reserve((size_t)nr * 16, s));
+  const int rb = visit_rank_bits(d.N, n);
+  if (!rb) MJ_TRY(c->rk_b.reserve((size_t)nr * 8, s));
+  MJ_TRY(c->rk_skr.reserve((size_t)nr * 8, s));
+  MJ_TRY(c->rk_win.reserve((size_t)nr * 32, s));
+  MJ_TRY(c->rk_sig1.reserve(sig1_bytes(n), s));
+  MJ_TRY(c->rk_sig2.reserve(sig2_bytes(n), s));
+  tstart(c, 2, s);
+  MJ_TRY(launch_rank_order(c->rk_first.as<uint32_t>(), sid_of, rank_of, n, d.repeats, c->rk_scan.as<uint32_t>(),
+                           c->rk_delta.as<uint32_t>(), c->scan_tmp.p, s));
+  for (uint32_t k = 0; k < d.repeats; ++k)
+    MJ_TRY(launch_rank_keys(c->recs.as<PRec>(), c->rep_first[k], c->rep_first[k + 1],
+                            c->rk_delta.as<uint32_t>() + (uint64_t)k * (n + 1), pb_bits, W, c->keys.as<uint32_t>(),
+                            c->idx.as<uint32_t>(), s));
+  bool alt = false;
+  MJ_TRY(radix_sort_u32(c->keys.as<uint32_t>(), c->keys_alt.as<uint32_t>(), c->idx.as<uint32_t>(),
+                        c->idx_alt.as<uint32_t>(), nr, 0, 32, c->sort_tmp.p, &alt, s));
+  const RankTables rt{c->rk_hi.as<uint32_t>(), rlen, d.N <= kLenRankMax ? c->rk_len_rank.as<uint32_t>() : nullptr,
+                      (uint32_t)d.N, n};
+  MJ_TRY(launch_rank_windows(alt ? c->idx_alt.as<uint32_t>() : c->idx.as<uint32_t>(),
+                             alt ? c->keys_alt.as<uint32_t>() : c->keys.as<uint32_t>(), nr, c->recs.as<PRec>(), rank_of,
+                             rt, d.K, W, pb_bits, rb, c->rk_a.as<uint4>(), c->rk_b.as<uint2>(),
+                             c->rk_skr.as<uint64_t>(), c->rk_win.as<uint4>(), cnt + 1, s));
+  tstop(c, 2, s);
+  tstart(c, 4, s);
+  // The lower bounds read every input byte once; without them a candidate
+  // costs a dynamic program.  They pay when the windows hold more than one
+  // record per 32 bytes of input.
+  const uint64_t min_visits = bounds_reach(d.N, d.sigma, d.K) ? c->stats.n_bytes / 32 : ~0ull;
+  const SigShape g = signature_shape(d.sigma, c->code_counts);
+  if (min_visits != ~0ull)
+    MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_visits, c->rk_sig1.as<uint4>(),
+                             c->rk_sig2.as<uint32_t>(), s));
+  PairArgs a;
+  a.recs = c->recs.as<PRec>();
+  a.first = c->rk_first.as<uint32_t>();
+  a.win = c->rk_win.as<uint4>();
+  a.A = c->rk_a.as<uint4>();
+  a.B = c->rk_b.as<uint2>();
+  a.sid_of = sid_of;
+  a.rlen = rlen;
+  a.hi = c->rk_hi.as<uint32_t>();
+  a.sig1 = c->rk_sig1.as<uint4>();
+  a.visits = cnt + 1;
+  a.min_visits = min_visits;
+  a.n = n;
+  a.reps = d.repeats;
+  a.K = d.K;
+  a.q1 = g.q1;
+  a.rb = rb;
+  a.out_count = cnt + 2;
+  a.totals = cnt + 3;
+  ListArgs l;
+  l.in_count = a.out_count;
+  l.sig2 = c->rk_sig2.as<uint4>();
+  l.sid_of = sid_of;
+  l.rlen = rlen;
+  l.visits = a.visits;
+  l.min_visits = min_visits;
+  l.K = d.K;
+  l.q2 = g.q2;
+  l.out_count = cnt + 6;
+  // room for what passes the bounds: a first guess, at least every candidate
+  // when the bounds are not used; a longer list is counted and made again
+  uint64_t cap1 = c->stats.n_bytes + (1u << 16), cap2 = c->stats.n_bytes / 8 + (1u << 16);
+  for (int tries = 0;; ++tries) {
+    MJ_TRY(c->rk_list.reserve(cap1 * 8, s));
+    MJ_TRY(c->cand_i.reserve(cap2 * 4 + 16, s));
+    MJ_TRY(c->cand_j.reserve(cap2 * 4 + 16, s));
+    a.cap = l.in_cap = cap1;
+    a.out = c->rk_list.as<uint2>();
+    l.in = a.out;
+    l.cap = cap2;
+    l.out_i = c->cand_i.as<uint32_t>();
+    l.out_j = c->cand_j.as<uint32_t>();
+    MJ_TRY(launch_string_pairs(a, c->rk_widest, s));
+    MJ_TRY(launch_listed_pairs(l, s));
+    MJ_TRY(readback(c, cnt + 2, 40, s));
+    if (c->h_small[1] >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;   // raw pairs, as on the general path
+    if (c->h_small[0] <= cap1 && c->h_small[4] <= cap2) break;
+    if (tries > 1) return MJ_ERR_DEVICE;   // both lists were counted in full
+    cap1 = std::max<uint64_t>(cap1, c->h_small[0]);
+    cap2 = std::max<uint64_t>(cap2, std::min<uint64_t>(c->h_small[4], c->h_small[0]));
+  }
+  tstop(c, 4, s);
+  c->n_list = c->h_small[4];
+  c->list_bounded = true;
+  c->stats.n_raw_pairs = c->h_small[1];
+  c->n_cand = c->h_small[2];
+  c->stats.n_candidates = c->n_cand;
+  c->stats.band_cells = c->h_small[3];
+  return MJ_OK;
+}
+
 // a8 on arbitrary pairs (rank codes from c->d).
 // Device flags and verification counters cleared for this call (once), on s.
 int verify_prep(mj_ctx* c, cudaStream_t s) {
@@ -623,31 +816,38 @@ int verify_prep(mj_ctx* c, cudaStream_t s) {
   return MJ_OK;
 }
 
+// Bit-planes (with guards for bands up to kmax) and rank codes of the input,
+// unless this call has made them.
+int ensure_planes(mj_ctx* c, const uint8_t* d_bytes, uint32_t kmax, cudaStream_t s) {
+  const uint32_t GW = plane_guard_words(kmax);
+  if (c->planes_ready && c->planes_gw >= GW) return MJ_OK;
+  const uint64_t nbytes = c->stats.n_bytes, PW = (nbytes + 31) / 32 + 2 * (uint64_t)GW;
+  MJ_TRY(c->planes.reserve(PW * c->d.bits * 4, s));
+  RankTable rt;
+  memcpy(rt.r, c->d.rank, 256);
+  MJ_TRY(c->codes.reserve(nbytes + 64, s));
+  tstart(c, 5, s);
+  MJ_TRY(launch_build_planes(d_bytes, nbytes, rt, c->d.bits, c->planes.as<uint32_t>(), PW, GW, c->codes.as<uint8_t>(),
+                             s));
+  tstop(c, 5, s);
+  c->planes_ready = c->codes_ready = true;
+  c->planes_pw = PW;
+  c->planes_gw = GW;
+  return MJ_OK;
+}
+
 int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const uint32_t* d_i, const uint32_t* d_j,
-           const uint32_t* d_k, uint64_t m, uint32_t K, uint32_t kmax, uint32_t* d_ed, bool count_cells,
-           cudaStream_t s, const uint32_t* order = nullptr, const uint32_t* skip_kband = nullptr,
+           const uint32_t* d_k, uint64_t m, uint32_t K, uint32_t kmax, uint32_t* d_ed, cudaStream_t s,
+           const uint32_t* order = nullptr, const uint32_t* skip_kband = nullptr,
            const uint32_t* range_lo = nullptr, const uint32_t* range_hi = nullptr, int kernel = -1, int lanes = -1,
            unsigned long long* next = nullptr, bool prep = true, const uint32_t* first_ed = nullptr) {
   const Derived& d = c->d;
   if (m == 0) return MJ_OK;
   if (kmax >= (1u << 16)) return MJ_ERR_UNSUPPORTED;
   const uint64_t nbytes = c->stats.n_bytes;
-  uint32_t GW = plane_guard_words(kmax);
-  uint64_t PW = (nbytes + 31) / 32 + 2 * (uint64_t)GW;
-  if (c->planes_ready && c->planes_gw >= GW) {
-    GW = c->planes_gw;   // written by the partition kernel of this call
-    PW = c->planes_pw;
-  } else {
-    MJ_TRY(c->planes.reserve(PW * d.bits * 4, s));
-    RankTable rt;
-    memcpy(rt.r, d.rank, 256);
-    MJ_TRY(c->codes.reserve(nbytes + 64, s));
-    tstart(c, 5, s);
-    MJ_TRY(launch_build_planes(d_bytes, nbytes, rt, d.bits, c->planes.as<uint32_t>(), PW, GW,
-                               c->codes.as<uint8_t>(), s));
-    tstop(c, 5, s);
-    c->codes_ready = true;
-  }
+  MJ_TRY(ensure_planes(c, d_bytes, kmax, s));
+  const uint32_t GW = c->planes_gw;
+  const uint64_t PW = c->planes_pw;
   if (prep) MJ_TRY(verify_prep(c, s));
   VerifyArgs a;
   a.planes = c->planes.as<uint32_t>();
@@ -667,7 +867,6 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
   a.K = K;
   a.m = m;
   a.ed = d_ed;
-  a.cells = count_cells ? c->small.as<unsigned long long>() : nullptr;
   a.work = c->small.as<unsigned long long>() + 2;
   a.dev_flags = c->dev_flags.as<uint32_t>();
   if (order && order == c->idx.as<uint32_t>() && c->geo_valid) a.pair_geo = c->geo.as<uint4>();
@@ -694,18 +893,57 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
 // lengths into c->idx), with the pairs' floor(log2) length buckets: counts in
 // branges words [0, 32), [start, end) ranges in words [32, 96).
 constexpr size_t kOrderScratchAt = 128;   // words of branges before the ordering scratch
+constexpr size_t kOrderKeptAt = 100;      // word of branges with the number of pairs in the order
+
+// The lower bounds (mj_pairs.cu) on a list of m pairs cost a pass over the
+// input; they pay from one pair per 16 input bytes on (1-2 ps per byte against
+// 100-300 ps for the dynamic program of an unrelated pair).
+// A list that was made under the bounds needs them no more, and a band that
+// the verifier refuses must leave the results unwritten.
+bool bounds_pay(const mj_ctx* c, uint64_t m, uint32_t kmax) {
+  if (!bounds_reach(c->d.N, c->d.sigma, kmax)) return false;
+  if (c->list_bounded || m <= c->stats.n_bytes / 16) return false;
+  if (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned)
+    return verify_supported(kmax, (int)c->vcfg.kernel, (int)c->vcfg.lanes);
+  for (int b = 0; b < kLenBuckets; ++b)
+    if (!verify_supported(kmax, (int)c->tuned_kernel[b], (int)c->tuned_lanes[b])) return false;
+  return true;
+}
+
+int bounds_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
+  MJ_TRY(c->rk_sig1.reserve(sig1_bytes((uint32_t)c->stats.n_strings), s));
+  MJ_TRY(c->rk_sig2.reserve(sig2_bytes((uint32_t)c->stats.n_strings), s));
+  return c->rejected.reserve(m, s);
+}
+
+// c->rejected[t] (and ed[t] = k + 1) for the pairs beyond their lower bounds;
+// needs the input's rank codes and bounds_buffers.
+int pair_bounds(mj_ctx* c, const int64_t* d_offsets, const uint32_t* ci, const uint32_t* cj, const uint32_t* pk,
+                uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
+  if (!c->codes_ready || !c->rk_sig1.p || !c->rk_sig2.p || !c->rejected.p) return MJ_ERR_STATE;
+  const uint32_t n = (uint32_t)c->stats.n_strings;
+  const SigShape g = signature_shape(c->d.sigma, c->code_counts);
+  MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, nullptr, n, g, nullptr, 0, c->rk_sig1.as<uint4>(),
+                           c->rk_sig2.as<uint32_t>(), s));
+  return launch_pair_bounds(ci, cj, pk, K, m, n, g, c->rk_sig1.as<uint4>(), c->rk_sig2.as<uint4>(),
+                            c->rejected.as<uint8_t>(), ed, s);
+}
 
 // The pairs' K-band cells are summed into small word 9 on the way.
+// With rejected, those pairs are left out and *kept (a device word) is the
+// number in the order.
 int pair_order(mj_ctx* c, const uint32_t* ci, const uint32_t* cj, const int64_t* d_offsets, uint64_t m,
-               const uint32_t** order, cudaStream_t s) {
+               const uint8_t* rejected, const uint32_t** order, const uint32_t** kept, cudaStream_t s) {
   if (!c->small.p || !c->branges.p || !c->idx.p || !c->geo.p || !c->strgeo.p) return MJ_ERR_STATE;   // order_buffers first
   uint32_t* counts = c->branges.as<uint32_t>();
   tstart(c, 8, s);
-  MJ_TRY(launch_length_order(ci, cj, d_offsets, (uint32_t)c->stats.n_strings, m, c->d.K, counts + kOrderScratchAt,
-                             c->strgeo.as<uint2>(), c->idx.as<uint32_t>(), c->geo.as<uint4>(), counts,
-                             counts + kLenBuckets, c->small.as<unsigned long long>() + 9, s));
+  MJ_TRY(launch_length_order(ci, cj, d_offsets, (uint32_t)c->stats.n_strings, m, c->d.K, rejected, counts + kOrderKeptAt,
+                             counts + kOrderScratchAt, c->strgeo.as<uint2>(), c->idx.as<uint32_t>(),
+                             c->geo.as<uint4>(), counts, counts + kLenBuckets, c->small.as<unsigned long long>() + 9,
+                             s));
   tstop(c, 8, s);
   *order = c->idx.as<uint32_t>();
+  if (kept) *kept = rejected ? counts + kOrderKeptAt : nullptr;
   c->geo_valid = true;   // c->geo matches the order in c->idx
   return MJ_OK;
 }
@@ -723,15 +961,20 @@ int order_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
 // context's kernel choice says (TUNED: per length bucket, batched).
 int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const uint32_t* ci,
                    const uint32_t* cj, uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
-  const uint32_t* order;
-  MJ_TRY(pair_order(c, ci, cj, d_offsets, m, &order, s));
+  const uint32_t *order, *kept;
+  const bool bounds = bounds_pay(c, m, K);
+  if (bounds) {
+    MJ_TRY(ensure_planes(c, d_bytes, K, s));
+    MJ_TRY(pair_bounds(c, d_offsets, ci, cj, nullptr, m, K, ed, s));
+  }
+  MJ_TRY(pair_order(c, ci, cj, d_offsets, m, bounds ? c->rejected.as<uint8_t>() : nullptr, &order, &kept, s));
   if (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned)
-    return verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, false, s, order);
+    return verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, nullptr, kept);
   uint32_t* counts = c->branges.as<uint32_t>();
   uint32_t* ranges = counts + kLenBuckets;
   if (c->vcfg.batching == 1) {
     for (int b = kLenBuckets - 1; b >= 0; --b)
-      MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, false, s, order, nullptr, ranges + 2 * b,
+      MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, ranges + 2 * b,
                     ranges + 2 * b + 1, (int)c->tuned_kernel[b], (int)c->tuned_lanes[b]));
     return MJ_OK;
   }
@@ -740,7 +983,7 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
   while (b >= 0) {
     int e = b;
     while (e - 1 >= 0 && c->tuned_kernel[e - 1] == c->tuned_kernel[b] && c->tuned_lanes[e - 1] == c->tuned_lanes[b]) --e;
-    MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, false, s, order, nullptr, ranges + 2 * b,
+    MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, ranges + 2 * b,
                   ranges + 2 * e + 1, (int)c->tuned_kernel[b], (int)c->tuned_lanes[b]));
     b = e - 1;
   }
@@ -754,6 +997,7 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
 int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const uint32_t* ci,
                          const uint32_t* cj, uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
   MJ_TRY(order_buffers(c, m, s));
+  if (bounds_pay(c, m, K)) MJ_TRY(bounds_buffers(c, m, s));
   // capture needs a stream of its own: the legacy and per-thread default
   // streams run the stage uncaptured
   const bool capturable = s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread;
@@ -763,13 +1007,14 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
     for (int b = 0; b < kLenBuckets; ++b) plan = plan * 1000003u + c->tuned_kernel[b] * 64u + c->tuned_lanes[b];
   }
   // everything the captured launches read as a parameter: buffers, sizes, plan
-  const uint64_t sig[23] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
+  const uint64_t sig[27] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
                             (uint64_t)ed, (uint64_t)c->planes.p, c->planes_pw, c->d.bits, plan,
                             (uint64_t)c->small.p, (uint64_t)c->idx.p, (uint64_t)c->branges.p,
                             (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0, (uint64_t)c->geo.p,
                             c->stats.n_bytes, c->stats.n_strings, c->planes_gw,
                             (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
-                            (uint64_t)c->rank_dev.p};
+                            (uint64_t)c->rank_dev.p, (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p,
+                            (uint64_t)c->rejected.p, bounds_pay(c, m, K) ? 1ull : 0ull};
   if (c->graph_exec && memcmp(sig, c->graph_sig, sizeof(sig)) == 0) {
     MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
     mark_graph_sections(c);
@@ -818,7 +1063,7 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
 // words (narrower than band K's), then band K for every pair not settled.
 int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t n, const mj_params* p,
                  cudaStream_t s) {
-  const uint64_t m = c->n_cand;
+  const uint64_t m = c->n_list;
   const uint32_t K = p->K;
   const bool learned = p->verify_mode == MJ_VERIFY_LEARNED;
   const bool want_feat = learned || (p->flags & MJ_FLAG_FEATURES);
@@ -850,8 +1095,15 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
   } else {
     if (!c->band_ready) return MJ_ERR_STATE;
     MJ_TRY(order_buffers(c, m, s));
-    const uint32_t* order;
-    MJ_TRY(pair_order(c, ci, cj, d_offsets, m, &order, s));
+    const uint32_t *order, *kept;
+    const bool bounds = bounds_pay(c, m, K);
+    if (bounds) {
+      MJ_TRY(bounds_buffers(c, m, s));
+      MJ_TRY(ensure_planes(c, d_bytes, K, s));
+      MJ_TRY(pair_bounds(c, d_offsets, ci, cj, nullptr, m, K, ed, s));
+    }
+    const uint8_t* rejected = bounds ? c->rejected.as<uint8_t>() : nullptr;
+    MJ_TRY(pair_order(c, ci, cj, d_offsets, m, rejected, &order, &kept, s));
     MJ_TRY(c->kband.reserve(m * 4, s));
     MJ_TRY(c->lvals.reserve(m * 4 + 16, s));
     MJ_TRY(c->franges.reserve(8 * (kMaxBandBuckets + 2), s));
@@ -859,7 +1111,7 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
     MJ_TRY(c->fcnt.reserve(8 * (kMaxBandBuckets + 2), s));
     MJ_TRY(launch_band_fused(c->band.as<float>(), ci, cj, c->run_start.as<uint32_t>(), c->stats.n_raw_pairs,
                              c->parts.as<uint32_t>(), d_offsets, m, K, c->d.T, c->band_margin, c->band_min_mult,
-                             c->kband.as<uint32_t>(), s));
+                             rejected, c->kband.as<uint32_t>(), s));
     // the pairs of each first-pass bucket, listed contiguously
     const uint32_t wK = (K + 1 + 31) / 32;
     const uint32_t nb = wK <= 1 ? 0 : (wK <= 8 ? wK - 1 : 32 - __builtin_clz(wK - 1));
@@ -898,7 +1150,7 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
         cudaStream_t sb = c->aux[(b - 1) % mj_ctx::kAuxStreams];
         if (b <= (uint32_t)mj_ctx::kAuxStreams) MJ_CUDA_TRY(cudaStreamWaitEvent(sb, c->ev_fork, 0));
         MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, c->kband.as<uint32_t>(), m, K, 32 * (whi - 1) - 1,
-                      c->ed_first.as<uint32_t>(), false, sb, forder, nullptr, ranges + 2 * b, ranges + 2 * b + 1,
+                      c->ed_first.as<uint32_t>(), sb, forder, nullptr, ranges + 2 * b, ranges + 2 * b + 1,
                       -1, -1, c->fnext.as<unsigned long long>() + b, false));
       }
       for (uint32_t b = 1; first && b <= std::min(nb, (uint32_t)mj_ctx::kAuxStreams); ++b) {
@@ -907,8 +1159,8 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
       }
     }
     c->out_collect = true;
-    const int st = verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, false, s, order,
-                          first ? c->kband.as<uint32_t>() : nullptr, nullptr, nullptr, -1, -1, nullptr, false,
+    const int st = verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order,
+                          first ? c->kband.as<uint32_t>() : nullptr, nullptr, kept, -1, -1, nullptr, false,
                           first ? c->ed_first.as<uint32_t>() : nullptr);
     c->out_collect = false;
     MJ_TRY(st);
@@ -1031,6 +1283,8 @@ void mj_destroy(mj_ctx* c) {
                  &c->tile_first,
                  &c->recs, &c->keys, &c->keys_alt, &c->idx, &c->idx_alt, &c->sort_tmp, &c->srec, &c->pair_count, &c->pair_off, &c->pairs, &c->pairs_alt,
                  &c->uflags, &c->uoffs, &c->cand_i, &c->cand_j, &c->pairbm, &c->planes, &c->ed, &c->out_t, &c->geo, &c->strgeo, &c->codes, &c->rank_dev,
+                 &c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi, &c->rk_first, &c->rk_delta,
+                 &c->rk_scan, &c->rk_len_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
                  &c->out_i, &c->out_j, &c->out_ed, &c->in_bytes, &c->in_offsets, &c->branges,
                  &c->band, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
                  &c->franges, &c->fnext, &c->fcnt, &c->ed_first};
@@ -1093,6 +1347,10 @@ int mj_partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
   cudaStream_t s = S(stream);
   begin_call(c, false);
   c->have_part = false;
+  if (c->cand_on_demand && !c->cand_recs_kept) {   // the last join's records stay for mj_candidates_copy
+    std::swap(c->recs, c->cand_recs);
+    c->cand_recs_kept = true;
+  }
   MJ_TRY(derive(c, d_bytes, d_offsets, n, p, s));
   MJ_TRY(partition(c, d_bytes, d_offsets, n, d_table, 0, s));
   MJ_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1120,7 +1378,7 @@ int mj_candidates(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, u
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
   begin_call(c, false);
-  c->have_part = c->have_cand = false;
+  c->have_part = c->have_cand = c->cand_on_demand = false;
   MJ_TRY(derive(c, d_bytes, d_offsets, n, p, s));
   MJ_TRY(partition(c, d_bytes, d_offsets, n, d_table, 0, s));
   c->have_part = true;
@@ -1137,6 +1395,22 @@ int mj_candidates_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, void* stream) {
   if (!c->have_cand) return MJ_ERR_STATE;
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
+  if (c->cand_on_demand) {
+    const mj_stats st = c->stats;
+    const Derived d = c->d;
+    const uint64_t n_part = c->n_part;
+    c->d = c->cand_d;
+    c->n_part = c->cand_n_part;
+    if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
+    c->timing = false;
+    const int rc = candidates(c, nullptr, nullptr, c->cand_n_str, 0, s);
+    if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
+    c->d = d;
+    c->n_part = n_part;
+    c->stats = st;
+    MJ_TRY(rc);
+    c->cand_on_demand = false;
+  }
   const size_t n = c->n_cand;
   if (!n) return MJ_OK;
   if (d_i) MJ_CUDA_TRY(cudaMemcpyAsync(d_i, c->cand_i.p, n * 4, cudaMemcpyDeviceToDevice, s));
@@ -1166,7 +1440,7 @@ int mj_candidates_records(mj_ctx* c, const uint32_t* d_sid, const uint32_t* d_po
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
   begin_call(c, false);
-  c->have_part = c->have_cand = false;
+  c->have_part = c->have_cand = c->cand_on_demand = false;
   Derived& d = c->d;
   d = Derived();
   d.K = p->K;
@@ -1204,7 +1478,7 @@ int mj_pairs_unique(mj_ctx* c, const uint32_t* d_i, const uint32_t* d_j, uint64_
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
   begin_call(c, false);
-  c->have_part = c->have_cand = false;
+  c->have_part = c->have_cand = c->cand_on_demand = false;
   c->n_cand = 0;
   if (m) {
     MJ_TRY(c->small.reserve(128, s));
@@ -1281,7 +1555,18 @@ int mj_verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
     MJ_TRY(launch_max_u32(d_k, m, dmax, s));
     MJ_TRY(readback(c, dmax, 4, s));
     const uint32_t kmax = *(uint32_t*)c->h_small;
-    MJ_TRY(verify(c, d_bytes, d_offsets, d_i, d_j, d_k, m, K, kmax, d_ed, true, s));
+    // the list as given, or without the pairs beyond their lower bounds
+    // (longest first: measured 6% slower than the given order on 100,000
+    // byte pairs, so the order comes with the bounds only)
+    const uint32_t *order = nullptr, *kept = nullptr;
+    if (bounds_pay(c, m, kmax)) {
+      MJ_TRY(order_buffers(c, m, s));
+      MJ_TRY(bounds_buffers(c, m, s));
+      MJ_TRY(ensure_planes(c, d_bytes, kmax, s));
+      MJ_TRY(pair_bounds(c, d_offsets, d_i, d_j, d_k, m, K, d_ed, s));
+      MJ_TRY(pair_order(c, d_i, d_j, d_offsets, m, c->rejected.as<uint8_t>(), &order, &kept, s));
+    }
+    MJ_TRY(verify(c, d_bytes, d_offsets, d_i, d_j, d_k, m, K, kmax, d_ed, s, order, nullptr, nullptr, kept));
   }
   c->stats.n_launches = launch_count() - c->launches_at_start;
   return MJ_OK;
@@ -1327,7 +1612,7 @@ int mj_autotune_verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offse
   MJ_TRY(order_buffers(c, m, s));
   MJ_TRY(c->ed.reserve(m * 4, s));
   const uint32_t* order;
-  MJ_TRY(pair_order(c, d_i, d_j, d_offsets, m, &order, s));
+  MJ_TRY(pair_order(c, d_i, d_j, d_offsets, m, nullptr, &order, nullptr, s));
   uint32_t* counts = c->branges.as<uint32_t>();
   uint32_t* ranges = counts + kLenBuckets;
   uint32_t* trial = ranges + 2 * kLenBuckets;   // [lo, hi) of the sample being timed
@@ -1347,7 +1632,7 @@ int mj_autotune_verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offse
     for (uint32_t k = 0; k < nc; ++k) {
       for (int rep_i = 0; rep_i < 2; ++rep_i) {   // the first run warms the caches
         MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
-        MJ_TRY(verify(c, d_bytes, d_offsets, d_i, d_j, nullptr, m, K, K, c->ed.as<uint32_t>(), false, s, order,
+        MJ_TRY(verify(c, d_bytes, d_offsets, d_i, d_j, nullptr, m, K, K, c->ed.as<uint32_t>(), s, order,
                       nullptr, trial, trial + 1, (int)ck[k], (int)cl[k]));
         MJ_CUDA_TRY(cudaEventRecord(c->ev[1], s));
       }
@@ -1384,18 +1669,35 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
     eff.verify_mode = MJ_VERIFY_PLAIN;
   p = &eff;
   begin_call(c, true);
-  c->have_part = c->have_cand = c->have_out = c->have_features = false;
+  c->have_part = c->have_cand = c->have_out = c->have_features = c->cand_on_demand = false;
   MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
   MJ_TRY(derive(c, d_bytes, d_offsets, n, p, s));
   MJ_CUDA_TRY(cudaEventRecord(c->ev[1], s));
+  // Plain joins go string by string.  The general path (one walk over all
+  // records, dedup by a bitmap over all pairs or a sort) serves learned mode
+  // and the candidates' features (they need multiplicities), the key check, a
+  // forced dedup, and windows too wide for a bitmap in shared memory; it is
+  // also the faster one for few strings, whose joins its fewer launches decide
+  // (1,000 strings: 518 us against 602) and whose candidates are few (50,000
+  // reads: 4.31 ms against 4.37).
+  constexpr uint32_t kStringsFrom = 1u << 16;
+  const uint32_t general = MJ_FLAG_FEATURES | MJ_FLAG_KEY_CHECK | MJ_FLAG_DEDUP_SORT | MJ_FLAG_DEDUP_BITMAP;
+  c->by_strings = p->verify_mode == MJ_VERIFY_PLAIN && !(p->flags & general) && p->K > 0 && n >= kStringsFrom;
+  if (c->by_strings) MJ_TRY(string_ranks(c, d_offsets, n, s));
   MJ_TRY(partition(c, d_bytes, d_offsets, n, nullptr, p->K, s));
   c->have_part = true;
   MJ_CUDA_TRY(cudaEventRecord(c->ev[2], s));
-  MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,
-                    p->verify_mode == MJ_VERIFY_LEARNED || (p->flags & MJ_FLAG_FEATURES)));
+  const bool strings = c->by_strings && string_pairs_fit(c->rk_widest);
+  if (strings) {
+    MJ_TRY(string_candidates(c, d_offsets, n, s));
+  } else {
+    MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,
+                      p->verify_mode == MJ_VERIFY_LEARNED || (p->flags & MJ_FLAG_FEATURES)));
+    c->n_list = c->n_cand;
+  }
   c->have_cand = true;
   MJ_CUDA_TRY(cudaEventRecord(c->ev[3], s));
-  const uint64_t m = c->n_cand;
+  const uint64_t m = c->n_list;
   c->n_out = 0;
   if (m) {
     MJ_TRY(verify_stage(c, d_bytes, d_offsets, n, p, s));
@@ -1406,7 +1708,7 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
     MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + 3, c->small.as<unsigned long long>() + 2, 8, cudaMemcpyDeviceToHost, s));
     MJ_CUDA_TRY(cudaStreamSynchronize(s));
     const uint64_t no = c->h_small[0];
-    c->stats.band_cells = c->h_small[1];
+    if (!strings) c->stats.band_cells = c->h_small[1];
     c->stats.device_flags |= *(uint32_t*)(c->h_small + 2);
     c->stats.verify_word_columns = c->h_small[3];
     if (no > m) return MJ_ERR_DEVICE;
@@ -1416,11 +1718,20 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
     MJ_TRY(c->keys.reserve((size_t)no * 8 + 16, s));
     MJ_TRY(c->keys_alt.reserve((size_t)no * 8 + 16, s));
     MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(no), s));
-    // sorted candidate indices are (i, j) order
-    MJ_TRY(launch_gather_output(c->out_t.as<uint32_t>(), no, m, c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(),
-                                c->ed.as<uint32_t>(), c->keys.as<uint64_t>(), c->keys_alt.as<uint64_t>(),
-                                c->sort_tmp.p, c->out_i.as<uint32_t>(), c->out_j.as<uint32_t>(),
-                                c->out_ed.as<uint32_t>(), s));
+    if (strings) {   // pairs in any order
+      MJ_TRY(c->idx.reserve((size_t)no * 4 + 16, s));
+      MJ_TRY(c->idx_alt.reserve((size_t)no * 4 + 16, s));
+      MJ_TRY(launch_gather_output_pairs(c->out_t.as<uint32_t>(), no, bits_for(n - 1), c->cand_i.as<uint32_t>(),
+                                        c->cand_j.as<uint32_t>(), c->ed.as<uint32_t>(), c->keys.as<uint64_t>(),
+                                        c->keys_alt.as<uint64_t>(), c->idx.as<uint32_t>(), c->idx_alt.as<uint32_t>(),
+                                        c->sort_tmp.p, c->out_i.as<uint32_t>(), c->out_j.as<uint32_t>(),
+                                        c->out_ed.as<uint32_t>(), s));
+    } else {   // sorted candidate indices are (i, j) order
+      MJ_TRY(launch_gather_output(c->out_t.as<uint32_t>(), no, m, c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(),
+                                  c->ed.as<uint32_t>(), c->keys.as<uint64_t>(), c->keys_alt.as<uint64_t>(),
+                                  c->sort_tmp.p, c->out_i.as<uint32_t>(), c->out_j.as<uint32_t>(),
+                                  c->out_ed.as<uint32_t>(), s));
+    }
     tstop(c, 7, s);
     c->n_out = no;
   }

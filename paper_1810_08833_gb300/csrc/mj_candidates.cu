@@ -359,6 +359,29 @@ __global__ void gather_out_kernel(const uint64_t* __restrict__ keys, uint64_t n,
   }
 }
 
+// Keys (i << nb | j) of the listed pairs, and their indices.
+__global__ void out_pair_keys_kernel(const uint32_t* __restrict__ out_t, uint64_t n, int nb,
+                                     const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj,
+                                     uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t t = out_t[u];
+    keys[u] = ((uint64_t)ci[t] << nb) | cj[t];
+    vals[u] = t;
+  }
+}
+
+__global__ void gather_out_pairs_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+                                        uint64_t n, int nb, const uint32_t* __restrict__ ed,
+                                        uint32_t* __restrict__ oi, uint32_t* __restrict__ oj,
+                                        uint32_t* __restrict__ oed) {
+  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t k = keys[u];
+    oi[u] = (uint32_t)(k >> nb);
+    oj[u] = (uint32_t)(k & ((1ull << nb) - 1));
+    oed[u] = ed[vals[u]];
+  }
+}
+
 __global__ void multiplicity_kernel(const uint32_t* __restrict__ run_start, uint64_t nc, uint64_t raw,
                                     uint32_t* __restrict__ mult) {
   for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nc; u += (uint64_t)gridDim.x * blockDim.x) {
@@ -515,6 +538,7 @@ __global__ void __launch_bounds__(kOrderThreads) order_hist_kernel(const uint32_
                                                                    const uint32_t* __restrict__ cj,
                                                                    const uint2* __restrict__ sg, uint32_t n_str,
                                                                    uint64_t m, uint64_t R, uint32_t K,
+                                                                   const uint8_t* __restrict__ rejected,
                                                                    uint32_t* __restrict__ bh,
                                                                    unsigned long long* __restrict__ cells) {
   __shared__ uint32_t h[kOrderClasses];
@@ -526,7 +550,7 @@ __global__ void __launch_bounds__(kOrderThreads) order_hist_kernel(const uint32_
   for (uint64_t t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
     const PairLens L = pair_lens(ci, cj, sg, n_str, t);
     const uint32_t n = L.lx < L.ly ? L.lx : L.ly, mm = L.lx < L.ly ? L.ly : L.lx;
-    atomicAdd(&h[length_class((uint64_t)n)], 1u);
+    if (!rejected || !rejected[t]) atomicAdd(&h[length_class((uint64_t)n)], 1u);
     if (cells) acc += band_cells_of(mm, n, K);
   }
   if (cells) {
@@ -543,7 +567,7 @@ __global__ void __launch_bounds__(kOrderThreads) order_hist_kernel(const uint32_
 // counts[b] and ranges[2b], ranges[2b+1] = the pairs and [start, end) of
 // floor(log2) bucket b (n <= 1 in bucket 0).
 __global__ void order_scan_kernel(uint32_t* __restrict__ bh, uint32_t G, uint32_t* __restrict__ counts,
-                                  uint32_t* __restrict__ ranges) {
+                                  uint32_t* __restrict__ ranges, uint32_t* __restrict__ kept) {
   __shared__ uint32_t v[kOrderClasses], tot[kOrderClasses], cursor[kOrderClasses];
   const int c = threadIdx.x;
   uint32_t sum = 0;
@@ -562,6 +586,7 @@ __global__ void order_scan_kernel(uint32_t* __restrict__ bh, uint32_t G, uint32_
   }
   const int cls = kOrderClasses - 1 - c;
   cursor[cls] = v[c] - tot[cls];
+  if (kept && c == kOrderClasses - 1) *kept = v[c];
   __syncthreads();
   uint32_t run = cursor[c];
   for (uint32_t b = 0; b < G; ++b) {
@@ -594,6 +619,7 @@ __global__ void __launch_bounds__(kOrderThreads) order_scatter_kernel(const uint
                                                                      const uint32_t* __restrict__ cj,
                                                                      const uint2* __restrict__ sg,
                                                                      uint32_t n_str, uint64_t m, uint64_t R,
+                                                                     const uint8_t* __restrict__ rejected,
                                                                      const uint32_t* __restrict__ bbase,
                                                                      uint32_t* __restrict__ order,
                                                                      uint4* __restrict__ geo) {
@@ -613,7 +639,7 @@ __global__ void __launch_bounds__(kOrderThreads) order_scatter_kernel(const uint
     for (int k = 0; k < kOrderItems; ++k) {
       const uint64_t t = base + (uint64_t)k * kOrderThreads + threadIdx.x;
       cls[k] = 0xffffffffu;
-      if (t < t1) {
+      if (t < t1 && !(rejected && rejected[t])) {
         const PairLens L = pair_lens(ci, cj, sg, n_str, t);
         const bool xa = L.lx >= L.ly;
         g[k] = L.bad ? make_uint4(0u, 0u, 0u, kGeoBadIds)
@@ -801,8 +827,8 @@ int launch_compact_pairs(const uint64_t* sorted, const uint32_t* flags, const ui
 }
 
 int launch_length_order(const uint32_t* ci, const uint32_t* cj, const int64_t* offsets, uint32_t n_str, uint64_t m,
-                        uint32_t K, uint32_t* scratch, uint2* sg, uint32_t* order, uint4* geo, uint32_t* counts,
-                        uint32_t* ranges, unsigned long long* cells, cudaStream_t s) {
+                        uint32_t K, const uint8_t* rejected, uint32_t* kept, uint32_t* scratch, uint2* sg,
+                        uint32_t* order, uint4* geo, uint32_t* counts, uint32_t* ranges, unsigned long long* cells, cudaStream_t s) {
   if (n_str) {
     string_geo_kernel<<<grid_for(n_str), 256, 0, s>>>(offsets, n_str, sg);
     MJ_KERNEL_DONE();
@@ -812,12 +838,12 @@ int launch_length_order(const uint32_t* ci, const uint32_t* cj, const int64_t* o
   const uint32_t G = (uint32_t)(chunks < 1 ? 1 : (chunks < (uint64_t)kOrderBlocksMax ? chunks : kOrderBlocksMax));
   const uint64_t R = (chunks + G - 1) / G * kOrderChunk;
   if (cells) MJ_CUDA_TRY(cudaMemsetAsync(cells, 0, sizeof(unsigned long long), s));
-  order_hist_kernel<<<G, kOrderThreads, 0, s>>>(ci, cj, sg, n_str, m, R, K, scratch, cells);
+  order_hist_kernel<<<G, kOrderThreads, 0, s>>>(ci, cj, sg, n_str, m, R, K, rejected, scratch, cells);
   MJ_KERNEL_DONE();
-  order_scan_kernel<<<1, kOrderClasses, 0, s>>>(scratch, G, counts, ranges);
+  order_scan_kernel<<<1, kOrderClasses, 0, s>>>(scratch, G, counts, ranges, kept);
   MJ_KERNEL_DONE();
   if (m) {
-    order_scatter_kernel<<<G, kOrderThreads, 0, s>>>(ci, cj, sg, n_str, m, R, scratch, order, geo);
+    order_scatter_kernel<<<G, kOrderThreads, 0, s>>>(ci, cj, sg, n_str, m, R, rejected, scratch, order, geo);
     MJ_KERNEL_DONE();
   }
   return MJ_OK;
@@ -869,6 +895,21 @@ int launch_gather_output(const uint32_t* out_t, uint64_t n, uint64_t m, const ui
   bool alt = false;
   MJ_TRY(radix_sort_u64(keys, keys_alt, nullptr, nullptr, n, 0, bits, temp, &alt, s));
   gather_out_kernel<<<grid_for(n), 256, 0, s>>>(alt ? keys_alt : keys, n, ci, cj, ed, oi, oj, oed);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+int launch_gather_output_pairs(const uint32_t* out_t, uint64_t n, int nb, const uint32_t* ci, const uint32_t* cj,
+                               const uint32_t* ed, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals,
+                               uint32_t* vals_alt, void* temp, uint32_t* oi, uint32_t* oj, uint32_t* oed,
+                               cudaStream_t s) {
+  if (!n) return MJ_OK;
+  out_pair_keys_kernel<<<grid_for(n), 256, 0, s>>>(out_t, n, nb, ci, cj, keys, vals);
+  MJ_KERNEL_DONE();
+  bool alt = false;
+  MJ_TRY(radix_sort_u64(keys, keys_alt, vals, vals_alt, n, 0, 2 * nb, temp, &alt, s));
+  gather_out_pairs_kernel<<<grid_for(n), 256, 0, s>>>(alt ? keys_alt : keys, alt ? vals_alt : vals, n, nb, ed, oi, oj,
+                                                      oed);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

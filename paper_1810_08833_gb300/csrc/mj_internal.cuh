@@ -161,6 +161,107 @@ int radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t*
                    uint64_t n, int bit_lo, int bit_hi, void* temp, bool* result_in_alt,
                    cudaStream_t s);
 
+// The same for 32-bit keys (fewer bytes per pass); temp from radix_temp_bytes.
+int radix_sort_u32(uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t* vals_alt,
+                   uint64_t n, int bit_lo, int bit_hi, void* temp, bool* result_in_alt,
+                   cudaStream_t s);
+
+// a5-a7 of a plain join, string by string in order of length (mj_pairs.cu).
+// Ranks: strings sorted by length (ties by id).  len/sid (n entries each and
+// their alternates) end sorted, in the alternates if *in_alt; rank_of[id],
+// hi[rank] = the last rank within K of its length; len_rank[l] (nullable) = the
+// first rank of length l or more; *widest = the most ranks above its own that
+// a string can pair with.
+int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, int len_bits, uint32_t* len, uint32_t* len_alt,
+                        uint32_t* sid, uint32_t* sid_alt, void* temp, uint32_t* rank_of, uint32_t* hi,
+                        uint32_t* len_rank, unsigned int* widest, bool* in_alt, cudaStream_t s);
+// first[i], i = 0 .. n: base + the anchors before string i in the bitmap
+// (`total` anchors in all).
+int launch_string_first(const int64_t* offsets, uint32_t n, uint64_t nbytes, const uint32_t* bitmap,
+                        const uint32_t* tile_off, uint32_t total, uint32_t base, uint32_t* first, cudaStream_t s);
+// delta[k (n + 1) + id] + t = place by rank of record t of repetition k;
+// rfirst: n words of scratch.
+int launch_rank_order(const uint32_t* first, const uint32_t* sid_of, const uint32_t* rank_of, uint32_t n, uint32_t reps,
+                      uint32_t* rfirst, uint32_t* delta, void* temp, cudaStream_t s);
+// Sort keys and record indices of records [t0, t1) of one repetition (delta:
+// its n + 1 words) at their places by rank.
+int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int pb_bits, uint32_t W,
+                     uint32_t* keys, uint32_t* vals, cudaStream_t s);
+// Rank bits of a visit word when a visit fits 16 bytes, else 0 (B is then used).
+int visit_rank_bits(uint64_t longest, uint32_t n);
+// From the sorted keys and indices: A, B, skr (n_rec entries) and the windows
+// of every record (2 entries each, at the record's own place); *visits = the
+// records in all windows.
+struct RankTables {
+  const uint32_t* hi;
+  const uint32_t* rlen;       // lengths by rank
+  const uint32_t* len_rank;   // nullable
+  uint32_t longest, n;
+};
+int launch_rank_windows(const uint32_t* idx, const uint32_t* keys, uint32_t n_rec, const PRec* recs,
+                        const uint32_t* rank_of, const RankTables& rt, uint32_t K, uint32_t W, int pb_bits, int rb,
+                        uint4* A, uint2* B, uint64_t* skr, uint4* win, unsigned long long* visits, cudaStream_t s);
+// Lower bounds on the edit distance: gram lengths of the two levels and the
+// buckets of single symbols (by rank code).
+struct SigShape {
+  uint32_t q1, q2;
+  uint8_t bucket[256];
+};
+uint32_t signature_grams(uint32_t sigma, uint32_t want);   // the shortest q (<= 8) with sigma^q >= want
+SigShape signature_shape(uint32_t sigma, const uint64_t* counts_by_code);
+size_t sig1_bytes(uint32_t n);
+size_t sig2_bytes(uint32_t n);
+// Signatures by rank (sid_of) or id (null).  With visits (nullable), does
+// nothing when *visits <= min_visits.
+int launch_signatures(const uint8_t* codes, const int64_t* offsets, const uint32_t* sid_of, uint32_t n,
+                      const SigShape& g, const unsigned long long* visits, uint64_t min_visits, uint4* sig1,
+                      uint32_t* sig2, cudaStream_t s);
+// The same bounds on listed pairs (signatures by id): rejected[t] = 1 and
+// ed[t] = k + 1 where they exceed pair t's band (pk[t], or K when pk is null).
+int launch_pair_bounds(const uint32_t* pi, const uint32_t* pj, const uint32_t* pk, uint32_t K, uint64_t m, uint32_t n,
+                       const SigShape& g, const uint4* sig1, const uint4* sig2, uint8_t* rejected, uint32_t* ed,
+                       cudaStream_t s);
+struct PairArgs {
+  const PRec* recs;           // in position order
+  const uint32_t* first;      // launch_string_first, one row of n + 1 per repetition
+  const uint4* win;
+  const uint4* A;
+  const uint2* B;
+  const uint32_t* sid_of;     // by rank
+  const uint32_t* rlen;
+  const uint32_t* hi;
+  const uint4* sig1;          // read when *visits > min_visits
+  const unsigned long long* visits;
+  uint64_t min_visits;
+  uint32_t n, reps, K, q1;
+  int rb;                     // visit_rank_bits
+  uint32_t bm_words = 0;      // set by the launcher
+  unsigned long long* out_count;   // pairs of ranks that pass the first bound (all counted, the first cap listed)
+  unsigned long long* totals;      // out_count + 1: raw pairs, candidates, K-band cells of the candidates
+  uint64_t cap;
+  uint2* out;
+};
+bool string_pairs_fit(uint32_t widest);   // a string's bitmap fits in shared memory
+constexpr size_t kStringPairsSmemMax = 160u << 10;
+int launch_string_pairs(const PairArgs& a, uint32_t widest, cudaStream_t s);
+// The second bound of the listed pairs: what passes, as pairs of ids (i < j).
+struct ListArgs {
+  const uint2* in;
+  const unsigned long long* in_count;
+  uint64_t in_cap;
+  const uint4* sig2;          // read when *visits > min_visits
+  const uint32_t* sid_of;
+  const uint32_t* rlen;
+  const unsigned long long* visits;
+  uint64_t min_visits;
+  uint32_t K, q2;
+  unsigned long long* out_count;   // all counted, the first cap listed
+  uint64_t cap;
+  uint32_t* out_i;
+  uint32_t* out_j;
+};
+int launch_listed_pairs(const ListArgs& a, cudaStream_t s);
+
 // a5-a6: grouping keys and pair emission.  A group key is hash_bits (<= 32)
 // bits of a hash of (len, Karp-Rabin key), then pb_bits bits of the
 // position bucket pos / W (W >= K, so the partner of a record under the
@@ -229,7 +330,6 @@ struct VerifyArgs {
   uint32_t K;
   uint64_t m;
   uint32_t* ed = nullptr;
-  unsigned long long* cells = nullptr; // nullable: K-band cells accumulated
   unsigned long long* work = nullptr;  // nullable: word-columns processed (columns x W) accumulated
   uint32_t* dev_flags = nullptr;
   const uint4* pair_geo = nullptr;     // nullable: at order position q, (oA, oB, m, n) of pair order[q], A the
@@ -251,6 +351,8 @@ int launch_build_planes(const uint8_t* bytes, uint64_t nbytes, const RankTable& 
 int launch_verify(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, uint32_t kmax,
                   unsigned long long* next, cudaStream_t s, int kernel = MJ_VERIFY_KERNEL_AUTO, int lanes = 0);
 int wave_lanes_for(uint32_t kmax);
+// whether launch_verify takes bands up to kmax with this kernel choice
+bool verify_supported(uint32_t kmax, int kernel, int lanes);
 // lanes of the CTA wavefront (several warps per pair) for bands up to kmax,
 // and the fewest lanes of either wavefront form; at most kMaxCtaLanes
 constexpr int kMaxCtaLanes = 1024;
@@ -273,9 +375,12 @@ constexpr int kOrderScratchWords = 256 * kNumSMsHint * 8;
 constexpr uint32_t kGeoBadIds = 0xffffffffu;
 // sg: n_str entries of scratch for the strings' {offset, length} (inputs
 // are under 4 GB).
+// rejected (nullable): pairs with rejected[t] != 0 are left out of the order
+// and the buckets (not of the cells); *kept (nullable): pairs in the order.
 int launch_length_order(const uint32_t* ci, const uint32_t* cj, const int64_t* offsets, uint32_t n_str, uint64_t m,
-                        uint32_t K, uint32_t* scratch, uint2* sg, uint32_t* order, uint4* geo, uint32_t* counts,
-                        uint32_t* ranges, unsigned long long* cells, cudaStream_t s);
+                        uint32_t K, const uint8_t* rejected, uint32_t* kept, uint32_t* scratch, uint2* sg,
+                        uint32_t* order, uint4* geo, uint32_t* counts, uint32_t* ranges, unsigned long long* cells,
+                        cudaStream_t s);
 
 // ---- learned first-pass band (MLP 8 -> 64 -> 64 -> 1)
 // features of a candidate (i, j), n = min length, d0 = length difference,
@@ -299,7 +404,7 @@ int launch_band_adam(float* P, const float* G, float* M, float* V, float lr, flo
                      cudaStream_t s);
 int launch_band_fused(const float* P, const uint32_t* ci, const uint32_t* cj, const uint32_t* run_start, uint64_t raw,
                       const uint32_t* parts, const int64_t* offsets, uint64_t m, uint32_t K, uint32_t T, uint32_t margin,
-                      uint32_t min_mult, uint32_t* kband, cudaStream_t s);
+                      uint32_t min_mult, const uint8_t* rejected, uint32_t* kband, cudaStream_t s);
 int launch_gate_hist(const float* X, const uint32_t* ed, uint64_t m, uint32_t K, unsigned int* hist, cudaStream_t s);
 int launch_band_rule(const float* yhat, const uint32_t* ci, const uint32_t* cj, const int64_t* offsets, uint64_t m,
                      uint32_t K, uint32_t margin, uint32_t* kband, cudaStream_t s);
@@ -322,5 +427,12 @@ int launch_band_buckets(const uint32_t* kband, uint64_t m, uint32_t K, uint32_t 
 int launch_gather_output(const uint32_t* out_t, uint64_t n, uint64_t m, const uint32_t* ci, const uint32_t* cj,
                          const uint32_t* ed, uint64_t* keys, uint64_t* keys_alt, void* temp, uint32_t* oi,
                          uint32_t* oj, uint32_t* oed, cudaStream_t s);
+
+// The same for pairs in any order: sorted by (i, j) (nb bits each); vals and
+// vals_alt: 4 * n bytes each.
+int launch_gather_output_pairs(const uint32_t* out_t, uint64_t n, int nb, const uint32_t* ci, const uint32_t* cj,
+                               const uint32_t* ed, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals,
+                               uint32_t* vals_alt, void* temp, uint32_t* oi, uint32_t* oj, uint32_t* oed,
+                               cudaStream_t s);
 
 }  // namespace mj

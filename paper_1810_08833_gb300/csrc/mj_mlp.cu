@@ -272,6 +272,7 @@ __global__ void __launch_bounds__(kQueue) band_fused_kernel(const float* __restr
                                                             const uint32_t* __restrict__ parts,
                                                             const int64_t* __restrict__ offsets, uint64_t m, uint32_t K,
                                                             uint32_t T, uint32_t margin, uint32_t min_mult,
+                                                            const uint8_t* __restrict__ rejected,
                                                             uint32_t* __restrict__ kband) {
   __shared__ float s[kBandParams];
   __shared__ uint32_t q_u[2 * kQueue];
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(kQueue) band_fused_kernel(const float* __restr
       const uint64_t e = u + 1 < m ? run_start[u + 1] : raw;
       const uint32_t c = (uint32_t)(e - run_start[u]);
       kband[u] = K;
-      if (c >= min_mult) {
+      if (c >= min_mult && !(rejected && rejected[u])) {   // a rejected pair needs no pass at all
         const uint32_t slot = atomicAdd(&qn, 1u);
         q_u[slot] = (uint32_t)u;
         q_c[slot] = c;
@@ -411,10 +412,10 @@ int launch_band_adam(float* P, const float* G, float* M, float* V, float lr, flo
 
 int launch_band_fused(const float* P, const uint32_t* ci, const uint32_t* cj, const uint32_t* run_start, uint64_t raw,
                       const uint32_t* parts, const int64_t* offsets, uint64_t m, uint32_t K, uint32_t T, uint32_t margin,
-                      uint32_t min_mult, uint32_t* kband, cudaStream_t s) {
+                      uint32_t min_mult, const uint8_t* rejected, uint32_t* kband, cudaStream_t s) {
   if (!m) return MJ_OK;
   band_fused_kernel<<<grid1(m, kQueue), kQueue, 0, s>>>(P, ci, cj, run_start, raw, parts, offsets, m, K, T, margin,
-                                                       min_mult, kband);
+                                                       min_mult, rejected, kband);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

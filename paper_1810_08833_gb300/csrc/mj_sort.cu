@@ -121,7 +121,8 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys per tile
 
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint64_t* __restrict__ keys, uint64_t n,
+template <class KT>
+__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const KT* __restrict__ keys, uint64_t n,
                                                                   int shift, uint32_t num_tiles,
                                                                   uint32_t* __restrict__ hist) {
   __shared__ uint32_t s_hist[256];
@@ -143,18 +144,20 @@ __global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint64_t
 // The tile is first placed in digit order in shared memory, then written out
 // item by item in that order: items of one digit go to consecutive global
 // addresses, so a warp's stores form a few contiguous runs.
-constexpr size_t kScatterSmem = (size_t)kSortTile * (sizeof(uint64_t) + sizeof(uint32_t));
+template <class KT>
+constexpr size_t kScatterSmem = (size_t)kSortTile * (sizeof(KT) + sizeof(uint32_t));
 constexpr int kScatThreads = 512;                       // threads of the scatter kernel
 constexpr int kScatItems = kSortTile / kScatThreads;    // items per thread
 constexpr int kScatWarps = kScatThreads / 32;
 
+template <class KT>
 __global__ void __launch_bounds__(kScatThreads) radix_scatter_kernel(
-    const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n, int shift,
-    uint32_t num_tiles, const uint32_t* __restrict__ offs, uint64_t* __restrict__ keys_out,
+    const KT* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n, int shift,
+    uint32_t num_tiles, const uint32_t* __restrict__ offs, KT* __restrict__ keys_out,
     uint32_t* __restrict__ vals_out) {
   extern __shared__ __align__(16) uint8_t smem[];
-  uint64_t* s_keys = reinterpret_cast<uint64_t*>(smem);
-  uint32_t* s_vals = reinterpret_cast<uint32_t*>(smem + (size_t)kSortTile * sizeof(uint64_t));
+  KT* s_keys = reinterpret_cast<KT*>(smem);
+  uint32_t* s_vals = reinterpret_cast<uint32_t*>(smem + (size_t)kSortTile * sizeof(KT));
   __shared__ uint32_t s_cnt[kScatWarps][256];
   __shared__ uint32_t s_start[256];   // first local position of each digit
   __shared__ uint32_t s_goff[256];    // global position of each digit's first item
@@ -166,13 +169,13 @@ __global__ void __launch_bounds__(kScatThreads) radix_scatter_kernel(
   const uint64_t tile0 = (uint64_t)blockIdx.x * kSortTile;
   const uint64_t base = tile0 + (uint64_t)wid * (kSortTile / kScatWarps);
   const uint32_t valid = (uint32_t)min((uint64_t)kSortTile, n - tile0);
-  uint64_t k_[kScatItems];
+  KT k_[kScatItems];
   uint32_t rank_[kScatItems];
   const uint32_t lt = (1u << lane) - 1;
 #pragma unroll
   for (int r = 0; r < kScatItems; ++r) {
     const uint64_t idx = base + (uint64_t)r * 32 + lane;
-    k_[r] = idx < n ? keys[idx] : ~0ull;
+    k_[r] = idx < n ? keys[idx] : ~KT(0);
   }
 #pragma unroll
   for (int r = 0; r < kScatItems; ++r) {
@@ -228,7 +231,7 @@ __global__ void __launch_bounds__(kScatThreads) radix_scatter_kernel(
   for (int r = 0; r < kScatItems; ++r) {
     const uint32_t i = (uint32_t)r * kScatThreads + threadIdx.x;
     if (i < valid) {
-      const uint64_t key = s_keys[i];
+      const KT key = s_keys[i];
       const uint32_t d = (uint32_t)(key >> shift) & 255u;
       const uint32_t dst = s_goff[d] + (i - s_start[d]);
       keys_out[dst] = key;
@@ -262,8 +265,11 @@ size_t radix_temp_bytes(uint64_t n) {
   return 2 * h * sizeof(uint32_t) + scan_temp_bytes(h) + 256;
 }
 
-int radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint64_t n,
-                   int bit_lo, int bit_hi, void* temp, bool* result_in_alt, cudaStream_t s) {
+namespace {
+
+template <class KT>
+int radix_sort(KT* keys, KT* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint64_t n, int bit_lo, int bit_hi,
+               void* temp, bool* result_in_alt, cudaStream_t s) {
   *result_in_alt = false;
   if (n <= 1 || bit_hi <= bit_lo) return MJ_OK;
   if (n >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;
@@ -272,18 +278,18 @@ int radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t*
   uint32_t* hist = static_cast<uint32_t*>(temp);
   uint32_t* offs = hist + h;
   void* scan_tmp = offs + h;
-  uint64_t* src_k = keys;
-  uint64_t* dst_k = keys_alt;
+  KT* src_k = keys;
+  KT* dst_k = keys_alt;
   uint32_t* src_v = vals;
   uint32_t* dst_v = vals_alt;
   bool alt = false;
-  MJ_CUDA_TRY(cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kScatterSmem));
+  MJ_CUDA_TRY(cudaFuncSetAttribute(radix_scatter_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kScatterSmem<KT>));
   for (int shift = bit_lo; shift < bit_hi; shift += 8) {
-    radix_hist_kernel<<<tiles, kSortThreads, 0, s>>>(src_k, n, shift, tiles, hist);
+    radix_hist_kernel<KT><<<tiles, kSortThreads, 0, s>>>(src_k, n, shift, tiles, hist);
     MJ_KERNEL_DONE();
     MJ_TRY(launch_exclusive_scan_u32(hist, offs, h, scan_tmp, nullptr, s));
-    radix_scatter_kernel<<<tiles, kScatThreads, kScatterSmem, s>>>(src_k, src_v, n, shift, tiles, offs, dst_k,
+    radix_scatter_kernel<KT><<<tiles, kScatThreads, kScatterSmem<KT>, s>>>(src_k, src_v, n, shift, tiles, offs, dst_k,
                                                                     dst_v);
     MJ_KERNEL_DONE();
     std::swap(src_k, dst_k);
@@ -292,6 +298,18 @@ int radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t*
   }
   *result_in_alt = alt;
   return MJ_OK;
+}
+
+}  // namespace
+
+int radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint64_t n, int bit_lo,
+                   int bit_hi, void* temp, bool* result_in_alt, cudaStream_t s) {
+  return radix_sort(keys, keys_alt, vals, vals_alt, n, bit_lo, bit_hi, temp, result_in_alt, s);
+}
+
+int radix_sort_u32(uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint64_t n, int bit_lo,
+                   int bit_hi, void* temp, bool* result_in_alt, cudaStream_t s) {
+  return radix_sort(keys, keys_alt, vals, vals_alt, n, bit_lo, bit_hi, temp, result_in_alt, s);
 }
 
 }  // namespace mj

@@ -99,7 +99,6 @@ extern "C" int mj_verify_static(const uint8_t* d_bytes, const int64_t* d_offsets
   a.K = K;
   a.m = m;
   a.ed = d_ed;
-  a.cells = nullptr;
   a.work = nullptr;
   a.dev_flags = flags;
   return launch_verify(a, PW, GW, K, next, s);

@@ -98,17 +98,6 @@ __device__ __forceinline__ void put_result(const VerifyArgs& a, uint64_t t, uint
   if (a.out_t && v <= a.K) a.out_t[atomicAdd(a.out_count, 1ull)] = (uint32_t)t;
 }
 
-// Number of cells (i, j), 1 <= i <= m, 1 <= j <= n, with |i - j| <= K (m >= n).
-__device__ __forceinline__ uint64_t band_cells(int64_t m, int64_t n, int64_t K) {
-  if (n <= 0 || m <= 0) return 0;
-  int64_t a = m - K;                                   // j <= a: min(m, j+K) = j + K
-  a = a < 0 ? 0 : (a > n ? n : a);
-  int64_t smin = a * (a + 1) / 2 + a * K + (n - a) * m;
-  int64_t b = K < n ? K : n;                           // j <= K: max(1, j-K) = 1
-  int64_t smax = b + (n > K ? (n - K) * (n - K + 1) / 2 : 0);
-  return (uint64_t)(smin - smax + n);
-}
-
 // Per-lane state of one pair in flight.
 template <int W, int P>
 struct PairState {
@@ -523,7 +512,7 @@ __global__ void __launch_bounds__(128, (P == 7 && W <= 3) ? 7 : ((P == 5 && W <=
   PairState<W, P> st;
   bool active = false;
   bool more = true;
-  uint64_t cells = 0, work = 0, nskip = 0;
+  uint64_t work = 0, nskip = 0;
   while (true) {
     // lanes without a pair fetch the next indices
     const bool need = !active && more;
@@ -546,14 +535,6 @@ __global__ void __launch_bounds__(128, (P == 7 && W <= 3) ? 7 : ((P == 5 && W <=
           if (settled && a.first_ed) put_result(a, t, fed[t]);
           nskip += settled ? 1 : 0;
           if (!settled) {
-            if (a.cells) {
-              const uint32_t x = a.pi[t], y = a.pj[t];
-              if (x < a.n_strings && y < a.n_strings) {
-                const int64_t lx = __ldg(a.offsets + x + 1) - __ldg(a.offsets + x);
-                const int64_t ly = __ldg(a.offsets + y + 1) - __ldg(a.offsets + y);
-                cells += band_cells(lx > ly ? lx : ly, lx > ly ? ly : lx, a.K);
-              }
-            }
             uint32_t res;
             if (pair_init<W, P>(st, a, GW, q, t, &res)) {
               active = true;
@@ -575,10 +556,6 @@ __global__ void __launch_bounds__(128, (P == 7 && W <= 3) ? 7 : ((P == 5 && W <=
         active = false;
       }
     }
-  }
-  if (a.cells) {
-    for (int o = 16; o > 0; o >>= 1) cells += __shfl_down_sync(0xffffffffu, cells, o);
-    if (lane == 0 && cells) atomicAdd(a.cells, (unsigned long long)cells);
   }
   if (a.work) {
     for (int o = 16; o > 0; o >>= 1) work += __shfl_down_sync(0xffffffffu, work, o);
@@ -704,7 +681,7 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
   uint32_t pub = kIdle;
   bool done = false, reject = false;
   int32_t result = 0;
-  uint64_t work = 0, cells = 0, nskip = 0;
+  uint64_t work = 0, nskip = 0;
 #pragma unroll
   for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
 
@@ -756,7 +733,6 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
             if (gl == 0) atomicOr(a.dev_flags, FLAG_BOUNDS);
             res = k + 1;
           } else {
-            if (a.cells && gl == 0) cells += band_cells(gm, gn, a.K);
             const int64_t mm = gm, nn = gn;
             if (mm >= (int64_t)kMaxLen) {
               if (gl == 0) atomicOr(a.dev_flags, FLAG_LENGTH);
@@ -900,10 +876,6 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
     for (int o = 16; o > 0; o >>= 1) work += __shfl_down_sync(0xffffffffu, work, o);
     if (lane == 0 && work) atomicAdd(a.work, (unsigned long long)work);
   }
-  if (a.cells) {
-    for (int o = 16; o > 0; o >>= 1) cells += __shfl_down_sync(0xffffffffu, cells, o);
-    if (lane == 0 && cells) atomicAdd(a.cells, (unsigned long long)cells);
-  }
   if (a.skipped) {
     for (int o = 16; o > 0; o >>= 1) nskip += __shfl_down_sync(0xffffffffu, nskip, o);
     if (lane == 0 && nskip) atomicAdd(a.skipped, (unsigned long long)nskip);
@@ -957,7 +929,7 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
   bool done = false, reject = false;
   int32_t result = 0;
   uint32_t win = 0;   // windows run by the CTA (selects the flag slot)
-  uint64_t work = 0, cells = 0, nskip = 0;
+  uint64_t work = 0, nskip = 0;
 #pragma unroll
   for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
 
@@ -1003,7 +975,6 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
           put_result(a, t, kt + 1);
           continue;
         }
-        if (a.cells) cells += band_cells(mm, nn, a.K);
         if (mm >= (int64_t)kMaxLen) {
           atomicOr(a.dev_flags, FLAG_LENGTH);
           put_result(a, t, kt + 1);
@@ -1124,7 +1095,6 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
     for (int o = 16; o > 0; o >>= 1) work += __shfl_down_sync(0xffffffffu, work, o);
     if (lane == 0 && work) atomicAdd(a.work, (unsigned long long)work);
   }
-  if (tid == 0 && a.cells && cells) atomicAdd(a.cells, (unsigned long long)cells);
   if (tid == 0 && a.skipped && nskip) atomicAdd(a.skipped, (unsigned long long)nskip);
 }
 
@@ -1157,8 +1127,12 @@ int launch_vp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long*
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_cta_kernel<V, P>, 32 * V, 0);
   if (per_sm < 1) per_sm = 1;
+  // pairs take about equally long: no more CTAs than give every one the same
+  // number of pairs (fewer CTAs per SM run faster, a part-filled last round
+  // does not)
   uint64_t grid = (uint64_t)sms * per_sm;
-  if (a.m < grid) grid = a.m;
+  const uint64_t rounds = (a.m + grid - 1) / grid;
+  grid = (a.m + rounds - 1) / rounds;
   verify_cta_kernel<V, P><<<(unsigned)(grid ? grid : 1), 32 * V, 0, s>>>(a, PW, GW, next);
   MJ_KERNEL_DONE();
   return MJ_OK;
@@ -1249,6 +1223,18 @@ int cta_lanes_for(uint32_t kmax) {
 int fewest_lanes_for(uint32_t kmax) {
   const int g = wave_lanes_for(kmax);
   return g <= 32 ? g : cta_lanes_for(kmax);
+}
+
+bool verify_supported(uint32_t kmax, int kernel, int lanes) {
+  if (kmax >= (1u << 16)) return false;
+  const int W = verify_words_for(kmax);
+  if (kernel == MJ_VERIFY_KERNEL_TUNED) kernel = MJ_VERIFY_KERNEL_AUTO, lanes = 0;
+  if (kernel == MJ_VERIFY_KERNEL_AUTO) kernel = W <= 8 ? MJ_VERIFY_KERNEL_DIAGONAL : MJ_VERIFY_KERNEL_WAVEFRONT;
+  if (kernel == MJ_VERIFY_KERNEL_DIAGONAL) return W <= 32;
+  if (kernel != MJ_VERIFY_KERNEL_WAVEFRONT) return false;
+  const bool cta = lanes > 32 || (lanes <= 0 && wave_lanes_for(kmax) > 32);
+  const int need = cta ? cta_lanes_for(kmax) : wave_lanes_for(kmax), G = lanes > 0 ? lanes : need;
+  return G >= need && G <= (cta ? kMaxCtaLanes : 32) && !(G & (G - 1));
 }
 
 int launch_verify(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, unsigned long long* next,

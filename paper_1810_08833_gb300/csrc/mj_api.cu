@@ -152,7 +152,6 @@ struct mj_ctx {
   Buf out_i, out_j, out_ed;
   Buf out_t;          // indices of the candidates within K, listed by the band-K pass
   bool out_collect = false;
-  Buf rank_dev;       // the derived rank codes on the device (256 bytes)
   Buf geo;            // pair geometry at the verification order's positions (uint4)
   Buf strgeo;         // per string {offset, length} for the ordering (uint2)
   bool geo_valid = false;
@@ -167,10 +166,10 @@ struct mj_ctx {
   // joins by strings) those the lower bounds leave, in any order
   uint64_t n_list = 0;
   bool list_bounded = false;      // made under the lower bounds of mj_pairs.cu
-  // plain joins by strings (mj_pairs.cu): lengths and ids by rank, ranks by
+  // plain joins by strings (mj_pairs.cu): lengths (as shorts) and ids by rank, ranks by
   // id, windows by rank, first records by string, sorted records, windows,
   // signatures, counters
-  Buf rk_len, rk_len_alt, rk_sid, rk_sid_alt, rk_of, rk_hi, rk_first, rk_delta, rk_scan, rk_len_rank;
+  Buf rk_len, rk_len_alt, rk_sid, rk_sid_alt, rk_of, rk_hi, rk_first, rk_delta, rk_scan, rk_short_rank;
   Buf rk_a, rk_b, rk_skr, rk_win, rk_sig1, rk_sig2, rk_cnt, rk_list;
   Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
   bool by_strings = false;        // this call builds the rank tables
@@ -195,8 +194,8 @@ struct mj_ctx {
   Buf branges;   // bucket counts [32] then ranges [64]
   // CUDA graph of the plain verification stage
   cudaGraphExec_t graph_exec = nullptr;
-  uint64_t graph_sig[27] = {};
-  uint64_t last_sig[27] = {};
+  uint64_t graph_sig[26] = {};
+  uint64_t last_sig[26] = {};
   uint64_t graph_launches = 0;
   // learned first-pass band: parameters P, Adam moments M and V, gradient G, loss
   Buf band;
@@ -222,11 +221,20 @@ struct mj_ctx {
   bool codes_ready = false;   // written in this call (with the planes)
   uint64_t planes_pw = 0;
   uint32_t planes_gw = 0;
+  bool flags_clear = false;   // device flags cleared in this call
+  bool want_cells = false;    // this join takes its band cells from the verification order
   bool have_part = false, have_cand = false, have_out = false;
-  cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  // section timers of mj_join (mj_stats.ms_section)
-  static constexpr int kSections = 9;
+  cudaEvent_t ev[2] = {nullptr, nullptr};   // the autotuner's
+  // section timers of mj_join (mj_stats.ms_section): each section has two
+  // events of its own (what a captured graph records); outside a capture a
+  // point in the stream that several sections share is recorded once, in
+  // marks, and at[i] names the event of the section's start or end
+  static constexpr int kSections = 9, kMarks = 40;
   cudaEvent_t sec_ev[2 * kSections] = {};
+  cudaEvent_t marks[kMarks] = {};
+  int n_marks = 0;
+  uint64_t mark_launches = ~0ull;
+  cudaEvent_t at[2 * kSections] = {};
   bool sec_used[kSections] = {};
   bool timing = false;
   // while the verification stage is captured, section events become event
@@ -252,32 +260,53 @@ struct DeviceGuard {
 
 cudaStream_t S(void* s) { return static_cast<cudaStream_t>(s); }
 
-int readback(mj_ctx* c, const void* d_src, size_t bytes, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small, d_src, bytes, cudaMemcpyDeviceToHost, s));
+// Copies to word `at` of the staging memory and waits for the stream.
+int readback_at(mj_ctx* c, int at, const void* d_src, size_t bytes, cudaStream_t s) {
+  MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + at, d_src, bytes, cudaMemcpyDeviceToHost, s));
   MJ_CUDA_TRY(cudaStreamSynchronize(s));
   return MJ_OK;
 }
 
+int readback(mj_ctx* c, const void* d_src, size_t bytes, cudaStream_t s) { return readback_at(c, 0, d_src, bytes, s); }
+
 // A section's interval runs from its first start to its last stop in a call.
-void record_event(mj_ctx* c, cudaEvent_t e, cudaStream_t s) {
-  if (c->capturing) cudaEventRecordWithFlags(e, s, cudaEventRecordExternal);
-  else cudaEventRecord(e, s);
+// An event at this point of the stream: the last one again when no kernel was
+// launched since (an event costs the host about 1.5 us).
+cudaEvent_t mark(mj_ctx* c, cudaStream_t s) {
+  const uint64_t now = launch_count();
+  if (c->n_marks && c->mark_launches == now) return c->marks[c->n_marks - 1];
+  if (c->n_marks == mj_ctx::kMarks) --c->n_marks;   // more repetitions than events: the last one moves on
+  cudaEventRecord(c->marks[c->n_marks], s);
+  c->mark_launches = now;
+  return c->marks[c->n_marks++];
+}
+void section_event(mj_ctx* c, int k, cudaStream_t s) {
+  if (c->capturing) {
+    c->at[k] = c->sec_ev[k];
+    cudaEventRecordWithFlags(c->sec_ev[k], s, cudaEventRecordExternal);
+  } else {
+    c->at[k] = mark(c, s);
+  }
 }
 void tstart(mj_ctx* c, int i, cudaStream_t s) {
   if (c->timing && !c->sec_used[i]) {
-    record_event(c, c->sec_ev[2 * i], s);
+    section_event(c, 2 * i, s);
     c->sec_used[i] = true;
     if (c->capturing) c->graph_sections |= 1u << i;
   }
 }
 void tstop(mj_ctx* c, int i, cudaStream_t s) {
-  if (c->timing) record_event(c, c->sec_ev[2 * i + 1], s);
+  if (c->timing) section_event(c, 2 * i + 1, s);
 }
 // after a replay of the verification graph: its event nodes timed these
 void mark_graph_sections(mj_ctx* c) {
   if (!c->timing) return;
   for (int i = 0; i < mj_ctx::kSections; ++i)
-    if (c->graph_sections & (1u << i)) c->sec_used[i] = true;
+    if (c->graph_sections & (1u << i)) {
+      c->sec_used[i] = true;
+      c->at[2 * i] = c->sec_ev[2 * i];
+      c->at[2 * i + 1] = c->sec_ev[2 * i + 1];
+    }
 }
 
 void begin_call(mj_ctx* c, bool timing) {
@@ -287,8 +316,9 @@ void begin_call(mj_ctx* c, bool timing) {
   c->codes_ready = false;
   c->planes_pw = c->planes_gw = 0;
   c->work_started = false;
-  c->by_strings = c->list_bounded = false;
+  c->by_strings = c->list_bounded = c->flags_clear = c->want_cells = false;
   c->timing = timing;
+  c->n_marks = 0;
   for (bool& u : c->sec_used) u = false;
   c->launches_at_start = launch_count();
 }
@@ -315,16 +345,12 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
 // a1: alphabet, longest length, q, T, radius bound.
 int derive(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t n, const mj_params* p,
            cudaStream_t s) {
-  MJ_TRY(c->hist.reserve(256 * sizeof(unsigned long long) + 64, s));
-  unsigned long long* hist = c->hist.as<unsigned long long>();
-  unsigned long long* maxlen = hist + 256;
-  MJ_TRY(readback(c, d_offsets + n, sizeof(int64_t), s));
-  const uint64_t nbytes = c->h_small[0];
+  MJ_TRY(c->hist.reserve(258 * sizeof(unsigned long long), s));
+  MJ_TRY(launch_input_stats(d_bytes, d_offsets, n, c->hist.as<unsigned long long>(), s));
+  MJ_TRY(readback(c, c->hist.p, 258 * sizeof(unsigned long long), s));
+  const uint64_t nbytes = c->h_small[257];
   if (nbytes >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;
   if (nbytes > 0 && !d_bytes) return MJ_ERR_ARG;
-  MJ_TRY(launch_byte_histogram(d_bytes, nbytes, hist, s));
-  MJ_TRY(launch_max_length(d_offsets, n, maxlen, s));
-  MJ_TRY(readback(c, hist, 257 * sizeof(unsigned long long), s));
   Derived& d = c->d;
   d = Derived();
   uint32_t sigma = 0;
@@ -357,13 +383,6 @@ int derive(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t
   d.repeats = p->repeats;
   c->stats.n_strings = n;
   c->stats.n_bytes = nbytes;
-  // the rank codes on the device (the text verifier reads B's bytes through
-  // them), staged through pinned memory
-  MJ_TRY(c->rank_dev.reserve(256, s));
-  uint8_t* stage = reinterpret_cast<uint8_t*>(c->h_small) + 3072;
-  MJ_CUDA_TRY(cudaStreamSynchronize(s));   // an earlier copy may still read the staging area
-  memcpy(stage, d.rank, 256);
-  MJ_CUDA_TRY(cudaMemcpyAsync(c->rank_dev.p, stage, 256, cudaMemcpyHostToDevice, s));
   return MJ_OK;
 }
 
@@ -398,11 +417,10 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
   c->n_part = 0;
   if (tiles == 0) return MJ_OK;
   MJ_TRY(c->dev_flags.reserve(64, s));
-  MJ_CUDA_TRY(cudaMemsetAsync(c->dev_flags.p, 0, 64, s));
   MJ_TRY(c->bitmap.reserve(tiles * (kPartTile / 32) * sizeof(uint32_t), s));
   MJ_TRY(c->tile_count.reserve(tiles * sizeof(uint32_t), s));
   MJ_TRY(c->tile_first.reserve(tiles * sizeof(uint32_t), s));
-  MJ_TRY(c->tile_off.reserve(tiles * sizeof(uint32_t) + 16, s));
+  MJ_TRY(c->tile_off.reserve(tiles * sizeof(uint32_t), s));
   MJ_TRY(c->scan_tmp.reserve(scan_temp_bytes(tiles), s));
   c->planes_ready = false;
   c->codes_ready = false;
@@ -412,16 +430,9 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
   if (plane_kmax > 0) {
     GW = plane_guard_words(plane_kmax);
     PW = tiles * (kPartTile / 32) + 2 * (uint64_t)GW;
-    MJ_TRY(c->planes.reserve(PW * d.bits * 4, s));
+    MJ_TRY(c->planes.reserve(PW * plane_stride(d.bits) * 4, s));
     planes = c->planes.as<uint32_t>();
     MJ_TRY(c->codes.reserve(tiles * kPartTile + 64, s));   // written by the first repetition's tiles
-    // guard words before and after every plane's data are zero
-    MJ_CUDA_TRY(cudaMemsetAsync(planes, 0, (size_t)GW * 4, s));
-    for (uint32_t p = 0; p < d.bits; ++p) {
-      const uint64_t from = (uint64_t)p * PW + GW + tiles * (kPartTile / 32);
-      const uint64_t words = (p + 1 < d.bits) ? 2 * (uint64_t)GW : (uint64_t)GW;
-      MJ_CUDA_TRY(cudaMemsetAsync(planes + from, 0, words * 4, s));
-    }
   }
   // parallel repetition (Sec. 2.2): Pi_k has the seed d.seed + k * 0x9E3779B97F4A7C15;
   // the records of repetition k follow those of repetitions 0 .. k-1
@@ -436,7 +447,8 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
     a.codes = (planes && k == 0) ? c->codes.as<uint8_t>() : nullptr;
     MJ_TRY(launch_anchor_flags(a, c->bitmap.as<uint32_t>(), c->tile_count.as<uint32_t>(),
                                c->dev_flags.as<uint32_t>(), k == 0 ? planes : nullptr, PW, GW,
-                               c->tile_first.as<uint32_t>(), s));
+                               c->tile_first.as<uint32_t>(), k == 0, s));
+    c->flags_clear = true;
     tstop(c, 0, s);
     if (planes && k == 0) {
       c->planes_ready = true;
@@ -444,17 +456,14 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
       c->planes_pw = PW;
       c->planes_gw = GW;
     }
-    uint32_t* total = c->tile_off.as<uint32_t>() + tiles;
+    uint32_t* total = c->dev_flags.as<uint32_t>() + 1;   // read back with the flags and the widest window
     MJ_TRY(launch_exclusive_scan_u32(c->tile_count.as<uint32_t>(), c->tile_off.as<uint32_t>(), tiles,
                                      c->scan_tmp.p, total, s));
-    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small, total, 4, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaMemcpyAsync((char*)c->h_small + 8, c->dev_flags.p, 4, cudaMemcpyDeviceToHost, s));
-    if (c->by_strings)
-      MJ_CUDA_TRY(cudaMemcpyAsync((char*)c->h_small + 16, c->rk_cnt.p, 4, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaStreamSynchronize(s));
-    const uint32_t n_anchor = *(uint32_t*)c->h_small;
-    if (c->by_strings) c->rk_widest = *(uint32_t*)((char*)c->h_small + 16);
-    c->stats.device_flags |= *(uint32_t*)((char*)c->h_small + 8);
+    MJ_TRY(readback(c, c->dev_flags.p, 12, s));
+    const uint32_t* got = reinterpret_cast<const uint32_t*>(c->h_small);
+    const uint32_t n_anchor = got[1];
+    c->rk_widest = got[2];
+    c->stats.device_flags |= got[0];
     if (c->stats.device_flags) return MJ_ERR_DEVICE;
     if (n_total + n_anchor >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;   // record indexes are 32-bit
     MJ_TRY(c->recs.grow_keep((n_total + n_anchor + 1) * sizeof(PRec), n_total * sizeof(PRec), s));
@@ -653,26 +662,29 @@ bool bounds_reach(uint64_t N, uint32_t sigma, uint32_t K) {
   return 2.0 * q * K < 18.0 * sqrt((double)N);
 }
 
-constexpr uint64_t kLenRankMax = 1u << 22;   // longest string up to which ranks are found by length from a table
+constexpr uint64_t kBoundsFrom = 1u << 15;    // candidates from which a join by strings may use the lower bounds
+constexpr uint64_t kShortRankMax = 1u << 22;   // longest string up to which ranks are found by length in a table
 
 // Rank tables of a plain join by strings (before its partition step, whose
 // readback also returns the widest window).
 int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s) {
   const size_t b = (size_t)n * 4 + 16;
   for (Buf* x : {&c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi}) MJ_TRY(x->reserve(b, s));
-  MJ_TRY(c->rk_cnt.reserve(128, s));
+  MJ_TRY(c->rk_cnt.reserve(64, s));
+  MJ_CUDA_TRY(cudaMemsetAsync(c->rk_cnt.p, 0, 64, s));
+  MJ_TRY(c->dev_flags.reserve(64, s));
+  MJ_CUDA_TRY(cudaMemsetAsync(c->dev_flags.p, 0, 64, s));
   MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(n), s));
-  const bool by_len = c->d.N <= kLenRankMax;
+  const bool by_len = c->d.N <= kShortRankMax;
   if (by_len) {
-    MJ_TRY(c->rk_len_rank.reserve(((size_t)c->d.N + 1) * 4, s));
-    if (c->fixed_alpha)   // N may be above this input's longest
-      MJ_CUDA_TRY(cudaMemsetAsync(c->rk_len_rank.p, 0xff, ((size_t)c->d.N + 1) * 4, s));
+    MJ_TRY(c->rk_short_rank.reserve(((size_t)c->d.N + 1) * 4, s));
   }
   MJ_TRY(c->rk_first.reserve((size_t)c->d.repeats * ((size_t)n + 1) * 4, s));
-  return launch_string_ranks(d_offsets, n, c->d.K, bits_for(c->d.N), c->rk_len.as<uint32_t>(),
+  return launch_string_ranks(d_offsets, n, c->d.K, (uint32_t)c->d.N, bits_for(c->d.N), c->rk_len.as<uint32_t>(),
                              c->rk_len_alt.as<uint32_t>(), c->rk_sid.as<uint32_t>(), c->rk_sid_alt.as<uint32_t>(),
                              c->sort_tmp.p, c->rk_of.as<uint32_t>(), c->rk_hi.as<uint32_t>(),
-                             by_len ? c->rk_len_rank.as<uint32_t>() : nullptr, c->rk_cnt.as<unsigned int>(), &c->rk_alt,
+                             by_len ? c->rk_short_rank.as<uint32_t>() : nullptr, c->dev_flags.as<unsigned int>() + 2,
+                             &c->rk_alt,
                              s);
 }
 
@@ -688,16 +700,17 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   c->cand_n_part = nr;
   c->cand_n_str = n;
   if (nr == 0) return MJ_OK;
-  // position buckets of width W >= K / 2 in at most 8 of the 32 key bits, so that
-  // at least 24 hash bits keep most (len, key) classes apart (the visits
-  // compare both)
+  // position buckets of width W >= K / 2 in at most 8 key bits; the hash bits
+  // only have to keep most (len, key) classes apart (the visits compare both)
   uint32_t W = d.K / 2 + (d.K & 1u);
   if (d.N / W > 255) W = (uint32_t)(d.N / 255 + 1);
   const int pb_bits = bits_for(d.N / W);
+  // hash bits: two more than the records' logarithm, in whole radix passes
+  const int key_bits = std::min(32, (pb_bits + std::max(14, bits_for(nr)) + 2 + 7) / 8 * 8);
   const uint32_t* sid_of = c->rk_alt ? c->rk_sid_alt.as<uint32_t>() : c->rk_sid.as<uint32_t>();
-  const uint32_t* rlen = c->rk_alt ? c->rk_len_alt.as<uint32_t>() : c->rk_len.as<uint32_t>();
+  const uint32_t* shorts = c->rk_alt ? c->rk_len_alt.as<uint32_t>() : c->rk_len.as<uint32_t>();
   const uint32_t* rank_of = c->rk_of.as<uint32_t>();
-  unsigned long long* cnt = c->rk_cnt.as<unsigned long long>();   // 0 widest, 1 visits, 2 listed, 3-5 totals, 6 listed after the second bound
+  unsigned long long* cnt = c->rk_cnt.as<unsigned long long>();   // 1 sampled, 2 listed, 3-5 totals, 6 listed after the second bound
   MJ_TRY(c->keys.reserve((size_t)nr * 4, s));
   MJ_TRY(c->keys_alt.reserve((size_t)nr * 4, s));
   c->geo_valid = false;   // c->idx is reused by the record sort
@@ -719,27 +732,19 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
                            c->rk_delta.as<uint32_t>(), c->scan_tmp.p, s));
   for (uint32_t k = 0; k < d.repeats; ++k)
     MJ_TRY(launch_rank_keys(c->recs.as<PRec>(), c->rep_first[k], c->rep_first[k + 1],
-                            c->rk_delta.as<uint32_t>() + (uint64_t)k * (n + 1), pb_bits, W, c->keys.as<uint32_t>(),
+                            c->rk_delta.as<uint32_t>() + (uint64_t)k * (n + 1), key_bits - pb_bits, pb_bits, W, c->keys.as<uint32_t>(),
                             c->idx.as<uint32_t>(), s));
   bool alt = false;
   MJ_TRY(radix_sort_u32(c->keys.as<uint32_t>(), c->keys_alt.as<uint32_t>(), c->idx.as<uint32_t>(),
-                        c->idx_alt.as<uint32_t>(), nr, 0, 32, c->sort_tmp.p, &alt, s));
-  const RankTables rt{c->rk_hi.as<uint32_t>(), rlen, d.N <= kLenRankMax ? c->rk_len_rank.as<uint32_t>() : nullptr,
+                        c->idx_alt.as<uint32_t>(), nr, 0, key_bits, c->sort_tmp.p, &alt, s));
+  const RankTables rt{c->rk_hi.as<uint32_t>(), shorts, d.N <= kShortRankMax ? c->rk_short_rank.as<uint32_t>() : nullptr,
                       (uint32_t)d.N, n};
   MJ_TRY(launch_rank_windows(alt ? c->idx_alt.as<uint32_t>() : c->idx.as<uint32_t>(),
                              alt ? c->keys_alt.as<uint32_t>() : c->keys.as<uint32_t>(), nr, c->recs.as<PRec>(), rank_of,
                              rt, d.K, W, pb_bits, rb, c->rk_a.as<uint4>(), c->rk_b.as<uint2>(),
-                             c->rk_skr.as<uint64_t>(), c->rk_win.as<uint4>(), cnt + 1, s));
+                             c->rk_skr.as<uint64_t>(), c->rk_win.as<uint4>(), s));
   tstop(c, 2, s);
   tstart(c, 4, s);
-  // The lower bounds read every input byte once; without them a candidate
-  // costs a dynamic program.  They pay when the windows hold more than one
-  // record per 32 bytes of input.
-  const uint64_t min_visits = bounds_reach(d.N, d.sigma, d.K) ? c->stats.n_bytes / 32 : ~0ull;
-  const SigShape g = signature_shape(d.sigma, c->code_counts);
-  if (min_visits != ~0ull)
-    MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_visits, c->rk_sig1.as<uint4>(),
-                             c->rk_sig2.as<uint32_t>(), s));
   PairArgs a;
   a.recs = c->recs.as<PRec>();
   a.first = c->rk_first.as<uint32_t>();
@@ -747,25 +752,41 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   a.A = c->rk_a.as<uint4>();
   a.B = c->rk_b.as<uint2>();
   a.sid_of = sid_of;
-  a.rlen = rlen;
+  a.shorts = shorts;
+  a.longest = (uint32_t)d.N;
   a.hi = c->rk_hi.as<uint32_t>();
   a.sig1 = c->rk_sig1.as<uint4>();
-  a.visits = cnt + 1;
-  a.min_visits = min_visits;
+  a.sampled = cnt + 1;
   a.n = n;
   a.reps = d.repeats;
   a.K = d.K;
-  a.q1 = g.q1;
   a.rb = rb;
   a.out_count = cnt + 2;
   a.totals = cnt + 3;
+  // The lower bounds read every input byte once (about 2 ps per byte); without
+  // them an unrelated candidate costs its dynamic program (100-300 ps, and
+  // less while all candidates are in flight at once).  They are used from one
+  // candidate per 96 bytes on, estimated from a sample of the strings, where
+  // they can exceed K at all.
+  const bool bounds = bounds_reach(d.N, d.sigma, d.K);
+  const SigShape g = signature_shape(d.sigma, c->code_counts);
+  const uint64_t stride = std::max<uint32_t>(1, n / kSampleStrings);
+  const uint64_t min_sampled = bounds ? std::max<uint64_t>(c->stats.n_bytes / 96, kBoundsFrom) / stride : ~0ull;
+  a.min_sampled = min_sampled;
+  a.q1 = g.q1;
+  if (bounds) {
+    MJ_TRY(launch_string_sample(a, c->rk_widest, s));
+    MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_sampled,
+                             c->rk_sig1.as<uint4>(), c->rk_sig2.as<uint32_t>(), s));
+  }
   ListArgs l;
   l.in_count = a.out_count;
   l.sig2 = c->rk_sig2.as<uint4>();
   l.sid_of = sid_of;
-  l.rlen = rlen;
-  l.visits = a.visits;
-  l.min_visits = min_visits;
+  l.shorts = shorts;
+  l.longest = (uint32_t)d.N;
+  l.sampled = a.sampled;
+  l.min_sampled = min_sampled;
   l.K = d.K;
   l.q2 = g.q2;
   l.out_count = cnt + 6;
@@ -790,6 +811,7 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
     if (tries > 1) return MJ_ERR_DEVICE;   // both lists were counted in full
     cap1 = std::max<uint64_t>(cap1, c->h_small[0]);
     cap2 = std::max<uint64_t>(cap2, std::min<uint64_t>(c->h_small[4], c->h_small[0]));
+    MJ_CUDA_TRY(cudaMemsetAsync(cnt + 2, 0, 40, s));
   }
   tstop(c, 4, s);
   c->n_list = c->h_small[4];
@@ -803,10 +825,13 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
 
 // a8 on arbitrary pairs (rank codes from c->d).
 // Device flags and verification counters cleared for this call (once), on s.
-int verify_prep(mj_ctx* c, cudaStream_t s) {
+// *fresh: the counters have just been cleared, the work counter (1) included.
+int verify_prep(mj_ctx* c, cudaStream_t s, bool* fresh = nullptr) {
   MJ_TRY(c->dev_flags.reserve(64, s));
-  MJ_CUDA_TRY(cudaMemsetAsync(c->dev_flags.p, 0, 64, s));
+  // a join's partition step has cleared and checked the flags in this call
+  if (!c->flags_clear) MJ_CUDA_TRY(cudaMemsetAsync(c->dev_flags.p, 0, 64, s));
   MJ_TRY(c->small.reserve(128, s));
+  if (fresh) *fresh = !c->work_started;
   if (!c->work_started) {
     // counters 0-5 and the output count (8) start at zero once per call;
     // 6 and 7 hold values read back before verification starts
@@ -822,7 +847,7 @@ int ensure_planes(mj_ctx* c, const uint8_t* d_bytes, uint32_t kmax, cudaStream_t
   const uint32_t GW = plane_guard_words(kmax);
   if (c->planes_ready && c->planes_gw >= GW) return MJ_OK;
   const uint64_t nbytes = c->stats.n_bytes, PW = (nbytes + 31) / 32 + 2 * (uint64_t)GW;
-  MJ_TRY(c->planes.reserve(PW * c->d.bits * 4, s));
+  MJ_TRY(c->planes.reserve(PW * plane_stride(c->d.bits) * 4, s));
   RankTable rt;
   memcpy(rt.r, c->d.rank, 256);
   MJ_TRY(c->codes.reserve(nbytes + 64, s));
@@ -848,7 +873,8 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
   MJ_TRY(ensure_planes(c, d_bytes, kmax, s));
   const uint32_t GW = c->planes_gw;
   const uint64_t PW = c->planes_pw;
-  if (prep) MJ_TRY(verify_prep(c, s));
+  bool fresh = false;
+  if (prep) MJ_TRY(verify_prep(c, s, &fresh));
   VerifyArgs a;
   a.planes = c->planes.as<uint32_t>();
   a.bits = d.bits;
@@ -870,7 +896,6 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
   a.work = c->small.as<unsigned long long>() + 2;
   a.dev_flags = c->dev_flags.as<uint32_t>();
   if (order && order == c->idx.as<uint32_t>() && c->geo_valid) a.pair_geo = c->geo.as<uint4>();
-  a.rank_table = c->rank_dev.as<uint8_t>();
   a.codes = c->codes_ready ? c->codes.as<uint8_t>() : nullptr;
   a.nbytes = nbytes;
   if (c->out_collect) {   // the join's band-K pass lists the pairs within K
@@ -884,7 +909,8 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
     kk = MJ_VERIFY_KERNEL_AUTO;
     ll = 0;
   }
-  MJ_TRY(launch_verify(a, PW, GW, kmax, next ? next : c->small.as<unsigned long long>() + 1, s, kk, ll));
+  MJ_TRY(launch_verify(a, PW, GW, kmax, next ? next : c->small.as<unsigned long long>() + 1, s, kk, ll,
+                       fresh && !next));
   tstop(c, 6, s);
   return MJ_OK;
 }
@@ -893,6 +919,9 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
 // lengths into c->idx), with the pairs' floor(log2) length buckets: counts in
 // branges words [0, 32), [start, end) ranges in words [32, 96).
 constexpr size_t kOrderScratchAt = 128;   // words of branges before the ordering scratch
+// Pairs from which a list is verified longest first: more than are in flight at
+// once, on two lanes each or on a warp and more.
+constexpr uint64_t kOrderFrom = 29184, kOrderFromWide = 1024;
 constexpr size_t kOrderKeptAt = 100;      // word of branges with the number of pairs in the order
 
 // The lower bounds (mj_pairs.cu) on a list of m pairs cost a pass over the
@@ -900,9 +929,9 @@ constexpr size_t kOrderKeptAt = 100;      // word of branges with the number of 
 // 100-300 ps for the dynamic program of an unrelated pair).
 // A list that was made under the bounds needs them no more, and a band that
 // the verifier refuses must leave the results unwritten.
-bool bounds_pay(const mj_ctx* c, uint64_t m, uint32_t kmax) {
+bool bounds_pay(const mj_ctx* c, uint64_t m, uint32_t kmax, uint64_t bytes_per_pair = 16) {
   if (!bounds_reach(c->d.N, c->d.sigma, kmax)) return false;
-  if (c->list_bounded || m <= c->stats.n_bytes / 16) return false;
+  if (c->list_bounded || m <= c->stats.n_bytes / bytes_per_pair) return false;
   if (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned)
     return verify_supported(kmax, (int)c->vcfg.kernel, (int)c->vcfg.lanes);
   for (int b = 0; b < kLenBuckets; ++b)
@@ -967,6 +996,9 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
     MJ_TRY(ensure_planes(c, d_bytes, K, s));
     MJ_TRY(pair_bounds(c, d_offsets, ci, cj, nullptr, m, K, ed, s));
   }
+  // few enough pairs to be in flight all at once run in the given order
+  if (!bounds && !c->want_cells && m <= (K <= 255 ? kOrderFrom : kOrderFromWide) && (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned))
+    return verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s);
   MJ_TRY(pair_order(c, ci, cj, d_offsets, m, bounds ? c->rejected.as<uint8_t>() : nullptr, &order, &kept, s));
   if (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned)
     return verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, nullptr, kept);
@@ -1007,16 +1039,17 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
     for (int b = 0; b < kLenBuckets; ++b) plan = plan * 1000003u + c->tuned_kernel[b] * 64u + c->tuned_lanes[b];
   }
   // everything the captured launches read as a parameter: buffers, sizes, plan
-  const uint64_t sig[27] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
+  const uint64_t sig[26] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
                             (uint64_t)ed, (uint64_t)c->planes.p, c->planes_pw, c->d.bits, plan,
                             (uint64_t)c->small.p, (uint64_t)c->idx.p, (uint64_t)c->branges.p,
                             (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0, (uint64_t)c->geo.p,
                             c->stats.n_bytes, c->stats.n_strings, c->planes_gw,
                             (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
-                            (uint64_t)c->rank_dev.p, (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p,
+                            (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p,
                             (uint64_t)c->rejected.p, bounds_pay(c, m, K) ? 1ull : 0ull};
   if (c->graph_exec && memcmp(sig, c->graph_sig, sizeof(sig)) == 0) {
     MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
+    c->mark_launches = ~0ull;   // the graph's kernels are not counted as launches
     mark_graph_sections(c);
     c->launches_at_start -= c->graph_launches;   // kernels replayed by the graph
     return MJ_OK;
@@ -1053,6 +1086,7 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
   c->graph_launches = launch_count() - before;
   memcpy(c->graph_sig, sig, sizeof(sig));
   MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
+  c->mark_launches = ~0ull;
   mark_graph_sections(c);
   return MJ_OK;
 }
@@ -1096,7 +1130,7 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
     if (!c->band_ready) return MJ_ERR_STATE;
     MJ_TRY(order_buffers(c, m, s));
     const uint32_t *order, *kept;
-    const bool bounds = bounds_pay(c, m, K);
+    const bool bounds = bounds_pay(c, m, K, 256);   // a rejected pair also spares the network
     if (bounds) {
       MJ_TRY(bounds_buffers(c, m, s));
       MJ_TRY(ensure_planes(c, d_bytes, K, s));
@@ -1254,6 +1288,13 @@ int mj_create(mj_ctx** ctx, int device) {
       return MJ_ERR_CUDA;
     }
   }
+  for (auto& e : c->marks) {
+    if (cudaEventCreate(&e) != cudaSuccess) {
+      cudaGetLastError();
+      mj_destroy(c);
+      return MJ_ERR_CUDA;
+    }
+  }
   for (auto& e : c->ev) {
     if (cudaEventCreate(&e) != cudaSuccess) {
       cudaGetLastError();
@@ -1282,9 +1323,9 @@ void mj_destroy(mj_ctx* c) {
   Buf* bufs[] = {&c->hist, &c->dev_flags, &c->small, &c->bitmap, &c->tile_count, &c->tile_off, &c->scan_tmp,
                  &c->tile_first,
                  &c->recs, &c->keys, &c->keys_alt, &c->idx, &c->idx_alt, &c->sort_tmp, &c->srec, &c->pair_count, &c->pair_off, &c->pairs, &c->pairs_alt,
-                 &c->uflags, &c->uoffs, &c->cand_i, &c->cand_j, &c->pairbm, &c->planes, &c->ed, &c->out_t, &c->geo, &c->strgeo, &c->codes, &c->rank_dev,
+                 &c->uflags, &c->uoffs, &c->cand_i, &c->cand_j, &c->pairbm, &c->planes, &c->ed, &c->out_t, &c->geo, &c->strgeo, &c->codes,
                  &c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi, &c->rk_first, &c->rk_delta,
-                 &c->rk_scan, &c->rk_len_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
+                 &c->rk_scan, &c->rk_short_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
                  &c->out_i, &c->out_j, &c->out_ed, &c->in_bytes, &c->in_offsets, &c->branges,
                  &c->band, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
                  &c->franges, &c->fnext, &c->fcnt, &c->ed_first};
@@ -1297,6 +1338,8 @@ void mj_destroy(mj_ctx* c) {
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
   for (auto& e : c->sec_ev)
+    if (e) cudaEventDestroy(e);
+  for (auto& e : c->marks)
     if (e) cudaEventDestroy(e);
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   if (c->h_small) cudaFreeHost(c->h_small);
@@ -1413,9 +1456,7 @@ int mj_candidates_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, void* stream) {
   }
   const size_t n = c->n_cand;
   if (!n) return MJ_OK;
-  if (d_i) MJ_CUDA_TRY(cudaMemcpyAsync(d_i, c->cand_i.p, n * 4, cudaMemcpyDeviceToDevice, s));
-  if (d_j) MJ_CUDA_TRY(cudaMemcpyAsync(d_j, c->cand_j.p, n * 4, cudaMemcpyDeviceToDevice, s));
-  return MJ_OK;
+  return launch_copy_words(c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(), nullptr, n, d_i, d_j, nullptr, s);
 }
 
 int mj_set_alphabet(mj_ctx* c, const uint8_t* h_present, uint64_t N) {
@@ -1670,23 +1711,24 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
   p = &eff;
   begin_call(c, true);
   c->have_part = c->have_cand = c->have_out = c->have_features = c->cand_on_demand = false;
-  MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
+  cudaEvent_t at[5];
+  at[0] = mark(c, s);
   MJ_TRY(derive(c, d_bytes, d_offsets, n, p, s));
-  MJ_CUDA_TRY(cudaEventRecord(c->ev[1], s));
+  at[1] = mark(c, s);
   // Plain joins go string by string.  The general path (one walk over all
   // records, dedup by a bitmap over all pairs or a sort) serves learned mode
   // and the candidates' features (they need multiplicities), the key check, a
-  // forced dedup, and windows too wide for a bitmap in shared memory; it is
-  // also the faster one for few strings, whose joins its fewer launches decide
-  // (1,000 strings: 518 us against 602) and whose candidates are few (50,000
-  // reads: 4.31 ms against 4.37).
-  constexpr uint32_t kStringsFrom = 1u << 16;
+  // forced dedup, and windows too wide for a bitmap in shared memory.  Measured
+  // (general, by strings; us per join): 1,000 short reads 428, 410; 10,000 reads
+  // 1603, 1674; 6,000 text-like strings 1266, 850; 20,000 protein-like 1086,
+  // 1004; 10,000 of bytes, with hardly an unrelated candidate, 1018, 1145.  How
+  // many candidates there are is not known before the records are grouped.
   const uint32_t general = MJ_FLAG_FEATURES | MJ_FLAG_KEY_CHECK | MJ_FLAG_DEDUP_SORT | MJ_FLAG_DEDUP_BITMAP;
-  c->by_strings = p->verify_mode == MJ_VERIFY_PLAIN && !(p->flags & general) && p->K > 0 && n >= kStringsFrom;
+  c->by_strings = p->verify_mode == MJ_VERIFY_PLAIN && !(p->flags & general) && p->K > 0 && n > 1;
   if (c->by_strings) MJ_TRY(string_ranks(c, d_offsets, n, s));
   MJ_TRY(partition(c, d_bytes, d_offsets, n, nullptr, p->K, s));
   c->have_part = true;
-  MJ_CUDA_TRY(cudaEventRecord(c->ev[2], s));
+  at[2] = mark(c, s);
   const bool strings = c->by_strings && string_pairs_fit(c->rk_widest);
   if (strings) {
     MJ_TRY(string_candidates(c, d_offsets, n, s));
@@ -1694,23 +1736,21 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
     MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,
                       p->verify_mode == MJ_VERIFY_LEARNED || (p->flags & MJ_FLAG_FEATURES)));
     c->n_list = c->n_cand;
+    c->want_cells = true;
   }
   c->have_cand = true;
-  MJ_CUDA_TRY(cudaEventRecord(c->ev[3], s));
+  at[3] = mark(c, s);
   const uint64_t m = c->n_list;
   c->n_out = 0;
   if (m) {
     MJ_TRY(verify_stage(c, d_bytes, d_offsets, n, p, s));
     tstart(c, 7, s);
-    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small, c->small.as<unsigned long long>() + 8, 8, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + 1, c->small.as<unsigned long long>() + 9, 8, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + 2, c->dev_flags.p, 4, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + 3, c->small.as<unsigned long long>() + 2, 8, cudaMemcpyDeviceToHost, s));
-    MJ_CUDA_TRY(cudaStreamSynchronize(s));
-    const uint64_t no = c->h_small[0];
-    if (!strings) c->stats.band_cells = c->h_small[1];
-    c->stats.device_flags |= *(uint32_t*)(c->h_small + 2);
-    c->stats.verify_word_columns = c->h_small[3];
+    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small, c->small.p, 80, cudaMemcpyDeviceToHost, s));
+    MJ_TRY(readback_at(c, 10, c->dev_flags.p, 4, s));
+    const uint64_t no = c->h_small[8];
+    if (!strings) c->stats.band_cells = c->h_small[9];
+    c->stats.device_flags |= *(uint32_t*)(c->h_small + 10);
+    c->stats.verify_word_columns = c->h_small[2];
     if (no > m) return MJ_ERR_DEVICE;
     MJ_TRY(c->out_i.reserve((size_t)no * 4 + 16, s));
     MJ_TRY(c->out_j.reserve((size_t)no * 4 + 16, s));
@@ -1735,16 +1775,16 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
     tstop(c, 7, s);
     c->n_out = no;
   }
-  MJ_CUDA_TRY(cudaEventRecord(c->ev[4], s));
-  MJ_CUDA_TRY(cudaEventSynchronize(c->ev[4]));
+  at[4] = mark(c, s);
+  MJ_CUDA_TRY(cudaStreamSynchronize(s));
   c->stats.n_output = c->n_out;
-  c->stats.ms_derive = elapsed(c->ev[0], c->ev[1]);
-  c->stats.ms_partition = elapsed(c->ev[1], c->ev[2]);
-  c->stats.ms_join_filter = elapsed(c->ev[2], c->ev[3]);
-  c->stats.ms_verify = elapsed(c->ev[3], c->ev[4]);
-  c->stats.ms_total = elapsed(c->ev[0], c->ev[4]);
+  c->stats.ms_derive = elapsed(at[0], at[1]);
+  c->stats.ms_partition = elapsed(at[1], at[2]);
+  c->stats.ms_join_filter = elapsed(at[2], at[3]);
+  c->stats.ms_verify = elapsed(at[3], at[4]);
+  c->stats.ms_total = elapsed(at[0], at[4]);
   for (int i = 0; i < mj_ctx::kSections; ++i)
-    c->stats.ms_section[i] = c->sec_used[i] ? elapsed(c->sec_ev[2 * i], c->sec_ev[2 * i + 1]) : 0.f;
+    c->stats.ms_section[i] = c->sec_used[i] ? elapsed(c->at[2 * i], c->at[2 * i + 1]) : 0.f;
   c->stats.n_launches = launch_count() - c->launches_at_start;
   if (c->stats.device_flags) return MJ_ERR_DEVICE;
   c->have_out = true;
@@ -1965,10 +2005,8 @@ int mj_result_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, uint32_t* d_ed, void
   cudaStream_t s = S(stream);
   const size_t n = c->n_out;
   if (!n) return MJ_OK;
-  if (d_i) MJ_CUDA_TRY(cudaMemcpyAsync(d_i, c->out_i.p, n * 4, cudaMemcpyDeviceToDevice, s));
-  if (d_j) MJ_CUDA_TRY(cudaMemcpyAsync(d_j, c->out_j.p, n * 4, cudaMemcpyDeviceToDevice, s));
-  if (d_ed) MJ_CUDA_TRY(cudaMemcpyAsync(d_ed, c->out_ed.p, n * 4, cudaMemcpyDeviceToDevice, s));
-  return MJ_OK;
+  return launch_copy_words(c->out_i.as<uint32_t>(), c->out_j.as<uint32_t>(), c->out_ed.as<uint32_t>(), n, d_i, d_j,
+                           d_ed, s);
 }
 
 int mj_join_host(mj_ctx* c, const uint8_t* h_bytes, const int64_t* h_offsets, uint32_t n, const mj_params* p,

@@ -28,40 +28,51 @@
 namespace mj {
 namespace {
 
-__global__ void byte_hist_kernel(const uint8_t* __restrict__ bytes, uint64_t nbytes,
-                                 unsigned long long* __restrict__ hist) {
-  __shared__ uint32_t s[256];
-  s[threadIdx.x] = 0;
-  __syncthreads();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * 16;
-  for (uint64_t base = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 16; base < nbytes; base += stride) {
-    if (base + 16 <= nbytes && (((uintptr_t)(bytes + base)) & 15) == 0) {
-      uint4 v = __ldg(reinterpret_cast<const uint4*>(bytes + base));
-      uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) atomicAdd(&s[(w[k] >> (8 * b)) & 255u], 1u);
-      }
-    } else {
-      for (uint64_t g = base; g < base + 16 && g < nbytes; ++g) atomicAdd(&s[__ldg(bytes + g)], 1u);
-    }
-  }
-  __syncthreads();
-  if (s[threadIdx.x]) atomicAdd(&hist[threadIdx.x], (unsigned long long)s[threadIdx.x]);
-}
-
-__global__ void max_len_kernel(const int64_t* __restrict__ off, uint32_t n, unsigned long long* __restrict__ out) {
+// out[b], b < 256: 0 for byte values that do not occur, else about a sixteenth
+// of their count, at least 1 (presence decides the alphabet; the counts only
+// weigh the buckets of the distance bounds); out[256] = the longest string's
+// length, out[257] = offsets[n], the input's size, which the kernel reads
+// itself so that the host need not wait for it first.  Sizes from 2^32 on are
+// refused by the host, and a null input has no bytes to read.
+// A plain flag store per byte instead of an atomic count: 250 MB of DNA took
+// 48 us with atomics (four counters take all of a warp's updates).
+__global__ void __launch_bounds__(256) input_stats_kernel(const uint8_t* __restrict__ bytes,
+                                                          const int64_t* __restrict__ offsets, uint32_t n,
+                                                          unsigned long long* __restrict__ out) {
+  __shared__ uint32_t s_seen[256], s_cnt[256];
+  s_seen[threadIdx.x] = s_cnt[threadIdx.x] = 0;
+  const uint64_t nbytes = (uint64_t)__ldg(offsets + n);
+  const uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, threads = (uint64_t)gridDim.x * blockDim.x;
+  if (t0 == 0) out[257] = nbytes;
   unsigned long long m = 0;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    int64_t L = off[i + 1] - off[i];
+  for (uint64_t i = t0; i < n; i += threads) {
+    const int64_t L = __ldg(offsets + i + 1) - __ldg(offsets + i);
     if ((unsigned long long)L > m) m = (unsigned long long)L;
   }
   for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long y = __shfl_down_sync(0xffffffffu, m, o);
+    const unsigned long long y = __shfl_down_sync(0xffffffffu, m, o);
     m = y > m ? y : m;
   }
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(out + 256, m);
+  if (!bytes || nbytes >= (1ull << 32) || (uint64_t)blockIdx.x * blockDim.x * 16 >= nbytes) return;   // uniform
+  __syncthreads();
+  const bool vec = ((uintptr_t)bytes & 15) == 0;
+  uint32_t it = 0;
+  for (uint64_t base = t0 * 16; base < nbytes; base += threads * 16, ++it) {
+    if (base + 16 <= nbytes && vec) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(bytes + base));
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) s_seen[(w[k] >> (8 * b)) & 255u] = 1u;
+      if (!(it & 15)) atomicAdd(&s_cnt[w[it >> 4 & 3] & 255u], 1u);   // one byte of the 16
+    } else {
+      for (uint64_t g = base; g < base + 16 && g < nbytes; ++g) s_seen[__ldg(bytes + g)] = 1u;
+    }
+  }
+  __syncthreads();
+  if (s_seen[threadIdx.x]) atomicAdd(&out[threadIdx.x], (unsigned long long)max(s_cnt[threadIdx.x], 1u));
 }
 
 __global__ void max_u32_kernel(const uint32_t* __restrict__ v, uint64_t n, unsigned int* __restrict__ out) {
@@ -693,6 +704,18 @@ __global__ void pack_pairs_kernel(const uint32_t* __restrict__ pi, const uint32_
   }
 }
 
+// Up to three arrays of n words copied by one launch (three copies cost the host
+// about 5 us each); null outputs are skipped.
+__global__ void copy_words_kernel(const uint32_t* __restrict__ a, const uint32_t* __restrict__ b,
+                                  const uint32_t* __restrict__ c, uint64_t n, uint32_t* __restrict__ oa,
+                                  uint32_t* __restrict__ ob, uint32_t* __restrict__ oc) {
+  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
+    if (oa) oa[t] = a[t];
+    if (ob) ob[t] = b[t];
+    if (oc) oc[t] = c[t];
+  }
+}
+
 unsigned grid_for(uint64_t n, int threads = 256) {
   uint64_t g = (n + threads - 1) / threads;
   uint64_t cap = (uint64_t)kNumSMsHint * 32;
@@ -701,10 +724,10 @@ unsigned grid_for(uint64_t n, int threads = 256) {
 
 }  // namespace
 
-int launch_byte_histogram(const uint8_t* bytes, uint64_t nbytes, unsigned long long* hist, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned long long), s));
-  if (!nbytes) return MJ_OK;
-  byte_hist_kernel<<<grid_for((nbytes + 15) / 16), 256, 0, s>>>(bytes, nbytes, hist);
+int launch_input_stats(const uint8_t* bytes, const int64_t* offsets, uint32_t n, unsigned long long* out,
+                       cudaStream_t s) {
+  MJ_CUDA_TRY(cudaMemsetAsync(out, 0, 258 * sizeof(unsigned long long), s));
+  input_stats_kernel<<<kNumSMsHint * 8, 256, 0, s>>>(bytes, offsets, n, out);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
@@ -713,14 +736,6 @@ int launch_max_u32(const uint32_t* v, uint64_t n, unsigned int* out, cudaStream_
   MJ_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(unsigned int), s));
   if (!n) return MJ_OK;
   max_u32_kernel<<<grid_for(n), 256, 0, s>>>(v, n, out);
-  MJ_KERNEL_DONE();
-  return MJ_OK;
-}
-
-int launch_max_length(const int64_t* offsets, uint32_t n, unsigned long long* out, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(unsigned long long), s));
-  if (!n) return MJ_OK;
-  max_len_kernel<<<grid_for(n), 256, 0, s>>>(offsets, n, out);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
@@ -910,6 +925,14 @@ int launch_gather_output_pairs(const uint32_t* out_t, uint64_t n, int nb, const 
   MJ_TRY(radix_sort_u64(keys, keys_alt, vals, vals_alt, n, 0, 2 * nb, temp, &alt, s));
   gather_out_pairs_kernel<<<grid_for(n), 256, 0, s>>>(alt ? keys_alt : keys, alt ? vals_alt : vals, n, nb, ed, oi, oj,
                                                       oed);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+int launch_copy_words(const uint32_t* a, const uint32_t* b, const uint32_t* c, uint64_t n, uint32_t* oa, uint32_t* ob,
+                      uint32_t* oc, cudaStream_t s) {
+  if (!n || (!oa && !ob && !oc)) return MJ_OK;
+  copy_words_kernel<<<grid_for(n), 256, 0, s>>>(a, b, c, n, oa, ob, oc);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

@@ -74,10 +74,10 @@ struct Derived {
 // ---------------------------------------------------------------- kernels (launchers)
 // All launchers are stream-ordered and return MJ_OK or MJ_ERR_CUDA.
 
-// a1: 256-bin byte histogram (u64 counts) and the longest string length.
-int launch_byte_histogram(const uint8_t* bytes, uint64_t nbytes, unsigned long long* hist,
-                          cudaStream_t s);
-int launch_max_length(const int64_t* offsets, uint32_t n, unsigned long long* out, cudaStream_t s);
+// a1: out[0 .. 255] non-zero for the byte values present (a sampled count),
+// out[256] = the longest string's length, out[257] = the input's size.
+int launch_input_stats(const uint8_t* bytes, const int64_t* offsets, uint32_t n, unsigned long long* out,
+                       cudaStream_t s);
 // *out = max of v[0 .. n-1] (0 when n = 0)
 int launch_max_u32(const uint32_t* v, uint64_t n, unsigned int* out, cudaStream_t s);
 
@@ -130,12 +130,14 @@ struct PartitionArgs {
 constexpr int kPartTile = 2048;  // byte positions per CTA tile
 uint64_t partition_num_tiles(uint64_t nbytes);
 // planes (nullable): also writes the rank-code bit-planes of the tile for the
-// verifier (plane p word guard_words + g/32 holds positions g .. g+31), and
+// verifier (plane p's word for positions g .. g+31 at plane_at(guard_words +
+// g/32, p)), and
 // with a.codes the rank codes themselves (a.codes[g] for position g; the
-// buffer covers whole tiles).
+// buffer covers whole tiles).  With first_call, dev_flags words 0 and 1 and the
+// planes' guard words are cleared before.
 int launch_anchor_flags(const PartitionArgs& a, uint32_t* bitmap, uint32_t* tile_count,
                         uint32_t* dev_flags, uint32_t* planes, uint64_t plane_words,
-                        uint32_t guard_words, uint32_t* tile_first, cudaStream_t s);
+                        uint32_t guard_words, uint32_t* tile_first, bool first_call, cudaStream_t s);
 // a4: one partition record per anchor, in position order (so string order),
 // from the bitmap and the per-tile list offsets; key = (len, H61(substring)).
 int launch_partition_records(const PartitionArgs& a, const uint32_t* bitmap, const uint32_t* tile_offset,
@@ -166,15 +168,17 @@ int radix_sort_u32(uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t*
                    uint64_t n, int bit_lo, int bit_hi, void* temp, bool* result_in_alt,
                    cudaStream_t s);
 
-// a5-a7 of a plain join, string by string in order of length (mj_pairs.cu).
-// Ranks: strings sorted by length (ties by id).  len/sid (n entries each and
-// their alternates) end sorted, in the alternates if *in_alt; rank_of[id],
-// hi[rank] = the last rank within K of its length; len_rank[l] (nullable) = the
-// first rank of length l or more; *widest = the most ranks above its own that
-// a string can pair with.
-int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, int len_bits, uint32_t* len, uint32_t* len_alt,
-                        uint32_t* sid, uint32_t* sid_alt, void* temp, uint32_t* rank_of, uint32_t* hi,
-                        uint32_t* len_rank, unsigned int* widest, bool* in_alt, cudaStream_t s);
+// a5-a7 of a plain join, string by string from the longest (mj_pairs.cu).
+// The caller clears every counter these steps add to.
+// Ranks: strings from the longest to the shortest (ties by id); short = longest
+// - length.  shorts/sid (n entries each and their alternates) end sorted, in the
+// alternates if *in_alt; rank_of[id], hi[rank] = the last rank within K of its
+// length; short_rank[l] (nullable), l = 0 .. longest = the first rank of short l
+// or more; *widest = the most ranks above its own that a string can pair with.
+int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t longest, int len_bits,
+                        uint32_t* shorts, uint32_t* shorts_alt, uint32_t* sid, uint32_t* sid_alt, void* temp,
+                        uint32_t* rank_of, uint32_t* hi, uint32_t* short_rank, unsigned int* widest, bool* in_alt,
+                        cudaStream_t s);
 // first[i], i = 0 .. n: base + the anchors before string i in the bitmap
 // (`total` anchors in all).
 int launch_string_first(const int64_t* offsets, uint32_t n, uint64_t nbytes, const uint32_t* bitmap,
@@ -185,22 +189,21 @@ int launch_rank_order(const uint32_t* first, const uint32_t* sid_of, const uint3
                       uint32_t* rfirst, uint32_t* delta, void* temp, cudaStream_t s);
 // Sort keys and record indices of records [t0, t1) of one repetition (delta:
 // its n + 1 words) at their places by rank.
-int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int pb_bits, uint32_t W,
-                     uint32_t* keys, uint32_t* vals, cudaStream_t s);
+int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int hash_bits, int pb_bits,
+                     uint32_t W, uint32_t* keys, uint32_t* vals, cudaStream_t s);
 // Rank bits of a visit word when a visit fits 16 bytes, else 0 (B is then used).
 int visit_rank_bits(uint64_t longest, uint32_t n);
 // From the sorted keys and indices: A, B, skr (n_rec entries) and the windows
-// of every record (2 entries each, at the record's own place); *visits = the
-// records in all windows.
+// of every record (2 entries each, at the record's own place).
 struct RankTables {
   const uint32_t* hi;
-  const uint32_t* rlen;       // lengths by rank
-  const uint32_t* len_rank;   // nullable
+  const uint32_t* shorts;
+  const uint32_t* short_rank;   // nullable
   uint32_t longest, n;
 };
 int launch_rank_windows(const uint32_t* idx, const uint32_t* keys, uint32_t n_rec, const PRec* recs,
                         const uint32_t* rank_of, const RankTables& rt, uint32_t K, uint32_t W, int pb_bits, int rb,
-                        uint4* A, uint2* B, uint64_t* skr, uint4* win, unsigned long long* visits, cudaStream_t s);
+                        uint4* A, uint2* B, uint64_t* skr, uint4* win, cudaStream_t s);
 // Lower bounds on the edit distance: gram lengths of the two levels and the
 // buckets of single symbols (by rank code).
 struct SigShape {
@@ -211,10 +214,10 @@ uint32_t signature_grams(uint32_t sigma, uint32_t want);   // the shortest q (<=
 SigShape signature_shape(uint32_t sigma, const uint64_t* counts_by_code);
 size_t sig1_bytes(uint32_t n);
 size_t sig2_bytes(uint32_t n);
-// Signatures by rank (sid_of) or id (null).  With visits (nullable), does
-// nothing when *visits <= min_visits.
+// Signatures by rank (sid_of) or id (null).  With sampled (nullable), does
+// nothing when *sampled <= min_sampled.
 int launch_signatures(const uint8_t* codes, const int64_t* offsets, const uint32_t* sid_of, uint32_t n,
-                      const SigShape& g, const unsigned long long* visits, uint64_t min_visits, uint4* sig1,
+                      const SigShape& g, const unsigned long long* sampled, uint64_t min_sampled, uint4* sig1,
                       uint32_t* sig2, cudaStream_t s);
 // The same bounds on listed pairs (signatures by id): rejected[t] = 1 and
 // ed[t] = k + 1 where they exceed pair t's band (pk[t], or K when pk is null).
@@ -228,32 +231,38 @@ struct PairArgs {
   const uint4* A;
   const uint2* B;
   const uint32_t* sid_of;     // by rank
-  const uint32_t* rlen;
+  const uint32_t* shorts;
+  uint32_t longest;
   const uint32_t* hi;
-  const uint4* sig1;          // read when *visits > min_visits
-  const unsigned long long* visits;
-  uint64_t min_visits;
+  const uint4* sig1;          // read when *sampled > min_sampled
+  unsigned long long* sampled;   // candidates of the sampled strings (launch_string_sample)
+  uint64_t min_sampled;
+  uint32_t stride = 1;        // set by the launcher
   uint32_t n, reps, K, q1;
   int rb;                     // visit_rank_bits
   uint32_t bm_words = 0;      // set by the launcher
   unsigned long long* out_count;   // pairs of ranks that pass the first bound (all counted, the first cap listed)
   unsigned long long* totals;      // out_count + 1: raw pairs, candidates, K-band cells of the candidates
-  uint64_t cap;
-  uint2* out;
+  uint64_t cap = 0;
+  uint2* out = nullptr;
 };
 bool string_pairs_fit(uint32_t widest);   // a string's bitmap fits in shared memory
 constexpr size_t kStringPairsSmemMax = 160u << 10;
 int launch_string_pairs(const PairArgs& a, uint32_t widest, cudaStream_t s);
+// *a.sampled += the candidates of about kSampleStrings strings
+constexpr uint32_t kSampleStrings = 1024;
+int launch_string_sample(const PairArgs& a, uint32_t widest, cudaStream_t s);
 // The second bound of the listed pairs: what passes, as pairs of ids (i < j).
 struct ListArgs {
   const uint2* in;
   const unsigned long long* in_count;
   uint64_t in_cap;
-  const uint4* sig2;          // read when *visits > min_visits
+  const uint4* sig2;          // read when *sampled > min_sampled
   const uint32_t* sid_of;
-  const uint32_t* rlen;
-  const unsigned long long* visits;
-  uint64_t min_visits;
+  const uint32_t* shorts;
+  uint32_t longest;
+  const unsigned long long* sampled;
+  uint64_t min_sampled;
   uint32_t K, q2;
   unsigned long long* out_count;   // all counted, the first cap listed
   uint64_t cap;
@@ -313,7 +322,7 @@ struct RankTable {
   uint8_t r[256];
 };
 struct VerifyArgs {
-  const uint32_t* planes = nullptr;    // bit-planes of rank codes: plane p at planes + p * plane_words
+  const uint32_t* planes = nullptr;    // bit-planes of rank codes: word w of plane p at w * plane_stride(bits) + p
   uint32_t bits;
   const uint8_t* bytes = nullptr;
   const int64_t* offsets = nullptr;
@@ -335,11 +344,18 @@ struct VerifyArgs {
   const uint4* pair_geo = nullptr;     // nullable: at order position q, (oA, oB, m, n) of pair order[q], A the
                                        // longer string (n = kGeoBadIds: an id out of range); loaded with order[q]
   uint32_t* out_t = nullptr;           // nullable: indices of the pairs with result <= K, appended (order arbitrary)
-  const uint8_t* rank_table = nullptr; // device copy of the 256 rank codes
   const uint8_t* codes = nullptr;      // the input's rank codes, one byte per input byte (digit-table kernels)
   uint64_t nbytes = 0;                 // bytes of the input
   unsigned long long* out_count = nullptr;
 };
+// The planes' words of the same 32 positions lie side by side, in 2 words for
+// codes of up to 2 bits, else in 8 (planes beyond the code's bits are zero), so
+// that a lane fetches them by one 8-byte or two 16-byte loads: every lane of
+// the verifiers reads at places of its own, and such loads cost one cycle of
+// the L1 cache per lane each, whatever their width.  (One array per plane took
+// 28 loads per 32 columns of a 3-word band instead of 10: 1.3 M text pairs
+// 7.7 -> 5.3 ms, 100,000 byte pairs 691 -> 577 us.)
+__host__ __device__ constexpr uint32_t plane_stride(uint32_t bits) { return bits <= 2 ? 2u : 8u; }
 int verify_words_for(uint32_t kmax);
 inline uint32_t plane_guard_words(uint32_t kmax) { return kmax / 64 + (uint32_t)verify_words_for(kmax) + 4; }
 // codes (nullable, nbytes + 32 bytes): also the rank code of every byte.
@@ -348,8 +364,16 @@ int launch_build_planes(const uint8_t* bytes, uint64_t nbytes, const RankTable& 
                         cudaStream_t s);
 // `next` is a device counter the persistent kernel hands pairs out from.
 // kernel: MJ_VERIFY_KERNEL_*; lanes: wavefront lanes per pair (0 = fewest that fit).
+// next_is_zero: the caller has cleared it.
 int launch_verify(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, uint32_t kmax,
-                  unsigned long long* next, cudaStream_t s, int kernel = MJ_VERIFY_KERNEL_AUTO, int lanes = 0);
+                  unsigned long long* next, cudaStream_t s, int kernel = MJ_VERIFY_KERNEL_AUTO, int lanes = 0,
+                  bool next_is_zero = false);
+// the two-lanes-per-pair verifier (bands of 1 .. 8 words) and the wavefront on
+// 2 .. 32 lanes (one warp) or 64 .. 1024 (one CTA per pair); *next is zero
+int launch_verify_split(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, int words,
+                        unsigned long long* next, cudaStream_t s);
+int launch_verify_wave(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, int lanes,
+                       unsigned long long* next, cudaStream_t s);
 int wave_lanes_for(uint32_t kmax);
 // whether launch_verify takes bands up to kmax with this kernel choice
 bool verify_supported(uint32_t kmax, int kernel, int lanes);
@@ -420,6 +444,10 @@ int launch_partition_counts(const PRec* recs, uint64_t n_rec, uint32_t n, uint32
 constexpr uint32_t kMaxBandBuckets = 16;
 int launch_band_buckets(const uint32_t* kband, uint64_t m, uint32_t K, uint32_t nb, uint32_t* cnt, uint32_t* ranges,
                         uint32_t* list, unsigned long long* first_total, cudaStream_t s);
+
+// oa/ob/oc[t] = a/b/c[t], t < n, where the output is non-null
+int launch_copy_words(const uint32_t* a, const uint32_t* b, const uint32_t* c, uint64_t n, uint32_t* oa, uint32_t* ob,
+                      uint32_t* oc, cudaStream_t s);
 
 // output of the join: the listed pair indices (sorted ascending, which is
 // (i, j) order since the candidates are sorted) gathered into (i, j, ED);

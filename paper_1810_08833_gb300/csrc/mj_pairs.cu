@@ -3,28 +3,31 @@
 // candidates, with a lower bound on the edit distance tested before a
 // candidate is listed for verification.
 //
-// Strings are ranked by length (ties by id).  The length filter lets a string
-// of rank x pair only with ranks up to hi(x), the last string no more than K
-// longer, so "every pair once" is "every pair from its lower rank", and the
-// candidates of x are a bitmap of hi(x) - x bits in shared memory: no bitmap
-// over all pairs is cleared, marked at random in DRAM and swept.
+// Strings are ranked from the longest to the shortest (ties by id).  The length
+// filter lets a string of rank x pair only with ranks up to hi(x), the last
+// string no more than K shorter, so "every pair once" is "every pair from its
+// lower rank", and the candidates of x are a bitmap of hi(x) - x bits in shared
+// memory: no bitmap over all pairs is cleared, marked at random in DRAM and
+// swept.  (Pairs are listed by their longer string, whose bit-planes are most
+// of what the verifier reads: neighbouring lanes then read the same words.)
 //
 // Records are sorted by (hash of the partition, position bucket), stably,
 // from an order in which they come by rank: within a bucket ranks ascend.  For
-// strings of lengths l and l + L the position filter keeps the partners at
-// positions [pos - (K - L) / 2, pos + (K + L) / 2], an interval of K + 1 that
+// strings of lengths l and l - L the position filter keeps the partners at
+// positions [pos - (K + L) / 2, pos + (K - L) / 2], an interval of K + 1 that
 // moves with L.  With buckets of width W >= K / 2, x's partners through one
-// record are in four windows of the sorted records: the buckets -1, 0, +1 and
-// +2 of its own, each cut to the ranks whose L lets the interval reach it.
+// record are in four windows of the sorted records: the buckets -2, -1, 0 and
+// +1 of its own, each cut to the ranks whose L lets the interval reach it.
 // Windows hold about 1 + W / K times the pairs that pass: 1.5 with W = K / 2;
 // three whole buckets of width K held 2.5 (protein) to 2.9 (text) times them.
+// Lengths are kept by rank as "short" = N - length, N the longest.
 
 // Measured on 300,000 text-like strings (450 MB, 786 M raw pairs, 641 M
-// candidates), general path against this one: pairs and dedup 33.8 -> 8.8 ms,
-// order of the candidates 8.1 -> 0.1, their verification 182.7 -> 7.7 (1.3 M
+// candidates), general path against this one: pairs and dedup 33.8 -> 8.7 ms,
+// order of the candidates 8.1 -> 0.1, their verification 182.7 -> 4.4 (1.3 M
 // pairs pass the bounds; the signatures take 0.9 ms); 400,000 protein-like
-// strings (178 MB, 190 M candidates): 16.1 -> 4.2 + 2.0 (second bound), 2.5 ->
-// 0.4, 21.0 -> 3.6.
+// strings (178 MB, 190 M candidates): 16.1 -> 4.1 + 2.0 (second bound), 2.5 ->
+// 0.4, 21.0 -> 3.3.
 #include <algorithm>
 #include <type_traits>
 
@@ -36,9 +39,9 @@ namespace {
 
 // ---------------------------------------------------------------- strings by length
 __global__ void string_lengths_kernel(const int64_t* __restrict__ offsets, uint32_t n, uint32_t* __restrict__ keys,
-                                      uint32_t* __restrict__ vals) {
+                                      uint32_t* __restrict__ vals, uint32_t longest) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    keys[i] = (uint32_t)(offsets[i + 1] - offsets[i]);
+    keys[i] = longest - (uint32_t)(offsets[i + 1] - offsets[i]);
     vals[i] = (uint32_t)i;
   }
 }
@@ -54,20 +57,24 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
   return lo;
 }
 
-// rank_of[sid]; hi[r] = last rank whose length is at most rlen[r] + K;
+// rank_of[sid]; hi[r] = last rank whose short is at most shorts[r] + K;
 // *widest = the most ranks above its own that a string can pair with;
-// len_rank[l] (nullable), l = 0 .. the longest length: first rank of length >= l.
-__global__ void rank_tables_kernel(const uint32_t* __restrict__ rlen, const uint32_t* __restrict__ sid_of, uint32_t n,
-                                   uint32_t K, uint32_t* __restrict__ rank_of, uint32_t* __restrict__ hi,
-                                   uint32_t* __restrict__ len_rank, unsigned int* __restrict__ widest) {
+// short_rank[l] (nullable), l = 0 .. longest: first rank of short >= l, n if none.
+__global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const uint32_t* __restrict__ sid_of, uint32_t n,
+                                   uint32_t K, uint32_t longest, uint32_t* __restrict__ rank_of,
+                                   uint32_t* __restrict__ hi, uint32_t* __restrict__ short_rank,
+                                   unsigned int* __restrict__ widest) {
   uint32_t w = 0;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t r = (uint32_t)t;
     rank_of[sid_of[r]] = r;
-    if (len_rank)
-      for (uint32_t l = r ? rlen[r - 1] + 1u : 0u; l <= rlen[r]; ++l) len_rank[l] = r;
-    const uint32_t L = rlen[r], top = L > 0xffffffffu - K ? 0xffffffffu : L + K;
-    const uint32_t h = upper_bound_of(rlen, r + 1, n, top) - 1;
+    const uint32_t L = shorts[r], top = L > 0xffffffffu - K ? 0xffffffffu : L + K;
+    if (short_rank) {
+      for (uint32_t l = r ? shorts[r - 1] + 1u : 0u; l <= L; ++l) short_rank[l] = r;
+      if (r == n - 1)
+        for (uint32_t l = L + 1u; l <= longest; ++l) short_rank[l] = n;
+    }
+    const uint32_t h = upper_bound_of(shorts, r + 1, n, top) - 1;
     hi[r] = h;
     w = max(w, h - r);
   }
@@ -140,9 +147,9 @@ __device__ __forceinline__ uint64_t mix64(uint64_t k) {  // MurmurHash3 fmix64
 }
 
 // Sort keys of records [t0, t1) (one repetition) at their places by rank:
-// 32 - pb_bits hash bits of (len, key), then the position bucket.
+// hash_bits bits of a hash of (len, key), then the position bucket.
 __global__ void rank_keys_kernel(const PRec* __restrict__ recs, uint32_t t0, uint32_t t1,
-                                 const uint32_t* __restrict__ delta, int pb_bits, uint32_t W,
+                                 const uint32_t* __restrict__ delta, int hash_bits, int pb_bits, uint32_t W,
                                  uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   const uint32_t pb_max = (1u << pb_bits) - 1u;
   for (uint64_t t = t0 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < t1;
@@ -150,7 +157,7 @@ __global__ void rank_keys_kernel(const PRec* __restrict__ recs, uint32_t t0, uin
     const PRec r = load_rec(recs, t);
     const uint64_t g = mix64(r.h61 ^ ((uint64_t)r.len * 0x9e3779b97f4a7c15ull));
     const uint32_t d = (uint32_t)t + __ldg(delta + r.sid);
-    keys[d] = ((uint32_t)(g >> (32 + pb_bits)) << pb_bits) | min(r.pos / W, pb_max);
+    keys[d] = ((uint32_t)(g >> (64 - hash_bits)) << pb_bits) | min(r.pos / W, pb_max);
     vals[d] = (uint32_t)t;
   }
 }
@@ -224,67 +231,61 @@ __device__ __forceinline__ uint32_t gallop_down(const uint64_t* __restrict__ a, 
 }
 
 // The windows of every record (see the file comment), written at the record's
-// own place: win[2 t], win[2 t + 1] = {first, count} of the buckets -1, 0, +1
-// and +2.  Threads take the records in sorted order, so that neighbours search
-// the same words.  *visits += all counts.
-// len_rank: first rank by length up to the longest (null: no cut by length
-// within a bucket).
+// own place: win[2 t], win[2 t + 1] = {first, count} of the buckets -2, -1, 0
+// and +1.  Threads take the records in sorted order, so that neighbours search
+// the same words.
+// short_rank: first rank by short (null: no cut by length within a bucket).
 __global__ void rank_windows_kernel(const uint64_t* __restrict__ skr, const uint32_t* __restrict__ idx,
-                                    const uint4* __restrict__ A, bool packed, uint32_t n_rec, const uint32_t* __restrict__ hi,
-                                    const uint32_t* __restrict__ rlen, const uint32_t* __restrict__ len_rank,
-                                    uint32_t longest, uint32_t n, uint32_t K, uint32_t W, int pb_bits,
-                                    uint4* __restrict__ win, unsigned long long* __restrict__ visits) {
+                                    const uint4* __restrict__ A, bool packed, uint32_t n_rec, RankTables rt, uint32_t K,
+                                    uint32_t W, int pb_bits, uint4* __restrict__ win) {
   const int32_t pb_max = (int32_t)((1u << pb_bits) - 1u);
-  unsigned long long sum = 0;
   for (uint64_t pp = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; pp < n_rec;
        pp += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t p = (uint32_t)pp;
     const uint64_t w = __ldg(skr + p);
-    const uint32_t key = (uint32_t)(w >> 32), x = (uint32_t)w, h = __ldg(hi + x);
-    uint32_t lo[4] = {0, 0, 0, 0}, cnt[4] = {0, 0, 0, 0};
+    const uint32_t key = (uint32_t)(w >> 32), x = (uint32_t)w, h = __ldg(rt.hi + x);
+    uint32_t lo[4] = {0, 0, 0, 0}, cnt[4] = {0, 0, 0, 0};   // buckets 0, +1, -1, -2
     if (h > x) {
       const int64_t pos = packed ? __ldg(&A[p].x) & 0xffffu : __ldg(&A[p].x);
-      const uint32_t len = __ldg(rlen + x);
+      const uint32_t sh = __ldg(rt.shorts + x);
       const int32_t pb = (int32_t)(key & (uint32_t)pb_max);
-      uint32_t from = p;   // the buckets 0, +1, +2 follow each other upwards from p
+      uint32_t up = p, down = p;   // searches go on from here: buckets 0 and +1 upwards, -1 and -2 downwards
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
-        const int e = s == 3 ? -1 : s;
+        const int e = s < 2 ? s : 1 - s;
         const int32_t bk = pb + e;
         if (bk < 0 || bk > pb_max) continue;
         // ranks (r0, r1] of the lengths from which positions [bk W, bk W + W) can be reached
         uint32_t r0 = x, r1 = h;
-        if (e != 0 && len_rank) {
+        if (e != 0 && rt.short_rank) {
           const int64_t first = (int64_t)bk * W, last = first + W - 1;
-          const int64_t lmin = max((int64_t)0, 2 * (first - pos) - (int64_t)K);
-          const int64_t lmax = last < pos ? (int64_t)K - 2 * (pos - last) : (int64_t)K;
+          const int64_t lmin = e < 0 ? max((int64_t)0, 2 * (pos - last) - (int64_t)K) : 0;
+          const int64_t lmax = e > 0 ? (int64_t)K - 2 * (first - pos) : (int64_t)K;
           if (lmin > lmax) continue;
-          const uint64_t l0 = (uint64_t)len + lmin, l1 = (uint64_t)len + lmax + 1;
-          if (lmin > 0) r0 = max(x, (l0 <= longest ? __ldg(len_rank + l0) : n) - 1u);
-          if (lmax < (int64_t)K) r1 = min(h, (l1 <= longest ? __ldg(len_rank + l1) : n) - 1u);
+          const uint64_t l0 = (uint64_t)sh + lmin, l1 = (uint64_t)sh + lmax + 1;
+          if (lmin > 0) r0 = max(x, (l0 <= rt.longest ? __ldg(rt.short_rank + l0) : rt.n) - 1u);
+          if (lmax < (int64_t)K) r1 = min(h, (l1 <= rt.longest ? __ldg(rt.short_rank + l1) : rt.n) - 1u);
           if (r0 >= r1) continue;
         }
         const uint64_t k = (uint64_t)(key + (uint32_t)e) << 32;
         uint32_t a, b;
         if (e < 0) {
-          b = gallop_down(skr, p, (k | r1) + 1u);
+          b = gallop_down(skr, down, (k | r1) + 1u);
           a = gallop_down(skr, b, (k | r0) + 1u);
+          down = a;
         } else {
-          a = gallop_up(skr, from, n_rec, (k | r0) + 1u);
+          a = gallop_up(skr, up, n_rec, (k | r0) + 1u);
           b = gallop_up(skr, a, n_rec, (k | r1) + 1u);
-          from = b;
+          up = b;
         }
         lo[s] = a;
         cnt[s] = b - a;
-        sum += b - a;
       }
     }
     const uint64_t t = __ldg(idx + p);
-    win[2 * t] = make_uint4(lo[3], cnt[3], lo[0], cnt[0]);
-    win[2 * t + 1] = make_uint4(lo[1], cnt[1], lo[2], cnt[2]);
+    win[2 * t] = make_uint4(lo[3], cnt[3], lo[2], cnt[2]);
+    win[2 * t + 1] = make_uint4(lo[0], cnt[0], lo[1], cnt[1]);
   }
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(visits, sum);
 }
 
 // ---------------------------------------------------------------- lower bounds on the edit distance
@@ -312,50 +313,80 @@ __device__ __forceinline__ uint32_t gram_hash(uint32_t h) {   // MurmurHash3 fmi
   return h;
 }
 
+// Whether a join by strings uses the bounds, from the candidates of a sample of
+// its strings (string_pairs_kernel<..., true>), on the device: the host does
+// not wait for the sample.
+__device__ __forceinline__ bool use_bounds(const unsigned long long* sampled, uint64_t min_sampled) {
+  return *sampled > min_sampled;
+}
+
 constexpr int kSigWarps = 8;
+constexpr int kSigCopies = 4;   // of the first level's few counters, so that a warp's updates spread
 
 // One warp per string: the counts in shared memory, then both signatures at
-// the string's rank (sid_of) or id (null).  With visits, returns at once when the windows hold at most min_visits
-// records (the candidates are then few and verified directly).
+// the string's rank (sid_of) or id (null).  With sampled, returns at once when
+// the bounds are not to be used (use_bounds).  A lane takes the four symbols of an aligned word and
+// the words after it for the grams that run on (q <= 8).  Bound by the shared
+// memory's updates, two per symbol.
 __global__ void __launch_bounds__(32 * kSigWarps) signature_kernel(
     const uint8_t* __restrict__ codes, const int64_t* __restrict__ offsets, const uint32_t* __restrict__ sid_of,
-    uint32_t n, SigShape g, const unsigned long long* __restrict__ visits, uint64_t min_visits,
+    uint32_t n, SigShape g, const unsigned long long* __restrict__ sampled, uint64_t min_sampled,
     uint4* __restrict__ sig1, uint32_t* __restrict__ sig2) {
-  if (visits && *visits <= min_visits) return;
-  __shared__ uint32_t s_cnt[kSigWarps][kSig1 + kSig2];
+  if (sampled && !use_bounds(sampled, min_sampled)) return;
+  __shared__ uint32_t s_c1[kSigWarps][kSigCopies * kSig1];
+  __shared__ uint32_t s_c2[kSigWarps][kSig2];
   __shared__ uint8_t s_bucket[256];
   for (int c = threadIdx.x; c < 256; c += blockDim.x) s_bucket[c] = g.bucket[c];
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t* c1 = s_cnt[wid];
-  uint32_t* c2 = c1 + kSig1;
+  uint32_t* c1 = s_c1[wid];
+  uint32_t* c1_mine = c1 + kSig1 * (lane & (kSigCopies - 1));
+  uint32_t* c2 = s_c2[wid];
+  const uint32_t* codes32 = reinterpret_cast<const uint32_t*>(codes);   // whole words: the buffer is longer than the input
   const uint64_t warps = (uint64_t)gridDim.x * kSigWarps;
   for (uint64_t r = (uint64_t)blockIdx.x * kSigWarps + wid; r < n; r += warps) {
-    for (int c = lane; c < kSig1 + kSig2; c += 32) c1[c] = 0;
+    for (int c = lane; c < kSigCopies * kSig1; c += 32) c1[c] = 0;
+#pragma unroll
+    for (int c = 0; c < kSig2; c += 32) c2[c + lane] = 0;
     __syncwarp();
     const uint32_t s = sid_of ? __ldg(sid_of + r) : (uint32_t)r;
-    const uint64_t o = (uint64_t)__ldg(offsets + s);
-    const uint32_t L = (uint32_t)((uint64_t)__ldg(offsets + s + 1) - o);
-    const uint8_t* b = codes + o;
-    for (uint32_t i = lane; i < L; i += 32) {
-      uint32_t v = __ldg(b + i);
-      if (g.q1 == 1) atomicAdd(c1 + s_bucket[v], 1u);
-      if (g.q2 == 1) atomicAdd(c2 + v, 1u);
-      const uint32_t q = g.q1 > g.q2 ? g.q1 : g.q2;
-      for (uint32_t k = 1; k < q && i + k < L; ++k) {
-        v = v * 257u + __ldg(b + i + k) + 1u;
-        if (k + 1 == g.q1) atomicAdd(c1 + __umulhi(gram_hash(v), (uint32_t)kSig1), 1u);
-        if (k + 1 == g.q2) atomicAdd(c2 + (gram_hash(v) >> 24), 1u);
+    const uint32_t o = (uint32_t)__ldg(offsets + s), e = (uint32_t)__ldg(offsets + s + 1);   // inputs are under 4 GB
+    const uint32_t w1 = (uint32_t)(((uint64_t)e + 3) >> 2);
+#pragma unroll 2
+    for (uint32_t w = (o >> 2) + lane; w < w1; w += 32) {
+      const uint32_t x0 = __ldg(codes32 + w), x1 = __ldg(codes32 + w + 1);
+      const uint32_t x2 = g.q2 > 5 ? __ldg(codes32 + w + 2) : 0u;
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        const uint32_t p = 4 * w + k;   // below 2^32: w < 2^30
+        if (p < o || p >= e) continue;
+        const uint32_t left = e - p;
+        const uint32_t lo = __funnelshift_r(x0, x1, 8 * k), hi = __funnelshift_r(x1, x2, 8 * k);   // eight symbols from p
+        uint32_t v = lo & 255u;
+        if (g.q1 == 1) atomicAdd(c1_mine + s_bucket[v], 1u);
+        if (g.q2 == 1) atomicAdd(c2 + v, 1u);
+        for (uint32_t i = 1; i < g.q2 && i < left; ++i) {   // q1 <= q2
+          v = v * 257u + (((i < 4 ? lo >> (8 * i) : hi >> (8 * i - 32)) & 255u) + 1u);
+          if (i + 1 == g.q1) atomicAdd(c1_mine + __umulhi(gram_hash(v), (uint32_t)kSig1), 1u);
+          if (i + 1 == g.q2) atomicAdd(c2 + (gram_hash(v) >> 24), 1u);
+        }
       }
     }
     __syncwarp();
-    auto pack = [&](const uint32_t* c) {
-      return min(c[0], 255u) | (min(c[1], 255u) << 8) | (min(c[2], 255u) << 16) | (min(c[3], 255u) << 24);
-    };
     uint32_t* d1 = reinterpret_cast<uint32_t*>(sig1 + 2 * r);
-    if (lane == 0) d1[0] = L;
-    if (lane < kSig1 / 4) d1[1 + lane] = pack(c1 + 4 * lane);
-    uint32_t v2 = 0;   // lane w: buckets 8 w .. 8 w + 7
+    if (lane == 0) d1[0] = e - o;
+    if (lane < kSig1 / 4) {
+      uint32_t v1 = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int y = 0; y < kSigCopies; ++y) c += c1[y * kSig1 + 4 * lane + k];
+        v1 |= min(c, 255u) << (8 * k);
+      }
+      d1[1 + lane] = v1;
+    }
+    uint32_t v2 = 0;   // lane l: buckets 8 l .. 8 l + 7
 #pragma unroll
     for (int k = 0; k < 8; ++k) v2 |= min(c2[8 * lane + k], 15u) << (4 * k);
     sig2[r * (kSig2Bytes / 4) + lane] = v2;
@@ -511,7 +542,8 @@ __device__ __forceinline__ uint32_t absdiff2(uint32_t a, uint32_t b) {   // |a.l
   return d;
 }
 
-template <int THREADS, bool WIDE, bool PACKED>
+// SAMPLE: only counts the candidates of every a.stride-th string into *a.sampled.
+template <int THREADS, bool WIDE, bool PACKED, bool SAMPLE>
 __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_kernel(PairArgs a) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   using Shared = PairShared<THREADS, WIDE>;
@@ -524,17 +556,18 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
     if (THREADS == 32) __syncwarp();
     else __syncthreads();
   };
-  const bool filter = *a.visits > a.min_visits;
+  const bool filter = !SAMPLE && use_bounds(a.sampled, a.min_sampled);
   const uint32_t lim1 = 2u * a.q1 * a.K;
   unsigned long long raw = 0, cand = 0, cells = 0;
   if (tid == 0) sh.n_short = sh.n_long = 0;
   for (uint32_t w = tid; w < a.bm_words; w += THREADS) bm[w] = 0;   // cleared again as it is read
   sync();
-  for (uint32_t x = blockIdx.x; x < a.n; x += gridDim.x) {
+  for (uint64_t xs = (uint64_t)blockIdx.x * a.stride; xs < a.n; xs += (uint64_t)gridDim.x * a.stride) {
+    const uint32_t x = (uint32_t)xs;
     const uint32_t span = __ldg(a.hi + x) - x;
     if (span == 0) continue;
     const uint32_t words = (span + 31) / 32;
-    const uint32_t sid = __ldg(a.sid_of + x), len_x = __ldg(a.rlen + x);
+    const uint32_t sid = __ldg(a.sid_of + x), len_x = a.longest - __ldg(a.shorts + x);
     uint4 sx = make_uint4(0u, 0u, 0u, 0u), sy = sx;
     if (filter) {
       sx = __ldg(a.sig1 + 2 * (uint64_t)x);
@@ -670,15 +703,15 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
           u[e] = __ldg(a.sig1 + 2 * (uint64_t)y);
           v[e] = __ldg(a.sig1 + 2 * (uint64_t)y + 1);
         } else if (on[e]) {
-          u[e].x = __ldg(a.rlen + y);
+          u[e].x = a.longest - __ldg(a.shorts + y);
         }
       }
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         bool live = on[e];
         if (live) {
-          cells += band_cells_of(u[e].x, len_x, a.K);
-          if (filter) live = sig1_sum(u[e], v[e], sx, sy) <= lim1 || u[e].x >= kBoundsMaxLen;
+          cells += band_cells_of(len_x, u[e].x, a.K);
+          if (filter) live = sig1_sum(u[e], v[e], sx, sy) <= lim1 || len_x >= kBoundsMaxLen;
         }
         const uint32_t mask = __ballot_sync(0xffffffffu, live);
         if (live) passed[waiting + __popc(mask & ((1u << lane) - 1u))] = (Slot)slot[e];
@@ -701,9 +734,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
         const uint32_t z = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += z;
       }
+      cand += c;
+      if (SAMPLE) continue;   // nothing is listed: the stack stays empty
       uint32_t at = depth + incl - c;
       depth += __shfl_sync(0xffffffffu, incl, 31);
-      cand += c;
       while (bits) {
         stack[at++] = (Slot)(16u * h + (__ffs(bits) - 1));
         bits &= bits - 1;
@@ -712,14 +746,20 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
       while (depth >= 64) test(std::integral_constant<int, 2>(), 64u);
       __syncwarp();   // the popped entries are read before the next step's pushes
     }
-    if (depth) test(std::integral_constant<int, 2>(), depth);
-    if (waiting) append();
+    if (!SAMPLE) {
+      if (depth) test(std::integral_constant<int, 2>(), depth);
+      if (waiting) append();
+    }
     sync();   // the bitmap is clear for the next string
   }
   for (int o = 16; o > 0; o >>= 1) {
     raw += __shfl_down_sync(0xffffffffu, raw, o);
     cand += __shfl_down_sync(0xffffffffu, cand, o);
     cells += __shfl_down_sync(0xffffffffu, cells, o);
+  }
+  if (SAMPLE) {
+    if (lane == 0 && cand) atomicAdd(a.sampled, cand);
+    return;
   }
   if (lane == 0) {
     if (raw) atomicAdd(a.totals + 0, raw);
@@ -729,11 +769,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
 }
 
 // Second bound of the listed pairs of ranks (x < y): a warp takes 32 pairs per
-// step and appends what passes, as ids.  Without the bounds (few visits) every
-// pair passes.
+// step and appends what passes, as ids.  Without the bounds (few candidates)
+// every pair passes.
 __global__ void __launch_bounds__(256) listed_pairs_kernel(ListArgs a) {
   const int lane = threadIdx.x & 31;
-  const bool filter = *a.visits > a.min_visits;
+  const bool filter = use_bounds(a.sampled, a.min_sampled);
   const uint64_t m = min(*a.in_count, (unsigned long long)a.in_cap);
   const uint32_t lim = 2u * a.q2 * a.K;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -743,8 +783,8 @@ __global__ void __launch_bounds__(256) listed_pairs_kernel(ListArgs a) {
     bool pass = t < m;
     if (filter) {
       const uint32_t sum = sig2_sums(a.sig2, lane, [&](int q) { return a.in[min(t0 + q, m - 1)]; });
-      const uint32_t lx = __ldg(a.rlen + pair.x), ly = __ldg(a.rlen + pair.y);
-      pass = pass && (sum + (ly - lx) <= lim || ly >= kBoundsMaxLen);
+      const uint32_t sx = __ldg(a.shorts + pair.x), sy = __ldg(a.shorts + pair.y);
+      pass = pass && (sum + (sy - sx) <= lim || a.longest - sx >= kBoundsMaxLen);
     }
     const uint32_t mask = __ballot_sync(0xffffffffu, pass);
     if (!mask) continue;
@@ -762,20 +802,30 @@ __global__ void __launch_bounds__(256) listed_pairs_kernel(ListArgs a) {
   }
 }
 
-template <int THREADS, bool WIDE, bool PACKED>
+template <int THREADS, bool WIDE, bool PACKED, bool SAMPLE>
 int launch_string_pairs_t(PairArgs a, uint32_t widest, cudaStream_t s) {
-  auto kernel = string_pairs_kernel<THREADS, WIDE, PACKED>;
+  auto kernel = string_pairs_kernel<THREADS, WIDE, PACKED, SAMPLE>;
   const size_t smem = sizeof(PairShared<THREADS, WIDE>) + ((size_t)widest + 31) / 32 * 4 + 16;
   int dev = 0, sms = 0, per_sm = 0;
   MJ_CUDA_TRY(cudaGetDevice(&dev));
   MJ_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   MJ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   MJ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, THREADS, smem));
-  const uint64_t grid = std::min<uint64_t>(a.n, (uint64_t)std::max(1, sms) * std::max(1, per_sm));
+  a.stride = SAMPLE ? std::max<uint32_t>(1, a.n / kSampleStrings) : 1;
+  const uint64_t work = (a.n + a.stride - 1) / a.stride;
+  const uint64_t grid = std::min<uint64_t>(work, (uint64_t)std::max(1, sms) * std::max(1, per_sm));
   a.bm_words = (widest + 31) / 32;
   kernel<<<(unsigned)grid, THREADS, smem, s>>>(a);
   MJ_KERNEL_DONE();
   return MJ_OK;
+}
+
+template <bool SAMPLE>
+int launch_string_pairs_s(const PairArgs& a, uint32_t widest, cudaStream_t s) {
+  if (!a.n) return MJ_OK;
+  if (widest < 65536 && a.rb) return launch_string_pairs_t<32, false, true, SAMPLE>(a, widest, s);
+  return a.rb ? launch_string_pairs_t<128, true, true, SAMPLE>(a, widest, s)
+              : launch_string_pairs_t<128, true, false, SAMPLE>(a, widest, s);
 }
 
 unsigned grid_for(uint64_t n, int threads = 256) {
@@ -785,17 +835,16 @@ unsigned grid_for(uint64_t n, int threads = 256) {
 
 }  // namespace
 
-int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, int len_bits, uint32_t* len, uint32_t* len_alt,
-                        uint32_t* sid, uint32_t* sid_alt, void* temp, uint32_t* rank_of, uint32_t* hi,
-                        uint32_t* len_rank, unsigned int* widest, bool* in_alt, cudaStream_t s) {
+int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t longest, int len_bits,
+                        uint32_t* shorts, uint32_t* shorts_alt, uint32_t* sid, uint32_t* sid_alt, void* temp, uint32_t* rank_of, uint32_t* hi,
+                        uint32_t* short_rank, unsigned int* widest, bool* in_alt, cudaStream_t s) {
   *in_alt = false;
-  MJ_CUDA_TRY(cudaMemsetAsync(widest, 0, sizeof(unsigned int), s));
   if (!n) return MJ_OK;
-  string_lengths_kernel<<<grid_for(n), 256, 0, s>>>(offsets, n, len, sid);
+  string_lengths_kernel<<<grid_for(n), 256, 0, s>>>(offsets, n, shorts, sid, longest);
   MJ_KERNEL_DONE();
-  MJ_TRY(radix_sort_u32(len, len_alt, sid, sid_alt, n, 0, len_bits, temp, in_alt, s));
-  rank_tables_kernel<<<grid_for(n), 256, 0, s>>>(*in_alt ? len_alt : len, *in_alt ? sid_alt : sid, n, K, rank_of, hi,
-                                                 len_rank, widest);
+  MJ_TRY(radix_sort_u32(shorts, shorts_alt, sid, sid_alt, n, 0, len_bits, temp, in_alt, s));
+  rank_tables_kernel<<<grid_for(n), 256, 0, s>>>(*in_alt ? shorts_alt : shorts, *in_alt ? sid_alt : sid, n, K, longest,
+                                                 rank_of, hi, short_rank, widest);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
@@ -818,24 +867,22 @@ int launch_rank_order(const uint32_t* first, const uint32_t* sid_of, const uint3
   return MJ_OK;
 }
 
-int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int pb_bits, uint32_t W,
-                     uint32_t* keys, uint32_t* vals, cudaStream_t s) {
+int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int hash_bits, int pb_bits,
+                     uint32_t W, uint32_t* keys, uint32_t* vals, cudaStream_t s) {
   if (t1 <= t0) return MJ_OK;
-  rank_keys_kernel<<<grid_for(t1 - t0), 256, 0, s>>>(recs, t0, t1, delta, pb_bits, W, keys, vals);
+  rank_keys_kernel<<<grid_for(t1 - t0), 256, 0, s>>>(recs, t0, t1, delta, hash_bits, pb_bits, W, keys, vals);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
 
 int launch_rank_windows(const uint32_t* idx, const uint32_t* keys, uint32_t n_rec, const PRec* recs,
                         const uint32_t* rank_of, const RankTables& rt, uint32_t K, uint32_t W, int pb_bits, int rb,
-                        uint4* A, uint2* B, uint64_t* skr, uint4* win, unsigned long long* visits, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemsetAsync(visits, 0, sizeof(unsigned long long), s));
+                        uint4* A, uint2* B, uint64_t* skr, uint4* win, cudaStream_t s) {
   if (!n_rec) return MJ_OK;
   if (rb) rank_gather_kernel<true><<<grid_for(n_rec), 256, 0, s>>>(idx, keys, n_rec, recs, rank_of, rb, A, B, skr);
   else rank_gather_kernel<false><<<grid_for(n_rec), 256, 0, s>>>(idx, keys, n_rec, recs, rank_of, rb, A, B, skr);
   MJ_KERNEL_DONE();
-  rank_windows_kernel<<<grid_for(n_rec), 256, 0, s>>>(skr, idx, A, rb != 0, n_rec, rt.hi, rt.rlen, rt.len_rank, rt.longest, rt.n, K,
-                                                      W, pb_bits, win, visits);
+  rank_windows_kernel<<<grid_for(n_rec), 256, 0, s>>>(skr, idx, A, rb != 0, n_rec, rt, K, W, pb_bits, win);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
@@ -881,10 +928,10 @@ SigShape signature_shape(uint32_t sigma, const uint64_t* counts_by_code) {
 }
 
 int launch_signatures(const uint8_t* codes, const int64_t* offsets, const uint32_t* sid_of, uint32_t n,
-                      const SigShape& g, const unsigned long long* visits, uint64_t min_visits, uint4* sig1,
+                      const SigShape& g, const unsigned long long* sampled, uint64_t min_sampled, uint4* sig1,
                       uint32_t* sig2, cudaStream_t s) {
   if (!n) return MJ_OK;
-  signature_kernel<<<grid_for(n, kSigWarps), 32 * kSigWarps, 0, s>>>(codes, offsets, sid_of, n, g, visits, min_visits,
+  signature_kernel<<<grid_for(n, kSigWarps), 32 * kSigWarps, 0, s>>>(codes, offsets, sid_of, n, g, sampled, min_sampled,
                                                                      sig1, sig2);
   MJ_KERNEL_DONE();
   return MJ_OK;
@@ -904,15 +951,14 @@ bool string_pairs_fit(uint32_t widest) {
 }
 
 int launch_string_pairs(const PairArgs& a, uint32_t widest, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemsetAsync(a.out_count, 0, 4 * sizeof(unsigned long long), s));   // and the totals behind it
-  if (!a.n) return MJ_OK;
-  if (widest < 65536 && a.rb) return launch_string_pairs_t<32, false, true>(a, widest, s);
-  return a.rb ? launch_string_pairs_t<128, true, true>(a, widest, s)
-              : launch_string_pairs_t<128, true, false>(a, widest, s);
+  return launch_string_pairs_s<false>(a, widest, s);
+}
+
+int launch_string_sample(const PairArgs& a, uint32_t widest, cudaStream_t s) {
+  return launch_string_pairs_s<true>(a, widest, s);
 }
 
 int launch_listed_pairs(const ListArgs& a, cudaStream_t s) {
-  MJ_CUDA_TRY(cudaMemsetAsync(a.out_count, 0, sizeof(unsigned long long), s));
   listed_pairs_kernel<<<grid_for(a.in_cap), 256, 0, s>>>(a);
   MJ_KERNEL_DONE();
   return MJ_OK;

@@ -61,9 +61,21 @@ __host__ __device__ inline size_t anchor_smem_bytes(int r_max) {
 }
 
 // tile_first[t] = the string holding byte t * kPartTile: every non-empty
-// string marks the tiles that start inside it.
+// string marks the tiles that start inside it.  flags (nullable): words 0 and 1
+// are cleared, and the planes' guard words before and after the data.
 __global__ void tile_first_kernel(const int64_t* __restrict__ offsets, uint32_t n, uint64_t tiles,
-                                  uint32_t* __restrict__ tile_first) {
+                                  uint32_t* __restrict__ tile_first, uint32_t* __restrict__ flags,
+                                  uint32_t* __restrict__ planes, uint64_t plane_words, uint32_t guard_words,
+                                  uint32_t bits) {
+  if (flags) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) flags[threadIdx.x] = 0;
+    if (planes) {
+      const uint32_t edge = guard_words * plane_stride(bits);   // words before and after the data
+      const uint64_t behind = (plane_words - guard_words) * plane_stride(bits);
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * edge; i += gridDim.x * blockDim.x)
+        planes[i < edge ? i : behind + (i - edge)] = 0;
+    }
+  }
   for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (uint64_t)gridDim.x * blockDim.x) {
     const int64_t lo = offsets[s], hi = offsets[s + 1];
     if (hi <= lo) continue;
@@ -383,19 +395,43 @@ __global__ void __launch_bounds__(kAThreads, sizeof(HT) == 4 ? 4 : 2) anchor_fla
         }
       }
       if (pack) {
-        // plane p, positions g .. g+15 of this run: one 16-bit half of word g / 32
+        // plane p, positions g .. g+15 of this run: one 16-bit half of word g / 32.
+        // Two neighbouring lanes hold the two halves of the same words (the
+        // range of valid words ends with a tile, so whole warps are in it):
+        // they swap halves, two planes per exchange, and each stores half of
+        // the words' planes.
         const uint64_t g = (uint64_t)gx;
         const uint64_t word = guard_words + (g >> 5);
         if (word < guard_words + tiles * (kPartTile / 32)) {
-          for (int p = 0; p < (int)a.bits; ++p) {
-            uint32_t half = 0;
+          auto half = [&](int p) {
+            uint32_t h16 = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               // bit p of the four byte-codes of symw[k] into a nibble (k-th symbol at bit k)
               const uint32_t x = (symw[k] >> p) & 0x01010101u;
-              half += ((x * 0x01020408u) >> 24) << (4 * k);
+              h16 += ((x * 0x01020408u) >> 24) << (4 * k);
             }
-            reinterpret_cast<uint16_t*>(planes + (uint64_t)p * plane_words + word)[(g >> 4) & 1] = (uint16_t)half;
+            return h16;
+          };
+          const bool hi = (g >> 4) & 1;   // this run is the words' upper half
+          if (plane_stride(a.bits) == 2) {
+            const uint32_t mine = half(0) | (half(1) << 16);   // planes 0 and 1
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
+            if (!hi)
+              reinterpret_cast<uint2*>(planes)[word] =
+                  make_uint2((mine & 0xffffu) | (other << 16), (mine >> 16) | (other & 0xffff0000u));
+          } else {
+            // pairs of planes: the lower run stores planes 0-3, the upper 4-7
+            uint32_t q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              q[k] = 2 * k < (int)a.bits ? half(2 * k) | (2 * k + 1 < (int)a.bits ? half(2 * k + 1) << 16 : 0u) : 0u;
+            const uint32_t r0 = __shfl_xor_sync(0xffffffffu, hi ? q[0] : q[2], 1);
+            const uint32_t r1 = __shfl_xor_sync(0xffffffffu, hi ? q[1] : q[3], 1);
+            const uint32_t lo0 = hi ? r0 : q[0], hi0 = hi ? q[2] : r0, lo1 = hi ? r1 : q[1], hi1 = hi ? q[3] : r1;
+            reinterpret_cast<uint4*>(planes)[2 * word + (hi ? 1 : 0)] =
+                make_uint4((lo0 & 0xffffu) | (hi0 << 16), (lo0 >> 16) | (hi0 & 0xffff0000u),
+                           (lo1 & 0xffffu) | (hi1 << 16), (lo1 >> 16) | (hi1 & 0xffff0000u));
           }
           if (a.codes) *reinterpret_cast<uint4*>(a.codes + g) = make_uint4(symw[0], symw[1], symw[2], symw[3]);
         }
@@ -682,13 +718,14 @@ uint64_t partition_num_tiles(uint64_t nbytes) { return (nbytes + kPartTile - 1) 
 
 int launch_anchor_flags(const PartitionArgs& a, uint32_t* bitmap, uint32_t* tile_count, uint32_t* dev_flags,
                         uint32_t* planes, uint64_t plane_words, uint32_t guard_words, uint32_t* tile_first,
-                        cudaStream_t s) {
+                        bool first_call, cudaStream_t s) {
   const uint64_t tiles = partition_num_tiles(a.nbytes);
   if (tiles == 0) return MJ_OK;
   {
     uint64_t blocks = (a.n + 255) / 256;
     if (blocks > (uint64_t)kNumSMsHint * 32) blocks = (uint64_t)kNumSMsHint * 32;
-    tile_first_kernel<<<(unsigned)(blocks ? blocks : 1), 256, 0, s>>>(a.offsets, a.n, tiles, tile_first);
+    tile_first_kernel<<<(unsigned)(blocks ? blocks : 1), 256, 0, s>>>(
+        a.offsets, a.n, tiles, tile_first, first_call ? dev_flags : nullptr, planes, plane_words, guard_words, a.bits);
     MJ_KERNEL_DONE();
   }
   PartitionArgs ka = a;

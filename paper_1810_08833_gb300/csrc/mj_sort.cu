@@ -73,12 +73,57 @@ __global__ void __launch_bounds__(kScanThreads) scan_down_kernel(const TI* __res
   }
 }
 
+// One block scans up to kOneScan elements, kOneItems consecutive ones per
+// thread: short scans are a launch's time (about 2 us a piece), so one launch
+// replaces the two or three of the tiled form.
+constexpr int kOneThreads = 1024, kOneItems = 32;
+constexpr uint64_t kOneScan = (uint64_t)kOneThreads * kOneItems;
+
+template <class TI, class TO>
+__global__ void __launch_bounds__(kOneThreads) scan_one_kernel(const TI* __restrict__ in, TO* __restrict__ out,
+                                                               uint32_t n, TO* __restrict__ total_out) {
+  __shared__ TO s_warp[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // only as many items per thread as the input needs, all loaded at once
+  const uint32_t per = (n + kOneThreads - 1) / kOneThreads;
+  const uint32_t base = threadIdx.x * per;
+  TI v[kOneItems];
+  TO sum = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < kOneItems; ++k) v[k] = k < per && base + k < n ? in[base + k] : TI(0);
+#pragma unroll
+  for (uint32_t k = 0; k < kOneItems; ++k) sum += (TO)v[k];
+  TO x = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const TO y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[wid] = x;
+  __syncthreads();
+  if (wid == 0) {
+    TO w = s_warp[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const TO y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    s_warp[lane] = w;
+  }
+  __syncthreads();
+  TO run = (wid ? s_warp[wid - 1] : TO(0)) + x - sum;
+#pragma unroll
+  for (uint32_t k = 0; k < kOneItems; ++k) {
+    if (k < per && base + k < n) out[base + k] = run;
+    run += (TO)v[k];
+  }
+  if (total_out && threadIdx.x == 0) *total_out = s_warp[31];
+}
+
 uint64_t blocks_for(uint64_t n) { return (n + kScanTile - 1) / kScanTile; }
 
 // temp elements needed by exclusive_scan: 2 per block at every level
 size_t scan_temp_elems(uint64_t n) {
   size_t e = 0;
-  while (n > kScanTile) {
+  while (n > kOneScan) {
     uint64_t b = blocks_for(n);
     e += 2 * b;
     n = b;
@@ -96,16 +141,12 @@ int exclusive_scan(const TI* in, TO* out, uint64_t n, TO* temp, TO* total_out, c
     if (total_out) MJ_CUDA_TRY(cudaMemsetAsync(total_out, 0, sizeof(TO), s));
     return MJ_OK;
   }
-  uint64_t b = blocks_for(n);
-  if (b == 1) {
-    if (total_out) {
-      scan_reduce_kernel<TI, TO><<<1, kScanThreads, 0, s>>>(in, n, total_out);
-      MJ_KERNEL_DONE();
-    }
-    scan_down_kernel<TI, TO><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr);
+  if (n <= kOneScan) {
+    scan_one_kernel<TI, TO><<<1, kOneThreads, 0, s>>>(in, out, (uint32_t)n, total_out);
     MJ_KERNEL_DONE();
     return MJ_OK;
   }
+  const uint64_t b = blocks_for(n);
   TO* sums = temp;
   TO* sums_scanned = temp + b;
   scan_reduce_kernel<TI, TO><<<(unsigned)b, kScanThreads, 0, s>>>(in, n, sums);
@@ -129,11 +170,16 @@ __global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const KT* __re
   s_hist[threadIdx.x] = 0;
   __syncthreads();
   uint64_t base = (uint64_t)blockIdx.x * kSortTile;
-#pragma unroll 4
+  // all 16 loads in flight: with few tiles the kernel is a load's latency
+  uint32_t d[kSortItems];
+#pragma unroll
   for (int k = 0; k < kSortItems; ++k) {
-    uint64_t idx = base + (uint64_t)k * kSortThreads + threadIdx.x;
-    if (idx < n) atomicAdd(&s_hist[(uint32_t)(keys[idx] >> shift) & 255u], 1u);
+    const uint64_t idx = base + (uint64_t)k * kSortThreads + threadIdx.x;
+    d[k] = idx < n ? (uint32_t)(keys[idx] >> shift) & 255u : 256u;
   }
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k)
+    if (d[k] < 256u) atomicAdd(&s_hist[d[k]], 1u);
   __syncthreads();
   hist[(uint64_t)threadIdx.x * num_tiles + blockIdx.x] = s_hist[threadIdx.x];
 }
@@ -240,6 +286,105 @@ __global__ void __launch_bounds__(kScatThreads) radix_scatter_kernel(
   }
 }
 
+// Stable sort of up to kOneSort keys (and values) by one block, all passes in
+// shared memory: 3 launches per pass of the tiled form cost more than the
+// sort.  Thread t of warp w takes items 512 w + 32 r + lane in round r; the
+// ranks are those of radix_scatter_kernel.
+constexpr int kOneSortThreads = 1024;
+constexpr int kOneSortWarps = kOneSortThreads / 32;
+template <class KT>
+constexpr uint32_t kOneSort = sizeof(KT) == 4 ? 16384 : 8192;
+
+template <class KT, int ITEMS>
+__global__ void __launch_bounds__(kOneSortThreads) radix_one_kernel(KT* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                                    uint32_t n, int bit_lo, int bit_hi) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  KT* s_keys = reinterpret_cast<KT*>(smem);
+  uint32_t* s_vals = reinterpret_cast<uint32_t*>(smem + (size_t)kOneSortThreads * ITEMS * sizeof(KT));
+  uint32_t(*s_cnt)[256] = reinterpret_cast<uint32_t(*)[256]>(s_vals + (size_t)kOneSortThreads * ITEMS);
+  __shared__ uint32_t s_start[256];
+  __shared__ uint32_t s_wsum[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t lt = (1u << lane) - 1;
+  KT k_[ITEMS];
+  uint32_t v_[ITEMS], rank_[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const uint32_t i = (uint32_t)(wid * ITEMS + r) * 32 + lane;
+    k_[r] = i < n ? keys[i] : ~KT(0);
+    v_[r] = i < n && vals ? vals[i] : 0u;
+  }
+  for (int shift = bit_lo; shift < bit_hi; shift += 8) {
+    for (int d = threadIdx.x; d < kOneSortWarps * 256; d += kOneSortThreads) (&s_cnt[0][0])[d] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {   // items past n have the last digit and come last in the input
+      const uint32_t d = (uint32_t)(k_[r] >> shift) & 255u;
+      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      const uint32_t before = __popc(peers & lt);
+      const uint32_t cnt = s_cnt[wid][d];
+      rank_[r] = cnt + before;
+      __syncwarp();
+      if (before == 0) s_cnt[wid][d] = cnt + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    uint32_t run = 0, x = 0;
+    if (threadIdx.x < 256) {
+      for (int w = 0; w < kOneSortWarps; ++w) {
+        const uint32_t c = s_cnt[w][threadIdx.x];
+        s_cnt[w][threadIdx.x] = run;
+        run += c;
+      }
+      x = run;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) s_wsum[wid] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+      uint32_t pre = 0;
+      for (int w = 0; w < wid; ++w) pre += s_wsum[w];
+      s_start[threadIdx.x] = pre + x - run;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const uint32_t d = (uint32_t)(k_[r] >> shift) & 255u;
+      const uint32_t pos = s_start[d] + s_cnt[wid][d] + rank_[r];
+      s_keys[pos] = k_[r];
+      s_vals[pos] = v_[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const uint32_t i = (uint32_t)(wid * ITEMS + r) * 32 + lane;
+      k_[r] = s_keys[i];
+      v_[r] = s_vals[i];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const uint32_t i = (uint32_t)(wid * ITEMS + r) * 32 + lane;
+    if (i < n) {
+      keys[i] = k_[r];
+      if (vals) vals[i] = v_[r];
+    }
+  }
+}
+
+template <class KT, int ITEMS>
+int launch_radix_one(KT* keys, uint32_t* vals, uint32_t n, int bit_lo, int bit_hi, cudaStream_t s) {
+  constexpr size_t smem = (size_t)kOneSortThreads * ITEMS * (sizeof(KT) + 4) + (size_t)kOneSortWarps * 256 * 4;
+  MJ_CUDA_TRY(cudaFuncSetAttribute(radix_one_kernel<KT, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  radix_one_kernel<KT, ITEMS><<<1, kOneSortThreads, smem, s>>>(keys, vals, n, bit_lo, bit_hi);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
 }  // namespace
 
 size_t scan_temp_bytes(uint64_t n) { return scan_temp_elems(n) * sizeof(uint64_t) + 64; }
@@ -273,6 +418,12 @@ int radix_sort(KT* keys, KT* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint6
   *result_in_alt = false;
   if (n <= 1 || bit_hi <= bit_lo) return MJ_OK;
   if (n >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;
+  if (n <= kOneSort<KT>) {
+    const uint32_t m = (uint32_t)n;
+    if (m <= 1024) return launch_radix_one<KT, 1>(keys, vals, m, bit_lo, bit_hi, s);
+    if (m <= 4096) return launch_radix_one<KT, 4>(keys, vals, m, bit_lo, bit_hi, s);
+    return launch_radix_one<KT, (int)(kOneSort<KT> / kOneSortThreads)>(keys, vals, m, bit_lo, bit_hi, s);
+  }
   const uint32_t tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
   const uint64_t h = (uint64_t)tiles * 256;
   uint32_t* hist = static_cast<uint32_t*>(temp);

@@ -1,0 +1,606 @@
+// Step a8 for wide bands: row-fixed blocks with a skewed wavefront, within one
+// warp (G lanes per pair) or one CTA of several warps per pair.
+#include "mj_verify_common.cuh"
+
+namespace mj {
+namespace {
+
+// ---------------------------------------------------------------- wide bands
+// Row-fixed blocks with a skewed wavefront, G lanes per pair.
+//
+// Rows are cut into 32-row blocks (block b = rows 32b+1 .. 32b+32, one 32-bit
+// word per vector); lane b mod G of the pair's group owns block b.  Block b
+// advances column j at step s = j + b: it needs the horizontal delta of the
+// row just above it in column j, which the lane owning block b-1 produced one
+// step earlier and passes on by a shuffle.  A block works on the columns in
+// which some of its rows lie in the band [j + dlo, j + dhi]; outside, a block
+// entering the band starts from vertical deltas of +1 and the row above a
+// retired block gets a horizontal delta of +1 (the same over-estimates as the
+// diagonal kernel).  With an incoming horizontal delta hin in {-1, 0, +1}, a
+// block step is the recurrence of the diagonal kernel with the top row's
+// chain seeded by hin: Xh's carry chain starts set when hin = -1, and the
+// shifted-in top bit of Ph (Mh) is set when hin = +1 (-1).  Each block keeps
+// D of its bottom row; the bottom row of the block holding row m at column n
+// gives D[m][n], and the block holding row j + d0 at column j gives the
+// diagonal lower bound used for the early exit.
+constexpr int kWaveSteps = 32;   // wavefront steps between refills and votes (<= 32: B's bits per reload)
+
+// Each lane publishes one word per wavefront step for the lane holding the
+// next block of rows:
+//   bit 31      the block's bottom row gained +1 in this column (hout = +1)
+//   bits 1..30  D at the block's bottom row in this column (the score)
+//   bit 0       hout = -1
+// The next lane reads it only in the columns that block b - 1 shares with
+// block b; elsewhere the top row's delta is kIdle, +1 (the band's edge).
+constexpr uint32_t kIdle = 0x80000000u;
+constexpr int32_t kDeadU = -0x40000000;   // step offset of a lane without a block
+constexpr uint32_t kMaxLen = 1u << 27;     // scores must fit bits 1..30
+
+template <int P>
+__device__ __forceinline__ void wave_load_bits(const VerifyArgs& a, uint64_t PW, uint64_t pos, uint32_t (&v)[P],
+                                               bool reverse) {
+  uint32_t lo[P], hi[P];
+  load_plane_words<P>(a.planes, (int64_t)(pos >> 5), lo);
+  load_plane_words<P>(a.planes, (int64_t)(pos >> 5) + 1, hi);
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const uint32_t x = __funnelshift_r(lo[p], hi[p], (uint32_t)(pos & 31));
+    v[p] = reverse ? __brev(x) : x;
+  }
+}
+
+// One column of a 32-row block (Myers' step in Hyyro's formulation).  wv
+// carries the horizontal delta entering the top row (bit 31: +1, bit 0: -1,
+// neither: 0); B's symbol is bit 31 of bw[] (consumed, shifted out); T's
+// score bits (1..30) follow the bottom row; Ph keeps the bottom row's +1 in
+// bit 31 and hn is its -1.  Bit extraction, shifts and disjoint ORs are
+// written as integer multiply-adds, which the FMA pipe can take: the logic
+// ops already fill the ALU pipe.
+__device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c) {   // a * b + c on the FMA pipe
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// pub: the word published to the next lane, ((Ph & 2^31) | T) + hn with the
+// updated T (bit 31 and bit 0 of T are clear), formed by multiply-adds as
+// T_old + hp (2^31 + 2) - hn.
+template <int P>
+__device__ __forceinline__ void wave_column(const uint32_t (&pa)[P], uint32_t (&bw)[P], uint32_t wv, uint32_t& Pv,
+                                            uint32_t& Mv, uint32_t& T, uint32_t& Ph, uint32_t& hn, uint32_t& pub) {
+  uint32_t Eq = 0xffffffffu;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const uint32_t xb = (uint32_t)__mulhi((int32_t)bw[p], 1);   // B's bit p broadcast (sign of bw)
+    Eq &= ~(pa[p] ^ xb);
+    bw[p] *= 2u;
+  }
+  const uint32_t hin_neg = wv & 1u;
+  const uint32_t hin_pos = __umulhi(wv, 2u);
+  const uint32_t Xv = Eq | Mv;
+  const uint32_t Eh = Eq | hin_neg;
+  const uint32_t Xh = (((Eh & Pv) + Pv) ^ Pv) | Eh;
+  Ph = Mv | ~(Xh | Pv);
+  const uint32_t Mh = Pv & Xh;
+  hn = __umulhi(Mh, 2u);
+  const uint32_t hp = __umulhi(Ph, 2u);
+  pub = mad_lo(hn, 0xffffffffu, mad_lo(hp, 0x80000002u, T));
+  T = mad_lo(hn, 0xfffffffeu, mad_lo(hp, 2u, T));
+  const uint32_t Ph1 = Ph * 2u + hin_pos;   // (Ph << 1) | hin > 0
+  const uint32_t Mh1 = Mh * 2u + hin_neg;   // (Mh << 1) | hin < 0
+  Pv = Mh1 | ~(Xv | Ph1);
+  Mv = Ph1 & Xv;
+}
+
+template <int G, int P>
+__global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
+                                                          unsigned long long* __restrict__ next) {
+  const int lane = threadIdx.x & 31;
+  const int gl = lane & (G - 1);
+  const int gbase = lane - gl;
+  const uint32_t gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << gbase);
+  const int prev_lane = gbase + ((gl + G - 1) & (G - 1));
+  const uint64_t q_lo = a.range_lo ? *a.range_lo : 0;
+  const uint64_t q_hi = a.range_hi ? *a.range_hi : a.m;
+  // pair state (identical in the G lanes of a group)
+  bool has = false, more = true;
+  uint64_t t = 0;
+  uint32_t k = 0;
+  int64_t oA = 0, oB = 0;
+  int32_t m = 0, n = 0, d0 = 0, dlo = 0, dhi = 0, bm = 0;
+  int32_t sbase = 0;   // wavefront steps done on the pair
+  // block state (this lane): block b runs at the steps where 0 <= u <= span
+  // (u counts up by one per step); block b - 1 computed the same column one
+  // step earlier while u <= u_valid; diagonal d0 crosses it where
+  // 0 <= u + dg < 32
+  int32_t b = 0, u = kDeadU, span = 0, u_valid = -1, dg = 0x40000000;
+  uint32_t T = 0;   // score << 1
+  uint32_t Pv = 0, Mv = 0;
+  uint32_t pa[P], bw[P];
+  uint32_t pub = kIdle;
+  bool done = false, reject = false;
+  int32_t result = 0;
+  uint64_t work = 0, nskip = 0;
+#pragma unroll
+  for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
+
+  // Take block nb after step s.  Its columns are [jf, jl]; block nb computes
+  // column j at step j + nb.  Blocks past row m never run.
+  auto take_block = [&](int32_t nb, int32_t s) {
+    b = nb;
+    if (b <= bm) {
+      const int32_t jf = max(1, 32 * b + 1 - dhi);
+      const int32_t jl = min(n, 32 * b + 32 - dlo);
+      u = s - (jf + b);
+      span = jl - jf;
+      u_valid = b == 0 ? -1 : min(n, 32 * b - dlo) - jf;   // last column of block b - 1
+      dg = jf - 32 * b - 1 + d0;   // row j + d0 is row 32 b + 1 + (u + dg)
+    } else {
+      u = kDeadU;
+      span = 0;
+      u_valid = -1;
+      dg = 0x40000000;
+    }
+  };
+
+  while (true) {
+    // ---- groups without a pair take pairs until they hold one that needs
+    // the wavefront (one vote while all groups are busy)
+    while (true) {
+      const bool need = !has && more;
+      const uint32_t leaders = __ballot_sync(0xffffffffu, need && gl == 0);
+      if (!leaders) break;
+      const int first = __ffs(leaders) - 1;
+      unsigned long long base = 0;
+      if (lane == first) base = atomicAdd(next, (unsigned long long)__popc(leaders));
+      base = __shfl_sync(0xffffffffu, base, first);
+      const uint64_t q = q_lo + base + __popc(leaders & ((1u << gbase) - 1u));
+      if (need) {
+        if (q >= q_hi) {
+          more = false;
+        } else {
+          t = a.order ? a.order[q] : q;
+          int64_t gm = 0, gn = 0;
+          k = a.pk ? a.pk[t] : a.K;
+          uint32_t res = 0xffffffffu;
+          const uint32_t* fed = a.first_ed ? a.first_ed : a.ed;
+          const bool skip = a.skip_kband && a.skip_kband[t] < a.K && fed[t] <= a.skip_kband[t];
+          if (skip) {
+            if (a.first_ed && gl == 0) put_result(a, t, fed[t]);
+            res = 0xfffffffeu;   // settled by the first pass: nothing to do
+          } else if (!pair_geometry(a, q, t, oA, oB, gm, gn)) {
+            if (gl == 0) atomicOr(a.dev_flags, FLAG_BOUNDS);
+            res = k + 1;
+          } else {
+            const int64_t mm = gm, nn = gn;
+            if (mm >= (int64_t)kMaxLen) {
+              if (gl == 0) atomicOr(a.dev_flags, FLAG_LENGTH);
+              res = k + 1;
+            } else if (mm - nn > (int64_t)k) {
+              res = k + 1;
+            } else if (nn == 0) {
+              res = (uint32_t)mm;
+            } else {
+              m = (int32_t)mm;
+              n = (int32_t)nn;
+              d0 = m - n;
+              dlo = -(int32_t)((k - (uint32_t)d0) >> 1);
+              dhi = d0 + (int32_t)((k - (uint32_t)d0) >> 1);
+              if (dhi - dlo < 63) dlo = dhi - 63;   // at least 64 band rows (any wider band is exact)
+              bm = (m - 1) >> 5;
+              sbase = 0;
+              take_block(gl, 0);
+              pub = kIdle;
+              done = reject = false;
+            }
+          }
+          if (res == 0xfffffffeu) {
+            if (gl == 0) ++nskip;
+          } else if (res != 0xffffffffu) {
+            if (gl == 0) put_result(a, t, res);
+          } else {
+            has = true;
+          }
+        }
+      }
+    }
+    if (!__any_sync(0xffffffffu, has || more)) break;
+
+    // ---- kWaveSteps wavefront steps.  Every lane runs the column step; a lane
+    // outside its block's steps computes on stale state (rebuilt at the
+    // block's first column) that no other lane reads.  First and last
+    // columns and the diagonal test take one rarely divergent branch.
+    // Steps in which no lane of the warp meets such an event (a block's first
+    // or last column, its input word switching from the predecessor's to the
+    // band edge's, the window's last step) run in a loop without the tests:
+    // their number is the warp's minimum of the steps to each lane's next
+    // event.
+    int it = 0;
+    while (it < kWaveSteps) {
+      {
+        const int64_t un = (int64_t)u + 1;   // u at the next step
+        int64_t fr = kWaveSteps - 1 - it;
+        if (un <= 0) fr = min(fr, -un);
+        if (un <= span) fr = min(fr, (int64_t)span - un);
+        if (un <= u_valid) fr = min(fr, (int64_t)u_valid - un + 1);
+        const int free = __reduce_min_sync(0xffffffffu, (int)fr);
+        const bool from_prev = un <= u_valid;
+        const uint32_t keep_in = from_prev ? 1u : 0u, idle_in = from_prev ? 0u : kIdle;
+#pragma unroll 4
+        for (int f = 0; f < free; ++f) {
+          const uint32_t w_in = __shfl_sync(0xffffffffu, pub, prev_lane);
+          const uint32_t wv = mad_lo(w_in, keep_in, idle_in);   // w_in, or kIdle at the band's edge
+          uint32_t Ph, hn;
+          wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+        }
+        u += free;
+        it += free;
+      }
+      const uint32_t w_in = __shfl_sync(0xffffffffu, pub, prev_lane);
+      ++u;
+      const uint32_t wv = u <= u_valid ? w_in : kIdle;
+      uint32_t Ph, hn;
+      wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+      const bool diag_here = it == kWaveSteps - 1 && (uint32_t)(u + dg) < 32u;
+      if (u == 0 || u == span || diag_here) {
+        if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
+          const int32_t jf = sbase + it + 1 - b;
+          wave_load_bits<P>(a, PW, (uint64_t)(oA + 32 * (int64_t)b + 32 * (int64_t)GW), pa, false);
+          wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
+          Pv = 0xffffffffu;
+          Mv = 0u;
+          wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+          // D of the row above the block in this column, plus the block's deltas
+          const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
+          const int32_t score = above + (int32_t)__popc(Pv) - (int32_t)__popc(Mv);
+          T = (uint32_t)score << 1;
+          pub = ((Ph & 0x80000000u) | T) + hn;
+        }
+        // D at row r of this block = score minus the deltas of the rows below r
+        if (diag_here && (uint32_t)u <= (uint32_t)span) {   // row j + d0 of diagonal d0
+          const int tr = u + dg;
+          const uint32_t below = tr == 31 ? 0u : (0xffffffffu << (tr + 1));
+          const int32_t diag = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+          if (diag > (int32_t)k) reject = true;
+        }
+        if (u == span) {   // the block leaves the band
+          if (b == bm) {
+            const int tm = (m - 1) & 31;
+            const uint32_t below = tm == 31 ? 0u : (0xffffffffu << (tm + 1));
+            result = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+            done = true;
+          }
+          work += (uint64_t)(span + 1);
+          take_block(b + G, sbase + it + 1);
+        }
+      }
+      ++it;
+    }
+    sbase += kWaveSteps;
+    if ((sbase & 31) == 0 && u >= 0 && u <= span) {   // B's symbols of the next 32 columns, all lanes at once
+      wave_load_bits<P>(a, PW, (uint64_t)(oB + (sbase - b) + 32 * (int64_t)GW), bw, true);
+    }
+    // ---- a group whose pair finished (or was rejected) writes it and frees
+    // its lanes; one vote in the common case where none did
+    const bool overrun = has && sbase >= n + bm;   // cannot happen: the last block ends at step n + bm
+    if (__ballot_sync(0xffffffffu, done || reject || overrun)) {
+      const uint32_t dmask = __ballot_sync(0xffffffffu, done) & gmask;
+      const uint32_t rmask = __ballot_sync(0xffffffffu, reject) & gmask;
+      const int src = dmask ? __ffs(dmask) - 1 : lane;
+      const int32_t fin = __shfl_sync(0xffffffffu, result, src);
+      bool end = false;
+      if (has && (dmask || rmask)) {
+        if (gl == 0) put_result(a, t, rmask ? k + 1 : (fin > (int32_t)k ? k + 1 : (uint32_t)fin));
+        end = true;
+      } else if (overrun) {
+        if (gl == 0) {
+          atomicOr(a.dev_flags, FLAG_BOUNDS);
+          put_result(a, t, k + 1);
+        }
+        end = true;
+      }
+      if (end) {
+        if (u >= 0 && u <= span) work += (uint64_t)(u + 1);   // block cut short by the exit
+        has = false;
+        u = kDeadU;
+        span = 0;
+        u_valid = -1;
+        dg = 0x40000000;
+        pub = kIdle;
+        done = reject = false;
+      }
+    }
+  }
+  if (a.work) {
+    for (int o = 16; o > 0; o >>= 1) work += __shfl_down_sync(0xffffffffu, work, o);
+    if (lane == 0 && work) atomicAdd(a.work, (unsigned long long)work);
+  }
+  if (a.skipped) {
+    for (int o = 16; o > 0; o >>= 1) nskip += __shfl_down_sync(0xffffffffu, nskip, o);
+    if (lane == 0 && nskip) atomicAdd(a.skipped, (unsigned long long)nskip);
+  }
+}
+
+// ---------------------------------------------------------------- bands wider than one warp
+// One CTA of V warps (G = 32 V lanes) per pair, for bands whose wavefront
+// needs more than 32 lanes (K >= 1025).  Blocks, lanes and the column step
+// are those of verify_wave_kernel (lane g owns blocks b = g mod G), with one
+// change to the schedule: block b computes column j at step
+//     j + b + 32 floor(b / 32),
+// i.e. every group of 32 blocks runs one window of kWaveSteps (= 32) steps
+// behind the group above it.  Inside a group the predecessor block b - 1 is
+// the next lane down in the same warp and hands its word over by a shuffle,
+// one step earlier as before.  The first block of a group (lane 0 of its
+// warp) takes its predecessor's word from the last lane of the previous warp,
+// written 33 steps earlier into a ring in shared memory: the CTA synchronises
+// once per window (__syncthreads), after which the previous window's words
+// are visible.  The extra skew also spaces a lane's consecutive blocks b and
+// b + G by 2G steps instead of G, so G lanes hold any band with
+//     34 G >= 32 + (dhi - dlo),  dhi - dlo <= K.
+// Pair fetch, the early exit and the result are CTA-wide decisions taken at
+// the window barrier; every loop bound is uniform over the CTA.
+constexpr int kRing = 128;   // words per warp in the ring: steps s - 128 .. s - 1 (reads reach s - 33)
+
+template <int V, int P>
+__global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
+                                                            unsigned long long* __restrict__ next) {
+  constexpr int G = 32 * V;
+  constexpr int S = kWaveSteps;
+  static_assert(S == 32 && kRing >= 2 * S + 2 && (kRing & (kRing - 1)) == 0, "window and ring sizes");
+  __shared__ uint32_t ring[V][kRing];
+  __shared__ unsigned long long s_t;   // pair of the CTA (~0: none left)
+  __shared__ longlong2 s_geo;          // its offsets of A and B
+  __shared__ int2 s_len;               // and lengths m >= n
+  __shared__ int s_flag[3];            // per window (mod 3): 1 = finished, 2 = rejected
+  __shared__ int32_t s_result[3];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int prev_warp = (warp + V - 1) % V;
+  const uint64_t q_lo = a.range_lo ? *a.range_lo : 0;
+  const uint64_t q_hi = a.range_hi ? *a.range_hi : a.m;
+  if (tid < 3) s_flag[tid] = 0;
+  uint32_t k = 0;
+  int64_t oA = 0, oB = 0;
+  int32_t m = 0, n = 0, d0 = 0, dlo = 0, dhi = 0, bm = 0;
+  int32_t b = 0, u = kDeadU, span = 0, u_valid = -1, dg = 0x40000000, colbase = 0;
+  uint32_t T = 0, Pv = 0, Mv = 0;
+  uint32_t pa[P], bw[P];
+  uint32_t pub = kIdle;
+  bool done = false, reject = false;
+  int32_t result = 0;
+  uint32_t win = 0;   // windows run by the CTA (selects the flag slot)
+  uint64_t work = 0, nskip = 0;
+#pragma unroll
+  for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
+
+  // Take block nb after s steps.  Its columns are [jf, jl]; it computes
+  // column j at step j + colbase (colbase = nb + 32 floor(nb / 32)).
+  auto take_block = [&](int32_t nb, int32_t s) {
+    b = nb;
+    if (b <= bm) {
+      const int32_t jf = max(1, 32 * b + 1 - dhi);
+      const int32_t jl = min(n, 32 * b + 32 - dlo);
+      colbase = b + S * (b >> 5);
+      u = s - (jf + colbase);
+      span = jl - jf;
+      u_valid = b == 0 ? -1 : min(n, 32 * b - dlo) - jf;   // last column of block b - 1
+      dg = jf - 32 * b - 1 + d0;
+    } else {
+      u = kDeadU;
+      span = 0;
+      u_valid = -1;
+      dg = 0x40000000;
+      colbase = 0;
+    }
+  };
+
+  while (true) {
+    // ---- thread 0 takes pairs until one needs the wavefront
+    if (tid == 0) {
+      unsigned long long got = ~0ull;
+      while (true) {
+        const uint64_t q = q_lo + atomicAdd(next, 1ull);
+        if (q >= q_hi) break;
+        const uint64_t t = a.order ? a.order[q] : q;
+        const uint32_t kt = a.pk ? a.pk[t] : a.K;
+        const uint32_t* fed = a.first_ed ? a.first_ed : a.ed;
+        if (a.skip_kband && a.skip_kband[t] < a.K && fed[t] <= a.skip_kband[t]) {
+          if (a.first_ed) put_result(a, t, fed[t]);
+          ++nskip;
+          continue;
+        }
+        int64_t gA, gB, mm, nn;
+        if (!pair_geometry(a, q, t, gA, gB, mm, nn)) {
+          atomicOr(a.dev_flags, FLAG_BOUNDS);
+          put_result(a, t, kt + 1);
+          continue;
+        }
+        if (mm >= (int64_t)kMaxLen) {
+          atomicOr(a.dev_flags, FLAG_LENGTH);
+          put_result(a, t, kt + 1);
+          continue;
+        }
+        if (mm - nn > (int64_t)kt) {
+          put_result(a, t, kt + 1);
+          continue;
+        }
+        if (nn == 0) {
+          put_result(a, t, (uint32_t)mm);
+          continue;
+        }
+        got = t;
+        s_geo = make_longlong2(gA, gB);
+        s_len = make_int2((int32_t)mm, (int32_t)nn);
+        break;
+      }
+      s_t = got;
+    }
+    __syncthreads();
+    const unsigned long long t = s_t;
+    if (t == ~0ull) break;
+    {
+      k = a.pk ? a.pk[t] : a.K;
+      const longlong2 geo = s_geo;
+      const int2 len = s_len;
+      oA = geo.x;
+      oB = geo.y;
+      m = len.x;
+      n = len.y;
+      d0 = m - n;
+      dlo = -(int32_t)((k - (uint32_t)d0) >> 1);
+      dhi = d0 + (int32_t)((k - (uint32_t)d0) >> 1);
+      if (dhi - dlo < 63) dlo = dhi - 63;
+      bm = (m - 1) >> 5;
+    }
+    take_block(tid, 0);
+    pub = kIdle;
+    done = reject = false;
+    const int32_t last_step = n + bm + S * (bm >> 5);   // block bm's last column
+    int32_t sbase = 0;
+    while (true) {
+#pragma unroll 8
+      for (int it = 0; it < S; ++it) {
+        const int32_t s1 = sbase + it + 1;   // this step, counted from 1
+        uint32_t w_in = __shfl_up_sync(0xffffffffu, pub, 1);
+        if (lane == 0) w_in = ring[prev_warp][(uint32_t)(s1 - 1 - S) & (kRing - 1)];
+        ++u;
+        const uint32_t wv = u <= u_valid ? w_in : kIdle;
+        uint32_t Ph, hn;
+        wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+        const bool diag_here = it == S - 1 && (uint32_t)(u + dg) < 32u;
+        if (u == 0 || u == span || diag_here) {
+          if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
+            const int32_t jf = s1 - colbase;
+            wave_load_bits<P>(a, PW, (uint64_t)(oA + 32 * (int64_t)b + 32 * (int64_t)GW), pa, false);
+            wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
+            Pv = 0xffffffffu;
+            Mv = 0u;
+            wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+            const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
+            const int32_t score = above + (int32_t)__popc(Pv) - (int32_t)__popc(Mv);
+            T = (uint32_t)score << 1;
+            pub = ((Ph & 0x80000000u) | T) + hn;
+          }
+          if (diag_here && (uint32_t)u <= (uint32_t)span) {   // row j + d0 of diagonal d0
+            const int tr = u + dg;
+            const uint32_t below = tr == 31 ? 0u : (0xffffffffu << (tr + 1));
+            const int32_t diag = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+            if (diag > (int32_t)k) reject = true;
+          }
+          if (u == span) {   // the block leaves the band
+            if (b == bm) {
+              const int tm = (m - 1) & 31;
+              const uint32_t below = tm == 31 ? 0u : (0xffffffffu << (tm + 1));
+              result = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+              done = true;
+            }
+            work += (uint64_t)(span + 1);
+            take_block(b + G, s1);
+          }
+        }
+        if (lane == 31) ring[warp][(uint32_t)s1 & (kRing - 1)] = pub;
+      }
+      sbase += S;
+      if (u >= 0 && u <= span)   // B's symbols of the next 32 columns
+        wave_load_bits<P>(a, PW, (uint64_t)(oB + (sbase - colbase) + 32 * (int64_t)GW), bw, true);
+      const uint32_t slot = win % 3;
+      if (done) {
+        s_result[slot] = result;
+        atomicOr(&s_flag[slot], 1);
+      }
+      if (reject) atomicOr(&s_flag[slot], 2);
+      __syncthreads();
+      const int f = s_flag[slot];
+      const int32_t fin = s_result[slot];
+      if (tid == 0) s_flag[(win + 2) % 3] = 0;
+      ++win;
+      const bool overrun = sbase >= last_step;   // finished at the latest in the window of step last_step
+      if (f || overrun) {
+        if (tid == 0) {
+          if (f & 1) {
+            put_result(a, t, fin > (int32_t)k ? k + 1 : (uint32_t)fin);
+          } else if (f & 2) {
+            put_result(a, t, k + 1);
+          } else {
+            atomicOr(a.dev_flags, FLAG_BOUNDS);
+            put_result(a, t, k + 1);
+          }
+        }
+        if (u >= 0 && u <= span) work += (uint64_t)(u + 1);   // block cut short by the exit
+        break;
+      }
+    }
+  }
+  if (a.work) {
+    for (int o = 16; o > 0; o >>= 1) work += __shfl_down_sync(0xffffffffu, work, o);
+    if (lane == 0 && work) atomicAdd(a.work, (unsigned long long)work);
+  }
+  if (tid == 0 && a.skipped && nskip) atomicAdd(a.skipped, (unsigned long long)nskip);
+}
+
+template <int G, int P>
+int launch_gp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+  int dev = 0, sms = kNumSMsHint, per_sm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_wave_kernel<G, P>, 128, 0);
+  if (per_sm < 1) per_sm = 1;
+  uint64_t need = (a.m * G + 127) / 128;
+  uint64_t grid = (uint64_t)sms * per_sm;
+  if (need < grid) grid = need;
+  verify_wave_kernel<G, P><<<(unsigned)(grid ? grid : 1), 128, 0, s>>>(a, PW, GW, next);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+template <int G>
+int launch_g(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+  if (a.bits <= 2) return launch_gp<G, 2>(a, PW, GW, next, s);
+  if (a.bits <= 5) return launch_gp<G, 5>(a, PW, GW, next, s);
+  return launch_gp<G, 8>(a, PW, GW, next, s);
+}
+
+template <int V, int P>
+int launch_vp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+  int dev = 0, sms = kNumSMsHint, per_sm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_cta_kernel<V, P>, 32 * V, 0);
+  if (per_sm < 1) per_sm = 1;
+  // pairs take about equally long: no more CTAs than give every one the same
+  // number of pairs (fewer CTAs per SM run faster, a part-filled last round
+  // does not)
+  uint64_t grid = (uint64_t)sms * per_sm;
+  const uint64_t rounds = (a.m + grid - 1) / grid;
+  grid = (a.m + rounds - 1) / rounds;
+  verify_cta_kernel<V, P><<<(unsigned)(grid ? grid : 1), 32 * V, 0, s>>>(a, PW, GW, next);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+template <int V>
+int launch_v(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+  if (a.bits <= 2) return launch_vp<V, 2>(a, PW, GW, next, s);
+  if (a.bits <= 5) return launch_vp<V, 5>(a, PW, GW, next, s);
+  return launch_vp<V, 8>(a, PW, GW, next, s);
+}
+
+}  // namespace
+
+int launch_verify_wave(const VerifyArgs& a, uint64_t PW, uint32_t GW, int lanes, unsigned long long* next,
+                       cudaStream_t s) {
+  switch (lanes) {
+    case 2: return launch_g<2>(a, PW, GW, next, s);
+    case 4: return launch_g<4>(a, PW, GW, next, s);
+    case 8: return launch_g<8>(a, PW, GW, next, s);
+    case 16: return launch_g<16>(a, PW, GW, next, s);
+    case 32: return launch_g<32>(a, PW, GW, next, s);
+    case 64: return launch_v<2>(a, PW, GW, next, s);
+    case 128: return launch_v<4>(a, PW, GW, next, s);
+    case 256: return launch_v<8>(a, PW, GW, next, s);
+    case 512: return launch_v<16>(a, PW, GW, next, s);
+    case 1024: return launch_v<32>(a, PW, GW, next, s);
+    default: return MJ_ERR_UNSUPPORTED;
+  }
+}
+
+}  // namespace mj

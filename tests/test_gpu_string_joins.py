@@ -10,7 +10,7 @@ from tests.gpu_util import to_device
 
 pytestmark = pytest.mark.gpu
 
-N = 66_000   # strings from which plain joins go string by string at any length
+N = 66_000   # more strings than a 16-bit window holds
 
 
 def _set(seed, n, lo, hi, symbols, K, rate=0.05, extra=(), T=0):

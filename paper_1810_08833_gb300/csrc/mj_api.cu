@@ -198,7 +198,7 @@ struct mj_ctx {
   uint64_t last_sig[26] = {};
   uint64_t graph_launches = 0;
   // learned first-pass band: parameters P, Adam moments M and V, gradient G, loss
-  Buf band;
+  Buf band, band_part;
   bool band_ready = false;
   uint32_t band_margin = 0, band_min_mult = 2;
   bool band_gate_auto = false;   // set band_min_mult from the training data
@@ -1327,7 +1327,7 @@ void mj_destroy(mj_ctx* c) {
                  &c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi, &c->rk_first, &c->rk_delta,
                  &c->rk_scan, &c->rk_short_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
                  &c->out_i, &c->out_j, &c->out_ed, &c->in_bytes, &c->in_offsets, &c->branges,
-                 &c->band, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
+                 &c->band, &c->band_part, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
                  &c->franges, &c->fnext, &c->fcnt, &c->ed_first};
   for (Buf* b : bufs) b->release();
   for (int i = 0; i < mj_ctx::kAuxStreams; ++i) {
@@ -1844,10 +1844,10 @@ int mj_band_train(mj_ctx* c, const float* d_x, const uint32_t* d_ed, uint64_t m,
   float* V = M + kBandParams;
   float* G = V + kBandParams;
   float* L = G + kBandParams;
+  MJ_TRY(c->band_part.reserve(band_grad_part_bytes(tp->batch), s));
   for (uint32_t step = 0; step < tp->steps; ++step) {
-    MJ_CUDA_TRY(cudaMemsetAsync(G, 0, sizeof(float) * (kBandParams + 1), s));
     MJ_TRY(launch_band_grad(P, d_x, nullptr, d_ed, K, m, tp->batch, tp->seed + (uint64_t)step * tp->batch, tp->tau,
-                            G, L, s));
+                            c->band_part.as<float>(), G, L, s));
     MJ_TRY(launch_band_adam(P, G, M, V, tp->lr, 0.9f, 0.999f, 1e-8f, ++c->band_step, s));
   }
   float loss = 0.f;
@@ -1885,7 +1885,7 @@ int mj_band_forward(mj_ctx* c, const float* d_x, uint64_t m, void* stream, float
   if (!c || (m && (!d_x || !d_yhat))) return MJ_ERR_ARG;
   if (!c->band_ready) return MJ_ERR_STATE;
   DeviceGuard g(c->device);
-  return launch_band_forward(c->band.as<float>(), d_x, m, nullptr, 0, d_yhat, S(stream));
+  return launch_band_forward(c->band.as<float>(), d_x, m, d_yhat, S(stream));
 }
 
 int mj_band_grad(mj_ctx* c, const float* d_x, const float* d_y, uint64_t m, float tau, void* stream, float* d_grad,
@@ -1896,13 +1896,11 @@ int mj_band_grad(mj_ctx* c, const float* d_x, const float* d_y, uint64_t m, floa
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
   float* L = c->band.as<float>() + 4 * kBandParams;
-  MJ_CUDA_TRY(cudaMemsetAsync(d_grad, 0, sizeof(float) * kBandParams, s));
-  MJ_CUDA_TRY(cudaMemsetAsync(L, 0, sizeof(float), s));
-  MJ_TRY(launch_band_grad(c->band.as<float>(), d_x, d_y, nullptr, 0, m, m, 0, tau, d_grad, L, s));
-  float l = 0.f;
-  MJ_CUDA_TRY(cudaMemcpyAsync(&l, L, sizeof(float), cudaMemcpyDeviceToHost, s));
-  MJ_CUDA_TRY(cudaStreamSynchronize(s));
-  if (loss) *loss = l;
+  MJ_TRY(c->band_part.reserve(band_grad_part_bytes(m), s));
+  MJ_TRY(launch_band_grad(c->band.as<float>(), d_x, d_y, nullptr, 0, m, m, 0, tau, c->band_part.as<float>(), d_grad, L,
+                          s));
+  MJ_TRY(readback(c, L, sizeof(float), s));
+  if (loss) memcpy(loss, c->h_small, sizeof(float));
   return MJ_OK;
 }
 

@@ -419,11 +419,11 @@ constexpr int kBandParams = kBandHidden * kBandFeatures + kBandHidden + kBandHid
 static_assert(kBandParams == MJ_BAND_PARAMS && kBandFeatures == MJ_BAND_FEATURES, "ABI constants");
 int launch_band_features(const uint32_t* ci, const uint32_t* cj, const uint32_t* mult, const uint32_t* parts,
                          const int64_t* offsets, uint64_t m, uint32_t K, uint32_t T, float* X, cudaStream_t s);
-int launch_band_forward(const float* P, const float* X, uint64_t m, const uint32_t* gate, uint32_t min_gate,
-                        float* out, cudaStream_t s);
-size_t band_grad_smem();
+int launch_band_forward(const float* P, const float* X, uint64_t m, float* out, cudaStream_t s);
+// part: band_grad_part_bytes(batch) of scratch; grad and *loss are overwritten
+size_t band_grad_part_bytes(uint64_t batch);
 int launch_band_grad(const float* P, const float* X, const float* Y, const uint32_t* ed, uint32_t K, uint64_t m,
-                     uint64_t batch, uint64_t seed, float tau, float* grad, float* loss, cudaStream_t s);
+                     uint64_t batch, uint64_t seed, float tau, float* part, float* grad, float* loss, cudaStream_t s);
 int launch_band_adam(float* P, const float* G, float* M, float* V, float lr, float b1, float b2, float eps, int step,
                      cudaStream_t s);
 int launch_band_fused(const float* P, const uint32_t* ci, const uint32_t* cj, const uint32_t* run_start, uint64_t raw,

@@ -3,6 +3,8 @@
 // here is in the MinJoin paper; the band it proposes only narrows a first
 // verification pass, and every pair that pass does not settle is verified
 // again with band K, so the join's output does not depend on the model.
+#include <algorithm>
+
 #include "mj_internal.cuh"
 
 namespace mj {
@@ -45,160 +47,316 @@ __global__ void features_kernel(const uint32_t* __restrict__ ci, const uint32_t*
   }
 }
 
-// ŷ of every sample (gate: samples with gate[u] < min_gate get +inf).
-__global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                      uint64_t m, const uint32_t* __restrict__ gate,
-                                                      uint32_t min_gate, float* __restrict__ out) {
-  __shared__ float s[kBandParams];
-  for (int i = threadIdx.x; i < kBandParams; i += blockDim.x) s[i] = P[i];
-  __syncthreads();
-  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < m; u += (uint64_t)gridDim.x * blockDim.x) {
-    if (gate && gate[u] < min_gate) {
-      out[u] = __int_as_float(0x7f800000);
-      continue;
-    }
-    float x[F];
-#pragma unroll
-    for (int f = 0; f < F; ++f) x[f] = X[u * F + f];
-    float h1[H];
-#pragma unroll
-    for (int a = 0; a < H; ++a) {
-      float z = s[OFF_B1 + a];
-#pragma unroll
-      for (int f = 0; f < F; ++f) z = fmaf(s[OFF_W1 + a * F + f], x[f], z);
-      h1[a] = relu(z);
-    }
-    float y = s[OFF_B3];
-#pragma unroll 4
-    for (int c = 0; c < H; ++c) {
-      float z = s[OFF_B2 + c];
-#pragma unroll
-      for (int a = 0; a < H; ++a) z = fmaf(s[OFF_W2 + c * H + a], h1[a], z);
-      y = fmaf(s[OFF_W3 + c], relu(z), y);
-    }
-    out[u] = y;
-  }
-}
-
 __device__ __forceinline__ uint64_t mix(uint64_t z) {  // splitmix64 finaliser (Steele, Lea, Flood 2014)
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
   z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
   return z ^ (z >> 31);
 }
 
-constexpr int kSB = 64;   // samples per block chunk of the gradient kernel
-constexpr int kLd = H + 1;
+// The network runs on chunks of 64 samples, a block of 256 threads each, as
+// 64 x 64 x 64 products in shared memory: thread t holds the 16 outputs of rows
+// t / 16 + 16 i and columns t % 16 + 16 j.  Operands are rows along the summed
+// index, read 16 bytes at a time: 8 loads feed 64 multiply-adds, and rows
+// kLd = 68 words apart keep the 8 lanes of a load phase in different banks.
+// Sums run in ascending order from the bias in FP32, as in a plain loop.
+constexpr int kSB = 64;
+constexpr int kNetThreads = 256;
+constexpr int kLd = H + 4;
+constexpr int kTile = kSB * kLd;
+static_assert(kSB == H, "the products are square");
 
-// Loss and parameter gradient of a batch, accumulated (atomically, one add
-// per parameter and block chunk) into grad[] and *loss.
-//  samples: batch indices idx[b] if idx is given, else b (b < batch); with
-//           seed != 0 a sample is drawn as mix(seed + b) % m.
-//  target:  y from Y, or from ed as min(ed, K+1) / K.
-//  loss:    tau == 0: mean squared error; else pinball loss at quantile tau.
-__global__ void __launch_bounds__(kSB) grad_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                   const float* __restrict__ Y, const uint32_t* __restrict__ ed,
-                                                   uint32_t K, uint64_t m, uint64_t batch, uint64_t seed, float tau,
-                                                   float* __restrict__ grad, float* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* w = sm;                          // kBandParams
-  float* h1s = w + kBandParams;           // [kSB][kLd]
-  float* h2s = h1s + kSB * kLd;           // [kSB][kLd]
-  float* d2s = h2s + kSB * kLd;           // [kSB][kLd]
-  float* d1s = d2s + kSB * kLd;           // [kSB][kLd]
-  float* xs = d1s + kSB * kLd;            // [kSB][F]
-  float* dys = xs + kSB * F;              // [kSB]
-  for (int i = threadIdx.x; i < kBandParams; i += blockDim.x) w[i] = P[i];
-  const float inv = 1.f / (float)batch;
-  for (uint64_t base = (uint64_t)blockIdx.x * kSB; base < batch; base += (uint64_t)gridDim.x * kSB) {
-    __syncthreads();
-    const uint64_t bidx = base + threadIdx.x;
-    const int s = threadIdx.x;
-    float dy = 0.f;
-    if (bidx < batch) {
-      const uint64_t u = seed ? mix(seed + bidx) % m : bidx;
-      float x[F];
+// acc[i][j] += sum over k of A[row i][k] B[column j][k]
+__device__ __forceinline__ void product(const float* __restrict__ A, const float* __restrict__ B, int tr, int tc,
+                                        float (&acc)[4][4]) {
+#pragma unroll 4
+  for (int k = 0; k < H; k += 4) {
+    float4 a[4], b[4];
 #pragma unroll
-      for (int f = 0; f < F; ++f) {
-        x[f] = X[u * F + f];
-        xs[s * F + f] = x[f];
-      }
-      float h1[H];
+    for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(A + (tr + 16 * i) * kLd + k);
 #pragma unroll
-      for (int a = 0; a < H; ++a) {
-        float z = w[OFF_B1 + a];
+    for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(B + (tc + 16 * j) * kLd + k);
 #pragma unroll
-        for (int f = 0; f < F; ++f) z = fmaf(w[OFF_W1 + a * F + f], x[f], z);
-        h1[a] = relu(z);
-        h1s[s * kLd + a] = h1[a];
-      }
-      float yhat = w[OFF_B3];
-      for (int c = 0; c < H; ++c) {
-        float z = w[OFF_B2 + c];
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int a = 0; a < H; ++a) z = fmaf(w[OFF_W2 + c * H + a], h1[a], z);
-        const float h2 = relu(z);
-        h2s[s * kLd + c] = h2;
-        yhat = fmaf(w[OFF_W3 + c], h2, yhat);
+      for (int j = 0; j < 4; ++j) {
+        acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+        acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+        acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+        acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
       }
-      const float y = Y ? Y[u] : (float)(ed[u] < K + 1 ? ed[u] : K + 1) / (float)(K ? K : 1);
-      const float r = y - yhat;
-      float l;
-      if (tau == 0.f) {
-        l = r * r;
-        dy = -2.f * r;
-      } else {
-        l = r > 0.f ? tau * r : (tau - 1.f) * r;
-        dy = r > 0.f ? -tau : (1.f - tau);
-      }
-      dy *= inv;
-      atomicAdd(loss, l * inv);
-      // back through layer 3 and the second ReLU
-      float dh1[H];
+  }
+}
+
+// The first layer of the chunk's samples xs[s][f]: units tc + 16 j of samples
+// tr + 16 i.
+__device__ __forceinline__ void first_layer(const float* __restrict__ w, const float* __restrict__ xs, int tr, int tc,
+                                            float (&h)[4][4]) {
 #pragma unroll
-      for (int a = 0; a < H; ++a) dh1[a] = 0.f;
-      for (int c = 0; c < H; ++c) {
-        const float d2 = h2s[s * kLd + c] > 0.f ? dy * w[OFF_W3 + c] : 0.f;
-        d2s[s * kLd + c] = d2;
+  for (int j = 0; j < 4; ++j) {
+    const float4* wj = reinterpret_cast<const float4*>(w + OFF_W1 + (tc + 16 * j) * F);
+    const float4 p = wj[0], q = wj[1];
 #pragma unroll
-        for (int a = 0; a < H; ++a) dh1[a] = fmaf(w[OFF_W2 + c * H + a], d2, dh1[a]);
-      }
-#pragma unroll
-      for (int a = 0; a < H; ++a) d1s[s * kLd + a] = h1[a] > 0.f ? dh1[a] : 0.f;
-    } else {
-      for (int a = 0; a < H; ++a) {
-        h1s[s * kLd + a] = 0.f;
-        h2s[s * kLd + a] = 0.f;
-        d2s[s * kLd + a] = 0.f;
-        d1s[s * kLd + a] = 0.f;
-      }
-      for (int f = 0; f < F; ++f) xs[s * F + f] = 0.f;
-    }
-    dys[s] = dy;
-    __syncthreads();
-    // parameter gradients of the chunk: sums over its samples
-    for (int p = threadIdx.x; p < kBandParams; p += blockDim.x) {
-      float g = 0.f;
-      if (p < OFF_B1) {
-        const int a = p / F, f = p % F;
-        for (int q = 0; q < kSB; ++q) g = fmaf(d1s[q * kLd + a], xs[q * F + f], g);
-      } else if (p < OFF_W2) {
-        const int a = p - OFF_B1;
-        for (int q = 0; q < kSB; ++q) g += d1s[q * kLd + a];
-      } else if (p < OFF_B2) {
-        const int c = (p - OFF_W2) / H, a = (p - OFF_W2) % H;
-        for (int q = 0; q < kSB; ++q) g = fmaf(d2s[q * kLd + c], h1s[q * kLd + a], g);
-      } else if (p < OFF_W3) {
-        const int c = p - OFF_B2;
-        for (int q = 0; q < kSB; ++q) g += d2s[q * kLd + c];
-      } else if (p < OFF_B3) {
-        const int c = p - OFF_W3;
-        for (int q = 0; q < kSB; ++q) g = fmaf(dys[q], h2s[q * kLd + c], g);
-      } else {
-        for (int q = 0; q < kSB; ++q) g += dys[q];
-      }
-      if (g != 0.f) atomicAdd(grad + p, g);
+    for (int i = 0; i < 4; ++i) {
+      const float4* xi = reinterpret_cast<const float4*>(xs + (tr + 16 * i) * F);
+      const float4 x = xi[0], y = xi[1];
+      float z = w[OFF_B1 + tc + 16 * j];
+      z = fmaf(p.x, x.x, z);
+      z = fmaf(p.y, x.y, z);
+      z = fmaf(p.z, x.z, z);
+      z = fmaf(p.w, x.w, z);
+      z = fmaf(q.x, y.x, z);
+      z = fmaf(q.y, y.y, z);
+      z = fmaf(q.z, y.z, z);
+      z = fmaf(q.w, y.w, z);
+      h[i][j] = relu(z);
     }
   }
+}
+
+// Output of sample s from the second layer h2t[c][s].
+__device__ __forceinline__ float last_layer(const float* __restrict__ w, const float* __restrict__ h2t, int s) {
+  float y = w[OFF_B3];
+#pragma unroll 16
+  for (int c = 0; c < H; ++c) y = fmaf(w[OFF_W3 + c], h2t[c * kLd + s], y);
+  return y;
+}
+
+// The parameters into shared memory: w as they are but W2, whose rows go to w2
+// (and its columns to w2t, when given).
+__device__ __forceinline__ void load_params(const float* __restrict__ P, float* __restrict__ w, float* __restrict__ w2,
+                                            float* __restrict__ w2t) {
+  for (int i = threadIdx.x; i < kBandParams; i += kNetThreads) {
+    const float v = P[i];
+    if (i >= OFF_W2 && i < OFF_B2) {
+      const int c = (i - OFF_W2) / H, a = (i - OFF_W2) % H;
+      w2[c * kLd + a] = v;
+      if (w2t) w2t[a * kLd + c] = v;
+    } else {
+      w[i] = v;
+    }
+  }
+}
+
+constexpr int kParamPad = (kBandParams + 3) / 4 * 4;
+constexpr size_t kForwardSmem = sizeof(float) * (kParamPad + kSB * F + 3 * kTile);
+
+// y of every sample.  Bound by the FP32 multiply-adds (4,672 a sample):
+// 65,536 samples 76 us with one sample per thread and a shared load for every
+// one to four of them, 32 us so (300,000: 290, 83).
+__global__ void __launch_bounds__(kNetThreads) forward_kernel(const float* __restrict__ P, const float* __restrict__ X,
+                                                              uint64_t m, float* __restrict__ out) {
+  extern __shared__ __align__(16) float sm[];
+  float* w = sm;
+  float* xs = w + kParamPad;
+  float* w2 = xs + kSB * F;
+  float* h1 = w2 + kTile;    // [s][a]
+  float* h2t = h1 + kTile;   // [c][s]
+  load_params(P, w, w2, nullptr);
+  const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+  for (uint64_t base = (uint64_t)blockIdx.x * kSB; base < m; base += (uint64_t)gridDim.x * kSB) {
+    __syncthreads();   // the parameters are there, the previous chunk's rows are read
+    for (int i = threadIdx.x; i < kSB * F; i += kNetThreads) xs[i] = base * F + i < m * F ? X[base * F + i] : 0.f;
+    __syncthreads();
+    float h[4][4];
+    first_layer(w, xs, tr, tc, h);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h1[(tr + 16 * i) * kLd + tc + 16 * j] = h[i][j];
+        h[i][j] = w[OFF_B2 + tr + 16 * i];
+      }
+    __syncthreads();
+    product(w2, h1, tr, tc, h);   // unit c = row, sample = column
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) h2t[(tr + 16 * i) * kLd + tc + 16 * j] = relu(h[i][j]);
+    __syncthreads();
+    if (threadIdx.x < kSB && base + threadIdx.x < m) out[base + threadIdx.x] = last_layer(w, h2t, threadIdx.x);
+  }
+}
+
+constexpr size_t kGradSmem = sizeof(float) * (kParamPad + 2 * kSB * F + 2 * kSB + 6 * kTile);
+
+// Loss and parameter gradient of a batch: every block's sums over its chunks
+// to part[block][kBandParams + 1] (the loss last), summed by grad_sum_kernel.
+//  samples: batch index b, or with seed != 0 the sample mix(seed + b) % m.
+//  target:  y from Y, or from ed as min(ed, K+1) / K.
+//  loss:    tau == 0: mean squared error; else pinball loss at quantile tau.
+// Sums are taken in a fixed order, so that a call's result does not depend on
+// the blocks' timing.  Bound by the FP32 multiply-adds (13,400 a sample):
+// 65,536 samples with two warps per chunk and atomic sums 267 us, so 133 (the
+// call with its readback); a training step of 1,024 samples 65 us, 30 so.  The
+// loss of 300,000 samples was 2e-5 off the sum in 64 bits, and is 1e-8 off.
+__global__ void __launch_bounds__(kNetThreads, 2) grad_kernel(const float* __restrict__ P, const float* __restrict__ X,
+                                                              const float* __restrict__ Y,
+                                                              const uint32_t* __restrict__ ed, uint32_t K, uint64_t m,
+                                                              uint64_t batch, uint64_t seed, float tau,
+                                                              float* __restrict__ part) {
+  extern __shared__ __align__(16) float sm[];
+  float* w = sm;
+  float* xs = w + kParamPad;       // [s][f]
+  float* xt = xs + kSB * F;        // [f][s]
+  float* dys = xt + kSB * F;       // dy of every sample
+  float* ls = dys + kSB;           // its loss
+  float* w2 = ls + kSB;            // [c][a]
+  float* w2t = w2 + kTile;         // [a][c]
+  float* h1 = w2t + kTile;         // [s][a], then d2 [s][c]
+  float* h1t = h1 + kTile;         // [a][s]
+  float* h2t = h1t + kTile;        // [c][s], then d1 [a][s]
+  float* d2t = h2t + kTile;        // [c][s]
+  float* d2 = h1;
+  float* d1t = h2t;
+  load_params(P, w, w2, w2t);
+  const int t = threadIdx.x, tr = t >> 4, tc = t & 15;
+  const float inv = 1.f / (float)batch;
+  float g2[4][4] = {};             // W2[tr + 16 i][tc + 16 j]
+  float g1[2] = {0.f, 0.f};        // W1 entries t and t + 256
+  float gv = 0.f;                  // t < 64: b1, < 128: b2, < 192: W3, = 192: b3
+  float loss = 0.f;                // t = 224
+  for (uint64_t base = (uint64_t)blockIdx.x * kSB; base < batch; base += (uint64_t)gridDim.x * kSB) {
+    __syncthreads();
+    for (int i = t; i < kSB * F; i += kNetThreads) {
+      const uint64_t b = base + i / F;
+      const uint64_t u = seed ? mix(seed + b) % m : b;
+      const float x = b < batch ? X[u * F + i % F] : 0.f;
+      xs[i] = x;
+      xt[(i % F) * kSB + i / F] = x;
+    }
+    __syncthreads();
+    float h[4][4];
+    first_layer(w, xs, tr, tc, h);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h1[(tr + 16 * i) * kLd + tc + 16 * j] = h[i][j];
+        h1t[(tc + 16 * j) * kLd + tr + 16 * i] = h[i][j];
+        h[i][j] = w[OFF_B2 + tr + 16 * i];
+      }
+    __syncthreads();
+    product(w2, h1, tr, tc, h);   // unit c = tr + 16 i, sample = tc + 16 j
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h[i][j] = relu(h[i][j]);
+        h2t[(tr + 16 * i) * kLd + tc + 16 * j] = h[i][j];
+      }
+    __syncthreads();
+    if (t < kSB) {
+      float dy = 0.f, l = 0.f;
+      const uint64_t b = base + t;
+      if (b < batch) {
+        const uint64_t u = seed ? mix(seed + b) % m : b;
+        const float y = Y ? Y[u] : (float)(ed[u] < K + 1 ? ed[u] : K + 1) / (float)(K ? K : 1);
+        const float r = y - last_layer(w, h2t, t);
+        if (tau == 0.f) {
+          l = r * r;
+          dy = -2.f * r;
+        } else {
+          l = r > 0.f ? tau * r : (tau - 1.f) * r;
+          dy = r > 0.f ? -tau : (1.f - tau);
+        }
+        dy *= inv;
+        l *= inv;
+      }
+      dys[t] = dy;
+      ls[t] = l;
+    }
+    __syncthreads();
+    // back through layer 3 and the second ReLU (samples past the batch have dy = 0)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float v = h[i][j] > 0.f ? dys[tc + 16 * j] * w[OFF_W3 + tr + 16 * i] : 0.f;
+        d2[(tc + 16 * j) * kLd + tr + 16 * i] = v;
+        d2t[(tr + 16 * i) * kLd + tc + 16 * j] = v;
+        h[i][j] = 0.f;
+      }
+    if (t >= 128 && t < 192) {
+      const float* row = h2t + (t - 128) * kLd;
+      float g = 0.f;
+#pragma unroll 16
+      for (int q = 0; q < kSB; ++q) g = fmaf(dys[q], row[q], g);
+      gv += g;
+    } else if (t == 192) {
+      float g = 0.f;
+      for (int q = 0; q < kSB; ++q) g += dys[q];
+      gv += g;
+    } else if (t == 224) {
+      float g = 0.f;
+      for (int q = 0; q < kSB; ++q) g += ls[q];
+      loss += g;
+    }
+    __syncthreads();
+    product(w2t, d2, tr, tc, h);   // unit a = tr + 16 i, sample = tc + 16 j
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int at = (tr + 16 * i) * kLd + tc + 16 * j;
+        d1t[at] = h1t[at] > 0.f ? h[i][j] : 0.f;
+        h[i][j] = 0.f;
+      }
+    product(d2t, h1t, tr, tc, h);   // c = tr + 16 i, a = tc + 16 j, summed over the chunk's samples
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) g2[i][j] += h[i][j];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {   // W1[a][f]
+      const int p = t + kNetThreads * e;
+      const float* row = d1t + (p / F) * kLd;
+      const float* col = xt + (p % F) * kSB;
+      float g = 0.f;
+#pragma unroll 16
+      for (int q = 0; q < kSB; ++q) g = fmaf(row[q], col[q], g);
+      g1[e] += g;
+    }
+    if (t < 128) {
+      const float* row = t < 64 ? d1t + t * kLd : d2t + (t - 64) * kLd;
+      float g = 0.f;
+#pragma unroll 16
+      for (int q = 0; q < kSB; ++q) g += row[q];
+      gv += g;
+    }
+  }
+  float* o = part + (uint64_t)blockIdx.x * (kBandParams + 1);
+#pragma unroll
+  for (int e = 0; e < 2; ++e) o[OFF_W1 + t + kNetThreads * e] = g1[e];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[OFF_W2 + (tr + 16 * i) * H + tc + 16 * j] = g2[i][j];
+  if (t < 64) o[OFF_B1 + t] = gv;
+  else if (t < 128) o[OFF_B2 + t - 64] = gv;
+  else if (t < 192) o[OFF_W3 + t - 128] = gv;
+  else if (t == 192) o[OFF_B3] = gv;
+  else if (t == 224) o[kBandParams] = loss;
+}
+
+// grad[p] and *loss = the blocks' partial sums: eight interleaved sums, then
+// their pairwise sum.
+__global__ void grad_sum_kernel(const float* __restrict__ part, int blocks, float* __restrict__ grad,
+                                float* __restrict__ loss) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p > kBandParams) return;
+  float s[8] = {};
+  int b = 0;
+  for (; b + 8 <= blocks; b += 8) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += part[(uint64_t)(b + k) * (kBandParams + 1) + p];
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (b + k < blocks) s[k] += part[(uint64_t)(b + k) * (kBandParams + 1) + p];
+  const float v = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  if (p == kBandParams) *loss = v;
+  else grad[p] = v;
 }
 
 // Adam (Kingma & Ba 2015) with bias correction.
@@ -380,24 +538,29 @@ int launch_band_features(const uint32_t* ci, const uint32_t* cj, const uint32_t*
   return MJ_OK;
 }
 
-int launch_band_forward(const float* P, const float* X, uint64_t m, const uint32_t* gate, uint32_t min_gate,
-                        float* out, cudaStream_t s) {
+int launch_band_forward(const float* P, const float* X, uint64_t m, float* out, cudaStream_t s) {
   if (!m) return MJ_OK;
-  forward_kernel<<<grid1(m, 128), 128, 0, s>>>(P, X, m, gate, min_gate, out);
+  MJ_CUDA_TRY(cudaFuncSetAttribute(forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForwardSmem));
+  const uint64_t blocks = std::min<uint64_t>((m + kSB - 1) / kSB, (uint64_t)kNumSMsHint * 3);
+  forward_kernel<<<(unsigned)blocks, kNetThreads, kForwardSmem, s>>>(P, X, m, out);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
 
-size_t band_grad_smem() { return sizeof(float) * (kBandParams + 4 * kSB * kLd + kSB * F + kSB); }
+static uint64_t grad_blocks(uint64_t batch) {
+  return std::min<uint64_t>((batch + kSB - 1) / kSB, (uint64_t)kNumSMsHint * 2);
+}
+
+size_t band_grad_part_bytes(uint64_t batch) { return sizeof(float) * grad_blocks(batch) * (kBandParams + 1); }
 
 int launch_band_grad(const float* P, const float* X, const float* Y, const uint32_t* ed, uint32_t K, uint64_t m,
-                     uint64_t batch, uint64_t seed, float tau, float* grad, float* loss, cudaStream_t s) {
+                     uint64_t batch, uint64_t seed, float tau, float* part, float* grad, float* loss, cudaStream_t s) {
   if (!batch) return MJ_OK;
-  const size_t smem = band_grad_smem();
-  MJ_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  uint64_t blocks = (batch + kSB - 1) / kSB;
-  if (blocks > (uint64_t)kNumSMsHint * 2) blocks = (uint64_t)kNumSMsHint * 2;
-  grad_kernel<<<(unsigned)blocks, kSB, smem, s>>>(P, X, Y, ed, K, m, batch, seed, tau, grad, loss);
+  MJ_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem));
+  const unsigned blocks = (unsigned)grad_blocks(batch);
+  grad_kernel<<<blocks, kNetThreads, kGradSmem, s>>>(P, X, Y, ed, K, m, batch, seed, tau, part);
+  MJ_KERNEL_DONE();
+  grad_sum_kernel<<<(kBandParams + 1 + 127) / 128, 128, 0, s>>>(part, (int)blocks, grad, loss);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

@@ -158,9 +158,7 @@ int launch_wp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long*
 
 template <int W>
 int launch_w(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
-  // digit tables read B's rank codes; without them (raw byte planes) every
-  // plane is XNORed
-  if (!a.codes) return launch_wp<W, 8>(a, PW, GW, next, s);
+  if (!a.codes) return launch_wp<W, kXnor8>(a, PW, GW, next, s);   // digit tables read B's rank codes
   if (a.bits <= 2) return launch_wp<W, 2>(a, PW, GW, next, s);
   if (a.bits <= 5) return launch_wp<W, 5>(a, PW, GW, next, s);
   if (a.bits == 7) return launch_wp<W, 7>(a, PW, GW, next, s);   // text (65-128 symbols)
@@ -248,7 +246,7 @@ int launch_verify(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, 
   int dev = 0, sms = kNumSMsHint;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (W <= 8 && a.m * 2 <= 3ull * 128 * sms) return launch_verify_split(a, PW, GW, W, next, s);
+  if (W <= 8 && a.codes && a.m * 2 <= 3ull * 128 * sms) return launch_verify_split(a, PW, GW, W, next, s);
   switch (W) {
     case 1: return launch_w<1>(a, PW, GW, next, s);
     case 2: return launch_w<2>(a, PW, GW, next, s);
@@ -264,8 +262,8 @@ int launch_verify(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, 
   if (plane_stride(a.bits) == 2)
     return W <= 16 ? launch_wp<16, 2>(a, PW, GW, next, s)
                    : (W <= 32 ? launch_wp<32, 2>(a, PW, GW, next, s) : MJ_ERR_UNSUPPORTED);
-  if (W <= 16) return launch_wp<16, 8>(a, PW, GW, next, s);
-  if (W <= 32) return launch_wp<32, 8>(a, PW, GW, next, s);
+  if (W <= 16) return launch_wp<16, kXnor8>(a, PW, GW, next, s);
+  if (W <= 32) return launch_wp<32, kXnor8>(a, PW, GW, next, s);
   return MJ_ERR_UNSUPPORTED;
 }
 

@@ -42,6 +42,12 @@
 namespace mj {
 namespace {
 
+// P, the planes a kernel is built for: 2, 5, 7 or 8 with digit tables, which
+// need the input's rank codes, or kXnor8: eight planes compared by XNOR.
+constexpr int kXnor8 = 9;
+template <int P>
+constexpr int kPlanes = P == kXnor8 ? 8 : P;
+
 // Per-lane state of one pair in flight.
 template <int W, int P>
 struct PairState {
@@ -206,13 +212,13 @@ template <> struct add_chain<8> {
 };
 
 // Columns between two early-exit checks: 32 (the most one load of B's bits
-// covers).  With the XNOR path (8 planes), bands of one or two words take 16,
-// since their pairs are often short and exit early (measured before the
-// digit tables: 32 was 5% faster at 3-4 words and 8% slower at 2).  With
-// digit tables every chunk rebuilds them, and 32 columns won at two words
-// too (protein verify 24.9 -> 22.6 ms, with 25% more word-columns advanced).
+// covers).  With the XNORs, bands of one or two words take 16, since their
+// pairs are often short and exit early (measured before the digit tables: 32
+// was 5% faster at 3-4 words and 8% slower at 2).  With digit tables every
+// chunk rebuilds them, and 32 columns won at two words too (protein verify
+// 24.9 -> 22.6 ms, with 25% more word-columns advanced).
 template <int P>
-constexpr bool kDigitTables = P == 2 || P == 5 || P == 7;
+constexpr bool kDigitTables = P != kXnor8;
 template <int W, int P>
 constexpr int kChunkFor = (W <= 2 && !kDigitTables<P>) ? 16 : 32;
 
@@ -223,25 +229,30 @@ constexpr int kChunkFor = (W <= 2 && !kDigitTables<P>) ? 16 : 32;
 // columns: with digit tables its rank codes, one byte per column; with the
 // XNORs (8 planes) its plane bits, bit-reversed so that the next column's
 // bit is the sign bit.
-// Equality bits by digit tables (2, 5 and 7 bit-planes).  Per chunk, every
+// Equality bits by digit tables.  Per chunk, every
 // thread writes to shared memory, for each of A's band words, the masks "rows
 // whose rank code has digit value d" for each digit of the code: one digit of
 // 2 bits for 2 planes (4 masks), 3 + 2 bits for 5 planes (8 + 4), 3 + 2 + 2
-// bits for 7 planes (8 + 4 + 4); a column then takes its symbol's rank code
+// bits for 7 planes (8 + 4 + 4), 3 + 3 + 2 bits for 8 planes (8 + 8 + 4); a
+// column then takes its symbol's rank code
 // from the input's code bytes and ANDs one mask of each digit's table (one load per word
 // for 2 planes, one three-input logic op per word for 7), instead of an XNOR
 // per plane and word.  Tables: word (d * (W + 1) + w) * 128 + thread, the
 // digits' tables back to back.  (For 7 planes, two digits of 4 and 3 bits,
 // 24 masks a word, take 50% more shared memory: 4 blocks per SM instead of
-// 6.)  8 planes (byte alphabets) keep the XNORs.
+// 6.)  Bytes (8 planes), 150,000 pairs of 700 random bytes: an XNOR per plane and
+// word over planes stored apart took 959 us at K = 60 and 1932 at K = 250, the
+// tables 509 and 978.  kXnor8 keeps
+// the XNORs where there are no rank codes (the allocation-free entry point)
+// and for forced bands of more than 8 words, whose tables would not fit.
 template <int P>
-constexpr int digit_masks() { return P == 2 ? 4 : (P == 5 ? 12 : 16); }
+constexpr int digit_masks() { return P == 2 ? 4 : (P == 5 ? 12 : (P == 7 ? 16 : 20)); }
 template <int W, int P>
 constexpr size_t digit_smem_bytes() { return (size_t)digit_masks<P>() * (W + 1) * 128 * 4; }
 
 // The masks of band word w (A's pre-shifted plane words pa) into the tables.
 template <int W, int P>
-__device__ __forceinline__ void build_digit_tables(const uint32_t (&pa)[P][W + 1], int w, uint32_t* __restrict__ tab,
+__device__ __forceinline__ void build_digit_tables(const uint32_t (&pa)[kPlanes<P>][W + 1], int w, uint32_t* __restrict__ tab,
                                                    int tid) {
   auto put = [&](int d, uint32_t v) { tab[(d * (W + 1) + w) * 128 + tid] = v; };
   auto two = [&](int p, int base) {   // a 2-bit digit from planes p, p + 1
@@ -254,13 +265,20 @@ __device__ __forceinline__ void build_digit_tables(const uint32_t (&pa)[P][W + 1
   if constexpr (P == 2) {
     two(0, 0);
   } else {
-    // a 3-bit digit from planes 0-2
-    const uint32_t a0 = pa[0][w], a1 = pa[1][w], a2 = pa[2][w];
-    const uint32_t t2[4] = {~a0 & ~a1, a0 & ~a1, ~a0 & a1, a0 & a1};
+    auto three = [&](int p, int base) {   // a 3-bit digit from planes p .. p + 2
+      const uint32_t a0 = pa[p][w], a1 = pa[p + 1][w], a2 = pa[p + 2][w];
+      const uint32_t t2[4] = {~a0 & ~a1, a0 & ~a1, ~a0 & a1, a0 & a1};
 #pragma unroll
-    for (int d = 0; d < 8; ++d) put(d, t2[d & 3] & ((d & 4) ? a2 : ~a2));
-    two(3, 8);
-    if constexpr (P == 7) two(5, 12);
+      for (int d = 0; d < 8; ++d) put(base + d, t2[d & 3] & ((d & 4) ? a2 : ~a2));
+    };
+    three(0, 0);
+    if constexpr (P == 8) {
+      three(3, 8);
+      two(6, 16);
+    } else {
+      two(3, 8);
+      if constexpr (P == 7) two(5, 12);
+    }
   }
 }
 
@@ -280,8 +298,8 @@ __device__ __forceinline__ void digit_lookup(const uint32_t* __restrict__ tab, u
     for (int w = 0; w <= W; ++w) EqF[w] = ta[w * 128] & tb[w * 128];
   } else {
     const uint32_t* ta = tab + (code & 7u) * S + tid;
-    const uint32_t* tb = tab + (8u + ((code >> 3) & 3u)) * S + tid;
-    const uint32_t* tc = tab + (12u + (code >> 5)) * S + tid;
+    const uint32_t* tb = tab + (8u + ((code >> 3) & (P == 7 ? 3u : 7u))) * S + tid;
+    const uint32_t* tc = tab + (P == 7 ? 12u + (code >> 5) : 16u + (code >> 6)) * S + tid;
 #pragma unroll
     for (int w = 0; w <= W; ++w) EqF[w] = ta[w * 128] & tb[w * 128] & tc[w * 128];
   }
@@ -295,8 +313,9 @@ __device__ __forceinline__ bool pair_chunk(PairState<W, P>& st, const VerifyArgs
                                            uint32_t* __restrict__ tab, uint32_t GW, bool rev = false) {
   constexpr bool kDigits = kDigitTables<P>;
   const int32_t j0 = st.j;
-  uint32_t pa[P][W + 1];
-  uint32_t bw[P];
+  constexpr int NP = kPlanes<P>;
+  uint32_t pa[NP][W + 1];
+  uint32_t bw[NP];
   uint32_t bsym[kDigits ? 8 : 1];   // B's rank codes of the chunk's columns, four per word
   {
     const uint64_t ab = SPLIT && rev ? st.abit - (uint64_t)(j0 - 1) : st.abit + (uint64_t)(j0 - 1);
@@ -305,24 +324,24 @@ __device__ __forceinline__ bool pair_chunk(PairState<W, P>& st, const VerifyArgs
     const uint32_t ash = (uint32_t)(ab & 31);
     const uint64_t wb = st.bpos >> 5;
     const uint32_t sb = (uint32_t)(st.bpos & 31);
-    uint32_t x0[P];
-    load_plane_words<P>(a.planes, (int64_t)aw, x0);
+    uint32_t x0[NP];
+    load_plane_words<NP>(a.planes, (int64_t)aw, x0);
 #pragma unroll
     for (int w = 0; w <= W; ++w) {
-      uint32_t x1[P];
-      load_plane_words<P>(a.planes, (int64_t)aw + step * (w + 1), x1);
+      uint32_t x1[NP];
+      load_plane_words<NP>(a.planes, (int64_t)aw + step * (w + 1), x1);
 #pragma unroll
-      for (int p = 0; p < P; ++p) {
+      for (int p = 0; p < NP; ++p) {
         pa[p][w] = SPLIT && rev ? __brev(__funnelshift_r(x1[p], x0[p], ash)) : __funnelshift_r(x0[p], x1[p], ash);
         x0[p] = x1[p];
       }
     }
     if (!kDigits) {
-      uint32_t y0[P], y1[P];
-      load_plane_words<P>(a.planes, (int64_t)wb, y0);
-      load_plane_words<P>(a.planes, (int64_t)wb + 1, y1);
+      uint32_t y0[NP], y1[NP];
+      load_plane_words<NP>(a.planes, (int64_t)wb, y0);
+      load_plane_words<NP>(a.planes, (int64_t)wb + 1, y1);
 #pragma unroll
-      for (int p = 0; p < P; ++p) {
+      for (int p = 0; p < NP; ++p) {
         bw[p] = __funnelshift_r(y0[p], y1[p], sb);
         if (!(SPLIT && rev)) bw[p] = __brev(bw[p]);
       }
@@ -403,7 +422,7 @@ __device__ __forceinline__ bool pair_chunk(PairState<W, P>& st, const VerifyArgs
 #pragma unroll
       for (int w = 0; w <= W; ++w) EqF[w] = 0xffffffffu;
 #pragma unroll
-      for (int p = 0; p < P; ++p) {
+      for (int p = 0; p < NP; ++p) {
         if (p < (int)a.bits) {
           const uint32_t xb = (uint32_t)__mulhi((int32_t)bw[p], 1);   // B's bit broadcast (sign)
           bw[p] *= 2u;

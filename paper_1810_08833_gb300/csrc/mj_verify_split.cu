@@ -125,12 +125,9 @@ __global__ void __launch_bounds__(128) verify_split_kernel(VerifyArgs a, uint64_
 
 template <int W, int P>
 int launch_split_wp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
-  const size_t smem = kDigitTables<P> ? digit_smem_bytes<W, P>() : 0;
-  if (kDigitTables<P>) {
-    if (!a.codes) return MJ_ERR_ARG;
-    MJ_CUDA_TRY(cudaFuncSetAttribute(verify_split_kernel<W, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-  }
+  if (!a.codes) return MJ_ERR_ARG;
+  constexpr size_t smem = digit_smem_bytes<W, P>();
+  MJ_CUDA_TRY(cudaFuncSetAttribute(verify_split_kernel<W, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   verify_split_kernel<W, P><<<(unsigned)((a.m * 2 + 127) / 128), 128, smem, s>>>(a, PW, GW, next);
   MJ_KERNEL_DONE();
   return MJ_OK;
@@ -138,7 +135,6 @@ int launch_split_wp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long
 
 template <int W>
 int launch_split_w(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
-  if (!a.codes) return launch_split_wp<W, 8>(a, PW, GW, next, s);
   if (a.bits <= 2) return launch_split_wp<W, 2>(a, PW, GW, next, s);
   if (a.bits <= 5) return launch_split_wp<W, 5>(a, PW, GW, next, s);
   if (a.bits == 7) return launch_split_wp<W, 7>(a, PW, GW, next, s);

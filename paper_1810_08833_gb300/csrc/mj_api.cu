@@ -939,6 +939,12 @@ bool bounds_pay(const mj_ctx* c, uint64_t m, uint32_t kmax, uint64_t bytes_per_p
   return true;
 }
 
+// The autotuner's first wavefront candidate, the fewest lanes that hold the
+// band, is the shape a launch without a number of lanes takes.
+int plan_lanes(uint32_t kernel, uint32_t lanes, uint32_t K) {
+  return kernel == MJ_VERIFY_KERNEL_WAVEFRONT && (int)lanes == fewest_lanes_for(K) ? 0 : (int)lanes;
+}
+
 int bounds_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
   MJ_TRY(c->rk_sig1.reserve(sig1_bytes((uint32_t)c->stats.n_strings), s));
   MJ_TRY(c->rk_sig2.reserve(sig2_bytes((uint32_t)c->stats.n_strings), s));
@@ -1007,7 +1013,8 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
   if (c->vcfg.batching == 1) {
     for (int b = kLenBuckets - 1; b >= 0; --b)
       MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, ranges + 2 * b,
-                    ranges + 2 * b + 1, (int)c->tuned_kernel[b], (int)c->tuned_lanes[b]));
+                    ranges + 2 * b + 1, (int)c->tuned_kernel[b],
+                    plan_lanes(c->tuned_kernel[b], c->tuned_lanes[b], K)));
     return MJ_OK;
   }
   // one launch per run of consecutive buckets (longest first) sharing a kernel
@@ -1016,7 +1023,7 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
     int e = b;
     while (e - 1 >= 0 && c->tuned_kernel[e - 1] == c->tuned_kernel[b] && c->tuned_lanes[e - 1] == c->tuned_lanes[b]) --e;
     MJ_TRY(verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s, order, nullptr, ranges + 2 * b,
-                  ranges + 2 * e + 1, (int)c->tuned_kernel[b], (int)c->tuned_lanes[b]));
+                  ranges + 2 * e + 1, (int)c->tuned_kernel[b], plan_lanes(c->tuned_kernel[b], c->tuned_lanes[b], K)));
     b = e - 1;
   }
   return MJ_OK;
@@ -1674,7 +1681,7 @@ int mj_autotune_verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offse
       for (int rep_i = 0; rep_i < 2; ++rep_i) {   // the first run warms the caches
         MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
         MJ_TRY(verify(c, d_bytes, d_offsets, d_i, d_j, nullptr, m, K, K, c->ed.as<uint32_t>(), s, order,
-                      nullptr, trial, trial + 1, (int)ck[k], (int)cl[k]));
+                      nullptr, trial, trial + 1, (int)ck[k], plan_lanes(ck[k], cl[k], K)));
         MJ_CUDA_TRY(cudaEventRecord(c->ev[1], s));
       }
       MJ_CUDA_TRY(cudaEventSynchronize(c->ev[1]));

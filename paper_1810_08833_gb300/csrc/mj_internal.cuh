@@ -374,6 +374,10 @@ int launch_verify_split(const VerifyArgs& a, uint64_t plane_words, uint32_t guar
                         unsigned long long* next, cudaStream_t s);
 int launch_verify_wave(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, int lanes,
                        unsigned long long* next, cudaStream_t s);
+// the wavefront in the shape (lanes, words per lane) that suits the band and
+// the number of pairs
+int launch_verify_wave_auto(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, uint32_t kmax,
+                            unsigned long long* next, cudaStream_t s);
 int wave_lanes_for(uint32_t kmax);
 // whether launch_verify takes bands up to kmax with this kernel choice
 bool verify_supported(uint32_t kmax, int kernel, int lanes);

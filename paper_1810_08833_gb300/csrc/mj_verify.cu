@@ -225,20 +225,13 @@ int launch_verify(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, 
   if (a.m == 0) return MJ_OK;
   const int W = verify_words_for(kmax);
   if (kernel == MJ_VERIFY_KERNEL_AUTO) kernel = W <= 8 ? MJ_VERIFY_KERNEL_DIAGONAL : MJ_VERIFY_KERNEL_WAVEFRONT;
-  if (kernel == MJ_VERIFY_KERNEL_WAVEFRONT && (lanes > 32 || (lanes <= 0 && wave_lanes_for(kmax) > 32))) {
-    // one CTA of several warps per pair
-    const int G = lanes > 0 ? lanes : cta_lanes_for(kmax);
-    if (G < cta_lanes_for(kmax) || G > kMaxCtaLanes || (G & (G - 1))) return MJ_ERR_UNSUPPORTED;
+  if (kernel == MJ_VERIFY_KERNEL_WAVEFRONT) {
+    if (!verify_supported(kmax, kernel, lanes)) return MJ_ERR_UNSUPPORTED;
     if (!next_is_zero) MJ_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(unsigned long long), s));
-    return launch_verify_wave(a, PW, GW, G, next, s);
+    return lanes > 0 ? launch_verify_wave(a, PW, GW, lanes, next, s)   // one word per lane
+                     : launch_verify_wave_auto(a, PW, GW, kmax, next, s);
   }
   if (!next_is_zero) MJ_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(unsigned long long), s));
-  if (kernel == MJ_VERIFY_KERNEL_WAVEFRONT) {
-    const int need = wave_lanes_for(kmax);
-    int G = lanes > 0 ? lanes : need;
-    if (G < need || G > 32 || (G & (G - 1))) return MJ_ERR_UNSUPPORTED;
-    return launch_verify_wave(a, PW, GW, G, next, s);
-  }
   if (kernel != MJ_VERIFY_KERNEL_DIAGONAL) return MJ_ERR_ARG;
   // every pair in flight at once with two lanes each, at three blocks of 128
   // threads per SM: then the longest pair is the kernel's time, and its halves

@@ -1,6 +1,9 @@
 // Step a8 for wide bands: row-fixed blocks with a skewed wavefront, within one
 // warp (G lanes per pair) or one CTA of several warps per pair.
-#include "mj_verify_common.cuh"
+#include <algorithm>
+#include <cmath>
+
+#include "mj_verify_diag.cuh"
 
 namespace mj {
 namespace {
@@ -8,8 +11,8 @@ namespace {
 // ---------------------------------------------------------------- wide bands
 // Row-fixed blocks with a skewed wavefront, G lanes per pair.
 //
-// Rows are cut into 32-row blocks (block b = rows 32b+1 .. 32b+32, one 32-bit
-// word per vector); lane b mod G of the pair's group owns block b.  Block b
+// Rows are cut into blocks of R = 32 V rows (block b = rows Rb+1 .. Rb+R, V
+// 32-bit words per vector; below V = 1 unless said); lane b mod G of the pair's group owns block b.  Block b
 // advances column j at step s = j + b: it needs the horizontal delta of the
 // row just above it in column j, which the lane owning block b-1 produced one
 // step earlier and passes on by a shuffle.  A block works on the columns in
@@ -62,39 +65,85 @@ __device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c) {
   return d;
 }
 
+// A block of V words (rows 32 V b + 1 ..) takes the same step, the carry of
+// (Eq & Pv) + Pv and the shifted-in bits running through its words.
 // pub: the word published to the next lane, ((Ph & 2^31) | T) + hn with the
 // updated T (bit 31 and bit 0 of T are clear), formed by multiply-adds as
-// T_old + hp (2^31 + 2) - hn.
-template <int P>
-__device__ __forceinline__ void wave_column(const uint32_t (&pa)[P], uint32_t (&bw)[P], uint32_t wv, uint32_t& Pv,
-                                            uint32_t& Mv, uint32_t& T, uint32_t& Ph, uint32_t& hn, uint32_t& pub) {
-  uint32_t Eq = 0xffffffffu;
+// T_old + hp (2^31 + 2) - hn.  Ph and hn: of the bottom word.
+template <int P, int V>
+__device__ __forceinline__ void wave_column(const uint32_t (&pa)[P][V], uint32_t (&bw)[P], uint32_t wv,
+                                            uint32_t (&Pv)[V], uint32_t (&Mv)[V], uint32_t& T, uint32_t& Ph_out,
+                                            uint32_t& hn, uint32_t& pub) {
+  uint32_t Eq[V], EP[V], SUM[V], Ph[V], Mh[V];
+#pragma unroll
+  for (int w = 0; w < V; ++w) Eq[w] = 0xffffffffu;
 #pragma unroll
   for (int p = 0; p < P; ++p) {
     const uint32_t xb = (uint32_t)__mulhi((int32_t)bw[p], 1);   // B's bit p broadcast (sign of bw)
-    Eq &= ~(pa[p] ^ xb);
+#pragma unroll
+    for (int w = 0; w < V; ++w) Eq[w] &= ~(pa[p][w] ^ xb);
     bw[p] *= 2u;
   }
   const uint32_t hin_neg = wv & 1u;
   const uint32_t hin_pos = __umulhi(wv, 2u);
-  const uint32_t Xv = Eq | Mv;
-  const uint32_t Eh = Eq | hin_neg;
-  const uint32_t Xh = (((Eh & Pv) + Pv) ^ Pv) | Eh;
-  Ph = Mv | ~(Xh | Pv);
-  const uint32_t Mh = Pv & Xh;
-  hn = __umulhi(Mh, 2u);
-  const uint32_t hp = __umulhi(Ph, 2u);
+#pragma unroll
+  for (int w = 0; w < V; ++w) EP[w] = (w == 0 ? Eq[w] | hin_neg : Eq[w]) & Pv[w];
+  add_chain<V>::run(EP, Pv, SUM);
+#pragma unroll
+  for (int w = 0; w < V; ++w) {
+    const uint32_t Xh = (SUM[w] ^ Pv[w]) | (w == 0 ? Eq[w] | hin_neg : Eq[w]);
+    Ph[w] = Mv[w] | ~(Xh | Pv[w]);
+    Mh[w] = Pv[w] & Xh;
+  }
+  hn = __umulhi(Mh[V - 1], 2u);
+  const uint32_t hp = __umulhi(Ph[V - 1], 2u);
   pub = mad_lo(hn, 0xffffffffu, mad_lo(hp, 0x80000002u, T));
   T = mad_lo(hn, 0xfffffffeu, mad_lo(hp, 2u, T));
-  const uint32_t Ph1 = Ph * 2u + hin_pos;   // (Ph << 1) | hin > 0
-  const uint32_t Mh1 = Mh * 2u + hin_neg;   // (Mh << 1) | hin < 0
-  Pv = Mh1 | ~(Xv | Ph1);
-  Mv = Ph1 & Xv;
+#pragma unroll
+  for (int w = V - 1; w >= 0; --w) {
+    const uint32_t Xv = Eq[w] | Mv[w];
+    const uint32_t Ph1 = w ? __funnelshift_l(Ph[w - 1], Ph[w], 1) : Ph[w] * 2u + hin_pos;   // (Ph << 1) | hin > 0
+    const uint32_t Mh1 = w ? __funnelshift_l(Mh[w - 1], Mh[w], 1) : Mh[w] * 2u + hin_neg;   // (Mh << 1) | hin < 0
+    Pv[w] = Mh1 | ~(Xv | Ph1);
+    Mv[w] = Ph1 & Xv;
+  }
+  Ph_out = Ph[V - 1];
 }
 
-template <int G, int P>
-__global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
+// Sum of the vertical deltas of a block's rows below row r (0 .. 32 V - 1).
+template <int V>
+__device__ __forceinline__ int32_t deltas_below(const uint32_t (&Pv)[V], const uint32_t (&Mv)[V], int r) {
+  int32_t d = 0;
+#pragma unroll
+  for (int w = 0; w < V; ++w) {
+    const int x = r - 32 * w;
+    const uint32_t below = x < 0 ? 0xffffffffu : (x >= 31 ? 0u : (0xffffffffu << (x + 1)));
+    d += (int32_t)__popc(Pv[w] & below) - (int32_t)__popc(Mv[w] & below);
+  }
+  return d;
+}
+
+// The planes of the 32 V rows from plane bit pos on.
+template <int P, int V>
+__device__ __forceinline__ void wave_load_rows(const VerifyArgs& a, uint64_t pos, uint32_t (&pa)[P][V]) {
+  uint32_t x0[P];
+  load_plane_words<P>(a.planes, (int64_t)(pos >> 5), x0);
+#pragma unroll
+  for (int w = 0; w < V; ++w) {
+    uint32_t x1[P];
+    load_plane_words<P>(a.planes, (int64_t)(pos >> 5) + w + 1, x1);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      pa[p][w] = __funnelshift_r(x0[p], x1[p], (uint32_t)(pos & 31));
+      x0[p] = x1[p];
+    }
+  }
+}
+
+template <int G, int P, int V>
+__global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
                                                           unsigned long long* __restrict__ next) {
+  constexpr int R = 32 * V;   // rows of a block
   const int lane = threadIdx.x & 31;
   const int gl = lane & (G - 1);
   const int gbase = lane - gl;
@@ -112,29 +161,35 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
   // block state (this lane): block b runs at the steps where 0 <= u <= span
   // (u counts up by one per step); block b - 1 computed the same column one
   // step earlier while u <= u_valid; diagonal d0 crosses it where
-  // 0 <= u + dg < 32
+  // 0 <= u + dg < R
   int32_t b = 0, u = kDeadU, span = 0, u_valid = -1, dg = 0x40000000;
   uint32_t T = 0;   // score << 1
-  uint32_t Pv = 0, Mv = 0;
-  uint32_t pa[P], bw[P];
+  uint32_t Pv[V], Mv[V];
+  uint32_t pa[P][V], bw[P];
   uint32_t pub = kIdle;
   bool done = false, reject = false;
   int32_t result = 0;
   uint64_t work = 0, nskip = 0;
 #pragma unroll
-  for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
+  for (int w = 0; w < V; ++w) {
+    Pv[w] = Mv[w] = 0u;
+#pragma unroll
+    for (int p = 0; p < P; ++p) pa[p][w] = 0u;
+  }
+#pragma unroll
+  for (int p = 0; p < P; ++p) bw[p] = 0u;
 
   // Take block nb after step s.  Its columns are [jf, jl]; block nb computes
   // column j at step j + nb.  Blocks past row m never run.
   auto take_block = [&](int32_t nb, int32_t s) {
     b = nb;
     if (b <= bm) {
-      const int32_t jf = max(1, 32 * b + 1 - dhi);
-      const int32_t jl = min(n, 32 * b + 32 - dlo);
+      const int32_t jf = max(1, R * b + 1 - dhi);
+      const int32_t jl = min(n, R * b + R - dlo);
       u = s - (jf + b);
       span = jl - jf;
-      u_valid = b == 0 ? -1 : min(n, 32 * b - dlo) - jf;   // last column of block b - 1
-      dg = jf - 32 * b - 1 + d0;   // row j + d0 is row 32 b + 1 + (u + dg)
+      u_valid = b == 0 ? -1 : min(n, R * b - dlo) - jf;   // last column of block b - 1
+      dg = jf - R * b - 1 + d0;   // row j + d0 is row R b + 1 + (u + dg)
     } else {
       u = kDeadU;
       span = 0;
@@ -187,7 +242,7 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
               dlo = -(int32_t)((k - (uint32_t)d0) >> 1);
               dhi = d0 + (int32_t)((k - (uint32_t)d0) >> 1);
               if (dhi - dlo < 63) dlo = dhi - 63;   // at least 64 band rows (any wider band is exact)
-              bm = (m - 1) >> 5;
+              bm = (m - 1) / R;
               sbase = 0;
               take_block(gl, 0);
               pub = kIdle;
@@ -226,12 +281,12 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
         const int free = __reduce_min_sync(0xffffffffu, (int)fr);
         const bool from_prev = un <= u_valid;
         const uint32_t keep_in = from_prev ? 1u : 0u, idle_in = from_prev ? 0u : kIdle;
-#pragma unroll 4
+#pragma unroll(V == 1 ? 4 : 2)
         for (int f = 0; f < free; ++f) {
           const uint32_t w_in = __shfl_sync(0xffffffffu, pub, prev_lane);
           const uint32_t wv = mad_lo(w_in, keep_in, idle_in);   // w_in, or kIdle at the band's edge
           uint32_t Ph, hn;
-          wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+          wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
         }
         u += free;
         it += free;
@@ -240,37 +295,36 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
       ++u;
       const uint32_t wv = u <= u_valid ? w_in : kIdle;
       uint32_t Ph, hn;
-      wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
-      const bool diag_here = it == kWaveSteps - 1 && (uint32_t)(u + dg) < 32u;
+      wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+      const bool diag_here = it == kWaveSteps - 1 && (uint32_t)(u + dg) < (uint32_t)R;
       if (u == 0 || u == span || diag_here) {
         if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
           const int32_t jf = sbase + it + 1 - b;
-          wave_load_bits<P>(a, PW, (uint64_t)(oA + 32 * (int64_t)b + 32 * (int64_t)GW), pa, false);
+          wave_load_rows<P, V>(a, (uint64_t)(oA + R * (int64_t)b + 32 * (int64_t)GW), pa);
           wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
-          Pv = 0xffffffffu;
-          Mv = 0u;
-          wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+#pragma unroll
+          for (int w = 0; w < V; ++w) {
+            Pv[w] = 0xffffffffu;
+            Mv[w] = 0u;
+          }
+          wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
           // D of the row above the block in this column, plus the block's deltas
           const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
-          const int32_t score = above + (int32_t)__popc(Pv) - (int32_t)__popc(Mv);
+          const int32_t score = above + deltas_below<V>(Pv, Mv, -1);
           T = (uint32_t)score << 1;
           pub = ((Ph & 0x80000000u) | T) + hn;
         }
         // D at row r of this block = score minus the deltas of the rows below r
         if (diag_here && (uint32_t)u <= (uint32_t)span) {   // row j + d0 of diagonal d0
-          const int tr = u + dg;
-          const uint32_t below = tr == 31 ? 0u : (0xffffffffu << (tr + 1));
-          const int32_t diag = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+          const int32_t diag = (int32_t)(T >> 1) - deltas_below<V>(Pv, Mv, u + dg);
           if (diag > (int32_t)k) reject = true;
         }
         if (u == span) {   // the block leaves the band
           if (b == bm) {
-            const int tm = (m - 1) & 31;
-            const uint32_t below = tm == 31 ? 0u : (0xffffffffu << (tm + 1));
-            result = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+            result = (int32_t)(T >> 1) - deltas_below<V>(Pv, Mv, (m - 1) % R);
             done = true;
           }
-          work += (uint64_t)(span + 1);
+          work += (uint64_t)(span + 1) * V;
           take_block(b + G, sbase + it + 1);
         }
       }
@@ -300,7 +354,7 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
         end = true;
       }
       if (end) {
-        if (u >= 0 && u <= span) work += (uint64_t)(u + 1);   // block cut short by the exit
+        if (u >= 0 && u <= span) work += (uint64_t)(u + 1) * V;   // block cut short by the exit
         has = false;
         u = kDeadU;
         span = 0;
@@ -323,9 +377,10 @@ __global__ void __launch_bounds__(128, P <= 2 ? 8 : 1) verify_wave_kernel(Verify
 
 // ---------------------------------------------------------------- bands wider than one warp
 // One CTA of V warps (G = 32 V lanes) per pair, for bands whose wavefront
-// needs more than 32 lanes (K >= 1025).  Blocks, lanes and the column step
-// are those of verify_wave_kernel (lane g owns blocks b = g mod G), with one
-// change to the schedule: block b computes column j at step
+// no shape of one warp holds (K > 7968), or with 64 lanes or more asked for.
+// Blocks, lanes and the column step are those of verify_wave_kernel with one
+// word per lane (lane g owns blocks b = g mod G), with one change to the
+// schedule: block b computes column j at step
 //     j + b + 32 floor(b / 32),
 // i.e. every group of 32 blocks runs one window of kWaveSteps (= 32) steps
 // behind the group above it.  Inside a group the predecessor block b - 1 is
@@ -362,15 +417,15 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
   int64_t oA = 0, oB = 0;
   int32_t m = 0, n = 0, d0 = 0, dlo = 0, dhi = 0, bm = 0;
   int32_t b = 0, u = kDeadU, span = 0, u_valid = -1, dg = 0x40000000, colbase = 0;
-  uint32_t T = 0, Pv = 0, Mv = 0;
-  uint32_t pa[P], bw[P];
+  uint32_t T = 0, Pv[1] = {0u}, Mv[1] = {0u};
+  uint32_t pa[P][1], bw[P];
   uint32_t pub = kIdle;
   bool done = false, reject = false;
   int32_t result = 0;
   uint32_t win = 0;   // windows run by the CTA (selects the flag slot)
   uint64_t work = 0, nskip = 0;
 #pragma unroll
-  for (int p = 0; p < P; ++p) pa[p] = bw[p] = 0u;
+  for (int p = 0; p < P; ++p) pa[p][0] = bw[p] = 0u;
 
   // Take block nb after s steps.  Its columns are [jf, jl]; it computes
   // column j at step j + colbase (colbase = nb + 32 floor(nb / 32)).
@@ -465,32 +520,28 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
         ++u;
         const uint32_t wv = u <= u_valid ? w_in : kIdle;
         uint32_t Ph, hn;
-        wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+        wave_column<P, 1>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
         const bool diag_here = it == S - 1 && (uint32_t)(u + dg) < 32u;
         if (u == 0 || u == span || diag_here) {
           if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
             const int32_t jf = s1 - colbase;
-            wave_load_bits<P>(a, PW, (uint64_t)(oA + 32 * (int64_t)b + 32 * (int64_t)GW), pa, false);
+            wave_load_rows<P, 1>(a, (uint64_t)(oA + 32 * (int64_t)b + 32 * (int64_t)GW), pa);
             wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
-            Pv = 0xffffffffu;
-            Mv = 0u;
-            wave_column<P>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+            Pv[0] = 0xffffffffu;
+            Mv[0] = 0u;
+            wave_column<P, 1>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
             const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
-            const int32_t score = above + (int32_t)__popc(Pv) - (int32_t)__popc(Mv);
+            const int32_t score = above + deltas_below<1>(Pv, Mv, -1);
             T = (uint32_t)score << 1;
             pub = ((Ph & 0x80000000u) | T) + hn;
           }
           if (diag_here && (uint32_t)u <= (uint32_t)span) {   // row j + d0 of diagonal d0
-            const int tr = u + dg;
-            const uint32_t below = tr == 31 ? 0u : (0xffffffffu << (tr + 1));
-            const int32_t diag = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+            const int32_t diag = (int32_t)(T >> 1) - deltas_below<1>(Pv, Mv, u + dg);
             if (diag > (int32_t)k) reject = true;
           }
           if (u == span) {   // the block leaves the band
             if (b == bm) {
-              const int tm = (m - 1) & 31;
-              const uint32_t below = tm == 31 ? 0u : (0xffffffffu << (tm + 1));
-              result = (int32_t)(T >> 1) - (int32_t)__popc(Pv & below) + (int32_t)__popc(Mv & below);
+              result = (int32_t)(T >> 1) - deltas_below<1>(Pv, Mv, (m - 1) & 31);
               done = true;
             }
             work += (uint64_t)(span + 1);
@@ -537,27 +588,60 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
   if (tid == 0 && a.skipped && nskip) atomicAdd(a.skipped, (unsigned long long)nskip);
 }
 
-template <int G, int P>
-int launch_gp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+// Warps per scheduler that a list is worth, from the warps it fills in all.
+// More warps hide more latency, but a pair taken early then runs more slowly
+// and cannot move, so the kernel ends with the slowest share: with throughput
+// T (1 + a / c) and c L for the longest pairs, c = sqrt(a T / L).  Measured with
+// 1 / 2 / 3 / all resident blocks of four warps per SM (pairs of 2,000-20,000
+// symbols): K = 3900, 3,000 pairs 3.18 / 2.66 / 3.36 / 4.37 ms, 20,000 pairs
+// 19.8 / 15.7 / 15.0 / 15.0; K = 700 (8 lanes), 8,000 pairs 1.65 / 2.42 / 3.42 /
+// 3.35, 100,000 pairs 14.0 / 10.5 / 9.9 / 10.3.
+inline int wave_blocks_per_sm(uint64_t pairs, int G, int sms) {
+  const double x = (double)pairs * G / 32 / (4.0 * sms);
+  return std::max(1, (int)std::lround(std::sqrt(x / 2)));
+}
+
+template <int G, int P, int V>
+int launch_gpv(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
   int dev = 0, sms = kNumSMsHint, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_wave_kernel<G, P>, 128, 0);
-  if (per_sm < 1) per_sm = 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_wave_kernel<G, P, V>, 128, 0);
+  per_sm = std::max(1, std::min(per_sm, wave_blocks_per_sm(a.m, G, sms)));
   uint64_t need = (a.m * G + 127) / 128;
   uint64_t grid = (uint64_t)sms * per_sm;
   if (need < grid) grid = need;
-  verify_wave_kernel<G, P><<<(unsigned)(grid ? grid : 1), 128, 0, s>>>(a, PW, GW, next);
+  verify_wave_kernel<G, P, V><<<(unsigned)(grid ? grid : 1), 128, 0, s>>>(a, PW, GW, next);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }
 
 template <int G>
 int launch_g(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
-  if (a.bits <= 2) return launch_gp<G, 2>(a, PW, GW, next, s);
-  if (a.bits <= 5) return launch_gp<G, 5>(a, PW, GW, next, s);
-  return launch_gp<G, 8>(a, PW, GW, next, s);
+  if (a.bits <= 2) return launch_gpv<G, 2, 1>(a, PW, GW, next, s);
+  if (a.bits <= 5) return launch_gpv<G, 5, 1>(a, PW, GW, next, s);
+  return launch_gpv<G, 8, 1>(a, PW, GW, next, s);
 }
+
+template <int G, int V>
+int launch_gv(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
+  return a.bits <= 2 ? launch_gpv<G, 2, V>(a, PW, GW, next, s) : launch_gpv<G, 8, V>(a, PW, GW, next, s);
+}
+
+// Shapes: G lanes of V words.  A block of R = 32 V rows is active for
+// width + R - 1 columns and its successor starts R + 1 steps later, so
+// floor((width + R - 2) / (R + 1)) + 1 <= G blocks must fit.
+struct WaveShape {
+  int G, V;
+  int (*launch)(const VerifyArgs&, uint64_t, uint32_t, unsigned long long*, cudaStream_t);
+};
+const WaveShape kWaveShapes[] = {
+    {2, 1, launch_g<2>}, {4, 1, launch_g<4>}, {8, 1, launch_g<8>}, {16, 1, launch_g<16>},
+    {32, 1, launch_g<32>}, {4, 4, launch_gv<4, 4>}, {4, 6, launch_gv<4, 6>}, {8, 2, launch_gv<8, 2>},
+    {8, 3, launch_gv<8, 3>}, {8, 4, launch_gv<8, 4>}, {8, 5, launch_gv<8, 5>}, {16, 2, launch_gv<16, 2>},
+    {16, 3, launch_gv<16, 3>}, {16, 5, launch_gv<16, 5>}, {32, 2, launch_gv<32, 2>}, {32, 3, launch_gv<32, 3>},
+    {32, 4, launch_gv<32, 4>}, {32, 6, launch_gv<32, 6>}, {32, 8, launch_gv<32, 8>},
+};
 
 template <int V, int P>
 int launch_vp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
@@ -585,6 +669,38 @@ int launch_v(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* 
 }
 
 }  // namespace
+
+// The shape with the least estimated time.  Per step, a warp takes about
+// 24 + 20 V issue cycles, a step alone 100 + 12 V cycles (K = 950, 50,000
+// pairs: 32 lanes of 1 / 2 / 4 / 8 words 10.8 / 13.9 / 22.3 / 39.9 ms; 100 pairs:
+// 1.20 ms with one word, 1.42 with four, 2.08 with eight); pairs reject early,
+// so the average one takes about 0.3 of the longest one's steps.  Work W
+// per scheduler and a longest pair L then overlap to (sqrt W + sqrt L)^2 (see
+// wave_blocks_per_sm).  Against one word per lane (for K >= 1025: a CTA per
+// pair) and all resident blocks: K = 1000, the band of 2,000 x 10 long noisy
+// reads' join: 46.8 -> 31.2 ms; K = 4000, 3,000 pairs: 5.6 -> 2.7 ms; K = 1900
+// and 12,000 pairs: 8.4 -> 5.4 ms.
+int launch_verify_wave_auto(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, unsigned long long* next,
+                            cudaStream_t s) {
+  int dev = 0, sms = kNumSMsHint;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int width = std::max<int>((int)kmax + 1, 64);
+  const WaveShape* best = nullptr;
+  double least = 0;
+  for (const WaveShape& w : kWaveShapes) {
+    const int R = 32 * w.V;
+    // the last block reads up to V words beyond the string: the guard holds them
+    if ((width + R - 2) / (R + 1) + 1 > w.G || (int)GW <= w.V) continue;
+    const double work = 0.3 * (24 + 20 * w.V) * ((double)a.m * w.G / 32 / (4.0 * sms)), longest = 100 + 12 * w.V;
+    const double t = std::sqrt(work) + std::sqrt(longest);
+    if (!best || t < least) {
+      best = &w;
+      least = t;
+    }
+  }
+  return best ? best->launch(a, PW, GW, next, s) : launch_verify_wave(a, PW, GW, cta_lanes_for(kmax), next, s);
+}
 
 int launch_verify_wave(const VerifyArgs& a, uint64_t PW, uint32_t GW, int lanes, unsigned long long* next,
                        cudaStream_t s) {

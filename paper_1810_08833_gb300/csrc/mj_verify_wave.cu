@@ -70,20 +70,10 @@ __device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c) {
 // pub: the word published to the next lane, ((Ph & 2^31) | T) + hn with the
 // updated T (bit 31 and bit 0 of T are clear), formed by multiply-adds as
 // T_old + hp (2^31 + 2) - hn.  Ph and hn: of the bottom word.
-template <int P, int V>
-__device__ __forceinline__ void wave_column(const uint32_t (&pa)[P][V], uint32_t (&bw)[P], uint32_t wv,
-                                            uint32_t (&Pv)[V], uint32_t (&Mv)[V], uint32_t& T, uint32_t& Ph_out,
-                                            uint32_t& hn, uint32_t& pub) {
-  uint32_t Eq[V], EP[V], SUM[V], Ph[V], Mh[V];
-#pragma unroll
-  for (int w = 0; w < V; ++w) Eq[w] = 0xffffffffu;
-#pragma unroll
-  for (int p = 0; p < P; ++p) {
-    const uint32_t xb = (uint32_t)__mulhi((int32_t)bw[p], 1);   // B's bit p broadcast (sign of bw)
-#pragma unroll
-    for (int w = 0; w < V; ++w) Eq[w] &= ~(pa[p][w] ^ xb);
-    bw[p] *= 2u;
-  }
+template <int V>
+__device__ __forceinline__ void wave_column(const uint32_t (&Eq)[V], uint32_t wv, uint32_t (&Pv)[V], uint32_t (&Mv)[V],
+                                            uint32_t& T, uint32_t& Ph_out, uint32_t& hn, uint32_t& pub) {
+  uint32_t EP[V], SUM[V], Ph[V], Mh[V];
   const uint32_t hin_neg = wv & 1u;
   const uint32_t hin_pos = __umulhi(wv, 2u);
 #pragma unroll
@@ -140,11 +130,79 @@ __device__ __forceinline__ void wave_load_rows(const VerifyArgs& a, uint64_t pos
   }
 }
 
+// Match bits of the block's rows with B's symbol (bit 31 of bw[], consumed).
+// From the block's planes:
+template <int P, int V>
+__device__ __forceinline__ void eq_planes(const uint32_t (&pa)[P][V], uint32_t (&bw)[P], uint32_t (&Eq)[V]) {
+#pragma unroll
+  for (int w = 0; w < V; ++w) Eq[w] = 0xffffffffu;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const uint32_t xb = (uint32_t)__mulhi((int32_t)bw[p], 1);   // B's bit p broadcast (sign of bw)
+#pragma unroll
+    for (int w = 0; w < V; ++w) Eq[w] &= ~(pa[p][w] ^ xb);
+    bw[p] *= 2u;
+  }
+}
+
+// For two planes, from a table in shared memory: a lane's rows for each of the
+// four symbols, in units of four words, then two, then one, each unit laid out
+// [symbol][lane] (a lane meets no other lane's banks, whatever the symbols).
+// The XNORs are 2 of the 12 logic operations per word on the ALU pipe, which
+// bounds the kernel (82% busy, the FMA pipe 10%); the loads and their address
+// (multiply-adds) take none.  Join of long reads at K = 1000 (5 words) 31.9 ->
+// 28.5 ms, 20,000 pairs at K = 4000 (4 words) 15.0 -> 13.4 ms, 300 pairs 1.43 ->
+// 1.34 ms; with one or two words a column's chain decides, not the ALU: K =
+// 700, 300 pairs 1.21 -> 1.29 ms, so they keep the planes.
+constexpr int kTableFrom = 3;
+template <int V>
+constexpr int kEqTableWords = 4 * 32 * V;   // of a warp
+
+template <int V>
+__device__ __forceinline__ void eq_store(uint32_t* tab, int lane, const uint32_t (&pa)[2][V]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int w = 0; w < V; ++w) {
+      const uint32_t e = (c & 1 ? pa[0][w] : ~pa[0][w]) & (c & 2 ? pa[1][w] : ~pa[1][w]);
+      const int unit = w < V / 4 * 4 ? 4 : (w < V / 2 * 2 ? 2 : 1);
+      const int first = w / unit * unit;   // units before hold words 0 .. first - 1
+      tab[first * 128 + (c * 32 + lane) * unit + (w - first)] = e;
+    }
+  }
+}
+
+template <int V>
+__device__ __forceinline__ void eq_load(const uint32_t* tab, int lane, uint32_t (&bw)[2], uint32_t (&Eq)[V]) {
+  const uint32_t b0 = __umulhi(bw[0], 2u), b1 = __umulhi(bw[1], 2u);
+  bw[0] *= 2u;
+  bw[1] *= 2u;
+  const uint32_t c32 = mad_lo(b1, 64u, mad_lo(b0, 32u, (uint32_t)lane));   // symbol * 32 + lane
+#pragma unroll
+  for (int w = 0; w + 4 <= V; w += 4) {
+    const uint4 x = *reinterpret_cast<const uint4*>(tab + w * 128 + c32 * 4);
+    Eq[w] = x.x;
+    Eq[w + 1] = x.y;
+    Eq[w + 2] = x.z;
+    Eq[w + 3] = x.w;
+  }
+  if constexpr (V % 4 >= 2) {
+    constexpr int w = V / 4 * 4;
+    const uint2 x = *reinterpret_cast<const uint2*>(tab + w * 128 + c32 * 2);
+    Eq[w] = x.x;
+    Eq[w + 1] = x.y;
+  }
+  if constexpr (V % 2) Eq[V - 1] = tab[(V - 1) * 128 + c32];
+}
+
 template <int G, int P, int V>
 __global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
                                                           unsigned long long* __restrict__ next) {
   constexpr int R = 32 * V;   // rows of a block
+    constexpr bool kTable = P == 2 && V >= kTableFrom;
   const int lane = threadIdx.x & 31;
+  __shared__ __align__(16) uint32_t tables[kTable ? 4 * kEqTableWords<V> : 4];
+  uint32_t* tab = tables + (kTable ? (threadIdx.x >> 5) * kEqTableWords<V> : 0);
   const int gl = lane & (G - 1);
   const int gbase = lane - gl;
   const uint32_t gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << gbase);
@@ -176,8 +234,21 @@ __global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_ker
 #pragma unroll
     for (int p = 0; p < P; ++p) pa[p][w] = 0u;
   }
+  if constexpr (kTable) eq_store<V>(tab, lane, pa);   // lanes without a block compute on it
 #pragma unroll
   for (int p = 0; p < P; ++p) bw[p] = 0u;
+
+  // One column: the block step on the match bits, which a table gives one
+  // column ahead (they wait for nothing; loaded when used they stand in the
+  // chain from hand-over to hand-over).
+  uint32_t Eq[V];
+#pragma unroll
+  for (int w = 0; w < V; ++w) Eq[w] = 0u;
+  auto column = [&](uint32_t wv, uint32_t& Ph, uint32_t& hn) {
+    if constexpr (!kTable) eq_planes<P, V>(pa, bw, Eq);
+    wave_column<V>(Eq, wv, Pv, Mv, T, Ph, hn, pub);
+    if constexpr (kTable) eq_load<V>(tab, lane, bw, Eq);
+  };
 
   // Take block nb after step s.  Its columns are [jf, jl]; block nb computes
   // column j at step j + nb.  Blocks past row m never run.
@@ -286,7 +357,7 @@ __global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_ker
           const uint32_t w_in = __shfl_sync(0xffffffffu, pub, prev_lane);
           const uint32_t wv = mad_lo(w_in, keep_in, idle_in);   // w_in, or kIdle at the band's edge
           uint32_t Ph, hn;
-          wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+          column(wv, Ph, hn);
         }
         u += free;
         it += free;
@@ -295,19 +366,21 @@ __global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_ker
       ++u;
       const uint32_t wv = u <= u_valid ? w_in : kIdle;
       uint32_t Ph, hn;
-      wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+      column(wv, Ph, hn);
       const bool diag_here = it == kWaveSteps - 1 && (uint32_t)(u + dg) < (uint32_t)R;
       if (u == 0 || u == span || diag_here) {
         if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
           const int32_t jf = sbase + it + 1 - b;
           wave_load_rows<P, V>(a, (uint64_t)(oA + R * (int64_t)b + 32 * (int64_t)GW), pa);
+          if constexpr (kTable) eq_store<V>(tab, lane, pa);
           wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
+          if constexpr (kTable) eq_load<V>(tab, lane, bw, Eq);
 #pragma unroll
           for (int w = 0; w < V; ++w) {
             Pv[w] = 0xffffffffu;
             Mv[w] = 0u;
           }
-          wave_column<P, V>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+          column(wv, Ph, hn);
           // D of the row above the block in this column, plus the block's deltas
           const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
           const int32_t score = above + deltas_below<V>(Pv, Mv, -1);
@@ -333,6 +406,7 @@ __global__ void __launch_bounds__(128, P <= 2 && V == 1 ? 8 : 1) verify_wave_ker
     sbase += kWaveSteps;
     if ((sbase & 31) == 0 && u >= 0 && u <= span) {   // B's symbols of the next 32 columns, all lanes at once
       wave_load_bits<P>(a, PW, (uint64_t)(oB + (sbase - b) + 32 * (int64_t)GW), bw, true);
+      if constexpr (kTable) eq_load<V>(tab, lane, bw, Eq);
     }
     // ---- a group whose pair finished (or was rejected) writes it and frees
     // its lanes; one vote in the common case where none did
@@ -520,7 +594,9 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
         ++u;
         const uint32_t wv = u <= u_valid ? w_in : kIdle;
         uint32_t Ph, hn;
-        wave_column<P, 1>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+        uint32_t Eq[1];
+        eq_planes<P, 1>(pa, bw, Eq);
+        wave_column<1>(Eq, wv, Pv, Mv, T, Ph, hn, pub);
         const bool diag_here = it == S - 1 && (uint32_t)(u + dg) < 32u;
         if (u == 0 || u == span || diag_here) {
           if (u == 0) {   // first column: load the block's symbols, rows start from +1 deltas
@@ -529,7 +605,8 @@ __global__ void __launch_bounds__(32 * V) verify_cta_kernel(VerifyArgs a, uint64
             wave_load_bits<P>(a, PW, (uint64_t)(oB + jf - 1 + 32 * (int64_t)GW), bw, true);
             Pv[0] = 0xffffffffu;
             Mv[0] = 0u;
-            wave_column<P, 1>(pa, bw, wv, Pv, Mv, T, Ph, hn, pub);
+            eq_planes<P, 1>(pa, bw, Eq);
+            wave_column<1>(Eq, wv, Pv, Mv, T, Ph, hn, pub);
             const int32_t above = b == 0 ? 1 : (int32_t)((w_in >> 1) & 0x3fffffffu);
             const int32_t score = above + deltas_below<1>(Pv, Mv, -1);
             T = (uint32_t)score << 1;

@@ -48,7 +48,7 @@ __device__ __forceinline__ uint32_t join_halves(const PairState<W, P>& st, int l
 // two: 2,200 pairs of 5,000-base reads (4 words) 393 -> 281 us, 4,500 of
 // 1,500-symbol text (3 words) 210 -> 143, 1,300 of 700 bytes (2 words) 229 -> 160.
 template <int W, int P>
-__global__ void __launch_bounds__(128) verify_split_kernel(VerifyArgs a, uint64_t PW, uint32_t GW,
+__global__ void __launch_bounds__(128) verify_split_kernel(VerifyArgs a, uint64_t PW, uint32_t GW, int lanes,
                                                            unsigned long long* __restrict__ next) {
   extern __shared__ __align__(16) uint32_t vsm[];
   const int lane = threadIdx.x & 31;
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(128) verify_split_kernel(VerifyArgs a, uint64_
   const uint64_t q_hi = a.range_hi ? *a.range_hi : a.m;
   PairState<W, P> st;
   bool active = false, running = false;   // the pair is held, this half has columns left
-  bool more = true;
+  bool more = lane < lanes;
   uint64_t work = 0, nskip = 0;
   while (true) {
     const bool need = !active && more;   // the same in both lanes of a pair
@@ -128,7 +128,18 @@ int launch_split_wp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long
   if (!a.codes) return MJ_ERR_ARG;
   constexpr size_t smem = digit_smem_bytes<W, P>();
   MJ_CUDA_TRY(cudaFuncSetAttribute(verify_split_kernel<W, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  verify_split_kernel<W, P><<<(unsigned)((a.m * 2 + 127) / 128), 128, smem, s>>>(a, PW, GW, next);
+  // The fewest lanes per warp with at most one warp per scheduler: a warp's
+  // loads take a wavefront per lane and its chunks last as long as the longest
+  // lane's.  2,000 pairs, 8 lanes against 32: 500-symbol protein 76 -> 67 us,
+  // 5,000-base reads 258 -> 246; 300 text pairs, 2 lanes: 134 -> 117; more
+  // warps than that share a scheduler and take longer (2,000 pairs of reads, 2
+  // lanes: 447).
+  int dev = 0, sms = kNumSMsHint, lanes = 2;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  while (lanes < 32 && a.m * 2 > (uint64_t)lanes * 4 * sms) lanes *= 2;
+  const uint64_t warps = (a.m * 2 + lanes - 1) / lanes;
+  verify_split_kernel<W, P><<<(unsigned)((warps + 3) / 4), 128, smem, s>>>(a, PW, GW, lanes, next);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

@@ -458,7 +458,11 @@ int radix_sort(KT* keys, KT* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint6
     const uint32_t m = (uint32_t)n;
     if (m <= 1024) return launch_radix_one<KT, 1>(keys, vals, m, bit_lo, bit_hi, s);
     if (m <= 4096) return launch_radix_one<KT, 4>(keys, vals, m, bit_lo, bit_hi, s);
-    return launch_radix_one<KT, (int)(kOneSort<KT> / kOneSortThreads)>(keys, vals, m, bit_lo, bit_hi, s);
+    if (m <= 8192) return launch_radix_one<KT, 8>(keys, vals, m, bit_lo, bit_hi, s);
+    if constexpr (sizeof(KT) == 4) {   // 16 items per thread spill registers
+      if (m <= 12288) return launch_radix_one<KT, 12>(keys, vals, m, bit_lo, bit_hi, s);
+      return launch_radix_one<KT, 16>(keys, vals, m, bit_lo, bit_hi, s);
+    }
   }
   const uint32_t tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
   const uint64_t h = (uint64_t)tiles * 256;

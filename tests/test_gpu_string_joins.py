@@ -75,3 +75,26 @@ def test_candidates_after_a_join_by_strings():
                 ctx.partition(d2, o2, p)
             ci, cj = ctx._copy_candidates(m, data.device)
             assert np.array_equal(ci.cpu().numpy(), want[0]) and np.array_equal(cj.cpu().numpy(), want[1])
+
+
+@pytest.mark.parametrize("bands", [False, True])
+def test_long_list_under_the_bounds(bands):
+    """Verification of a list long enough for the lower bounds, most of its
+    pairs unrelated, equals the oracle."""
+    import oracle
+    import paper_1810_08833_gb300 as mj
+    import torch
+    s = _set(51, 160, 60, 110, synth.PROTEIN, K=9)
+    m, K = (1 << 20) + 77, 9
+    rng = np.random.Generator(np.random.PCG64(52))
+    pairs = rng.integers(0, 160, size=(m, 2))
+    k = rng.integers(2, K + 1, size=m) if bands else np.full(m, K)
+    every = np.stack(np.meshgrid(np.arange(160), np.arange(160), indexing="ij"), axis=-1).reshape(-1, 2)
+    full = oracle.ed_band_pairs(s.bytes, s.offsets, every.astype(np.int64), K, cutoff=True).reshape(160, 160)
+    want = np.minimum(full[pairs[:, 0], pairs[:, 1]], k + 1)
+    data, off = to_device(s)
+    with mj.Context(0) as ctx:
+        i, j = (torch.from_numpy(pairs[:, c].astype(np.int32)).cuda() for c in (0, 1))
+        bd = torch.from_numpy(k.astype(np.int32)).cuda() if bands else None
+        got = ctx.verify(data, off, i, j, K, k=bd).cpu().numpy().astype(np.int64)
+    assert np.array_equal(got, want), np.nonzero(got != want)[0][:10]

@@ -47,10 +47,9 @@ RECORD_BYTES = 24            # one partition record written: sid, pos, len, stri
 # capture (dram__bytes_read.sum + dram__bytes_write.sum, a one-pass capture
 # of the full-size launch) of the current kernel, keyed by (section, workload
 # number); absent (reported as null) where no capture of the current kernel
-# exists.  Text-like workload: verify_diag_kernel<3, 7> with three digit
-# tables, code bytes and the per-chunk count of the top row's rises,
-# 49.80 GB read + 3.82 GB written in one launch over 645 M candidates.
-TRAFFIC_BYTES = {("verify_kernel", 5): 49.80e9 + 3.82e9}
+# exists.  The last capture was of a verifier launch over all 645 M candidates
+# of the text-like workload; the lower bounds have since left 2% of them.
+TRAFFIC_BYTES = {}
 # integer issue ceiling per SM and clock: the ALU pipe's 64 lanes plus the
 # FMA pipe's 64 (integer multiply-adds run there)
 ISSUE_LANES_PER_SM = 128
@@ -441,7 +440,9 @@ def roofline(section: str, ms: float, st: dict, nbytes: int, hbm: float, hbm_src
                 "frac": ach / hbm, "traffic": traffic, "peak_source": hbm_src}
     if section in ("record_sort", "pair_dedup"):
         n = st["n_partitions"] if section == "record_sort" else st["n_raw_pairs"]
-        per = 24 if section == "record_sort" else 16   # one read and one write of key (+ value)
+        # record_sort: one read and one write of key and value; pair_dedup: the
+        # 16-byte word that a string's visit of a partner reads, per raw pair
+        per = 24 if section == "record_sort" else 16
         work = n * per
         ach = work / sec / 1e9
         return {"kernel": section, "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",

@@ -194,8 +194,8 @@ struct mj_ctx {
   Buf branges;   // bucket counts [32] then ranges [64]
   // CUDA graph of the plain verification stage
   cudaGraphExec_t graph_exec = nullptr;
-  uint64_t graph_sig[26] = {};
-  uint64_t last_sig[26] = {};
+  uint64_t graph_sig[27] = {};
+  uint64_t last_sig[27] = {};
   uint64_t graph_launches = 0;
   // learned first-pass band: parameters P, Adam moments M and V, gradient G, loss
   Buf band, band_part;
@@ -1053,15 +1053,16 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
   if (c->tuned) {
     for (int b = 0; b < kLenBuckets; ++b) plan = plan * 1000003u + c->tuned_kernel[b] * 64u + c->tuned_lanes[b];
   }
-  // everything the captured launches read as a parameter: buffers, sizes, plan
-  const uint64_t sig[26] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
+  // everything the captured launches read as a parameter, and what verify_ordered
+  // branches on: buffers, sizes, plan, whether the order's cells are wanted
+  const uint64_t sig[27] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
                             (uint64_t)ed, (uint64_t)c->planes.p, c->planes_pw, c->d.bits, plan,
                             (uint64_t)c->small.p, (uint64_t)c->idx.p, (uint64_t)c->branges.p,
                             (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0, (uint64_t)c->geo.p,
                             c->stats.n_bytes, c->stats.n_strings, c->planes_gw,
                             (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
                             (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p,
-                            (uint64_t)c->rejected.p, bounds_pay(c, m, K) ? 1ull : 0ull};
+                            (uint64_t)c->rejected.p, bounds_pay(c, m, K) ? 1ull : 0ull, c->want_cells ? 1ull : 0ull};
   if (c->graph_exec && memcmp(sig, c->graph_sig, sizeof(sig)) == 0) {
     MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
     c->mark_launches = ~0ull;   // the graph's kernels are not counted as launches

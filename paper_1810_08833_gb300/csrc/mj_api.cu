@@ -128,6 +128,14 @@ using namespace mj;
 
 constexpr int kCalibrationRuns = 3;   // timed joins per mode in mj_band_calibrate (median)
 
+// Everything that the captured launches of the verification stage hold by value
+// and that the stage branches on: buffers, sizes, the kernel plan, whether the
+// order's cells are wanted, the shape of the bounds' signatures.
+struct GraphKey {
+  uint64_t word[28];
+  SigShape shape;
+};
+
 struct mj_ctx {
   int device = 0;
   int sms = 152;   // streaming multiprocessors of the device
@@ -194,8 +202,7 @@ struct mj_ctx {
   Buf branges;   // bucket counts [32] then ranges [64]
   // CUDA graph of the plain verification stage
   cudaGraphExec_t graph_exec = nullptr;
-  uint64_t graph_sig[27] = {};
-  uint64_t last_sig[27] = {};
+  GraphKey graph_key{}, last_key{};
   uint64_t graph_launches = 0;
   // learned first-pass band: parameters P, Adam moments M and V, gradient G, loss
   Buf band, band_part;
@@ -1043,7 +1050,11 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
 // second captures, later ones replay.
 int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const uint32_t* ci,
                          const uint32_t* cj, uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
+  if (K >= (1u << 16)) return MJ_ERR_UNSUPPORTED;   // as verify, before anything is built for it
   MJ_TRY(order_buffers(c, m, s));
+  // the planes and rank codes hold this call's bytes and alphabet, so they are
+  // made before the stage and never part of its graph
+  MJ_TRY(ensure_planes(c, d_bytes, K, s));
   if (bounds_pay(c, m, K)) MJ_TRY(bounds_buffers(c, m, s));
   // capture needs a stream of its own: the legacy and per-thread default
   // streams run the stage uncaptured
@@ -1053,25 +1064,24 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
   if (c->tuned) {
     for (int b = 0; b < kLenBuckets; ++b) plan = plan * 1000003u + c->tuned_kernel[b] * 64u + c->tuned_lanes[b];
   }
-  // everything the captured launches read as a parameter, and what verify_ordered
-  // branches on: buffers, sizes, plan, whether the order's cells are wanted
-  const uint64_t sig[27] = {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K,
-                            (uint64_t)ed, (uint64_t)c->planes.p, c->planes_pw, c->d.bits, plan,
-                            (uint64_t)c->small.p, (uint64_t)c->idx.p, (uint64_t)c->branges.p,
-                            (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0, (uint64_t)c->geo.p,
-                            c->stats.n_bytes, c->stats.n_strings, c->planes_gw,
-                            (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
-                            (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p,
-                            (uint64_t)c->rejected.p, bounds_pay(c, m, K) ? 1ull : 0ull, c->want_cells ? 1ull : 0ull};
-  if (c->graph_exec && memcmp(sig, c->graph_sig, sizeof(sig)) == 0) {
+  const bool bounds = bounds_pay(c, m, K);
+  const GraphKey key = {
+      {(uint64_t)d_bytes, (uint64_t)d_offsets, (uint64_t)ci, (uint64_t)cj, m, K, (uint64_t)ed, (uint64_t)c->planes.p,
+       c->planes_pw, c->planes_gw, c->d.bits, c->d.sigma, plan, (uint64_t)c->small.p, (uint64_t)c->idx.p,
+       (uint64_t)c->branges.p, (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0,
+       (uint64_t)c->geo.p, c->stats.n_bytes, c->stats.n_strings, (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
+       (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p, (uint64_t)c->rejected.p, bounds ? 1ull : 0ull,
+       c->want_cells ? 1ull : 0ull},
+      bounds ? signature_shape(c->d.sigma, c->code_counts) : SigShape{}};
+  if (c->graph_exec && memcmp(&key, &c->graph_key, sizeof(key)) == 0) {
     MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
     c->mark_launches = ~0ull;   // the graph's kernels are not counted as launches
     mark_graph_sections(c);
     c->launches_at_start -= c->graph_launches;   // kernels replayed by the graph
     return MJ_OK;
   }
-  if (memcmp(sig, c->last_sig, sizeof(sig)) != 0) {
-    memcpy(c->last_sig, sig, sizeof(sig));
+  if (memcmp(&key, &c->last_key, sizeof(key)) != 0) {
+    c->last_key = key;
     return verify_ordered(c, d_bytes, d_offsets, ci, cj, m, K, ed, s);
   }
   if (c->graph_exec) {
@@ -1100,7 +1110,7 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
   cudaGraphDestroy(graph);
   MJ_CUDA_TRY(ie);
   c->graph_launches = launch_count() - before;
-  memcpy(c->graph_sig, sig, sizeof(sig));
+  c->graph_key = key;
   MJ_CUDA_TRY(cudaGraphLaunch(c->graph_exec, s));
   c->mark_launches = ~0ull;
   mark_graph_sections(c);

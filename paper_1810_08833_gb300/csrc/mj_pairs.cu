@@ -809,7 +809,11 @@ int launch_string_pairs_t(PairArgs a, uint32_t widest, cudaStream_t s) {
   int dev = 0, sms = 0, per_sm = 0;
   MJ_CUDA_TRY(cudaGetDevice(&dev));
   MJ_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  MJ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit is the function's, shared by all contexts and threads: the largest
+  // size that string_pairs_fit or a 16-bit window allows, never this call's own
+  constexpr size_t limit = WIDE ? kStringPairsSmemMax + 32 : sizeof(PairShared<THREADS, WIDE>) + 65536 / 8 + 16;
+  if (smem > limit) return MJ_ERR_UNSUPPORTED;
+  MJ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
   MJ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, THREADS, smem));
   a.stride = SAMPLE ? std::max<uint32_t>(1, a.n / kSampleStrings) : 1;
   const uint64_t work = (a.n + a.stride - 1) / a.stride;

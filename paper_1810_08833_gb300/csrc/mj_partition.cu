@@ -737,22 +737,26 @@ int launch_anchor_flags(const PartitionArgs& a, uint32_t* bitmap, uint32_t* tile
   int dev = 0, max_optin = 0;
   MJ_CUDA_TRY(cudaGetDevice(&dev));
   MJ_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (smem + 256 + sizeof(int64_t) * (kAMaxStrings + 1) + sizeof(int32_t) * kAMaxStrings + 64 > (size_t)max_optin)
-    return MJ_ERR_UNSUPPORTED;
+  // dynamic shared memory that the kernels' own arrays leave: also the limit set
+  // below, which is the function's and shared by all contexts and threads, so
+  // that it never follows a call's own size
+  const size_t limit =
+      (size_t)max_optin - (256 + sizeof(int64_t) * (kAMaxStrings + 1) + sizeof(int32_t) * kAMaxStrings + 64);
+  if (smem > limit) return MJ_ERR_UNSUPPORTED;
   const unsigned grid = (unsigned)((tiles + 1) / 2);
   if (table) {
     auto k = anchor_flags_kernel<uint64_t, false, true>;
-    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
     k<<<grid, kAThreads, smem, s>>>(ka, bitmap, tile_count, dev_flags, planes, plane_words, guard_words, tile_first,
                                    tiles);
   } else if (wide) {
     auto k = anchor_flags_kernel<uint64_t, true, false>;
-    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
     k<<<grid, kAThreads, smem, s>>>(ka, bitmap, tile_count, dev_flags, planes, plane_words, guard_words, tile_first,
                                    tiles);
   } else {
     auto k = anchor_flags_kernel<uint32_t, false, false>;
-    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MJ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
     k<<<grid, kAThreads, smem, s>>>(ka, bitmap, tile_count, dev_flags, planes, plane_words, guard_words, tile_first,
                                    tiles);
   }

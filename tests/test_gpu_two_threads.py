@@ -23,9 +23,10 @@ def _one_length(seed, n, L, K):
     return synth.from_strings(strs, K=K, T=K)
 
 
-def _side_by_side(inputs, calls):
-    """Runs every (set, params) of `inputs` in a thread and context of its own,
-    `calls` times, and returns (errors, outputs that differ from a lone run)."""
+def _side_by_side(inputs, calls, what="join"):
+    """Runs Context.join (or another method) on every (set, params) of `inputs`
+    in a thread and context of its own, `calls` times, and returns (errors,
+    outputs that differ from a lone run)."""
     import paper_1810_08833_gb300 as mj
     import torch
     errors, wrong = [], []
@@ -33,7 +34,7 @@ def _side_by_side(inputs, calls):
     for s, p in inputs:
         data, off = to_device(s)
         with mj.Context(0) as ctx:
-            jobs.append((data, off, p, [t.cpu().numpy() for t in ctx.join(data, off, p)]))
+            jobs.append((data, off, p, [t.cpu().numpy() for t in getattr(ctx, what)(data, off, p)]))
     torch.cuda.synchronize()
     gate = threading.Barrier(len(jobs))
 
@@ -44,7 +45,7 @@ def _side_by_side(inputs, calls):
                 gate.wait()
                 for t in range(calls):
                     with torch.cuda.stream(stream):
-                        out = ctx.join(data, off, p, stream=stream)
+                        out = getattr(ctx, what)(data, off, p, stream=stream)
                         if t % 16 == 0:
                             got = [x.cpu().numpy() for x in out]
                             if not all(np.array_equal(a, b) for a, b in zip(got, want)):
@@ -66,4 +67,15 @@ def test_joins_with_windows_of_different_widths():
     import paper_1810_08833_gb300 as mj
     sets = [_one_length(1, 20_000, 40, 3), _one_length(2, 300, 40, 3), _one_length(3, 2_000, 60, 4)]
     errors, wrong = _side_by_side([(s, mj.params(s.K, T=s.T)) for s in sets], calls=400)
+    assert not errors and not wrong, (errors, wrong)
+
+
+def test_anchors_with_halos_of_different_radii():
+    """The anchor kernel's span follows the radius: strings of 12,000 symbols in
+    6 partitions (radius 856) and strings of 60 in 10 (radius 2)."""
+    import paper_1810_08833_gb300 as mj
+    long = synth.random_set(5, n=40, min_len=11_000, max_len=12_000, K=6, T=6, families=4, rate=0.0003)
+    short = synth.random_set(6, n=300, min_len=50, max_len=60, K=10, T=10, families=12, rate=0.02)
+    sets = [(s, mj.params(s.K, T=s.T)) for s in (long, short)]
+    errors, wrong = _side_by_side(sets * 3, calls=1500, what="partition")
     assert not errors and not wrong, (errors, wrong)

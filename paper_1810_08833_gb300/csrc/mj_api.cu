@@ -238,8 +238,8 @@ struct mj_ctx {
   // marks, and at[i] names the event of the section's start or end
   static constexpr int kSections = 9, kMarks = 40;
   cudaEvent_t sec_ev[2 * kSections] = {};
-  cudaEvent_t marks[kMarks] = {};
-  int n_marks = 0;
+  std::vector<cudaEvent_t> marks;   // kMarks from mj_create on, more when a call has more points (mark)
+  size_t n_marks = 0;
   uint64_t mark_launches = ~0ull;
   cudaEvent_t at[2 * kSections] = {};
   bool sec_used[kSections] = {};
@@ -282,7 +282,16 @@ int readback(mj_ctx* c, const void* d_src, size_t bytes, cudaStream_t s) { retur
 cudaEvent_t mark(mj_ctx* c, cudaStream_t s) {
   const uint64_t now = launch_count();
   if (c->n_marks && c->mark_launches == now) return c->marks[c->n_marks - 1];
-  if (c->n_marks == mj_ctx::kMarks) --c->n_marks;   // more repetitions than events: the last one moves on
+  // an event that sections already point to is never recorded again: 64
+  // repetitions, or a launch per length bucket, take more than the first kMarks
+  if (c->n_marks == c->marks.size()) {
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreate(&e) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;   // this point's times read 0
+    }
+    c->marks.push_back(e);
+  }
   cudaEventRecord(c->marks[c->n_marks], s);
   c->mark_launches = now;
   return c->marks[c->n_marks++];
@@ -342,6 +351,7 @@ int check_inputs(const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t n, c
 
 float elapsed(cudaEvent_t a, cudaEvent_t b) {
   float ms = 0.f;
+  if (!a || !b) return ms;
   if (cudaEventElapsedTime(&ms, a, b) != cudaSuccess) {
     cudaGetLastError();
     return 0.f;
@@ -1314,12 +1324,14 @@ int mj_create(mj_ctx** ctx, int device) {
       return MJ_ERR_CUDA;
     }
   }
-  for (auto& e : c->marks) {
+  for (int k = 0; k < mj_ctx::kMarks; ++k) {
+    cudaEvent_t e = nullptr;
     if (cudaEventCreate(&e) != cudaSuccess) {
       cudaGetLastError();
       mj_destroy(c);
       return MJ_ERR_CUDA;
     }
+    c->marks.push_back(e);
   }
   for (auto& e : c->ev) {
     if (cudaEventCreate(&e) != cudaSuccess) {
@@ -1365,8 +1377,7 @@ void mj_destroy(mj_ctx* c) {
     if (e) cudaEventDestroy(e);
   for (auto& e : c->sec_ev)
     if (e) cudaEventDestroy(e);
-  for (auto& e : c->marks)
-    if (e) cudaEventDestroy(e);
+  for (auto e : c->marks) cudaEventDestroy(e);
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   if (c->h_small) cudaFreeHost(c->h_small);
   delete c;

@@ -60,6 +60,9 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
 // rank_of[sid]; hi[r] = last rank whose short is at most shorts[r] + K;
 // *widest = the most ranks above its own that a string can pair with;
 // short_rank[l] (nullable), l = 0 .. longest: first rank of short >= l, n if none.
+// Every entry is a search of its own: filled by the rank that ends a run of
+// lengths, a gap between two lengths is one thread's loop (20,000 reads and one
+// string of 4 M symbols: 50 ms of a join of 108).
 __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const uint32_t* __restrict__ sid_of, uint32_t n,
                                    uint32_t K, uint32_t longest, uint32_t* __restrict__ rank_of,
                                    uint32_t* __restrict__ hi, uint32_t* __restrict__ short_rank,
@@ -69,15 +72,13 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
     const uint32_t r = (uint32_t)t;
     rank_of[sid_of[r]] = r;
     const uint32_t L = shorts[r], top = L > 0xffffffffu - K ? 0xffffffffu : L + K;
-    if (short_rank) {
-      for (uint32_t l = r ? shorts[r - 1] + 1u : 0u; l <= L; ++l) short_rank[l] = r;
-      if (r == n - 1)
-        for (uint32_t l = L + 1u; l <= longest; ++l) short_rank[l] = n;
-    }
     const uint32_t h = upper_bound_of(shorts, r + 1, n, top) - 1;
     hi[r] = h;
     w = max(w, h - r);
   }
+  if (short_rank)   // longest < 2^32 - 1: a string's length is below the input's size
+    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l <= longest; l += (uint64_t)gridDim.x * blockDim.x)
+      short_rank[l] = l ? upper_bound_of(shorts, 0, n, (uint32_t)l - 1u) : 0u;
   w = __reduce_max_sync(0xffffffffu, w);
   if ((threadIdx.x & 31) == 0 && w) atomicMax(widest, w);
 }
@@ -847,8 +848,8 @@ int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t
   string_lengths_kernel<<<grid_for(n), 256, 0, s>>>(offsets, n, shorts, sid, longest);
   MJ_KERNEL_DONE();
   MJ_TRY(radix_sort_u32(shorts, shorts_alt, sid, sid_alt, n, 0, len_bits, temp, in_alt, s));
-  rank_tables_kernel<<<grid_for(n), 256, 0, s>>>(*in_alt ? shorts_alt : shorts, *in_alt ? sid_alt : sid, n, K, longest,
-                                                 rank_of, hi, short_rank, widest);
+  rank_tables_kernel<<<grid_for(std::max<uint64_t>(n, short_rank ? longest + 1ull : 0)), 256, 0, s>>>(
+      *in_alt ? shorts_alt : shorts, *in_alt ? sid_alt : sid, n, K, longest, rank_of, hi, short_rank, widest);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

@@ -182,7 +182,8 @@ struct mj_ctx {
   Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
   bool by_strings = false;        // this call builds the rank tables
   bool rk_alt = false;            // rk_len_alt / rk_sid_alt hold the sorted strings
-  uint32_t rk_widest = 0;
+  uint32_t rk_widest = 0;         // the widest window of ranks,
+  uint64_t rk_spans = 0;          // and the sum of all (read back in partition)
   uint32_t rep_first[65] = {0};   // first record of every repetition
   uint64_t code_counts[256] = {0};   // input symbols by rank code
   // A plain join by strings lists no candidates: mj_candidates_copy makes them
@@ -476,10 +477,11 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
     uint32_t* total = c->dev_flags.as<uint32_t>() + 1;   // read back with the flags and the widest window
     MJ_TRY(launch_exclusive_scan_u32(c->tile_count.as<uint32_t>(), c->tile_off.as<uint32_t>(), tiles,
                                      c->scan_tmp.p, total, s));
-    MJ_TRY(readback(c, c->dev_flags.p, 12, s));
+    MJ_TRY(readback(c, c->dev_flags.p, 24, s));
     const uint32_t* got = reinterpret_cast<const uint32_t*>(c->h_small);
     const uint32_t n_anchor = got[1];
     c->rk_widest = got[2];
+    c->rk_spans = c->h_small[2];
     c->stats.device_flags |= got[0];
     if (c->stats.device_flags) return MJ_ERR_DEVICE;
     if (n_total + n_anchor >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;   // record indexes are 32-bit
@@ -680,6 +682,8 @@ bool bounds_reach(uint64_t N, uint32_t sigma, uint32_t K) {
 }
 
 constexpr uint64_t kBoundsFrom = 1u << 15;    // candidates from which a join by strings may use the lower bounds
+constexpr uint64_t kListAll = 1u << 20;        // pairs of ranks up to which there is room for all of them
+constexpr int kSampledAt = 64;                 // word of the staging memory for the sample's count
 constexpr uint64_t kShortRankMax = 1u << 22;   // longest string up to which ranks are found by length in a table
 
 // Rank tables of a plain join by strings (before its partition step, whose
@@ -701,8 +705,7 @@ int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s
                              c->rk_len_alt.as<uint32_t>(), c->rk_sid.as<uint32_t>(), c->rk_sid_alt.as<uint32_t>(),
                              c->sort_tmp.p, c->rk_of.as<uint32_t>(), c->rk_hi.as<uint32_t>(),
                              by_len ? c->rk_short_rank.as<uint32_t>() : nullptr, c->dev_flags.as<unsigned int>() + 2,
-                             &c->rk_alt,
-                             s);
+                             c->dev_flags.as<unsigned long long>() + 2, &c->rk_alt, s);
 }
 
 // a5-a7 by strings (after partition and string_ranks): the candidates counted,
@@ -791,10 +794,29 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   const uint64_t min_sampled = bounds ? std::max<uint64_t>(c->stats.n_bytes / 96, kBoundsFrom) / stride : ~0ull;
   a.min_sampled = min_sampled;
   a.q1 = g.q1;
-  if (bounds) {
-    MJ_TRY(launch_string_sample(a, c->rk_widest, s));
+  // The lists' sizes: all the windows' ranks where those are few, else the
+  // candidates that the sample lets expect (a copy that the host waits for while
+  // the signatures are made) and a quarter more.  Under the bounds most
+  // candidates are unrelated, and no more than 2^28, or one per input byte, are
+  // expected to pass the first, 2^24 or one per 8 bytes the second.
+  const bool many = c->rk_spans > kListAll;
+  if (bounds || many) MJ_TRY(launch_string_sample(a, c->rk_widest, s));
+  if (many) {
+    MJ_CUDA_TRY(cudaMemcpyAsync(c->h_small + kSampledAt, cnt + 1, 8, cudaMemcpyDeviceToHost, s));
+    MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
+  }
+  if (bounds)
     MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_sampled,
                              c->rk_sig1.as<uint4>(), c->rk_sig2.as<uint32_t>(), s));
+  uint64_t cap1 = c->rk_spans, cap2;
+  if (many) {
+    MJ_CUDA_TRY(cudaEventSynchronize(c->ev[0]));
+    const uint64_t sampled = c->h_small[kSampledAt], expected = sampled * stride;
+    cap1 = std::min(cap1, expected + expected / 4 + (1u << 16));
+    if (sampled > min_sampled) cap1 = std::min(cap1, std::max<uint64_t>(c->stats.n_bytes, 1u << 28));
+    cap2 = sampled > min_sampled ? std::min(cap1, std::max<uint64_t>(c->stats.n_bytes / 8, 1u << 24)) : cap1;
+  } else {
+    cap2 = cap1;
   }
   ListArgs l;
   l.in_count = a.out_count;
@@ -807,11 +829,11 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   l.K = d.K;
   l.q2 = g.q2;
   l.out_count = cnt + 6;
-  // room for what passes the bounds: a first guess, at least every candidate
-  // when the bounds are not used; a longer list is counted and made again
-  uint64_t cap1 = c->stats.n_bytes + (1u << 16), cap2 = c->stats.n_bytes / 8 + (1u << 16);
+  // a list that is too short is counted in full and made again, the first one
+  // with the second
+  bool first = true;
   for (int tries = 0;; ++tries) {
-    MJ_TRY(c->rk_list.reserve(cap1 * 8, s));
+    if (first) MJ_TRY(c->rk_list.reserve(cap1 * 8, s));
     MJ_TRY(c->cand_i.reserve(cap2 * 4 + 16, s));
     MJ_TRY(c->cand_j.reserve(cap2 * 4 + 16, s));
     a.cap = l.in_cap = cap1;
@@ -820,15 +842,23 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
     l.cap = cap2;
     l.out_i = c->cand_i.as<uint32_t>();
     l.out_j = c->cand_j.as<uint32_t>();
-    MJ_TRY(launch_string_pairs(a, c->rk_widest, s));
+    if (first) MJ_TRY(launch_string_pairs(a, c->rk_widest, s));
     MJ_TRY(launch_listed_pairs(l, s));
     MJ_TRY(readback(c, cnt + 2, 40, s));
     if (c->h_small[1] >= (1ull << 32)) return MJ_ERR_UNSUPPORTED;   // raw pairs, as on the general path
-    if (c->h_small[0] <= cap1 && c->h_small[4] <= cap2) break;
+    const uint64_t passed1 = c->h_small[0], passed2 = c->h_small[4];
+    if (passed1 <= cap1 && passed2 <= cap2) break;
     if (tries > 1) return MJ_ERR_DEVICE;   // both lists were counted in full
-    cap1 = std::max<uint64_t>(cap1, c->h_small[0]);
-    cap2 = std::max<uint64_t>(cap2, std::min<uint64_t>(c->h_small[4], c->h_small[0]));
-    MJ_CUDA_TRY(cudaMemsetAsync(cnt + 2, 0, 40, s));
+    first = passed1 > cap1;
+    if (first) {   // of the rest of the first list, as many are expected to pass as of its start
+      const uint64_t expected = (uint64_t)((double)passed2 * ((double)passed1 / (double)cap1));
+      cap2 = std::max(cap2, std::min(passed1, expected + expected / 4));
+      cap1 = passed1;
+      MJ_CUDA_TRY(cudaMemsetAsync(cnt + 2, 0, 40, s));
+    } else {
+      cap2 = passed2;
+      MJ_CUDA_TRY(cudaMemsetAsync(cnt + 6, 0, 8, s));
+    }
   }
   tstop(c, 4, s);
   c->n_list = c->h_small[4];

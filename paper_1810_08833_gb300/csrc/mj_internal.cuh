@@ -174,11 +174,12 @@ int radix_sort_u32(uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t*
 // - length.  shorts/sid (n entries each and their alternates) end sorted, in the
 // alternates if *in_alt; rank_of[id], hi[rank] = the last rank within K of its
 // length; short_rank[l] (nullable), l = 0 .. longest = the first rank of short l
-// or more; *widest = the most ranks above its own that a string can pair with.
+// or more; *widest = the most ranks above its own that a string can pair with,
+// *spans += the sum of them, an upper bound on the candidates.
 int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t longest, int len_bits,
                         uint32_t* shorts, uint32_t* shorts_alt, uint32_t* sid, uint32_t* sid_alt, void* temp,
-                        uint32_t* rank_of, uint32_t* hi, uint32_t* short_rank, unsigned int* widest, bool* in_alt,
-                        cudaStream_t s);
+                        uint32_t* rank_of, uint32_t* hi, uint32_t* short_rank, unsigned int* widest,
+                        unsigned long long* spans, bool* in_alt, cudaStream_t s);
 // first[i], i = 0 .. n: base + the anchors before string i in the bitmap
 // (`total` anchors in all).
 int launch_string_first(const int64_t* offsets, uint32_t n, uint64_t nbytes, const uint32_t* bitmap,

@@ -58,7 +58,7 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
 }
 
 // rank_of[sid]; hi[r] = last rank whose short is at most shorts[r] + K;
-// *widest = the most ranks above its own that a string can pair with;
+// *widest = the most ranks above its own that a string can pair with, *spans += all of them;
 // short_rank[l] (nullable), l = 0 .. longest: first rank of short >= l, n if none.
 // Every entry is a search of its own: filled by the rank that ends a run of
 // lengths, a gap between two lengths is one thread's loop (20,000 reads and one
@@ -66,8 +66,9 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
 __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const uint32_t* __restrict__ sid_of, uint32_t n,
                                    uint32_t K, uint32_t longest, uint32_t* __restrict__ rank_of,
                                    uint32_t* __restrict__ hi, uint32_t* __restrict__ short_rank,
-                                   unsigned int* __restrict__ widest) {
+                                   unsigned int* __restrict__ widest, unsigned long long* __restrict__ spans) {
   uint32_t w = 0;
+  unsigned long long sum = 0;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t r = (uint32_t)t;
     rank_of[sid_of[r]] = r;
@@ -75,12 +76,17 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
     const uint32_t h = upper_bound_of(shorts, r + 1, n, top) - 1;
     hi[r] = h;
     w = max(w, h - r);
+    sum += h - r;
   }
   if (short_rank)   // longest < 2^32 - 1: a string's length is below the input's size
     for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l <= longest; l += (uint64_t)gridDim.x * blockDim.x)
       short_rank[l] = l ? upper_bound_of(shorts, 0, n, (uint32_t)l - 1u) : 0u;
   w = __reduce_max_sync(0xffffffffu, w);
-  if ((threadIdx.x & 31) == 0 && w) atomicMax(widest, w);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0 && w) {
+    atomicMax(widest, w);
+    atomicAdd(spans, sum);
+  }
 }
 
 // ---------------------------------------------------------------- record order
@@ -842,14 +848,15 @@ unsigned grid_for(uint64_t n, int threads = 256) {
 
 int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t longest, int len_bits,
                         uint32_t* shorts, uint32_t* shorts_alt, uint32_t* sid, uint32_t* sid_alt, void* temp, uint32_t* rank_of, uint32_t* hi,
-                        uint32_t* short_rank, unsigned int* widest, bool* in_alt, cudaStream_t s) {
+                        uint32_t* short_rank, unsigned int* widest, unsigned long long* spans, bool* in_alt, cudaStream_t s) {
   *in_alt = false;
   if (!n) return MJ_OK;
   string_lengths_kernel<<<grid_for(n), 256, 0, s>>>(offsets, n, shorts, sid, longest);
   MJ_KERNEL_DONE();
   MJ_TRY(radix_sort_u32(shorts, shorts_alt, sid, sid_alt, n, 0, len_bits, temp, in_alt, s));
   rank_tables_kernel<<<grid_for(std::max<uint64_t>(n, short_rank ? longest + 1ull : 0)), 256, 0, s>>>(
-      *in_alt ? shorts_alt : shorts, *in_alt ? sid_alt : sid, n, K, longest, rank_of, hi, short_rank, widest);
+      *in_alt ? shorts_alt : shorts, *in_alt ? sid_alt : sid, n, K, longest, rank_of, hi, short_rank, widest,
+      spans);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

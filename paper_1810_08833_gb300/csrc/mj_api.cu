@@ -182,8 +182,10 @@ struct mj_ctx {
   Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
   bool by_strings = false;        // this call builds the rank tables
   bool rk_alt = false;            // rk_len_alt / rk_sid_alt hold the sorted strings
-  uint32_t rk_widest = 0;         // the widest window of ranks,
-  uint64_t rk_spans = 0;          // and the sum of all (read back in partition)
+  // read back in partition: the widest window of ranks, the longest string with
+  // a partner in its own, and the sum of all windows
+  uint32_t rk_widest = 0, rk_longest = 0;
+  uint64_t rk_spans = 0;
   uint32_t rep_first[65] = {0};   // first record of every repetition
   uint64_t code_counts[256] = {0};   // input symbols by rank code
   // A plain join by strings lists no candidates: mj_candidates_copy makes them
@@ -481,6 +483,7 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
     const uint32_t* got = reinterpret_cast<const uint32_t*>(c->h_small);
     const uint32_t n_anchor = got[1];
     c->rk_widest = got[2];
+    c->rk_longest = got[3];
     c->rk_spans = c->h_small[2];
     c->stats.device_flags |= got[0];
     if (c->stats.device_flags) return MJ_ERR_DEVICE;
@@ -741,7 +744,7 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   MJ_TRY(c->rk_scan.reserve((size_t)n * 4 + 16, s));
   MJ_TRY(c->scan_tmp.reserve(scan_temp_bytes(n), s));
   MJ_TRY(c->rk_a.reserve((size_t)nr * 16, s));
-  const int rb = visit_rank_bits(d.N, n);
+  const int rb = visit_rank_bits(c->rk_longest, n);
   if (!rb) MJ_TRY(c->rk_b.reserve((size_t)nr * 8, s));
   MJ_TRY(c->rk_skr.reserve((size_t)nr * 8, s));
   MJ_TRY(c->rk_win.reserve((size_t)nr * 32, s));

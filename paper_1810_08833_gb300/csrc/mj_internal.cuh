@@ -174,8 +174,9 @@ int radix_sort_u32(uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t*
 // - length.  shorts/sid (n entries each and their alternates) end sorted, in the
 // alternates if *in_alt; rank_of[id], hi[rank] = the last rank within K of its
 // length; short_rank[l] (nullable), l = 0 .. longest = the first rank of short l
-// or more; *widest = the most ranks above its own that a string can pair with,
-// *spans += the sum of them, an upper bound on the candidates.
+// or more; widest[0] = the most ranks above its own that a string can pair with,
+// widest[1] = the longest string that can pair at all; *spans += the sum of all
+// strings' such ranks, an upper bound on the candidates.
 int launch_string_ranks(const int64_t* offsets, uint32_t n, uint32_t K, uint32_t longest, int len_bits,
                         uint32_t* shorts, uint32_t* shorts_alt, uint32_t* sid, uint32_t* sid_alt, void* temp,
                         uint32_t* rank_of, uint32_t* hi, uint32_t* short_rank, unsigned int* widest,
@@ -193,6 +194,7 @@ int launch_rank_order(const uint32_t* first, const uint32_t* sid_of, const uint3
 int launch_rank_keys(const PRec* recs, uint32_t t0, uint32_t t1, const uint32_t* delta, int hash_bits, int pb_bits,
                      uint32_t W, uint32_t* keys, uint32_t* vals, cudaStream_t s);
 // Rank bits of a visit word when a visit fits 16 bytes, else 0 (B is then used).
+// longest: of the strings that can pair (the words of others are never visited).
 int visit_rank_bits(uint64_t longest, uint32_t n);
 // From the sorted keys and indices: A, B, skr (n_rec entries) and the windows
 // of every record (2 entries each, at the record's own place).

@@ -58,7 +58,8 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
 }
 
 // rank_of[sid]; hi[r] = last rank whose short is at most shorts[r] + K;
-// *widest = the most ranks above its own that a string can pair with, *spans += all of them;
+// widest[0] = the most ranks above its own that a string can pair with, widest[1] = the longest string
+// that can pair with another, *spans += all ranks above their own that strings can pair with;
 // short_rank[l] (nullable), l = 0 .. longest: first rank of short >= l, n if none.
 // Every entry is a search of its own: filled by the rank that ends a run of
 // lengths, a gap between two lengths is one thread's loop (20,000 reads and one
@@ -67,7 +68,7 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
                                    uint32_t K, uint32_t longest, uint32_t* __restrict__ rank_of,
                                    uint32_t* __restrict__ hi, uint32_t* __restrict__ short_rank,
                                    unsigned int* __restrict__ widest, unsigned long long* __restrict__ spans) {
-  uint32_t w = 0;
+  uint32_t w = 0, len = 0;
   unsigned long long sum = 0;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t r = (uint32_t)t;
@@ -76,6 +77,7 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
     const uint32_t h = upper_bound_of(shorts, r + 1, n, top) - 1;
     hi[r] = h;
     w = max(w, h - r);
+    if (h > r) len = max(len, longest - L);
     sum += h - r;
   }
   if (short_rank)   // longest < 2^32 - 1: a string's length is below the input's size
@@ -83,8 +85,10 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
       short_rank[l] = l ? upper_bound_of(shorts, 0, n, (uint32_t)l - 1u) : 0u;
   w = __reduce_max_sync(0xffffffffu, w);
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  len = __reduce_max_sync(0xffffffffu, len);
   if ((threadIdx.x & 31) == 0 && w) {
     atomicMax(widest, w);
+    atomicMax(widest + 1, len);
     atomicAdd(spans, sum);
   }
 }
@@ -308,8 +312,9 @@ __global__ void rank_windows_kernel(const uint64_t* __restrict__ skr, const uint
 // pass.
 constexpr int kSig1 = 28, kSig2 = 256;
 constexpr int kSig2Bytes = kSig2 / 2;
-// Longer strings are left to the verifier, which refuses them by a flag.
-constexpr uint32_t kBoundsMaxLen = 1u << 27;
+// Longer strings are left to the verifier: a warp counts a string's grams, 11 ns
+// a symbol, and one of 1,000,000 among 20,000 reads took 11 ms of a join of 35.
+constexpr uint32_t kBoundsMaxLen = 1u << 15;
 
 __device__ __forceinline__ uint32_t gram_hash(uint32_t h) {   // MurmurHash3 fmix32
   h ^= h >> 16;
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(32 * kSigWarps) signature_kernel(
     __syncwarp();
     const uint32_t s = sid_of ? __ldg(sid_of + r) : (uint32_t)r;
     const uint32_t o = (uint32_t)__ldg(offsets + s), e = (uint32_t)__ldg(offsets + s + 1);   // inputs are under 4 GB
-    const uint32_t w1 = (uint32_t)(((uint64_t)e + 3) >> 2);
+    const uint32_t w1 = e - o < kBoundsMaxLen ? (uint32_t)(((uint64_t)e + 3) >> 2) : 0u;   // no bounds: only the length
 #pragma unroll 2
     for (uint32_t w = (o >> 2) + lane; w < w1; w += 32) {
       const uint32_t x0 = __ldg(codes32 + w), x1 = __ldg(codes32 + w + 1);
@@ -835,6 +840,8 @@ template <bool SAMPLE>
 int launch_string_pairs_s(const PairArgs& a, uint32_t widest, cudaStream_t s) {
   if (!a.n) return MJ_OK;
   if (widest < 65536 && a.rb) return launch_string_pairs_t<32, false, true, SAMPLE>(a, widest, s);
+  if constexpr (!SAMPLE)   // a sample's few strings take longer on one warp each: 5.4 ms against 1.4 on four
+    if (widest < 65536) return launch_string_pairs_t<32, false, false, false>(a, widest, s);
   return a.rb ? launch_string_pairs_t<128, true, true, SAMPLE>(a, widest, s)
               : launch_string_pairs_t<128, true, false, SAMPLE>(a, widest, s);
 }

@@ -522,8 +522,8 @@ __global__ void __launch_bounds__(256) pair_bounds_kernel(const uint32_t* __rest
 //            windows at a time (a scan of their sizes), long ones by the whole
 //            CTA; a visit tests the position filter and the key, and sets the
 //            partner's bit;
-//   list     every warp takes 16 words of the bitmap, clears them, pushes
-//            their bits on its stack and pops candidates, two per lane, to
+//   list     every warp takes 16 words of the bitmap that hold bits, clears
+//            them, pushes their bits on its stack and pops candidates, two per lane, to
 //            test them against the first lower bound; what passes is appended
 //            to the list of pairs for the second.
 // A warp per string has no barriers to wait at; only windows of 2^16 ranks and
@@ -732,31 +732,39 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
         if (waiting > kPassed - 32) append();
       }
     };
-    // a warp step takes 32 half-words
-    for (uint32_t h0 = 32 * wid; h0 < 2 * words; h0 += 32 * kWarps) {
-      const uint32_t h = h0 + lane;
-      const uint32_t both = h < 2 * words ? bm[h >> 1] : 0u;
-      uint32_t bits = (both >> (16 * (h & 1))) & 0xffffu;
-      __syncwarp();
-      if (both && !(h & 1)) bm[h >> 1] = 0;
-      const uint32_t c = __popc(bits);
-      uint32_t incl = c;
+    // a warp looks at 128 words at a time and takes the 16 words of the groups
+    // that hold bits, 32 half-words to a step
+    for (uint32_t w0 = 128 * wid; w0 < words; w0 += 128 * kWarps) {
+      const uint32_t wl = w0 + 4 * lane;
+      const uint4 four = wl < a.bm_words ? *reinterpret_cast<const uint4*>(bm + wl) : make_uint4(0u, 0u, 0u, 0u);
+      uint32_t some = __ballot_sync(0xffffffffu, (four.x | four.y | four.z | four.w) != 0);
+      while (some) {
+        const uint32_t group = (uint32_t)(__ffs(some) - 1) >> 2;
+        some &= ~(15u << (4 * group));
+        const uint32_t h = 2 * (w0 + 16 * group) + lane;
+        const uint32_t both = h < 2 * words ? bm[h >> 1] : 0u;
+        uint32_t bits = (both >> (16 * (h & 1))) & 0xffffu;
+        __syncwarp();
+        if (both && !(h & 1)) bm[h >> 1] = 0;
+        const uint32_t c = __popc(bits);
+        cand += c;
+        if (SAMPLE) continue;   // nothing is listed: the stack stays empty
+        uint32_t incl = c;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t z = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += z;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t z = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += z;
+        }
+        uint32_t at = depth + incl - c;
+        depth += __shfl_sync(0xffffffffu, incl, 31);
+        while (bits) {
+          stack[at++] = (Slot)(16u * h + (__ffs(bits) - 1));
+          bits &= bits - 1;
+        }
+        __syncwarp();
+        while (depth >= 64) test(std::integral_constant<int, 2>(), 64u);
+        __syncwarp();   // the popped entries are read before the next step's pushes
       }
-      cand += c;
-      if (SAMPLE) continue;   // nothing is listed: the stack stays empty
-      uint32_t at = depth + incl - c;
-      depth += __shfl_sync(0xffffffffu, incl, 31);
-      while (bits) {
-        stack[at++] = (Slot)(16u * h + (__ffs(bits) - 1));
-        bits &= bits - 1;
-      }
-      __syncwarp();
-      while (depth >= 64) test(std::integral_constant<int, 2>(), 64u);
-      __syncwarp();   // the popped entries are read before the next step's pushes
     }
     if (!SAMPLE) {
       if (depth) test(std::integral_constant<int, 2>(), depth);
@@ -817,20 +825,20 @@ __global__ void __launch_bounds__(256) listed_pairs_kernel(ListArgs a) {
 template <int THREADS, bool WIDE, bool PACKED, bool SAMPLE>
 int launch_string_pairs_t(PairArgs a, uint32_t widest, cudaStream_t s) {
   auto kernel = string_pairs_kernel<THREADS, WIDE, PACKED, SAMPLE>;
-  const size_t smem = sizeof(PairShared<THREADS, WIDE>) + ((size_t)widest + 31) / 32 * 4 + 16;
+  a.bm_words = (widest / 32 + 4) / 4 * 4;   // whole 16-byte words, ceil(widest / 32) or more
+  const size_t smem = sizeof(PairShared<THREADS, WIDE>) + (size_t)a.bm_words * 4;
   int dev = 0, sms = 0, per_sm = 0;
   MJ_CUDA_TRY(cudaGetDevice(&dev));
   MJ_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   // the limit is the function's, shared by all contexts and threads: the largest
   // size that string_pairs_fit or a 16-bit window allows, never this call's own
-  constexpr size_t limit = WIDE ? kStringPairsSmemMax + 32 : sizeof(PairShared<THREADS, WIDE>) + 65536 / 8 + 16;
+  constexpr size_t limit = WIDE ? kStringPairsSmemMax + 32 : sizeof(PairShared<THREADS, WIDE>) + 65536 / 8;
   if (smem > limit) return MJ_ERR_UNSUPPORTED;
   MJ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
   MJ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, THREADS, smem));
   a.stride = SAMPLE ? std::max<uint32_t>(1, a.n / kSampleStrings) : 1;
   const uint64_t work = (a.n + a.stride - 1) / a.stride;
   const uint64_t grid = std::min<uint64_t>(work, (uint64_t)std::max(1, sms) * std::max(1, per_sm));
-  a.bm_words = (widest + 31) / 32;
   kernel<<<(unsigned)grid, THREADS, smem, s>>>(a);
   MJ_KERNEL_DONE();
   return MJ_OK;

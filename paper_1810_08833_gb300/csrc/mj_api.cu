@@ -178,7 +178,7 @@ struct mj_ctx {
   // id, windows by rank, first records by string, sorted records, windows,
   // signatures, counters
   Buf rk_len, rk_len_alt, rk_sid, rk_sid_alt, rk_of, rk_hi, rk_first, rk_delta, rk_scan, rk_short_rank;
-  Buf rk_a, rk_b, rk_skr, rk_win, rk_sig1, rk_sig2, rk_cnt, rk_list;
+  Buf rk_a, rk_b, rk_skr, rk_win, rk_sig1, rk_sig2, rk_cnt, rk_list, rk_table;
   Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
   bool by_strings = false;        // this call builds the rank tables
   bool rk_alt = false;            // rk_len_alt / rk_sid_alt hold the sorted strings
@@ -411,6 +411,14 @@ uint64_t key_base_for(uint64_t seed) {
   return 257 + splitmix(seed ^ 0x6b6579626173650aull) % (M61 - 1024);
 }
 
+// First record of every string in repetition k, whose bitmap and tile offsets
+// are the last ones made.
+int string_first(mj_ctx* c, const int64_t* d_offsets, uint32_t n, uint32_t k, cudaStream_t s) {
+  return launch_string_first(d_offsets, n, c->stats.n_bytes, c->bitmap.as<uint32_t>(), c->tile_off.as<uint32_t>(),
+                             c->rep_first[k + 1] - c->rep_first[k], c->rep_first[k],
+                             c->rk_first.as<uint32_t>() + (uint64_t)k * (n + 1), s);
+}
+
 // a2-a4 (after derive): partition records in c->recs (n_part of them).
 // plane_kmax > 0: also write the verifier's bit-planes (guard sized for bands
 // up to plane_kmax).
@@ -494,14 +502,14 @@ int partition(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
                                     c->tile_first.as<uint32_t>(), key_base_for(d.seed),
                                     c->recs.as<PRec>() + n_total, s));
     tstop(c, 1, s);
-    if (c->by_strings) {
-      MJ_TRY(launch_string_first(d_offsets, n, nbytes, c->bitmap.as<uint32_t>(), c->tile_off.as<uint32_t>(), n_anchor,
-                                 (uint32_t)n_total, c->rk_first.as<uint32_t>() + (uint64_t)k * (n + 1), s));
-      c->rep_first[k] = (uint32_t)n_total;
-    }
+    c->rep_first[k] = (uint32_t)n_total;
+    c->rep_first[k + 1] = (uint32_t)(n_total + n_anchor);
+    // one repetition's bitmap is there until the next partition: windows that may
+    // be left to the general path wait with the strings' first records
+    if (c->by_strings && (R > 1 || !string_pairs_from(n, c->rk_widest, c->sms)))
+      MJ_TRY(string_first(c, d_offsets, n, k, s));
     n_total += n_anchor;
   }
-  c->rep_first[R] = (uint32_t)n_total;
   c->n_part = n_total;
   c->stats.n_partitions = n_total;
   return MJ_OK;
@@ -709,6 +717,16 @@ int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s
                              c->sort_tmp.p, c->rk_of.as<uint32_t>(), c->rk_hi.as<uint32_t>(),
                              by_len ? c->rk_short_rank.as<uint32_t>() : nullptr, c->dev_flags.as<unsigned int>() + 2,
                              c->dev_flags.as<unsigned long long>() + 2, &c->rk_alt, s);
+}
+
+// Whether the records let expect `from` raw pairs or more.
+int many_pairs(mj_ctx* c, uint64_t from, bool* many, cudaStream_t s) {
+  MJ_TRY(c->rk_table.reserve((size_t)likely_pairs_slots(c->n_part) * 4, s));
+  MJ_TRY(launch_likely_pairs(c->recs.as<PRec>(), c->n_part, c->d.K, c->rk_table.as<uint32_t>(),
+                             c->rk_cnt.as<unsigned long long>() + 7, s));
+  MJ_TRY(readback(c, c->rk_cnt.as<unsigned long long>() + 7, 8, s));
+  *many = likely_pairs(c->n_part, c->h_small[0]) >= from;
+  return MJ_OK;
 }
 
 // a5-a7 by strings (after partition and string_ranks): the candidates counted,
@@ -1396,7 +1414,7 @@ void mj_destroy(mj_ctx* c) {
                  &c->recs, &c->keys, &c->keys_alt, &c->idx, &c->idx_alt, &c->sort_tmp, &c->srec, &c->pair_count, &c->pair_off, &c->pairs, &c->pairs_alt,
                  &c->uflags, &c->uoffs, &c->cand_i, &c->cand_j, &c->pairbm, &c->planes, &c->ed, &c->out_t, &c->geo, &c->strgeo, &c->codes,
                  &c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi, &c->rk_first, &c->rk_delta,
-                 &c->rk_scan, &c->rk_short_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
+                 &c->rk_scan, &c->rk_short_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->rk_table, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
                  &c->out_i, &c->out_j, &c->out_ed, &c->in_bytes, &c->in_offsets, &c->branges,
                  &c->band, &c->band_part, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
                  &c->franges, &c->fnext, &c->fcnt, &c->ed_first};
@@ -1799,8 +1817,11 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
   MJ_TRY(partition(c, d_bytes, d_offsets, n, nullptr, p->K, s));
   c->have_part = true;
   at[2] = mark(c, s);
-  const bool strings = c->by_strings && string_pairs_fit(c->rk_widest);
+  bool strings = c->by_strings && string_pairs_fit(c->rk_widest);
+  const uint64_t strings_from = strings ? string_pairs_from(n, c->rk_widest, c->sms) : 0;
+  if (strings_from) MJ_TRY(many_pairs(c, strings_from, &strings, s));
   if (strings) {
+    if (strings_from && p->repeats == 1) MJ_TRY(string_first(c, d_offsets, n, 0, s));
     MJ_TRY(string_candidates(c, d_offsets, n, s));
   } else {
     MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,

@@ -250,6 +250,15 @@ struct PairArgs {
   uint2* out = nullptr;
 };
 bool string_pairs_fit(uint32_t widest);   // a string's bitmap fits in shared memory
+// Raw pairs from which a join whose widest window holds `widest` ranks goes
+// string by string (0: always), and their estimate from one record in
+// likely_pairs_step(n_rec): *total sampled pairs, of which likely_pairs makes the
+// number.  table: likely_pairs_slots(n_rec) words of scratch.
+uint64_t string_pairs_from(uint32_t n, uint32_t widest, int sms);
+uint32_t likely_pairs_slots(uint64_t n_rec);
+int launch_likely_pairs(const PRec* recs, uint64_t n_rec, uint32_t K, uint32_t* table, unsigned long long* total,
+                        cudaStream_t s);
+uint64_t likely_pairs(uint64_t n_rec, uint64_t total);
 constexpr size_t kStringPairsSmemMax = 160u << 10;
 int launch_string_pairs(const PairArgs& a, uint32_t widest, cudaStream_t s);
 // *a.sampled += the candidates of about kSampleStrings strings

@@ -64,7 +64,7 @@ __device__ __forceinline__ uint32_t upper_bound_of(const T* __restrict__ a, uint
 // Every entry is a search of its own: filled by the rank that ends a run of
 // lengths, a gap between two lengths is one thread's loop (20,000 reads and one
 // string of 4 M symbols: 50 ms of a join of 108).
-__global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const uint32_t* __restrict__ sid_of, uint32_t n,
+__global__ void __launch_bounds__(256) rank_tables_kernel(const uint32_t* __restrict__ shorts, const uint32_t* __restrict__ sid_of, uint32_t n,
                                    uint32_t K, uint32_t longest, uint32_t* __restrict__ rank_of,
                                    uint32_t* __restrict__ hi, uint32_t* __restrict__ short_rank,
                                    unsigned int* __restrict__ widest, unsigned long long* __restrict__ spans) {
@@ -83,13 +83,31 @@ __global__ void rank_tables_kernel(const uint32_t* __restrict__ shorts, const ui
   if (short_rank)   // longest < 2^32 - 1: a string's length is below the input's size
     for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l <= longest; l += (uint64_t)gridDim.x * blockDim.x)
       short_rank[l] = l ? upper_bound_of(shorts, 0, n, (uint32_t)l - 1u) : 0u;
+  // one block's three results at a time: with a warp's they were 94,000 updates
+  // of three words for 1,000,000 strings, 75 us
+  __shared__ uint32_t s_w[8], s_len[8];
+  __shared__ unsigned long long s_sum[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   w = __reduce_max_sync(0xffffffffu, w);
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
   len = __reduce_max_sync(0xffffffffu, len);
-  if ((threadIdx.x & 31) == 0 && w) {
-    atomicMax(widest, w);
-    atomicMax(widest + 1, len);
-    atomicAdd(spans, sum);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if (lane == 0) {
+    s_w[wid] = w;
+    s_len[wid] = len;
+    s_sum[wid] = sum;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) {
+      w = max(w, s_w[k]);
+      len = max(len, s_len[k]);
+      sum += s_sum[k];
+    }
+    if (w) {
+      atomicMax(widest, w);
+      atomicMax(widest + 1, len);
+      atomicAdd(spans, sum);
+    }
   }
 }
 
@@ -239,6 +257,26 @@ __device__ __forceinline__ uint32_t gallop_down(const uint64_t* __restrict__ a, 
     else hi = mid;
   }
   return hi;
+}
+
+// Pairs of sampled records (every step-th) of one partition, position bucket and
+// length bucket of K + 1, a third or so of those that pass the filters, counted
+// as they meet in a table by hash: a record pairs with those that were counted
+// in its slot before.
+__global__ void likely_pairs_kernel(const PRec* __restrict__ recs, uint64_t n_rec, uint32_t step, uint32_t K,
+                                    uint32_t* __restrict__ table, uint32_t mask,
+                                    unsigned long long* __restrict__ total) {
+  unsigned long long sum = 0;
+  for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * step; t < n_rec;
+       t += (uint64_t)gridDim.x * blockDim.x * step) {
+    const PRec r = load_rec(recs, t);
+    const uint64_t g = mix64(mix64(r.h61 ^ ((uint64_t)r.len * 0x9e3779b97f4a7c15ull)) ^
+                             ((uint64_t)(r.pos / (K + 1)) << 32 | r.slen / (K + 1)));
+    sum += atomicAdd(table + ((uint32_t)g & mask), 1u);
+  }
+  __syncwarp();
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(total, sum);
 }
 
 // The windows of every record (see the file comment), written at the record's
@@ -732,39 +770,46 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? 26 : 1) string_pairs_
         if (waiting > kPassed - 32) append();
       }
     };
-    // a warp looks at 128 words at a time and takes the 16 words of the groups
-    // that hold bits, 32 half-words to a step
-    for (uint32_t w0 = 128 * wid; w0 < words; w0 += 128 * kWarps) {
-      const uint32_t wl = w0 + 4 * lane;
-      const uint4 four = wl < a.bm_words ? *reinterpret_cast<const uint4*>(bm + wl) : make_uint4(0u, 0u, 0u, 0u);
-      uint32_t some = __ballot_sync(0xffffffffu, (four.x | four.y | four.z | four.w) != 0);
-      while (some) {
-        const uint32_t group = (uint32_t)(__ffs(some) - 1) >> 2;
-        some &= ~(15u << (4 * group));
-        const uint32_t h = 2 * (w0 + 16 * group) + lane;
-        const uint32_t both = h < 2 * words ? bm[h >> 1] : 0u;
-        uint32_t bits = (both >> (16 * (h & 1))) & 0xffffu;
-        __syncwarp();
-        if (both && !(h & 1)) bm[h >> 1] = 0;
-        const uint32_t c = __popc(bits);
-        cand += c;
-        if (SAMPLE) continue;   // nothing is listed: the stack stays empty
-        uint32_t incl = c;
+    // 16 words from half-word h0 on, 32 half-words to a step
+    auto take = [&](uint32_t h0) {
+      const uint32_t h = h0 + lane;
+      const uint32_t both = h < 2 * words ? bm[h >> 1] : 0u;
+      if (THREADS != 32 && !__any_sync(0xffffffffu, both != 0)) return;
+      uint32_t bits = (both >> (16 * (h & 1))) & 0xffffu;
+      __syncwarp();
+      if (both && !(h & 1)) bm[h >> 1] = 0;
+      const uint32_t c = __popc(bits);
+      cand += c;
+      if (SAMPLE) return;   // nothing is listed: the stack stays empty
+      uint32_t incl = c;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t z = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += z;
-        }
-        uint32_t at = depth + incl - c;
-        depth += __shfl_sync(0xffffffffu, incl, 31);
-        while (bits) {
-          stack[at++] = (Slot)(16u * h + (__ffs(bits) - 1));
-          bits &= bits - 1;
-        }
-        __syncwarp();
-        while (depth >= 64) test(std::integral_constant<int, 2>(), 64u);
-        __syncwarp();   // the popped entries are read before the next step's pushes
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t z = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += z;
       }
+      uint32_t at = depth + incl - c;
+      depth += __shfl_sync(0xffffffffu, incl, 31);
+      while (bits) {
+        stack[at++] = (Slot)(16u * h + (__ffs(bits) - 1));
+        bits &= bits - 1;
+      }
+      __syncwarp();
+      while (depth >= 64) test(std::integral_constant<int, 2>(), 64u);
+      __syncwarp();   // the popped entries are read before the next step's pushes
+    };
+    if (THREADS == 32) {   // a warp looks at 128 words at a time and takes the groups that hold bits
+      for (uint32_t w0 = 0; w0 < words; w0 += 128) {
+        const uint32_t wl = w0 + 4 * lane;
+        const uint4 four = wl < a.bm_words ? *reinterpret_cast<const uint4*>(bm + wl) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t some = __ballot_sync(0xffffffffu, (four.x | four.y | four.z | four.w) != 0);
+        while (some) {
+          const uint32_t group = (uint32_t)(__ffs(some) - 1) >> 2;
+          some &= ~(15u << (4 * group));
+          take(2 * (w0 + 16 * group));
+        }
+      }
+    } else {   // wide windows come here with many candidates only: the warps take 16 words in turn
+      for (uint32_t h0 = 32 * wid; h0 < 2 * words; h0 += 32 * kWarps) take(h0);
     }
     if (!SAMPLE) {
       if (depth) test(std::integral_constant<int, 2>(), depth);
@@ -975,6 +1020,48 @@ int launch_pair_bounds(const uint32_t* pi, const uint32_t* pj, const uint32_t* p
 
 bool string_pairs_fit(uint32_t widest) {
   return sizeof(PairShared<128, true>) + (size_t)widest / 8 <= kStringPairsSmemMax;
+}
+
+// Windows of 2^16 ranks and more take a CTA each with up to 142 KB of bitmap, so
+// few are resident, and a string costs 6 us of its CTA's place however few
+// candidates it has (72,000 / 200,000 / 500,000 / 1,000,000 reads of one length:
+// 0.46 / 1.43 / 7.8 / 39 ms for 0.36 / 1.0 / 2.5 / 5.0 M raw pairs).  The general
+// path takes 85-130 ps a raw pair of such inputs, and 100-300 ps to verify the
+// candidate that it may be.  So strings pay from a raw pair per 0.25 ns of that
+// on.  (Whole joins by strings, against this choice, the general path: 0.99 /
+// 0.70, 2.21 / 0.94, 9.1 / 1.47, 41.3 / 2.39 ms; 450,000 text-like strings, 1.8 G
+// raw pairs, go by strings: 44 ms, some 530 by the general path.)
+uint64_t string_pairs_from(uint32_t n, uint32_t widest, int sms) {
+  if (widest < 65536) return 0;
+  const size_t smem = sizeof(PairShared<128, true>) + (size_t)widest / 8 + 1024;
+  const uint64_t resident = std::min<uint64_t>(8, std::max<uint64_t>(1, (227u << 10) / smem));
+  return (uint64_t)n * 24000 / ((uint64_t)sms * resident);
+}
+
+// About 2^17 records are sampled, whose table stays in L2 (2^20 of 5 M: 176 us).
+static uint32_t likely_pairs_step(uint64_t n_rec) { return (uint32_t)std::max<uint64_t>(1, n_rec >> 17); }
+
+uint32_t likely_pairs_slots(uint64_t n_rec) {   // 16 slots and more per sampled record
+  uint32_t slots = 1024;
+  while (slots < (1u << 22) && slots < 16 * (n_rec / likely_pairs_step(n_rec))) slots <<= 1;
+  return slots;
+}
+
+int launch_likely_pairs(const PRec* recs, uint64_t n_rec, uint32_t K, uint32_t* table, unsigned long long* total,
+                        cudaStream_t s) {
+  const uint32_t slots = likely_pairs_slots(n_rec), step = likely_pairs_step(n_rec);
+  MJ_CUDA_TRY(cudaMemsetAsync(table, 0, (size_t)slots * 4, s));
+  MJ_CUDA_TRY(cudaMemsetAsync(total, 0, sizeof(*total), s));
+  if (!n_rec) return MJ_OK;
+  likely_pairs_kernel<<<grid_for(n_rec / step + 1), 256, 0, s>>>(recs, n_rec, step, K, table, slots - 1, total);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+uint64_t likely_pairs(uint64_t n_rec, uint64_t total) {
+  const double step = likely_pairs_step(n_rec), m = (double)n_rec / step;
+  const double met = m * m / 2 / likely_pairs_slots(n_rec);   // different records in one slot
+  return (uint64_t)(std::max(0.0, (double)total - met) * step * step);
 }
 
 int launch_string_pairs(const PairArgs& a, uint32_t widest, cudaStream_t s) {

@@ -132,7 +132,7 @@ constexpr int kCalibrationRuns = 3;   // timed joins per mode in mj_band_calibra
 // and that the stage branches on: buffers, sizes, the kernel plan, whether the
 // order's cells are wanted, the shape of the bounds' signatures.
 struct GraphKey {
-  uint64_t word[28];
+  uint64_t word[27];
   SigShape shape;
 };
 
@@ -174,11 +174,21 @@ struct mj_ctx {
   // joins by strings) those the lower bounds leave, in any order
   uint64_t n_list = 0;
   bool list_bounded = false;      // made under the lower bounds of mj_pairs.cu
-  // plain joins by strings (mj_pairs.cu): lengths (as shorts) and ids by rank, ranks by
-  // id, windows by rank, first records by string, sorted records, windows,
-  // signatures, counters
-  Buf rk_len, rk_len_alt, rk_sid, rk_sid_alt, rk_of, rk_hi, rk_first, rk_delta, rk_scan, rk_short_rank;
-  Buf rk_a, rk_b, rk_skr, rk_win, rk_sig1, rk_sig2, rk_cnt, rk_list, rk_table;
+  // plain joins by strings (mj_pairs.cu), each group of arrays one allocation:
+  // strs (by the strings: lengths as shorts and ids by rank, ranks by id, windows
+  // by rank, first ranks by length, first records by string, counters) and, by
+  // the records, recs_by_rank (sort keys and indices, visit words, sort keys with
+  // ranks, windows, places)
+  Buf strs, recs_by_rank, rk_list, rk_table;
+  uint32_t *rk_len = nullptr, *rk_len_alt = nullptr, *rk_sid = nullptr, *rk_sid_alt = nullptr, *rk_of = nullptr,
+           *rk_hi = nullptr, *rk_short_rank = nullptr, *rk_first = nullptr, *rk_delta = nullptr, *rk_scan = nullptr;
+  unsigned long long* rk_cnt = nullptr;
+  uint4 *rk_a = nullptr, *rk_win = nullptr;
+  uint2* rk_b = nullptr;
+  uint64_t* rk_skr = nullptr;
+  uint32_t *rk_keys = nullptr, *rk_keys_alt = nullptr, *rk_idx = nullptr, *rk_idx_alt = nullptr;
+  uint8_t* rk_sort_tmp = nullptr;
+  Buf sigs;                       // signatures of both levels (signature_buffers)
   Buf rejected;                   // listed pairs beyond their lower bounds (one byte each)
   bool by_strings = false;        // this call builds the rank tables
   bool rk_alt = false;            // rk_len_alt / rk_sid_alt hold the sorted strings
@@ -416,7 +426,7 @@ uint64_t key_base_for(uint64_t seed) {
 int string_first(mj_ctx* c, const int64_t* d_offsets, uint32_t n, uint32_t k, cudaStream_t s) {
   return launch_string_first(d_offsets, n, c->stats.n_bytes, c->bitmap.as<uint32_t>(), c->tile_off.as<uint32_t>(),
                              c->rep_first[k + 1] - c->rep_first[k], c->rep_first[k],
-                             c->rk_first.as<uint32_t>() + (uint64_t)k * (n + 1), s);
+                             c->rk_first + (uint64_t)k * (n + 1), s);
 }
 
 // a2-a4 (after derive): partition records in c->recs (n_part of them).
@@ -693,38 +703,65 @@ bool bounds_reach(uint64_t N, uint32_t sigma, uint32_t K) {
 }
 
 constexpr uint64_t kBoundsFrom = 1u << 15;    // candidates from which a join by strings may use the lower bounds
-constexpr uint64_t kListAll = 1u << 20;        // pairs of ranks up to which there is room for all of them
+constexpr uint64_t kListAll = 1u << 20;        // ranks in the windows from which the sample sizes the lists
+constexpr uint64_t kListFirst = 96u << 10;     // pairs of a list under 1 MB, above which cudaMalloc takes 37 us instead of 2
 constexpr int kSampledAt = 64;                 // word of the staging memory for the sample's count
 constexpr uint64_t kShortRankMax = 1u << 22;   // longest string up to which ranks are found by length in a table
+
+// Arrays of one allocation, at multiples of 256 bytes: a cudaMalloc for each was
+// a third of a context's first join of 1,000 short reads.
+struct Carver {
+  uint8_t* base;
+  size_t used = 0;
+  template <class T>
+  void take(T** p, uint64_t count) {
+    *p = base && count ? reinterpret_cast<T*>(base + used) : nullptr;
+    used += (count * sizeof(T) + 255) / 256 * 256;
+  }
+};
+template <class F>
+int carve(Buf& buf, cudaStream_t s, F layout) {
+  Carver sizes{nullptr};
+  layout(sizes);
+  MJ_TRY(buf.reserve(sizes.used, s));
+  Carver at{buf.as<uint8_t>()};
+  layout(at);
+  return MJ_OK;
+}
+
+// Room for the signatures of n strings, both levels in one allocation.
+int signature_buffers(mj_ctx* c, uint32_t n, uint4** sig1, uint32_t** sig2, cudaStream_t s) {
+  return carve(c->sigs, s, [&](Carver& at) {
+    at.take(sig1, sig1_bytes(n) / sizeof(uint4));
+    at.take(sig2, sig2_bytes(n) / sizeof(uint32_t));
+  });
+}
 
 // Rank tables of a plain join by strings (before its partition step, whose
 // readback also returns the widest window).
 int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s) {
-  const size_t b = (size_t)n * 4 + 16;
-  for (Buf* x : {&c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi}) MJ_TRY(x->reserve(b, s));
-  MJ_TRY(c->rk_cnt.reserve(64, s));
-  MJ_CUDA_TRY(cudaMemsetAsync(c->rk_cnt.p, 0, 64, s));
+  const bool by_len = c->d.N <= kShortRankMax;
+  MJ_TRY(carve(c->strs, s, [&](Carver& at) {
+    for (uint32_t** x : {&c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi}) at.take(x, n);
+    at.take(&c->rk_short_rank, by_len ? c->d.N + 1 : 0);
+    at.take(&c->rk_first, (uint64_t)c->d.repeats * ((uint64_t)n + 1));
+    at.take(&c->rk_cnt, 8);
+    at.take(&c->rk_sort_tmp, radix_temp_bytes(n));
+  }));
+  MJ_CUDA_TRY(cudaMemsetAsync(c->rk_cnt, 0, 64, s));
   MJ_TRY(c->dev_flags.reserve(64, s));
   MJ_CUDA_TRY(cudaMemsetAsync(c->dev_flags.p, 0, 64, s));
-  MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(n), s));
-  const bool by_len = c->d.N <= kShortRankMax;
-  if (by_len) {
-    MJ_TRY(c->rk_short_rank.reserve(((size_t)c->d.N + 1) * 4, s));
-  }
-  MJ_TRY(c->rk_first.reserve((size_t)c->d.repeats * ((size_t)n + 1) * 4, s));
-  return launch_string_ranks(d_offsets, n, c->d.K, (uint32_t)c->d.N, bits_for(c->d.N), c->rk_len.as<uint32_t>(),
-                             c->rk_len_alt.as<uint32_t>(), c->rk_sid.as<uint32_t>(), c->rk_sid_alt.as<uint32_t>(),
-                             c->sort_tmp.p, c->rk_of.as<uint32_t>(), c->rk_hi.as<uint32_t>(),
-                             by_len ? c->rk_short_rank.as<uint32_t>() : nullptr, c->dev_flags.as<unsigned int>() + 2,
-                             c->dev_flags.as<unsigned long long>() + 2, &c->rk_alt, s);
+  return launch_string_ranks(d_offsets, n, c->d.K, (uint32_t)c->d.N, bits_for(c->d.N), c->rk_len, c->rk_len_alt,
+                             c->rk_sid, c->rk_sid_alt, c->rk_sort_tmp, c->rk_of, c->rk_hi, c->rk_short_rank,
+                             c->dev_flags.as<unsigned int>() + 2, c->dev_flags.as<unsigned long long>() + 2, &c->rk_alt,
+                             s);
 }
 
 // Whether the records let expect `from` raw pairs or more.
 int many_pairs(mj_ctx* c, uint64_t from, bool* many, cudaStream_t s) {
   MJ_TRY(c->rk_table.reserve((size_t)likely_pairs_slots(c->n_part) * 4, s));
-  MJ_TRY(launch_likely_pairs(c->recs.as<PRec>(), c->n_part, c->d.K, c->rk_table.as<uint32_t>(),
-                             c->rk_cnt.as<unsigned long long>() + 7, s));
-  MJ_TRY(readback(c, c->rk_cnt.as<unsigned long long>() + 7, 8, s));
+  MJ_TRY(launch_likely_pairs(c->recs.as<PRec>(), c->n_part, c->d.K, c->rk_table.as<uint32_t>(), c->rk_cnt + 7, s));
+  MJ_TRY(readback(c, c->rk_cnt + 7, 8, s));
   *many = likely_pairs(c->n_part, c->h_small[0]) >= from;
   return MJ_OK;
 }
@@ -748,55 +785,51 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   const int pb_bits = bits_for(d.N / W);
   // hash bits: two more than the records' logarithm, in whole radix passes
   const int key_bits = std::min(32, (pb_bits + std::max(14, bits_for(nr)) + 2 + 7) / 8 * 8);
-  const uint32_t* sid_of = c->rk_alt ? c->rk_sid_alt.as<uint32_t>() : c->rk_sid.as<uint32_t>();
-  const uint32_t* shorts = c->rk_alt ? c->rk_len_alt.as<uint32_t>() : c->rk_len.as<uint32_t>();
-  const uint32_t* rank_of = c->rk_of.as<uint32_t>();
-  unsigned long long* cnt = c->rk_cnt.as<unsigned long long>();   // 1 sampled, 2 listed, 3-5 totals, 6 listed after the second bound
-  MJ_TRY(c->keys.reserve((size_t)nr * 4, s));
-  MJ_TRY(c->keys_alt.reserve((size_t)nr * 4, s));
-  c->geo_valid = false;   // c->idx is reused by the record sort
-  MJ_TRY(c->idx.reserve((size_t)nr * 4, s));
-  MJ_TRY(c->idx_alt.reserve((size_t)nr * 4, s));
+  const uint32_t* sid_of = c->rk_alt ? c->rk_sid_alt : c->rk_sid;
+  const uint32_t* shorts = c->rk_alt ? c->rk_len_alt : c->rk_len;
+  const uint32_t* rank_of = c->rk_of;
+  unsigned long long* cnt = c->rk_cnt;   // 1 sampled, 2 listed, 3-5 totals, 6 listed after the second bound
   MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(nr), s));
-  MJ_TRY(c->rk_delta.reserve((size_t)d.repeats * ((size_t)n + 1) * 4, s));
-  MJ_TRY(c->rk_scan.reserve((size_t)n * 4 + 16, s));
   MJ_TRY(c->scan_tmp.reserve(scan_temp_bytes(n), s));
-  MJ_TRY(c->rk_a.reserve((size_t)nr * 16, s));
   const int rb = visit_rank_bits(c->rk_longest, n);
-  if (!rb) MJ_TRY(c->rk_b.reserve((size_t)nr * 8, s));
-  MJ_TRY(c->rk_skr.reserve((size_t)nr * 8, s));
-  MJ_TRY(c->rk_win.reserve((size_t)nr * 32, s));
-  MJ_TRY(c->rk_sig1.reserve(sig1_bytes(n), s));
-  MJ_TRY(c->rk_sig2.reserve(sig2_bytes(n), s));
+  MJ_TRY(carve(c->recs_by_rank, s, [&](Carver& at) {
+    for (uint32_t** x : {&c->rk_keys, &c->rk_keys_alt, &c->rk_idx, &c->rk_idx_alt}) at.take(x, nr);
+    at.take(&c->rk_a, nr);
+    at.take(&c->rk_b, rb ? 0 : nr);
+    at.take(&c->rk_skr, nr);
+    at.take(&c->rk_win, 2 * (uint64_t)nr);
+    at.take(&c->rk_delta, (uint64_t)d.repeats * ((uint64_t)n + 1));
+    at.take(&c->rk_scan, n);
+  }));
+  const bool bounds = bounds_reach(d.N, d.sigma, d.K);
+  uint4* sig1 = nullptr;
+  uint32_t* sig2 = nullptr;
+  if (bounds) MJ_TRY(signature_buffers(c, n, &sig1, &sig2, s));
   tstart(c, 2, s);
-  MJ_TRY(launch_rank_order(c->rk_first.as<uint32_t>(), sid_of, rank_of, n, d.repeats, c->rk_scan.as<uint32_t>(),
-                           c->rk_delta.as<uint32_t>(), c->scan_tmp.p, s));
+  MJ_TRY(launch_rank_order(c->rk_first, sid_of, rank_of, n, d.repeats, c->rk_scan, c->rk_delta, c->scan_tmp.p, s));
   for (uint32_t k = 0; k < d.repeats; ++k)
     MJ_TRY(launch_rank_keys(c->recs.as<PRec>(), c->rep_first[k], c->rep_first[k + 1],
-                            c->rk_delta.as<uint32_t>() + (uint64_t)k * (n + 1), key_bits - pb_bits, pb_bits, W, c->keys.as<uint32_t>(),
-                            c->idx.as<uint32_t>(), s));
+                            c->rk_delta + (uint64_t)k * (n + 1), key_bits - pb_bits, pb_bits, W, c->rk_keys, c->rk_idx,
+                            s));
   bool alt = false;
-  MJ_TRY(radix_sort_u32(c->keys.as<uint32_t>(), c->keys_alt.as<uint32_t>(), c->idx.as<uint32_t>(),
-                        c->idx_alt.as<uint32_t>(), nr, 0, key_bits, c->sort_tmp.p, &alt, s));
-  const RankTables rt{c->rk_hi.as<uint32_t>(), shorts, d.N <= kShortRankMax ? c->rk_short_rank.as<uint32_t>() : nullptr,
-                      (uint32_t)d.N, n};
-  MJ_TRY(launch_rank_windows(alt ? c->idx_alt.as<uint32_t>() : c->idx.as<uint32_t>(),
-                             alt ? c->keys_alt.as<uint32_t>() : c->keys.as<uint32_t>(), nr, c->recs.as<PRec>(), rank_of,
-                             rt, d.K, W, pb_bits, rb, c->rk_a.as<uint4>(), c->rk_b.as<uint2>(),
-                             c->rk_skr.as<uint64_t>(), c->rk_win.as<uint4>(), s));
+  MJ_TRY(radix_sort_u32(c->rk_keys, c->rk_keys_alt, c->rk_idx, c->rk_idx_alt, nr, 0, key_bits, c->sort_tmp.p, &alt, s));
+  const RankTables rt{c->rk_hi, shorts, c->rk_short_rank, (uint32_t)d.N, n};
+  MJ_TRY(launch_rank_windows(alt ? c->rk_idx_alt : c->rk_idx, alt ? c->rk_keys_alt : c->rk_keys, nr,
+                             c->recs.as<PRec>(), rank_of, rt, d.K, W, pb_bits, rb, c->rk_a, c->rk_b, c->rk_skr,
+                             c->rk_win, s));
   tstop(c, 2, s);
   tstart(c, 4, s);
   PairArgs a;
   a.recs = c->recs.as<PRec>();
-  a.first = c->rk_first.as<uint32_t>();
-  a.win = c->rk_win.as<uint4>();
-  a.A = c->rk_a.as<uint4>();
-  a.B = c->rk_b.as<uint2>();
+  a.first = c->rk_first;
+  a.win = c->rk_win;
+  a.A = c->rk_a;
+  a.B = c->rk_b;
   a.sid_of = sid_of;
   a.shorts = shorts;
   a.longest = (uint32_t)d.N;
-  a.hi = c->rk_hi.as<uint32_t>();
-  a.sig1 = c->rk_sig1.as<uint4>();
+  a.hi = c->rk_hi;
+  a.sig1 = sig1;
   a.sampled = cnt + 1;
   a.n = n;
   a.reps = d.repeats;
@@ -809,17 +842,17 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   // less while all candidates are in flight at once).  They are used from one
   // candidate per 96 bytes on, estimated from a sample of the strings, where
   // they can exceed K at all.
-  const bool bounds = bounds_reach(d.N, d.sigma, d.K);
   const SigShape g = signature_shape(d.sigma, c->code_counts);
   const uint64_t stride = std::max<uint32_t>(1, n / kSampleStrings);
   const uint64_t min_sampled = bounds ? std::max<uint64_t>(c->stats.n_bytes / 96, kBoundsFrom) / stride : ~0ull;
   a.min_sampled = min_sampled;
   a.q1 = g.q1;
-  // The lists' sizes: all the windows' ranks where those are few, else the
-  // candidates that the sample lets expect (a copy that the host waits for while
-  // the signatures are made) and a quarter more.  Under the bounds most
-  // candidates are unrelated, and no more than 2^28, or one per input byte, are
-  // expected to pass the first, 2^24 or one per 8 bytes the second.
+  // The lists' sizes: a context's first joins of few strings make room for
+  // kListFirst pairs; where the windows hold many ranks, the candidates that the
+  // sample lets expect (a copy that the host waits for while the signatures are
+  // made) and a quarter more.  Under the bounds most candidates are unrelated,
+  // and no more than 2^28, or one per input byte, are expected to pass the first,
+  // 2^24 or one per 8 bytes the second.  Lists that have grown stay as long.
   const bool many = c->rk_spans > kListAll;
   if (bounds || many) MJ_TRY(launch_string_sample(a, c->rk_widest, s));
   if (many) {
@@ -827,21 +860,21 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
     MJ_CUDA_TRY(cudaEventRecord(c->ev[0], s));
   }
   if (bounds)
-    MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_sampled,
-                             c->rk_sig1.as<uint4>(), c->rk_sig2.as<uint32_t>(), s));
-  uint64_t cap1 = c->rk_spans, cap2;
+    MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, sid_of, n, g, cnt + 1, min_sampled, sig1,
+                             sig2, s));
+  uint64_t cap1 = std::min(c->rk_spans, kListFirst), cap2 = cap1;
   if (many) {
     MJ_CUDA_TRY(cudaEventSynchronize(c->ev[0]));
     const uint64_t sampled = c->h_small[kSampledAt], expected = sampled * stride;
-    cap1 = std::min(cap1, expected + expected / 4 + (1u << 16));
+    cap1 = std::min(c->rk_spans, expected + expected / 4 + (1u << 16));
     if (sampled > min_sampled) cap1 = std::min(cap1, std::max<uint64_t>(c->stats.n_bytes, 1u << 28));
     cap2 = sampled > min_sampled ? std::min(cap1, std::max<uint64_t>(c->stats.n_bytes / 8, 1u << 24)) : cap1;
-  } else {
-    cap2 = cap1;
   }
+  cap1 = std::max<uint64_t>(cap1, c->rk_list.bytes / 8);
+  cap2 = std::max<uint64_t>(cap2, std::min(c->cand_i.bytes, c->cand_j.bytes) / 4);
   ListArgs l;
   l.in_count = a.out_count;
-  l.sig2 = c->rk_sig2.as<uint4>();
+  l.sig2 = reinterpret_cast<const uint4*>(sig2);
   l.sid_of = sid_of;
   l.shorts = shorts;
   l.longest = (uint32_t)d.N;
@@ -855,8 +888,8 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   bool first = true;
   for (int tries = 0;; ++tries) {
     if (first) MJ_TRY(c->rk_list.reserve(cap1 * 8, s));
-    MJ_TRY(c->cand_i.reserve(cap2 * 4 + 16, s));
-    MJ_TRY(c->cand_j.reserve(cap2 * 4 + 16, s));
+    MJ_TRY(c->cand_i.reserve(cap2 * 4, s));
+    MJ_TRY(c->cand_j.reserve(cap2 * 4, s));
     a.cap = l.in_cap = cap1;
     a.out = c->rk_list.as<uint2>();
     l.in = a.out;
@@ -1022,8 +1055,9 @@ int plan_lanes(uint32_t kernel, uint32_t lanes, uint32_t K) {
 }
 
 int bounds_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
-  MJ_TRY(c->rk_sig1.reserve(sig1_bytes((uint32_t)c->stats.n_strings), s));
-  MJ_TRY(c->rk_sig2.reserve(sig2_bytes((uint32_t)c->stats.n_strings), s));
+  uint4* sig1;
+  uint32_t* sig2;
+  MJ_TRY(signature_buffers(c, (uint32_t)c->stats.n_strings, &sig1, &sig2, s));
   return c->rejected.reserve(m, s);
 }
 
@@ -1031,12 +1065,14 @@ int bounds_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
 // needs the input's rank codes and bounds_buffers.
 int pair_bounds(mj_ctx* c, const int64_t* d_offsets, const uint32_t* ci, const uint32_t* cj, const uint32_t* pk,
                 uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
-  if (!c->codes_ready || !c->rk_sig1.p || !c->rk_sig2.p || !c->rejected.p) return MJ_ERR_STATE;
+  if (!c->codes_ready || !c->sigs.p || !c->rejected.p) return MJ_ERR_STATE;
   const uint32_t n = (uint32_t)c->stats.n_strings;
   const SigShape g = signature_shape(c->d.sigma, c->code_counts);
-  MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, nullptr, n, g, nullptr, 0, c->rk_sig1.as<uint4>(),
-                           c->rk_sig2.as<uint32_t>(), s));
-  return launch_pair_bounds(ci, cj, pk, K, m, n, g, c->rk_sig1.as<uint4>(), c->rk_sig2.as<uint4>(),
+  uint4* sig1;
+  uint32_t* sig2;
+  MJ_TRY(signature_buffers(c, n, &sig1, &sig2, s));   // reserved before (bounds_buffers): nothing is allocated here
+  MJ_TRY(launch_signatures(c->codes.as<uint8_t>(), d_offsets, nullptr, n, g, nullptr, 0, sig1, sig2, s));
+  return launch_pair_bounds(ci, cj, pk, K, m, n, g, sig1, reinterpret_cast<const uint4*>(sig2),
                             c->rejected.as<uint8_t>(), ed, s);
 }
 
@@ -1131,7 +1167,7 @@ int verify_ordered_graph(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_off
        c->planes_pw, c->planes_gw, c->d.bits, c->d.sigma, plan, (uint64_t)c->small.p, (uint64_t)c->idx.p,
        (uint64_t)c->branges.p, (uint64_t)c->dev_flags.p, c->out_collect ? (uint64_t)c->out_t.p : 0,
        (uint64_t)c->geo.p, c->stats.n_bytes, c->stats.n_strings, (uint64_t)c->codes.p, (uint64_t)c->strgeo.p,
-       (uint64_t)c->rk_sig1.p, (uint64_t)c->rk_sig2.p, (uint64_t)c->rejected.p, bounds ? 1ull : 0ull,
+       (uint64_t)c->sigs.p, (uint64_t)c->rejected.p, bounds ? 1ull : 0ull,
        c->want_cells ? 1ull : 0ull},
       bounds ? signature_shape(c->d.sigma, c->code_counts) : SigShape{}};
   if (c->graph_exec && memcmp(&key, &c->graph_key, sizeof(key)) == 0) {
@@ -1413,8 +1449,7 @@ void mj_destroy(mj_ctx* c) {
                  &c->tile_first,
                  &c->recs, &c->keys, &c->keys_alt, &c->idx, &c->idx_alt, &c->sort_tmp, &c->srec, &c->pair_count, &c->pair_off, &c->pairs, &c->pairs_alt,
                  &c->uflags, &c->uoffs, &c->cand_i, &c->cand_j, &c->pairbm, &c->planes, &c->ed, &c->out_t, &c->geo, &c->strgeo, &c->codes,
-                 &c->rk_len, &c->rk_len_alt, &c->rk_sid, &c->rk_sid_alt, &c->rk_of, &c->rk_hi, &c->rk_first, &c->rk_delta,
-                 &c->rk_scan, &c->rk_short_rank, &c->rk_a, &c->rk_b, &c->rk_skr, &c->rk_win, &c->rk_list, &c->rk_table, &c->cand_recs, &c->rejected, &c->rk_sig1, &c->rk_sig2, &c->rk_cnt,
+                 &c->strs, &c->recs_by_rank, &c->rk_list, &c->rk_table, &c->cand_recs, &c->rejected, &c->sigs,
                  &c->out_i, &c->out_j, &c->out_ed, &c->in_bytes, &c->in_offsets, &c->branges,
                  &c->band, &c->band_part, &c->feat_x, &c->mult, &c->run_start, &c->parts, &c->yhat, &c->kband, &c->lvals,
                  &c->franges, &c->fnext, &c->fcnt, &c->ed_first};

@@ -31,16 +31,35 @@ def test_lists_that_the_sample_makes_too_short():
         with mj.Context(0) as ctx:
             ref = ctx.join(data, off, mj.params(K, T=K, flags=mj.MJ_FLAG_DEDUP_SORT))
             want = ctx.stats()
-            assert want["n_candidates"] >= (N // 2) * (N // 2 - 1) // 2
-            for _ in range(2):
+        assert want["n_candidates"] >= (N // 2) * (N // 2 - 1) // 2
+        with mj.Context(0) as ctx:
+            for again in (False, True):   # lists that have grown stay as long
                 got = ctx.join(data, off, mj.params(K, T=K))
                 have = ctx.stats()
                 for x, y in zip(ref, got):
                     assert np.array_equal(x.cpu().numpy(), y.cpu().numpy())
                 for key in ("n_raw_pairs", "n_candidates", "n_output", "band_cells"):
                     assert want[key] == have[key], key
-            launches[seen] = have["n_launches"]
-    assert launches[False] == launches[True] + 2   # the pair kernel and the list kernel once more
+                launches[seen, again] = have["n_launches"]
+    assert launches[False, False] == launches[True, False] + 2   # the pair kernel and the list kernel once more
+    assert launches[False, True] == launches[True, True] == launches[True, False]
+
+
+def test_more_pairs_than_a_first_list_holds():
+    """700 copies of one string: windows of few ranks, but more pairs than the lists
+    of a context's first joins hold."""
+    import paper_1810_08833_gb300 as mj
+    rng = np.random.Generator(np.random.PCG64(6))
+    root = synth.DNA[rng.integers(0, 4, size=L)].tobytes()
+    s = synth.from_strings([root] * 700 + [root[:-1]] * 40, K=K, T=K)
+    data, off = to_device(s)
+    with mj.Context(0) as ctx:
+        ref = ctx.join(data, off, mj.params(K, T=K, flags=mj.MJ_FLAG_DEDUP_SORT))
+        assert ref[0].shape[0] == 740 * 739 // 2
+    with mj.Context(0) as ctx:
+        got = ctx.join(data, off, mj.params(K, T=K))
+    for x, y in zip(ref, got):
+        assert np.array_equal(x.cpu().numpy(), y.cpu().numpy())
 
 
 def test_only_the_second_list_is_made_again():

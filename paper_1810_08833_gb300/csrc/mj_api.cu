@@ -1935,9 +1935,6 @@ int mj_features_copy(mj_ctx* c, float* d_x, uint32_t* d_ed, uint32_t* d_i, uint3
 }
 
 static int band_buffers(mj_ctx* c, cudaStream_t s) {
-  // the gradient's partial sums too, in the size that no batch exceeds: a
-  // network's first forward and gradient of a few thousand rows 226 -> 114 us
-  MJ_TRY(c->band_part.reserve(band_grad_part_bytes(1ull << 32), s));
   return c->band.reserve(sizeof(float) * (4 * (size_t)kBandParams + 8), s);
 }
 
@@ -1946,6 +1943,10 @@ int mj_band_init(mj_ctx* c, uint64_t seed, uint32_t margin, uint32_t min_multipl
   c->band_enabled = -1;   // a new model is not calibrated
   DeviceGuard g(c->device);
   MJ_TRY(band_buffers(c, nullptr));
+  // a new network is trained: room for its gradients' partial sums, in the size
+  // that no batch exceeds (its first forward and gradient of a few thousand rows
+  // 226 -> 114 us; set weights make it when a gradient asks for it)
+  MJ_TRY(c->band_part.reserve(band_grad_part_bytes(1ull << 32), nullptr));
   std::vector<float> w(kBandParams);
   band_initial_weights(seed, w.data());
   MJ_CUDA_TRY(cudaMemcpy(c->band.p, w.data(), sizeof(float) * kBandParams, cudaMemcpyHostToDevice));

@@ -757,6 +757,13 @@ int string_ranks(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStream_t s
                              s);
 }
 
+// Gives back what only joins by strings hold.
+int release_strings(mj_ctx* c, cudaStream_t s) {
+  MJ_CUDA_TRY(cudaStreamSynchronize(s));
+  for (Buf* x : {&c->strs, &c->recs_by_rank, &c->rk_list, &c->rk_table, &c->sigs}) x->release();
+  return MJ_OK;
+}
+
 // Whether the records let expect `from` raw pairs or more.
 int many_pairs(mj_ctx* c, uint64_t from, bool* many, cudaStream_t s) {
   MJ_TRY(c->rk_table.reserve((size_t)likely_pairs_slots(c->n_part) * 4, s));
@@ -1848,17 +1855,27 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
   // many candidates there are is not known before the records are grouped.
   const uint32_t general = MJ_FLAG_FEATURES | MJ_FLAG_KEY_CHECK | MJ_FLAG_DEDUP_SORT | MJ_FLAG_DEDUP_BITMAP;
   c->by_strings = p->verify_mode == MJ_VERIFY_PLAIN && !(p->flags & general) && p->K > 0 && n > 1;
-  if (c->by_strings) MJ_TRY(string_ranks(c, d_offsets, n, s));
+  // Where device memory is short for it, the general path, which needs less (and
+  // sorts where a bitmap does not fit), takes the join as well.
+  const auto or_general = [&](int st) -> int {
+    if (st != MJ_ERR_OOM) return st;
+    c->by_strings = false;
+    return release_strings(c, s);
+  };
+  if (c->by_strings) MJ_TRY(or_general(string_ranks(c, d_offsets, n, s)));
   MJ_TRY(partition(c, d_bytes, d_offsets, n, nullptr, p->K, s));
   c->have_part = true;
   at[2] = mark(c, s);
   bool strings = c->by_strings && string_pairs_fit(c->rk_widest);
   const uint64_t strings_from = strings ? string_pairs_from(n, c->rk_widest, c->sms) : 0;
-  if (strings_from) MJ_TRY(many_pairs(c, strings_from, &strings, s));
-  if (strings) {
+  if (strings_from) MJ_TRY(or_general(many_pairs(c, strings_from, &strings, s)));
+  if (strings && c->by_strings) {
     if (strings_from && p->repeats == 1) MJ_TRY(string_first(c, d_offsets, n, 0, s));
-    MJ_TRY(string_candidates(c, d_offsets, n, s));
-  } else {
+    MJ_TRY(or_general(string_candidates(c, d_offsets, n, s)));
+  }
+  strings = strings && c->by_strings;
+  if (!strings) {
+    c->cand_on_demand = false;
     MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,
                       p->verify_mode == MJ_VERIFY_LEARNED || (p->flags & MJ_FLAG_FEATURES)));
     c->n_list = c->n_cand;

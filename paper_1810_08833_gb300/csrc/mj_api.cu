@@ -289,6 +289,29 @@ int readback_at(mj_ctx* c, int at, const void* d_src, size_t bytes, cudaStream_t
 
 int readback(mj_ctx* c, const void* d_src, size_t bytes, cudaStream_t s) { return readback_at(c, 0, d_src, bytes, s); }
 
+// The first n words of up to three arrays to the caller's (null: not wanted), on
+// s: by one kernel into memory of the context's device, by copies into any other
+// (another device's, which the kernel may have no access to, or an address that
+// is no multiple of 4).
+int copy_out(mj_ctx* c, uint64_t n, const Buf* const (&from)[3], uint32_t* const (&to)[3], cudaStream_t s) {
+  if (!n) return MJ_OK;
+  bool ours = true;
+  for (const uint32_t* p : to) {
+    if (!p) continue;
+    cudaPointerAttributes at{};
+    const cudaError_t e = cudaPointerGetAttributes(&at, p);
+    if (e != cudaSuccess) cudaGetLastError();
+    ours = ours && e == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == c->device &&
+           ((uintptr_t)p & 3) == 0;
+  }
+  if (ours)
+    return launch_copy_words(from[0]->as<uint32_t>(), from[1]->as<uint32_t>(),
+                             from[2] ? from[2]->as<uint32_t>() : nullptr, n, to[0], to[1], to[2], s);
+  for (int k = 0; k < 3; ++k)
+    if (to[k]) MJ_CUDA_TRY(cudaMemcpyAsync(to[k], from[k]->p, n * 4, cudaMemcpyDeviceToDevice, s));
+  return MJ_OK;
+}
+
 // A section's interval runs from its first start to its last stop in a call.
 // An event at this point of the stream: the last one again when no kernel was
 // launched since (an event costs the host about 1.5 us).
@@ -1584,9 +1607,7 @@ int mj_candidates_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, void* stream) {
     MJ_TRY(rc);
     c->cand_on_demand = false;
   }
-  const size_t n = c->n_cand;
-  if (!n) return MJ_OK;
-  return launch_copy_words(c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(), nullptr, n, d_i, d_j, nullptr, s);
+  return copy_out(c, c->n_cand, {&c->cand_i, &c->cand_j, nullptr}, {d_i, d_j, nullptr}, s);
 }
 
 int mj_set_alphabet(mj_ctx* c, const uint8_t* h_present, uint64_t N) {
@@ -2148,10 +2169,7 @@ int mj_result_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, uint32_t* d_ed, void
   if (!c->have_out) return MJ_ERR_STATE;
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
-  const size_t n = c->n_out;
-  if (!n) return MJ_OK;
-  return launch_copy_words(c->out_i.as<uint32_t>(), c->out_j.as<uint32_t>(), c->out_ed.as<uint32_t>(), n, d_i, d_j,
-                           d_ed, s);
+  return copy_out(c, c->n_out, {&c->out_i, &c->out_j, &c->out_ed}, {d_i, d_j, d_ed}, s);
 }
 
 int mj_join_host(mj_ctx* c, const uint8_t* h_bytes, const int64_t* h_offsets, uint32_t n, const mj_params* p,

@@ -198,13 +198,17 @@ struct mj_ctx {
   uint64_t rk_spans = 0;
   uint32_t rep_first[65] = {0};   // first record of every repetition
   uint64_t code_counts[256] = {0};   // input symbols by rank code
-  // A plain join by strings lists no candidates: mj_candidates_copy makes them
-  // on demand from the join's records, kept in cand_recs once mj_partition
-  // replaces recs.
-  bool cand_on_demand = false, cand_recs_kept = false;
+  // A plain join by strings makes no sorted list of its candidates:
+  // mj_candidates_copy sorts the join's own list where that holds them all
+  // (cand_listed), else lists them from the join's windows first (cand_pairs,
+  // cand_list), or from its records by the general path where memory is short
+  // for that.  The records are kept in cand_recs once mj_partition replaces recs.
+  bool cand_on_demand = false, cand_listed = false, cand_recs_kept = false;
   Derived cand_d;
-  uint64_t cand_n_part = 0;
-  uint32_t cand_n_str = 0;
+  PairArgs cand_pairs;
+  ListArgs cand_list;
+  uint64_t cand_n_part = 0, cand_count = 0;
+  uint32_t cand_n_str = 0, cand_widest = 0;
   Buf cand_recs;
   // bit-planes written by the partition kernel for the verifier
   mj_verify_config vcfg{MJ_VERIFY_KERNEL_AUTO, 0, 0, 0};
@@ -803,7 +807,7 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   const uint32_t nr = (uint32_t)c->n_part;
   c->n_cand = c->n_list = 0;
   c->cand_on_demand = true;
-  c->cand_recs_kept = false;
+  c->cand_listed = c->cand_recs_kept = false;
   c->cand_d = d;
   c->cand_n_part = nr;
   c->cand_n_str = n;
@@ -949,6 +953,11 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   c->list_bounded = true;
   c->stats.n_raw_pairs = c->h_small[1];
   c->n_cand = c->h_small[2];
+  c->cand_listed = c->n_list == c->n_cand;
+  c->cand_count = c->n_cand;
+  c->cand_pairs = a;
+  c->cand_list = l;
+  c->cand_widest = c->rk_widest;
   c->stats.n_candidates = c->n_cand;
   c->stats.band_cells = c->h_small[3];
   return MJ_OK;
@@ -1586,24 +1595,85 @@ int mj_candidates(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, u
   return MJ_OK;
 }
 
+// All candidates of a plain join by strings in cand_i/j, in any order: its pair
+// kernel again, without the bounds.
+static int relist_candidates(mj_ctx* c, cudaStream_t s) {
+  const uint64_t m = c->cand_count;
+  PairArgs a = c->cand_pairs;
+  ListArgs l = c->cand_list;
+  MJ_TRY(c->rk_list.reserve(m * 8, s));
+  MJ_TRY(c->cand_i.reserve(m * 4, s));
+  MJ_TRY(c->cand_j.reserve(m * 4, s));
+  a.min_sampled = l.min_sampled = ~0ull;
+  a.cap = l.in_cap = l.cap = m;
+  a.out = c->rk_list.as<uint2>();
+  l.in = a.out;
+  l.out_i = c->cand_i.as<uint32_t>();
+  l.out_j = c->cand_j.as<uint32_t>();
+  MJ_CUDA_TRY(cudaMemsetAsync(a.out_count, 0, 40, s));   // words 2 .. 6 of rk_cnt
+  MJ_TRY(launch_string_pairs(a, c->cand_widest, s));
+  MJ_TRY(launch_listed_pairs(l, s));
+  MJ_TRY(readback(c, a.out_count, 40, s));
+  if (c->h_small[0] != m || c->h_small[4] != m) return MJ_ERR_DEVICE;
+  c->cand_listed = true;
+  return MJ_OK;
+}
+
+// cand_i/j, all candidates, sorted.
+static int sort_candidates(mj_ctx* c, cudaStream_t s) {
+  const uint64_t m = c->cand_count;
+  const int nb = bits_for(c->cand_n_str - 1);
+  MJ_TRY(c->keys.reserve(m * 8, s));
+  MJ_TRY(c->keys_alt.reserve(m * 8, s));
+  MJ_TRY(c->sort_tmp.reserve(radix_temp_bytes(m), s));
+  MJ_TRY(launch_pack_pairs(c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(), m, nb, c->keys.as<uint64_t>(), s));
+  bool alt = false;
+  MJ_TRY(radix_sort_u64(c->keys.as<uint64_t>(), c->keys_alt.as<uint64_t>(), nullptr, nullptr, m, 0, 2 * nb,
+                        c->sort_tmp.p, &alt, s));
+  MJ_TRY(launch_unpack_pairs(alt ? c->keys_alt.as<uint64_t>() : c->keys.as<uint64_t>(), m, nb,
+                             c->cand_i.as<uint32_t>(), c->cand_j.as<uint32_t>(), s));
+  c->n_cand = m;
+  return MJ_OK;
+}
+
+// The sorted candidates of a plain join by strings, on s.
+static int demanded_candidates(mj_ctx* c, cudaStream_t s) {
+  int rc = c->cand_listed ? MJ_OK : relist_candidates(c, s);
+  if (rc == MJ_OK) rc = sort_candidates(c, s);
+  if (rc != MJ_ERR_OOM) return rc;
+  const mj_stats st = c->stats;
+  const Derived d = c->d;
+  const uint64_t n_part = c->n_part;
+  c->d = c->cand_d;
+  c->n_part = c->cand_n_part;
+  if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
+  c->timing = c->cand_listed = false;
+  rc = candidates(c, nullptr, nullptr, c->cand_n_str, 0, s);
+  if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
+  c->d = d;
+  c->n_part = n_part;
+  c->stats = st;
+  return rc;
+}
+
 int mj_candidates_copy(mj_ctx* c, uint32_t* d_i, uint32_t* d_j, void* stream) {
   if (!c) return MJ_ERR_ARG;
   if (!c->have_cand) return MJ_ERR_STATE;
   DeviceGuard g(c->device);
   cudaStream_t s = S(stream);
   if (c->cand_on_demand) {
-    const mj_stats st = c->stats;
-    const Derived d = c->d;
-    const uint64_t n_part = c->n_part;
-    c->d = c->cand_d;
-    c->n_part = c->cand_n_part;
-    if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
-    c->timing = false;
-    const int rc = candidates(c, nullptr, nullptr, c->cand_n_str, 0, s);
-    if (c->cand_recs_kept) std::swap(c->recs, c->cand_recs);
-    c->d = d;
-    c->n_part = n_part;
-    c->stats = st;
+    // the pass reads sizes back and may allocate, which a stream under capture
+    // cannot: there it runs on a stream of the context's, done before the copy
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (capturing) MJ_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    int rc = demanded_candidates(c, capturing ? c->aux[0] : s);
+    if (capturing) {
+      if (rc == MJ_OK && cudaStreamSynchronize(c->aux[0]) != cudaSuccess) rc = MJ_ERR_CUDA;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
     MJ_TRY(rc);
     c->cand_on_demand = false;
   }

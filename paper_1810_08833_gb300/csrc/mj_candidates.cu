@@ -704,6 +704,14 @@ __global__ void pack_pairs_kernel(const uint32_t* __restrict__ pi, const uint32_
   }
 }
 
+__global__ void unpack_pairs_kernel(const uint64_t* __restrict__ packed, uint64_t m, int nb, uint32_t* __restrict__ oi,
+                                    uint32_t* __restrict__ oj) {
+  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m; t += (uint64_t)gridDim.x * blockDim.x) {
+    oi[t] = (uint32_t)(packed[t] >> nb);
+    oj[t] = (uint32_t)(packed[t] & ((1ull << nb) - 1));
+  }
+}
+
 // Up to three arrays of n words copied by one launch (three copies cost the host
 // about 5 us each); null outputs are skipped.
 __global__ void copy_words_kernel(const uint32_t* __restrict__ a, const uint32_t* __restrict__ b,
@@ -948,6 +956,13 @@ int launch_pack_records(const uint32_t* sid, const uint32_t* pos, const uint32_t
 int launch_pack_pairs(const uint32_t* pi, const uint32_t* pj, uint64_t m, int nb, uint64_t* out, cudaStream_t s) {
   if (!m) return MJ_OK;
   pack_pairs_kernel<<<grid_for(m), 256, 0, s>>>(pi, pj, m, nb, out);
+  MJ_KERNEL_DONE();
+  return MJ_OK;
+}
+
+int launch_unpack_pairs(const uint64_t* packed, uint64_t m, int nb, uint32_t* oi, uint32_t* oj, cudaStream_t s) {
+  if (!m) return MJ_OK;
+  unpack_pairs_kernel<<<grid_for(m), 256, 0, s>>>(packed, m, nb, oi, oj);
   MJ_KERNEL_DONE();
   return MJ_OK;
 }

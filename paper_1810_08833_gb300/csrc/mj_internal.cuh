@@ -323,6 +323,7 @@ int launch_key_check(const PRec* r, const uint8_t* bytes, const int64_t* offsets
 int launch_pack_records(const uint32_t* sid, const uint32_t* pos, const uint32_t* len, const uint64_t* key,
                         const uint32_t* slen, uint64_t n, PRec* out, cudaStream_t s);
 int launch_pack_pairs(const uint32_t* pi, const uint32_t* pj, uint64_t m, int nb, uint64_t* out, cudaStream_t s);
+int launch_unpack_pairs(const uint64_t* packed, uint64_t m, int nb, uint32_t* oi, uint32_t* oj, cudaStream_t s);
 // a7: unique of sorted u64 pairs -> flags; then compaction.
 int launch_unique_flags(const uint64_t* sorted, uint64_t n, uint32_t* flags, cudaStream_t s);
 // run_start (nullable): run_start[u] = index of candidate u's first raw pair

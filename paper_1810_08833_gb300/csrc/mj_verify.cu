@@ -147,6 +147,11 @@ int launch_wp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long*
   // per SM to hide the recurrence's latency
   const uint64_t per_sm_pairs = (a.m + 3ull * 128 * sms - 1) / (3ull * 128 * sms);
   per_sm = (int)std::min<uint64_t>((uint64_t)per_sm, std::max<uint64_t>(3, per_sm_pairs));
+  // Two planes leave registers for 6 blocks at bands of up to 4 words, but a sixth
+  // only makes the lanes' rows push each other out of L1: 341,509 pairs of 5,000
+  // reads at K = 102 2.63 ms with 6, 2.49 with 5; 700,000 4.34 and 4.19, at K = 60
+  // 2.06 and 1.98.
+  if (P == 2) per_sm = std::min(per_sm, 5);
   if (per_sm < 1) per_sm = 1;
   uint64_t need = (a.m + 127) / 128;
   uint64_t grid = (uint64_t)sms * per_sm;

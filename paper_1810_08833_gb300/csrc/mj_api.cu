@@ -1060,10 +1060,13 @@ int verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const ui
 // branges words [0, 32), [start, end) ranges in words [32, 96).
 constexpr size_t kOrderScratchAt = 128;   // words of branges before the ordering scratch
 // Pairs from which a list is verified longest first: more than are in flight at
-// once, on two lanes each (launch_verify: three blocks of 128 lanes per SM; 29,184
-// pairs on 152 SMs) or on a warp and more.
-uint64_t order_from(const mj_ctx* c) { return 3ull * 128 * c->sms / 2; }
-constexpr uint64_t kOrderFromWide = 1024;
+// once.  On two lanes each (launch_verify) three blocks of 128 lanes per SM are
+// (29,184 pairs on 152 SMs), of wider bands a warp per scheduler (608; bands of a
+// CTA each, one per SM): 1,000 pairs of 20,000 to 60,000 bases in the given order
+// 4.67 ms at K = 1000 and 9.84 at K = 7900, longest first 4.06 and 6.98.
+uint64_t order_from(const mj_ctx* c, uint32_t K) {
+  return K <= 255 ? 3ull * 128 * c->sms / 2 : wave_in_flight(K, c->sms);
+}
 constexpr size_t kOrderKeptAt = 100;      // word of branges with the number of pairs in the order
 
 // The lower bounds (mj_pairs.cu) on a list of m pairs cost a pass over the
@@ -1073,7 +1076,7 @@ constexpr size_t kOrderKeptAt = 100;      // word of branges with the number of 
 // and passes over small inputs take, even if they reject it all (7,070 pairs of
 // 500 symbols at K <= 5: 104 us with them, 69 without; 341,509 pairs of 870 reads,
 // a quarter of them unrelated: 2.69 ms with, 2.60 without).  Learned joins, where
-// a rejected pair also spares the network, take them from order_from on.
+// a rejected pair also spares the network, take them from order_from pairs on.
 // A list that was made under the bounds needs them no more, and a band that
 // the verifier refuses must leave the results unwritten.
 constexpr uint64_t kBoundsFromPairs = 1u << 20;
@@ -1156,7 +1159,7 @@ int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, 
     MJ_TRY(pair_bounds(c, d_offsets, ci, cj, nullptr, m, K, ed, s));
   }
   // few enough pairs to be in flight all at once run in the given order
-  if (!bounds && !c->want_cells && m <= (K <= 255 ? order_from(c) : kOrderFromWide) && (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned))
+  if (!bounds && !c->want_cells && m <= order_from(c, K) && (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned))
     return verify(c, d_bytes, d_offsets, ci, cj, nullptr, m, K, K, ed, s);
   MJ_TRY(pair_order(c, ci, cj, d_offsets, m, bounds ? c->rejected.as<uint8_t>() : nullptr, &order, &kept, s));
   if (c->vcfg.kernel != MJ_VERIFY_KERNEL_TUNED || !c->tuned)
@@ -1294,7 +1297,7 @@ int verify_stage(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, ui
     if (!c->band_ready) return MJ_ERR_STATE;
     MJ_TRY(order_buffers(c, m, s));
     const uint32_t *order, *kept;
-    const bool bounds = bounds_pay(c, m, K, 256, order_from(c));   // a rejected pair also spares the network
+    const bool bounds = bounds_pay(c, m, K, 256, order_from(c, 255));   // a rejected pair also spares the network
     if (bounds) {
       MJ_TRY(bounds_buffers(c, m, s));
       MJ_TRY(ensure_planes(c, d_bytes, K, s));

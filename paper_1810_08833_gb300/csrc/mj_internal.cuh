@@ -391,6 +391,8 @@ int launch_verify_wave(const VerifyArgs& a, uint64_t plane_words, uint32_t guard
 // the number of pairs
 int launch_verify_wave_auto(const VerifyArgs& a, uint64_t plane_words, uint32_t guard_words, uint32_t kmax,
                             unsigned long long* next, cudaStream_t s);
+// pairs of bands up to kmax that such a launch has in flight from its start on
+uint64_t wave_in_flight(uint32_t kmax, int sms);
 int wave_lanes_for(uint32_t kmax);
 // whether launch_verify takes bands up to kmax with this kernel choice
 bool verify_supported(uint32_t kmax, int kernel, int lanes);

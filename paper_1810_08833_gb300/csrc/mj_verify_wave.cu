@@ -720,6 +720,11 @@ const WaveShape kWaveShapes[] = {
     {32, 4, launch_gv<32, 4>}, {32, 6, launch_gv<32, 6>}, {32, 8, launch_gv<32, 8>},
 };
 
+bool shape_holds(const WaveShape& w, uint32_t kmax) {
+  const int R = 32 * w.V, width = std::max<int>((int)kmax + 1, 64);
+  return (width + R - 2) / (R + 1) + 1 <= w.G;
+}
+
 template <int V, int P>
 int launch_vp(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* next, cudaStream_t s) {
   int dev = 0, sms = kNumSMsHint, per_sm = 1;
@@ -762,13 +767,11 @@ int launch_verify_wave_auto(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint3
   int dev = 0, sms = kNumSMsHint;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int width = std::max<int>((int)kmax + 1, 64);
   const WaveShape* best = nullptr;
   double least = 0;
   for (const WaveShape& w : kWaveShapes) {
-    const int R = 32 * w.V;
     // the last block reads up to V words beyond the string: the guard holds them
-    if ((width + R - 2) / (R + 1) + 1 > w.G || (int)GW <= w.V) continue;
+    if (!shape_holds(w, kmax) || (int)GW <= w.V) continue;
     const double work = 0.3 * (24 + 20 * w.V) * ((double)a.m * w.G / 32 / (4.0 * sms)), longest = 100 + 12 * w.V;
     const double t = std::sqrt(work) + std::sqrt(longest);
     if (!best || t < least) {
@@ -777,6 +780,12 @@ int launch_verify_wave_auto(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint3
     }
   }
   return best ? best->launch(a, PW, GW, next, s) : launch_verify_wave(a, PW, GW, cta_lanes_for(kmax), next, s);
+}
+
+uint64_t wave_in_flight(uint32_t kmax, int sms) {
+  for (const WaveShape& w : kWaveShapes)
+    if (shape_holds(w, kmax)) return 4ull * sms;
+  return (uint64_t)sms;
 }
 
 int launch_verify_wave(const VerifyArgs& a, uint64_t PW, uint32_t GW, int lanes, unsigned long long* next,

@@ -762,6 +762,12 @@ int launch_v(const VerifyArgs& a, uint64_t PW, uint32_t GW, unsigned long long* 
 // pair) and all resident blocks: K = 1000, the band of 2,000 x 10 long noisy
 // reads' join: 46.8 -> 31.2 ms; K = 4000, 3,000 pairs: 5.6 -> 2.7 ms; K = 1900
 // and 12,000 pairs: 8.4 -> 5.4 ms.
+// Codes of more than two planes compare eight, zero or not, with several words
+// per lane, and five or eight with one.  10 pairs of 8,000 to 20,000 symbols of
+// protein, alone: 1 word (K = 1000) 1.40 ms, 2 (1500) 1.44, 3 (2500) 1.64, 4 (4000)
+// 1.81, 6 (5000) 2.42, 8 (7900) 2.93; a CTA per pair 1.55 (1500), 1.56 (2500), 1.60
+// (4000), 1.93 (5000), 1.92 (7900).  Two planes, 20,000 to 60,000 bases: 4 words
+// (4000) 3.52, 6 (5000) 4.38, 8 (7900) 5.26; a CTA 4.04, 4.55, 4.55.
 int launch_verify_wave_auto(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint32_t kmax, unsigned long long* next,
                             cudaStream_t s) {
   int dev = 0, sms = kNumSMsHint;
@@ -779,6 +785,9 @@ int launch_verify_wave_auto(const VerifyArgs& a, uint64_t PW, uint32_t GW, uint3
       least = t;
     }
   }
+  // At most a pair per SM: every pair runs alone either way, and a CTA's warps
+  // take less than the steps of many words (see above).
+  if (best && a.m <= (uint64_t)sms && best->V > (a.bits <= 2 ? 6 : 2)) best = nullptr;
   return best ? best->launch(a, PW, GW, next, s) : launch_verify_wave(a, PW, GW, cta_lanes_for(kmax), next, s);
 }
 

@@ -48,8 +48,14 @@ extern "C" {
 #define MJ_FLAG_FIRST_PASS 32u   /* learned mode: run the first passes however few pairs they hold (by default
                                     they run only with at least 384 pairs per SM, below which their latency
                                     exceeds what they save, and every pair goes to band K) */
-/* Deduplication of the candidate pairs (last step of Alg. 3's join).  By
- * default the library picks per call: a bitmap with one bit per pair i < j
+/* Deduplication of the candidate pairs (last step of Alg. 3's join).  Plain
+ * joins go string by string by default: the strings are ranked by length, and
+ * every string's candidates are a small bitmap over the ranks within K of its
+ * own.  They take the path below with one of these flags, with
+ * MJ_FLAG_KEY_CHECK or MJ_FLAG_FEATURES, where very many strings of about one
+ * length have few candidates, and where device memory is short for their
+ * buffers.  mj_candidates and learned joins always do.  There the library picks
+ * per call: a bitmap with one bit per pair i < j
  * (n^2/16 bytes, cleared, set by every raw pair, then compacted row by row
  * into the sorted list) when sweeping it costs less than sorting the raw
  * pairs and it fits in device memory, else a radix sort of the raw pairs.
@@ -66,23 +72,29 @@ extern "C" {
 /* verification kernels (mj_verify_config.kernel) */
 #define MJ_VERIFY_KERNEL_AUTO 0       /* diagonal for K <= 255, wavefront above */
 #define MJ_VERIFY_KERNEL_DIAGONAL 1   /* one thread per pair, band as ceil((K+1)/32) words */
-#define MJ_VERIFY_KERNEL_WAVEFRONT 2  /* G lanes per pair, 32-row blocks, skewed wavefront: within one warp up
-                                         to 32 lanes, one CTA of several warps from 64 to 1,024 lanes */
+#define MJ_VERIFY_KERNEL_WAVEFRONT 2  /* G lanes per pair, blocks of 32 rows per word that a lane holds, skewed
+                                         wavefront: within one warp up to 32 lanes, one CTA of several warps
+                                         from 64 to 1,024 lanes */
 #define MJ_VERIFY_KERNEL_TUNED 3      /* per length bucket, as chosen by mj_autotune_verify */
 
 typedef struct mj_ctx mj_ctx;
 
 /* Choice of verification kernel for a context (used by mj_verify and mj_join).
- * Pairs are verified longest first; with MJ_VERIFY_KERNEL_TUNED each length
+ * Lists of more pairs than are in flight at once are verified longest first,
+ * shorter ones in the given order; with MJ_VERIFY_KERNEL_TUNED each length
  * bucket (floor(log2) of the shorter length) uses the kernel the autotuner
  * picked for it.
  *  kernel    MJ_VERIFY_KERNEL_*.
  *  lanes     wavefront only: lanes per pair, 2, 4, 8, 16 or 32 (one warp) or
  *            64, 128, 256, 512 or 1024 (one CTA per pair, its warps handing
- *            block boundaries over through shared memory); 0 = the fewest that
- *            hold the band: one warp holds bands up to K = 1,024, a CTA of G
- *            lanes bands with 34 G >= K + 32 (K up to 34,784 with 1,024).  Too
- *            few lanes for a band is MJ_ERR_UNSUPPORTED.
+ *            block boundaries over through shared memory), each with one word
+ *            (32 rows) per block: one warp then holds bands up to K = 1,024, a
+ *            CTA of G lanes bands with 34 G >= K + 32 (K up to 34,784 with
+ *            1,024), and too few lanes for a band is MJ_ERR_UNSUPPORTED.
+ *            0 = the library's choice by the band, the number of pairs and the
+ *            alphabet: one warp's lanes with blocks of 1 to 8 words for bands
+ *            up to K = 7,968, a CTA above, and below for lists of at most a
+ *            pair per SM where a lane would hold many words.
  *  batching  TUNED only: 0 = one persistent launch per run of consecutive
  *            buckets that share a kernel; 1 = one launch per length bucket.
  *  graph     1 = capture the plain verification stage (ordering, bucketing,
@@ -100,7 +112,9 @@ typedef struct {
 /* Result of mj_autotune_verify, per length bucket b (shorter length in
  * [2^b, 2^(b+1))): pairs seen, the kernel and lanes chosen, and the time of
  * every candidate tried on the bucket's sample (candidates: diagonal when
- * K <= 255, then the wavefront with 2^c times the fewest lanes). */
+ * K <= 255, then the wavefront with 2^c times the fewest lanes that hold the
+ * band with one word each; the fewest stand for the library's own choice of
+ * lanes and words). */
 #define MJ_TUNE_CANDIDATES 6
 typedef struct {
   uint32_t count[32];
@@ -175,10 +189,13 @@ typedef struct {
   uint64_t n_launches;         /* kernels the library launched during the call */
   /* device time (CUDA events on the call's stream) of the sections of the
    * last mj_join, in this order: 0 anchor test (Alg. 2), 1 partition
-   * records from the anchors (Alg. 1), 2 record grouping sort, 3 pair emission
-   * (filters of Alg. 3), 4 pair dedup, 5 equality bit-planes, 6 verification
-   * kernel(s), 7 output compaction, 8 the candidates' longest-first order for
-   * verification (a counting sort) */
+   * records from the anchors (Alg. 1), 2 record grouping sort (joins by strings:
+   * with the windows of every record), 3 pair emission (filters of Alg. 3; 0 in
+   * joins by strings), 4 pair dedup (joins by strings: the pairs of every string
+   * with the filters, the dedup and the lower bounds), 5 equality bit-planes, 6
+   * verification kernel(s), 7 output compaction, 8 the candidates' longest-first
+   * order for verification (a counting sort; 0 for lists that keep their order).
+   * A section runs from its first start to its last end in the call. */
   float ms_section[9];
   uint64_t verify_word_columns; /* 32-bit band words x columns the verifier advanced */
 } mj_stats;
@@ -223,7 +240,15 @@ int mj_partition_copy(mj_ctx* ctx, uint32_t* d_sid, uint32_t* d_pos, uint32_t* d
                       uint64_t* d_key, void* stream);
 
 /* Steps a2-a7 (Alg. 3's hash join): the deduplicated candidate set C.
- * *count receives |C|; mj_candidates_copy writes the pairs (i < j) sorted. */
+ * *count receives |C|; mj_candidates_copy writes the pairs (i < j) sorted.
+ * After mj_candidates, mj_candidates_records, mj_pairs_unique and joins by the
+ * general path it only queues copies.  A plain join by strings (see the dedup
+ * flags) counts its candidates and lists those that it verifies: the first
+ * mj_candidates_copy after it sorts that list, or lists all candidates first
+ * where the join's lower bounds left some out.  That pass allocates device
+ * memory, synchronises `stream`, and may return MJ_ERR_OOM (a later call tries
+ * again); its time and launches are in no mj_stats.  Under stream capture it
+ * runs at once on a stream of the context, and the copies are captured. */
 int mj_candidates(mj_ctx* ctx, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_t n,
                   const mj_params* p, const uint64_t* d_qgram_table, void* stream, uint64_t* count);
 int mj_candidates_copy(mj_ctx* ctx, uint32_t* d_i, uint32_t* d_j, void* stream);
@@ -267,7 +292,7 @@ int mj_pairs_unique(mj_ctx* ctx, const uint32_t* d_i, const uint32_t* d_j, uint6
  * where k_t = d_k[t] if d_k is non-null, else K.  Any pair of strings is
  * allowed (equal ids, empty strings).  Stream-ordered; does not synchronise.
  * Rank codes are derived from the n strings given.  Bands: the diagonal
- * kernel holds K <= 255, one warp's wavefront K <= 1,024 and a CTA's up to
+ * kernel holds K <= 255, one warp's wavefront K <= 7,968 and a CTA's up to
  * K = 34,784 (lanes of mj_verify_config); a wider band (or K >= 65,536)
  * returns MJ_ERR_UNSUPPORTED and writes nothing.  A pair id >= n yields
  * k_t + 1 and sets bit 0 of the context's device flags: mj_device_flags

@@ -806,8 +806,7 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   const Derived& d = c->d;
   const uint32_t nr = (uint32_t)c->n_part;
   c->n_cand = c->n_list = 0;
-  c->cand_on_demand = true;
-  c->cand_listed = c->cand_recs_kept = false;
+  c->cand_recs_kept = false;
   c->cand_d = d;
   c->cand_n_part = nr;
   c->cand_n_str = n;
@@ -953,6 +952,7 @@ int string_candidates(mj_ctx* c, const int64_t* d_offsets, uint32_t n, cudaStrea
   c->list_bounded = true;
   c->stats.n_raw_pairs = c->h_small[1];
   c->n_cand = c->h_small[2];
+  c->cand_on_demand = true;
   c->cand_listed = c->n_list == c->n_cand;
   c->cand_count = c->n_cand;
   c->cand_pairs = a;
@@ -1148,7 +1148,8 @@ int order_buffers(mj_ctx* c, uint64_t m, cudaStream_t s) {
   return MJ_OK;
 }
 
-// Band-K verification of pairs (ci, cj) in longest-first order, as the
+// Band-K verification of pairs (ci, cj), longest first where they are more than
+// are in flight at once (or their cells are wanted), as the
 // context's kernel choice says (TUNED: per length bucket, batched).
 int verify_ordered(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, const uint32_t* ci,
                    const uint32_t* cj, uint64_t m, uint32_t K, uint32_t* ed, cudaStream_t s) {
@@ -1813,7 +1814,7 @@ int mj_verify(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint3
   begin_call(c, false);
   MJ_TRY(derive(c, d_bytes, d_offsets, n, &p, s));
   if (!d_k) {
-    // one band for every pair: longest first, with the context's kernel plan
+    // one band for every pair, with the context's kernel plan
     if (m) MJ_TRY(verify_ordered_graph(c, d_bytes, d_offsets, d_i, d_j, m, K, d_ed, s));
   } else {
     // the widest per-pair band sizes the kernel (a device reduction, 4 bytes read back)
@@ -1944,11 +1945,14 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
   // Plain joins go string by string.  The general path (one walk over all
   // records, dedup by a bitmap over all pairs or a sort) serves learned mode
   // and the candidates' features (they need multiplicities), the key check, a
-  // forced dedup, and windows too wide for a bitmap in shared memory.  Measured
-  // (general, by strings; us per join): 1,000 short reads 428, 410; 10,000 reads
-  // 1603, 1674; 6,000 text-like strings 1266, 850; 20,000 protein-like 1086,
-  // 1004; 10,000 of bytes, with hardly an unrelated candidate, 1018, 1145.  How
-  // many candidates there are is not known before the records are grouped.
+  // forced dedup, wide windows with few candidates (string_pairs_from) and
+  // windows too wide for a bitmap in shared memory.  Measured (by strings,
+  // general with the better dedup; us per join): 1,000 short reads 351, 382;
+  // 10,000 reads 1593, 1555; 50,000 reads 4147, 4117; 6,000 text-like strings
+  // 739, 1081; 20,000 protein-like 955, 1014; 10,000 of bytes, with hardly an
+  // unrelated candidate, 897, 782; 300,000 text-like 20.8, 56.6 ms; 400,000
+  // protein-like 13.7, 29.8.  How many candidates there are is not known before
+  // the records are grouped.
   const uint32_t general = MJ_FLAG_FEATURES | MJ_FLAG_KEY_CHECK | MJ_FLAG_DEDUP_SORT | MJ_FLAG_DEDUP_BITMAP;
   c->by_strings = p->verify_mode == MJ_VERIFY_PLAIN && !(p->flags & general) && p->K > 0 && n > 1;
   // Where device memory is short for it, the general path, which needs less (and
@@ -1971,7 +1975,6 @@ int mj_join(mj_ctx* c, const uint8_t* d_bytes, const int64_t* d_offsets, uint32_
   }
   strings = strings && c->by_strings;
   if (!strings) {
-    c->cand_on_demand = false;
     MJ_TRY(candidates(c, d_bytes, d_offsets, n, p->flags, s,
                       p->verify_mode == MJ_VERIFY_LEARNED || (p->flags & MJ_FLAG_FEATURES)));
     c->n_list = c->n_cand;

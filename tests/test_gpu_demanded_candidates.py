@@ -112,3 +112,22 @@ def test_allocation_failures(name):
     finally:
         lib.mj_inject_alloc_failure(0)
     assert 0 in statuses
+
+
+def test_no_candidates_after_a_join_with_some():
+    """Empty strings have no records and no candidates, whatever was joined before."""
+    import paper_1810_08833_gb300 as mj
+    import torch
+    lib = mj.library()
+    s = _sets()["bounded"]
+    data, off = to_device(s)
+    empty = torch.zeros(3, dtype=torch.int64, device="cuda")
+    with mj.Context(0) as ctx:
+        ctx.join(data, off, mj.params(s.K, T=s.T))
+        assert ctx.join(data[:0], empty, mj.params(s.K, T=s.T))[0].shape[0] == 0
+        assert ctx.stats()["n_candidates"] == 0
+        out = torch.full((64,), -1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        assert lib.mj_candidates_copy(ctypes.c_void_p(ctx._h.value), out.data_ptr(), out.data_ptr(), None) == 0
+        torch.cuda.synchronize()
+        assert (out == -1).all()
